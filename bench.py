@@ -439,7 +439,7 @@ class Bench:
         st = self.cache.status()
         if st != 0:
             raise RuntimeError(f"cache build failed: status {st}")
-        self.prebuild_launches = 2 * self.prebuild_calls + 1  # + the status kernel
+        self.prebuild_launches = self.prebuild_calls + 1  # + the status kernel
         print(f"prebuild_launches={self.prebuild_launches}", file=sys.stderr, flush=True)
         self.steps = [self._stage(i) for i in range(self.total_steps)]
 

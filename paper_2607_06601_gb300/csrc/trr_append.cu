@@ -1,14 +1,11 @@
 // trr_append.cu - trr_kv_append: quantise-on-write into the width-class page pools.
 //
-// Calls of up to 256 entries (decode steps) run as one kernel, append_fused_kernel
-// (below); larger ones as two:
-//   append_plan_kernel   one CTA, one thread per entry.  Validates every entry, ranks
-//                        it among the earlier entries of its (sequence, class), hands
-//                        out page ids in entry order, and commits the metadata only
-//                        when the whole call is valid (Sec. 3.8: each token's KV is
-//                        stored at its chosen width in a paged cache).
-//   append_write_kernel  one thread per (entry, KV head, K|V, group): the quantiser
-//                        Q_b of Sec. 3.2(C), Eq. 4, or a bf16 copy for b = 16.
+// One kernel, append_kernel (below), for calls of up to 1024 entries: validates every
+// entry, ranks it among the earlier entries of its (sequence, class), hands out page ids in
+// entry order, quantises the rows (Q_b of Sec. 3.2(C), Eq. 4, or a bf16 copy for b = 16)
+// and commits the metadata only when the whole call is valid (Sec. 3.8: each token's KV is
+// stored at its chosen width in a paged cache).
+#include <algorithm>
 #include <climits>
 
 #include "trr_internal.cuh"
@@ -53,325 +50,227 @@ __device__ __forceinline__ int entry_bits(const uint8_t* bits, const float* bit_
   return bit_logits ? 2 << hard_decision<4>(bit_logits + 4 * e) : bits[e];
 }
 
-__global__ void __launch_bounds__(1024) append_plan_kernel(LayerArgs a, int n, const int32_t* __restrict__ seq_ids,
-                                                           const int32_t* __restrict__ positions,
-                                                           const uint8_t* __restrict__ bits,
-                                                           const uint8_t* __restrict__ modes,
-                                                           const float* __restrict__ bit_logits,
-                                                           const float* __restrict__ mode_logits) {
-  __shared__ int s_seq[1024];
-  __shared__ int s_pos[1024];
-  __shared__ int s_cls[1024];   // width class when the entry stores KV, else -1
-  __shared__ int s_open[1024];  // class of the page the entry opens, else -1
-  __shared__ int s_first_err;
-  __shared__ int s_nopen[kClasses];
+// Entries of the small instance: a decode step's calls plan with 256 threads, larger ones
+// with 1024.  The instance is chosen by n alone.
+constexpr int kSmallAppend = 256;
 
-  pdl_wait();
-  pdl_trigger();
-  const int e = threadIdx.x;
-  const bool act = e < n;
-  int seq = -1, pos = 0, c = -1, err = 0;
-  bool writes = false;
-  if (act) {
-    seq = seq_ids[e];
-    pos = positions[e];
-    const int m = entry_mode(a, modes, mode_logits, e);
-    if (seq < 0 || seq >= a.S) {
-      err = TRR_ERR_INVALID_ARG;
-    } else {
-      c = class_of_bits(entry_bits(bits, bit_logits, e));
-      if (c < 0 || m > TRR_MODE_FULL) err = TRR_ERR_INVALID_ARG;
-      else if (pos < 0 || pos >= a.maxctx) err = TRR_ERR_BAD_POSITION;
-    }
-    writes = !err && (m != TRR_MODE_SKIP || a.skip_writes_kv);
-  }
-  s_seq[e] = (act && seq >= 0 && seq < a.S) ? seq : -1;
-  s_pos[e] = pos;
-  s_cls[e] = writes ? c : -1;
-  if (e == 0) s_first_err = INT_MAX;
-  if (e < kClasses) s_nopen[e] = 0;
-  __syncthreads();
+// Per-entry facts of a call, indexed by entry, that every CTA works out for itself.
+template <int T>
+struct AppendShared {
+  unsigned long long prefix[T];  // inclusive counts of the four classes' tokens in sorted order (16 bits each)
+  unsigned long long wsum[32], wmax[32], wopen[32];  // per warp (the rest zero): see the prefix passes
+  uint32_t key[T];  // sequence << 10 | entry, sorted
+  int pos[T];       // position; later the page that the list slot's token opens
+  int cls[T];       // width class when the entry stores KV, else -1
+  int tok[T];       // token index in its (sequence, class) list
+  int pid[T];       // page of the token
+  int end[T];       // by first sorted index of a sequence: its last one
+  int whead[32];
+  int next[kClasses];
+  int first_err, last;
+};
 
-  // Earlier entries of the same sequence: the largest position and, per class, how
-  // many store KV.  Later ones: whether this entry is the sequence's / class's last.
-  int prev_max = -1, rank = 0;
-  bool later_seq = false, later_cls = false;
-  if (act && s_seq[e] >= 0) {
-    for (int j = 0; j < n; ++j) {
-      if (s_seq[j] != seq) continue;
-      if (j < e) {
-        prev_max = max(prev_max, s_pos[j]);
-        rank += (writes && s_cls[j] == c);
-      } else if (j > e) {
-        later_seq = true;
-        later_cls |= (writes && s_cls[j] == c);
+// Sorts the T keys (one per thread, all distinct) ascending: bitonic, exchanges inside a
+// warp by shuffles.
+template <int T>
+__device__ __forceinline__ uint32_t sort_keys(uint32_t key, uint32_t* sh) {
+  const int i = threadIdx.x;
+#pragma unroll 1
+  for (int k = 2; k <= T; k <<= 1) {
+#pragma unroll 1
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      uint32_t other;
+      if (j >= 32) {
+        sh[i] = key;
+        __syncthreads();
+        other = sh[i ^ j];
+        __syncthreads();
+      } else {
+        other = __shfl_xor_sync(0xffffffffu, key, j);
       }
+      const bool low = (i & j) == 0, up = (i & k) == 0;
+      key = low == up ? min(key, other) : max(key, other);
     }
   }
-  int k = 0, slot = 0, kidx = 0;
-  bool opens = false;
-  if (act && !err && pos <= max(prev_max, a.last_pos[seq])) err = TRR_ERR_BAD_POSITION;
-  if (act && !err && writes) {
-    k = a.ntok[seq * 4 + c] + rank;
-    slot = k % a.P;
-    kidx = k / a.P;
-    opens = slot == 0;
-  }
-  s_open[e] = opens ? c : -1;
-  __syncthreads();
-
-  int pid = -1;
-  if (opens) {  // page ids in entry order: next_page + openers of this class before e
-    int before = 0;
-    for (int j = 0; j < e; ++j) before += (s_open[j] == c);
-    pid = a.ctrl[kNextPage + c] + before;
-    if (pid >= a.cap[c]) err = TRR_ERR_OUT_OF_PAGES;
-  }
-  if (act && err) atomicMin(&s_first_err, e);
-  __syncthreads();
-  if (s_first_err != INT_MAX) {  // the call is a no-op; record the lowest failing entry
-    if (e == s_first_err) set_status(a.ctrl, err);
-    if (e == 0) a.ctrl[kAppendOk] = 0;
-    return;
-  }
-
-  // Commit.  Openers first, so that later entries of the same page can read its id.
-  const int64_t row = (static_cast<int64_t>(seq) * 4 + c) * a.MP + kidx;
-  if (opens) {
-    a.pt[row] = pid;
-    a.pfirst[row] = pos;
-    atomicAdd(&s_nopen[c], 1);
-    if (a.head_modes)  // a new page starts with every presence bit (and the padding) clear
-      for (int j = 0; j < a.Hkv; ++j) {
-        head_mask(a, c, pid, j)[0] = 0ull;
-        head_mask(a, c, pid, j)[1] = 0ull;
-      }
-  }
-  __syncthreads();
-  if (act) {
-    AppendPlan p{-1, 0, 0, pos};
-    if (writes) {
-      if (!opens) pid = a.pt[row];
-      p.page = pid;
-      p.slot = slot;
-      p.cls = c;
-      if (!later_cls || slot == a.P - 1) a.plast[row] = pos;
-      if (!later_cls) {
-        a.ntok[seq * 4 + c] = k + 1;
-        a.lastpg[seq * 4 + c] = pid;
-      }
-      reinterpret_cast<int32_t*>(a.pool[c] + pid * a.page_bytes[c])[slot] = pos;
-      atomicOr(&a.presence[static_cast<int64_t>(seq) * a.W32 + pos / 32], 1u << (pos % 32));
-      if (a.head_modes)  // the slot's bit for every KV head the entry stores
-        for (int j = 0; j < a.Hkv; ++j)
-          if (head_stores(a, modes, e, j)) atomicOr(head_mask(a, c, pid, j), 1ull << slot);
-    }
-    a.aplan[e] = p;
-    if (!later_seq) a.last_pos[seq] = pos;
-  }
-  __syncthreads();
-  if (e < kClasses) a.ctrl[kNextPage + e] += s_nopen[e];
-  if (e == 0) a.ctrl[kAppendOk] = 1;
+  return key;
 }
 
-// Eq. 4 on 32 consecutive values (one chunk of a group): codes packed LSB-first.
-template <int B>
-__device__ __forceinline__ void quantise_chunk(const uint4* src, float z, float s, float rs, uint8_t* sl, int64_t off,
-                                               bool sw) {
-  constexpr int levels = (1 << B) - 1;
-  constexpr int per_word = 32 / B;
-  uint32_t words[B];
-#pragma unroll
-  for (int w = 0; w < B; ++w) words[w] = 0;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const uint4 u = src[q];
-    const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int h = 0; h < 8; ++h) {
-      const float x = (h & 1) ? bf16hi(wv[h >> 1]) : bf16lo(wv[h >> 1]);
-      const int code = s != 0.f ? code_of(x, z, s, rs, levels) : 0;
-      const int j = q * 8 + h;
-      words[j / per_word] |= static_cast<uint32_t>(code) << ((j % per_word) * B);
-    }
-  }
-#pragma unroll
-  for (int w = 0; w < B; ++w) {  // word w at byte off + 4 w of the slice (swizzled: sw)
-    const int64_t o = off + 4 * w;
-    *reinterpret_cast<uint32_t*>(sl + (sw ? swz_off(o) : o)) = words[w];
-  }
+// The warp's sum of four 16-bit counts (each sum below 65536).
+__device__ __forceinline__ unsigned long long add_packed(unsigned long long x) {
+  const uint32_t lo = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(x));
+  const uint32_t hi = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(x >> 32));
+  return static_cast<unsigned long long>(hi) << 32 | lo;
 }
 
-__global__ void __launch_bounds__(256) append_write_kernel(LayerArgs a, int n, const uint16_t* __restrict__ k,
-                                                           const uint16_t* __restrict__ v) {
-  pdl_wait();
-  pdl_trigger();
-  if (a.ctrl[kAppendOk] == 0) return;
-  const int ng = a.d / a.G;
-  const int per_entry = a.Hkv * 2 * ng;
-  const int64_t gid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (gid >= static_cast<int64_t>(n) * per_entry) return;
-  const int e = static_cast<int>(gid / per_entry);
-  const int r = static_cast<int>(gid % per_entry);
-  const int h = r / (2 * ng);
-  const int which = (r / ng) & 1;  // 0 = K, 1 = V
-  const int g = r % ng;
-  const AppendPlan p = a.aplan[e];
-  if (p.page < 0) return;
-  const int b = bits_of_class(p.cls);
-  const uint16_t* src = (which ? v : k) + (static_cast<int64_t>(e) * a.Hkv + h) * a.d + g * a.G;
-  uint8_t* sl = a.pool[p.cls] + p.page * a.page_bytes[p.cls] + a.hdr + static_cast<int64_t>(h) * a.slice[p.cls];
-  const uint4* s4 = reinterpret_cast<const uint4*>(src);
-  if (b == 16) {  // native precision: copy the bf16 bits, 16 bytes (one chunk) at a time
-    const int64_t off = static_cast<int64_t>(which) * a.P * a.d * 2 + static_cast<int64_t>(p.slot) * a.d * 2 + g * a.G * 2;
-    for (int i = 0; i < a.G / 8; ++i) {
-      const int64_t o = off + 16 * i;
-      *reinterpret_cast<uint4*>(sl + (a.swz ? swz_off(o) : o)) = s4[i];
-    }
-    return;
-  }
-  // min / max of the group; values binary16 cannot carry make the group all zeros
-  float mn = __int_as_float(0x7f800000), mx = -mn;
-  bool bad = false;
-  for (int i = 0; i < a.G / 8; ++i) {
-    const uint4 u = s4[i];
-    const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
+// 8 consecutive values of a row (raw, bf16) by one lane of the G/8 that hold the group:
+// Eq. 4 at b < 16 bits, the 8 codes packed LSB-first into `codes`, (s, z) into `sz`.  A
+// group holding a value binary16 cannot carry (non-finite or |x| > 65504) gets zeros and
+// bad = true.  Every lane of the warp calls it.
+__device__ __forceinline__ void quantise_8(const uint4 raw, int b, int GL, unsigned long long& codes, uint32_t& sz,
+                                           bool& bad) {
+  const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+  float x[8];
 #pragma unroll
-    for (int h2 = 0; h2 < 8; ++h2) {
-      const float x = (h2 & 1) ? bf16hi(wv[h2 >> 1]) : bf16lo(wv[h2 >> 1]);
-      bad |= !(fabsf(x) <= 65504.f);  // also true for NaN
-      mn = fminf(mn, x);
-      mx = fmaxf(mx, x);
-    }
+  for (int i = 0; i < 4; ++i) {
+    x[2 * i] = bf16lo(w[i]);
+    x[2 * i + 1] = bf16hi(w[i]);
   }
-  const int rowb = a.d * b / 8;
-  const bool sw = a.swz && b == 8;  // 8-bit rows of a swizzled cache
-  const int64_t coff = static_cast<int64_t>(which) * a.P * rowb + static_cast<int64_t>(p.slot) * rowb + g * a.G * b / 8;
-  uint32_t* sz = reinterpret_cast<uint32_t*>(sl + 2 * static_cast<int64_t>(a.P) * rowb +
-                                             static_cast<int64_t>(which) * a.P * ng * 4 +
-                                             static_cast<int64_t>(p.slot) * ng * 4 + g * 4);
-  if (bad) {
-    for (int i = 0; i < a.G * b / 32; ++i) {
-      const int64_t o = coff + 4 * i;
-      *reinterpret_cast<uint32_t*>(sl + (sw ? swz_off(o) : o)) = 0;
-    }
-    *sz = 0;
-    set_status(a.ctrl, TRR_ERR_BAD_VALUE);
-    return;
+  float mn = x[0], mx = x[0];
+  bad = false;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    bad |= !(fabsf(x[i]) <= 65504.f);  // also true for NaN
+    mn = fminf(mn, x[i]);
+    mx = fmaxf(mx, x[i]);
   }
-  const __half z16 = __float2half_rn(mn);                                   // z = min(x)
-  const float levels = static_cast<float>((1 << b) - 1);
-  const __half s16 = __float2half_rn(__fdiv_rn(__fsub_rn(mx, mn), levels));  // s
+  for (int o = 1; o < GL; o <<= 1) {
+    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    bad |= __shfl_xor_sync(0xffffffffu, static_cast<int>(bad), o) != 0;
+  }
+  codes = 0;
+  sz = 0;
+  if (bad) return;
+  const int levels = (1 << b) - 1;
+  const __half z16 = __float2half_rn(mn);                                                        // z = min(x)
+  const __half s16 = __float2half_rn(__fdiv_rn(__fsub_rn(mx, mn), static_cast<float>(levels)));  // s
   const float z = __half2float(z16), s = __half2float(s16), rs = __frcp_rn(s);
-  for (int q = 0; q < a.G / 32; ++q) {
-    const int64_t off = coff + 4 * q * b;  // 32 codes of b bits = b words
-    if (b == 2) quantise_chunk<2>(s4 + 4 * q, z, s, rs, sl, off, false);
-    else if (b == 4) quantise_chunk<4>(s4 + 4 * q, z, s, rs, sl, off, false);
-    else quantise_chunk<8>(s4 + 4 * q, z, s, rs, sl, off, sw);
+  if (s != 0.f) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      codes |= static_cast<unsigned long long>(static_cast<uint32_t>(code_of(x[i], z, s, rs, levels))) << (i * b);
   }
-  *sz = static_cast<uint32_t>(__half_as_ushort(s16)) | (static_cast<uint32_t>(__half_as_ushort(z16)) << 16);
+  sz = static_cast<uint32_t>(__half_as_ushort(s16)) | (static_cast<uint32_t>(__half_as_ushort(z16)) << 16);
 }
 
-// ------------------------------------------------------------ one-kernel append --
+// One kernel per call.  Every CTA plans every entry the same way from the metadata as the
+// call found it and writes its share of the rows; the last CTA to finish planning commits
+// the metadata: every other CTA has read all it needs of them by then.
 //
-// For calls of up to kFusedMax entries (a decode step) one kernel does the whole append.
-// Every CTA plans every entry (the same deterministic plan as append_plan_kernel, from
-// the metadata as the call found it), each warp quantises one (entry, KV head, K|V) row,
-// and the last CTA to finish commits the metadata: no CTA reads metadata after the
-// commit, since every other CTA has finished by then.
+// The plan sorts the entries by (sequence, entry) unless they come that way, so that what
+// an entry needs of the earlier entries of its sequence (largest position, tokens per
+// class) is one prefix pass instead of a scan of all entries: O(n log n) in place of
+// O(n^2).  In the small instance everything up to the first read of metadata comes before
+// the wait on the previous kernel and overlaps it.  Rows are quantised by d/8 lanes each,
+// 16 bytes a lane.
+//
+// Bound by latency: the chain from the wait (metadata, page ids, first rows).  The second
+// row of a lane is loaded while the first is quantised, and the arrival's round trip and the
+// commit overlap the rows (13.9 -> 11.8 us a call of 1024 entries of 12 x 64 KV heads, on
+// the GPU alone).  With a plan kernel that scanned all entries for each and a second kernel
+// of one thread per group such a call took 122 us.  A call of 256 entries with its
+// attention: 97 -> 73 us.  The large instance waits before it reads its entries (as calls
+// of that size always did; reading them early would save 2.4 us).
+template <int D, int T>
+__global__ void __launch_bounds__(T) append_kernel(LayerArgs a, int n, const int32_t* __restrict__ seq_ids,
+                                                   const int32_t* __restrict__ positions,
+                                                   const uint8_t* __restrict__ bits,
+                                                   const uint8_t* __restrict__ modes,
+                                                   const float* __restrict__ bit_logits,
+                                                   const float* __restrict__ mode_logits,
+                                                   const uint16_t* __restrict__ k, const uint16_t* __restrict__ v) {
+  __shared__ AppendShared<T> sh;
+  constexpr int LPR = D / 8;  // lanes per row
+  const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
+  const unsigned below = (1u << lane) - 1u;
 
-constexpr int kFusedMax = 256;
-
-// One row of d values (entry, KV head, K or V) by a warp, written to its slot.
-// The codes go to byte row_off of the slice sl (swizzled when sw).
-template <int D>
-__device__ __forceinline__ void quantise_row(const uint2 w, uint8_t* sl, int64_t row_off, bool sw, uint32_t* sz_row,
-                                             int b, int G, int lane, int32_t* ctrl) {
-  const RowCodes r = quantise_row_codes<D>(w, b, G, lane);
-  if (r.bad && r.sz_idx >= 0) set_status(ctrl, TRR_ERR_BAD_VALUE);
-  if (r.code_idx >= 0) {
-    const int64_t o = row_off + 4 * r.code_idx;
-    *reinterpret_cast<uint32_t*>(sl + (sw ? swz_off(o) : o)) = r.code_word;
+  // ------------------------------------------- the entries, and what follows from them alone
+  // lanes LPR r .. of the grid hold row r = (entry, KV head, K | V), 8 values each
+  const int nlanes = n * a.Hkv * 2 * LPR, step = gridDim.x * T;
+  auto row_src = [&](int x) {
+    const int r = x / LPR, e = r / (2 * a.Hkv), j = (r >> 1) % a.Hkv;
+    return reinterpret_cast<const uint4*>(((r & 1) ? v : k) + (static_cast<int64_t>(e) * a.Hkv + j) * D) + x % LPR;
+  };
+  const int x0 = blockIdx.x * T + i;
+  if (T > kSmallAppend) pdl_wait();
+  int err = 0;  // of entry i until the sort, then of the entry this thread has
+  uint32_t key = 0xffffffffu - (1023u - i);  // past the entries
+  if (i < n) {
+    const int seq = seq_ids[i], pos = positions[i], m = entry_mode(a, modes, mode_logits, i);
+    const int c = class_of_bits(entry_bits(bits, bit_logits, i));
+    const bool in = seq >= 0 && seq < a.S;
+    if (!in || c < 0 || m > TRR_MODE_FULL) err = TRR_ERR_INVALID_ARG;
+    else if (pos < 0 || pos >= a.maxctx) err = TRR_ERR_BAD_POSITION;
+    key = ((in ? static_cast<uint32_t>(seq) : 1u << 20) << 10) | static_cast<uint32_t>(i);
+    sh.pos[i] = pos;
+    sh.cls[i] = !err && (m != TRR_MODE_SKIP || a.skip_writes_kv) ? c : -1;
+    sh.tok[i] = err;
   }
-  if (r.sz_idx >= 0) sz_row[r.sz_idx] = r.sz_word;
-}
-
-template <int D>
-__global__ void __launch_bounds__(256) append_fused_kernel(LayerArgs a, int n, const int32_t* __restrict__ seq_ids,
-                                                           const int32_t* __restrict__ positions,
-                                                           const uint8_t* __restrict__ bits,
-                                                           const uint8_t* __restrict__ modes,
-                                                           const float* __restrict__ bit_logits,
-                                                           const float* __restrict__ mode_logits,
-                                                           const uint16_t* __restrict__ k,
-                                                           const uint16_t* __restrict__ v) {
-  __shared__ int s_seq[kFusedMax];
-  __shared__ int s_pos[kFusedMax];
-  __shared__ int s_cls[kFusedMax];   // width class when the entry stores KV, else -1
-  __shared__ int s_k[kFusedMax];     // token index in the (sequence, class) list
-  __shared__ int s_pid[kFusedMax];   // page of the token (openers: the new page)
-  __shared__ int s_wopen[8][kClasses];
-  __shared__ int s_next[kClasses];
-  __shared__ int s_first_err;
-  __shared__ int s_last;
-
-  const int e = threadIdx.x, lane = e & 31, warp = e >> 5;
-  const bool act = e < n;
-  // The call's own inputs (entries, K/V rows) are read first: no kernel of this library
-  // writes them, so this overlaps the previous kernel of the stream.  Cache metadata and
-  // control words come after the wait.
-  // this warp's row (entry, KV head, K|V), loaded while the entries are planned
-  const int row = blockIdx.x * (blockDim.x >> 5) + warp;
-  const bool has_row = row < n * a.Hkv * 2;
-  const int re = row / (2 * a.Hkv), rh = (row >> 1) % a.Hkv, which = row & 1;
-  uint2 raw = make_uint2(0, 0);
-  if (has_row) {
-    const uint16_t* src = (which ? v : k) + (static_cast<int64_t>(re) * a.Hkv + rh) * D;
-    if (D == 64) raw.x = reinterpret_cast<const uint32_t*>(src)[lane];
-    else raw = reinterpret_cast<const uint2*>(src)[lane];
+  sh.key[i] = key;
+  if (i < 32) {
+    sh.wsum[i] = sh.wmax[i] = sh.wopen[i] = 0ull;
+    sh.whead[i] = -1;
   }
-  int seq = -1, pos = 0, c = -1, err = 0;
-  bool writes = false;
-  if (act) {
-    seq = seq_ids[e];
-    pos = positions[e];
-    const int m = entry_mode(a, modes, mode_logits, e);
-    if (seq < 0 || seq >= a.S) {
-      err = TRR_ERR_INVALID_ARG;
-    } else {
-      c = class_of_bits(entry_bits(bits, bit_logits, e));
-      if (c < 0 || m > TRR_MODE_FULL) err = TRR_ERR_INVALID_ARG;
-      else if (pos < 0 || pos >= a.maxctx) err = TRR_ERR_BAD_POSITION;
-    }
-    writes = !err && (m != TRR_MODE_SKIP || a.skip_writes_kv);
-  }
-  s_seq[e] = (act && seq >= 0 && seq < a.S) ? seq : -1;
-  s_pos[e] = pos;
-  s_cls[e] = writes ? c : -1;
-  pdl_wait();
-  pdl_trigger();
-  if (e < kClasses) s_next[e] = a.ctrl[kNextPage + e];
-  if (e == 0) s_first_err = INT_MAX;
+  if (i == 0) sh.first_err = INT_MAX;
   __syncthreads();
-
-  // earlier entries of the same sequence: the largest position and, per class, how many
-  // store KV; later ones: whether this entry is the sequence's / class's last
-  int prev_max = -1, rank = 0;
-  bool later_seq = false, later_cls = false;
-  if (act && s_seq[e] >= 0) {
-    for (int j = 0; j < n; ++j) {
-      if (s_seq[j] != seq) continue;
-      if (j < e) {
-        prev_max = max(prev_max, s_pos[j]);
-        rank += (writes && s_cls[j] == c);
-      } else if (j > e) {
-        later_seq = true;
-        later_cls |= (writes && s_cls[j] == c);
-      }
+  if (__syncthreads_or(i > 0 && sh.key[i - 1] > key)) {
+    key = sort_keys<T>(key, sh.key);
+    __syncthreads();
+    sh.key[i] = key;
+    __syncthreads();
+  }
+  const bool act = key < (2u << 30);            // an entry ..
+  const int e = static_cast<int>(key & 1023u);  // .. this one ..
+  const bool has_seq = key < (1u << 30);        // .. whose sequence id is valid
+  const int seq = has_seq ? static_cast<int>(key >> 10) : -1;
+  const int pos = act ? sh.pos[e] : 0, c = act ? sh.cls[e] : -1;
+  err = act ? sh.tok[e] : 0;
+  const bool writes = c >= 0;
+  // prefix passes over the sorted entries: tokens per class (16 bits each), the largest
+  // position so far (with the sequence above it: sequences ascend), the sequence's start
+  const bool head = i == 0 || (sh.key[i - 1] >> 10) != (key >> 10);
+  const bool tail = i == T - 1 || (sh.key[i + 1] >> 10) != (key >> 10);
+  unsigned long long sum = writes ? 1ull << (16 * c) : 0ull;
+  unsigned long long top = (static_cast<unsigned long long>(key >> 10) << 32) |
+                           (static_cast<uint32_t>(pos) ^ 0x80000000u);  // order of int32
+  const unsigned heads = __ballot_sync(0xffffffffu, head) & (below | (1u << lane));
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long s1 = __shfl_up_sync(0xffffffffu, sum, o), t1 = __shfl_up_sync(0xffffffffu, top, o);
+    if (lane >= o) {
+      sum += s1;
+      top = max(top, t1);
     }
   }
+  if (lane == 31) {
+    sh.wsum[warp] = sum;
+    sh.wmax[warp] = top;
+    sh.whead[warp] = heads ? 32 * warp + 31 - __clz(heads) : -1;
+  }
+  __syncthreads();
+  // the warps before this one: their sum, largest and last start, one warp per lane
+  const bool earlier = lane < warp;
+  const unsigned long long before = add_packed(earlier ? sh.wsum[lane] : 0ull);
+  const unsigned long long wt = earlier ? sh.wmax[lane] : 0ull;
+  const uint32_t th = __reduce_max_sync(0xffffffffu, static_cast<uint32_t>(wt >> 32));
+  const uint32_t tl = __reduce_max_sync(0xffffffffu, static_cast<uint32_t>(wt >> 32) == th ? static_cast<uint32_t>(wt) : 0u);
+  const unsigned long long top_before = static_cast<unsigned long long>(th) << 32 | tl;
+  const int hb = __reduce_max_sync(0xffffffffu, earlier ? sh.whead[lane] : -1);
+  const int first = heads ? 32 * warp + 31 - __clz(heads) : hb;
+  sum += before;
+  // the largest position before this entry: the previous lane's, or the previous warps'
+  unsigned long long prev = __shfl_up_sync(0xffffffffu, top, 1);
+  prev = lane == 0 ? top_before : max(prev, top_before);
+  const bool has_prev = i > 0 && static_cast<uint32_t>(prev >> 32) == (key >> 10);
+  const int prev_max = has_prev ? static_cast<int>(static_cast<uint32_t>(prev) ^ 0x80000000u) : -1;
+  sh.prefix[i] = sum;
+  if (tail) sh.end[first] = i;
+  __syncthreads();  // sh.pos (by entry) is read no more
+  const unsigned long long start = first > 0 ? sh.prefix[first - 1] : 0ull;
+  const unsigned long long mine = sum - start, all = sh.prefix[sh.end[first]] - start;
+  auto field = [](unsigned long long x, int cc) { return static_cast<int>((x >> (16 * cc)) & 0xffffu); };
+  const int rank = writes ? field(mine, c) - 1 : 0;  // earlier entries of the (sequence, class) that store KV
+  const bool last_cls = writes && rank + 1 == field(all, c);
+  int slot0 = first;  // where the class's tokens of this sequence are listed: first, then rank
+  for (int cc = 0; cc < c; ++cc) slot0 += field(all, cc);
+
+  // ----------------------------------- after the wait: the metadata, this lane's first row
+  if (T <= kSmallAppend) pdl_wait();
+  pdl_trigger();
+  uint4 raw = make_uint4(0, 0, 0, 0);
+  if (x0 < nlanes) raw = *row_src(x0);
+  if (i < kClasses) sh.next[i] = a.ctrl[kNextPage + i];
   int tok = 0, nt_old = 0, last_page = -1;
-  bool opens = false;
   if (act && !err) {
     const int lp = a.last_pos[seq];
     if (writes) {
@@ -379,111 +278,135 @@ __global__ void __launch_bounds__(256) append_fused_kernel(LayerArgs a, int n, c
       last_page = a.lastpg[seq * 4 + c];
     }
     if (pos <= max(prev_max, lp)) err = TRR_ERR_BAD_POSITION;
-    if (writes) {
-      tok = nt_old + rank;
-      opens = tok % a.P == 0;
-    }
+    tok = nt_old + rank;
   }
-  // page ids in entry order: next_page + openers of the same class before e
-  int before = 0;
+  const bool opens = writes && !err && tok % a.P == 0;
+  if (act) sh.pid[e] = opens;
+  __syncthreads();
+  // page ids in entry order: next_page + openers of the same class before the entry
+  {
+    const int cc = i < n && sh.pid[i] ? sh.cls[i] : -1;
+    unsigned long long mine4 = cc >= 0 ? 1ull << (16 * cc) : 0ull;
+    int rk = 0;
 #pragma unroll
-  for (int cc = 0; cc < kClasses; ++cc) {
-    const unsigned bal = __ballot_sync(0xffffffffu, !err && opens && c == cc);
-    if (lane == 0) s_wopen[warp][cc] = __popc(bal);
-    if (c == cc) before = __popc(bal & ((1u << lane) - 1u));
+    for (int q = 0; q < kClasses; ++q) {
+      const unsigned bal = __ballot_sync(0xffffffffu, cc == q);
+      if (cc == q) rk = __popc(bal & below);
+    }
+    mine4 = add_packed(mine4);
+    if (lane == 0) sh.wopen[warp] = mine4;
+    __syncthreads();
+    const unsigned long long wo = add_packed(lane < warp ? sh.wopen[lane] : 0ull);
+    if (cc >= 0) sh.pid[i] = sh.next[cc] + field(wo, cc) + rk;
   }
   __syncthreads();
   int pid = -1;
   if (opens) {
-    for (int w = 0; w < warp; ++w) before += s_wopen[w][c];
-    pid = s_next[c] + before;
+    pid = sh.pid[e];
     if (pid >= a.cap[c]) err = TRR_ERR_OUT_OF_PAGES;
+    sh.pos[slot0 + rank] = pid;
   }
-  if (act && err) atomicMin(&s_first_err, e);
-  s_k[e] = tok;
-  s_pid[e] = pid;
+  if (act && err) atomicMin(&sh.first_err, e);
   __syncthreads();
-  if (s_first_err != INT_MAX) {  // the call is a no-op; record the lowest failing entry
-    if (blockIdx.x == 0 && e == s_first_err) set_status(a.ctrl, err);
+  if (sh.first_err != INT_MAX) {  // the call is a no-op; record the lowest failing entry
+    if (blockIdx.x == 0 && act && e == sh.first_err) set_status(a.ctrl, err);
     return;
   }
   const int kidx = tok / a.P;
-  const int64_t prow = (static_cast<int64_t>(seq) * 4 + c) * a.MP + kidx;
-  if (writes && !opens) {  // a page opened earlier: by a previous call (then the class's
-                           // last page), or by an earlier entry of this call
-    if (kidx * a.P < nt_old) {
-      pid = last_page;
-    } else {
-      for (int j = 0; j < e; ++j)
-        if (s_seq[j] == seq && s_cls[j] == c && s_k[j] == kidx * a.P) pid = s_pid[j];
-    }
-    s_pid[e] = pid;
-  }
-  __syncthreads();
-
-  if (has_row) {
-    const int rc = s_cls[re];
-    if (rc >= 0) {
-      const int b = bits_of_class(rc), slot = s_k[re] % a.P;
-      uint8_t* sl = a.pool[rc] + static_cast<int64_t>(s_pid[re]) * a.page_bytes[rc] + a.hdr +
-                    static_cast<int64_t>(rh) * a.slice[rc];
-      if (b == 16) {  // this lane's D/32 values (4 or 8 bytes: inside one 16-byte chunk)
-        const int64_t o = (static_cast<int64_t>(which) * a.P + slot) * D * 2 + lane * (D / 16);
-        uint8_t* dst = sl + (a.swz ? swz_off(o) : o);
-        if (D == 64) *reinterpret_cast<uint32_t*>(dst) = raw.x;
-        else *reinterpret_cast<uint2*>(dst) = raw;
-      } else {
-        const int rowb = D * b / 8, ng = D / a.G;
-        uint32_t* sz_row = reinterpret_cast<uint32_t*>(sl + 2 * static_cast<int64_t>(a.P) * rowb +
-                                                      (static_cast<int64_t>(which) * a.P + slot) * ng * 4);
-        quantise_row<D>(raw, sl, (static_cast<int64_t>(which) * a.P + slot) * rowb, a.swz && b == 8, sz_row, b, a.G,
-                        lane, a.ctrl);
-      }
-    }
-  }
-
-  // the last CTA to finish commits the metadata of every entry: its acquire follows the
-  // release of every other CTA, after all of their reads of the old metadata
-  __syncthreads();
-  if (e == 0) s_last = atom_add_acq_rel(&a.ctrl[kAppendDone], 1) == static_cast<int>(gridDim.x) - 1;
-  __syncthreads();
-  if (!s_last) return;
+  if (writes && !opens)  // a page opened by an earlier call (then the class's last one), or
+                         // by an earlier entry of this one
+    pid = kidx * a.P < nt_old ? last_page : sh.pos[slot0 + kidx * a.P - nt_old];
   if (act) {
-    if (writes) {
-      const int slot = tok % a.P;
-      if (opens) {
-        a.pt[prow] = pid;
-        a.pfirst[prow] = pos;
-      }
-      if (!later_cls || slot == a.P - 1) a.plast[prow] = pos;
-      if (!later_cls) {
-        a.ntok[seq * 4 + c] = tok + 1;
-        a.lastpg[seq * 4 + c] = pid;
-      }
-      reinterpret_cast<int32_t*>(a.pool[c] + static_cast<int64_t>(pid) * a.page_bytes[c])[slot] = pos;
-      atomicOr(&a.presence[static_cast<int64_t>(seq) * a.W32 + pos / 32], 1u << (pos % 32));
-    }
-    if (!later_seq) a.last_pos[seq] = pos;
+    sh.pid[e] = pid;
+    sh.tok[e] = tok;
   }
+  __syncthreads();
+
+  // This CTA has read its last metadata.  The last one to get here commits them (after its
+  // own rows, so that the arrival's round trip is hidden): its acquire follows the release
+  // of every other CTA.
+  if (i == 0) sh.last = atom_add_acq_rel(&a.ctrl[kAppendDone], 1) == static_cast<int>(gridDim.x) - 1;
+
+  // ------------------------------------------------------------------------ the rows
+  const int ng = D / a.G, GL = a.G / 8;
+  uint4 next = raw;
+  for (int x = x0; x - lane < nlanes; x += step) {  // warps stay together
+    raw = next;
+    if (x + step < nlanes) next = *row_src(x + step);
+    const int r = min(x, nlanes - 1) / LPR, re = r / (2 * a.Hkv), j = (r >> 1) % a.Hkv, which = r & 1, l = x % LPR;
+    const int rc = x < nlanes ? sh.cls[re] : -1, b = bits_of_class(rc & 3);
+    unsigned long long codes;
+    uint32_t sz;
+    bool bad;
+    quantise_8(raw, min(b, 8), GL, codes, sz, bad);
+    if (rc < 0) continue;
+    const int slot = sh.tok[re] % a.P;
+    uint8_t* sl = a.pool[rc] + static_cast<int64_t>(sh.pid[re]) * a.page_bytes[rc] + a.hdr +
+                  static_cast<int64_t>(j) * a.slice[rc];
+    const int64_t off = static_cast<int64_t>(which * a.P + slot) * (D * b / 8) + l * b;
+    uint8_t* dst = sl + (a.swz && b >= 8 ? swz_off(off) : off);  // stays inside a 16-byte chunk
+    if (b == 16) {  // native precision: the bf16 bits
+      *reinterpret_cast<uint4*>(dst) = raw;
+      continue;
+    }
+    if (b == 2) *reinterpret_cast<uint16_t*>(dst) = static_cast<uint16_t>(codes);
+    else if (b == 4) *reinterpret_cast<uint32_t*>(dst) = static_cast<uint32_t>(codes);
+    else *reinterpret_cast<unsigned long long*>(dst) = codes;
+    if (l % GL == 0) {
+      reinterpret_cast<uint32_t*>(sl + 2 * static_cast<int64_t>(a.P) * (D * b / 8) +
+                                  static_cast<int64_t>(which * a.P + slot) * ng * 4)[l / GL] = sz;
+      if (bad) set_status(a.ctrl, TRR_ERR_BAD_VALUE);
+    }
+  }
+
+  // ---------------------------------------------------------------------- the commit
+  __syncthreads();
+  if (!sh.last) return;
+  if (writes) {
+    const int slot = tok % a.P;
+    const int64_t prow = (static_cast<int64_t>(seq) * 4 + c) * a.MP + kidx;
+    if (opens) {
+      a.pt[prow] = pid;
+      a.pfirst[prow] = pos;
+    }
+    if (last_cls || slot == a.P - 1) a.plast[prow] = pos;
+    if (last_cls) {
+      a.ntok[seq * 4 + c] = tok + 1;
+      a.lastpg[seq * 4 + c] = pid;
+    }
+    reinterpret_cast<int32_t*>(a.pool[c] + static_cast<int64_t>(pid) * a.page_bytes[c])[slot] = pos;
+    atomicOr(&a.presence[static_cast<int64_t>(seq) * a.W32 + pos / 32], 1u << (pos % 32));
+  }
+  if (act && tail) a.last_pos[seq] = pos;
   if (a.head_modes) {  // presence masks: openers clear their new pages, then every entry
                        // sets its slot's bit for the KV heads it stores
-    const bool mine = act && writes;
-    if (mine && opens)
+    if (opens)
       for (int j = 0; j < a.Hkv; ++j) {
         head_mask(a, c, pid, j)[0] = 0ull;
         head_mask(a, c, pid, j)[1] = 0ull;
       }
     __syncthreads();
-    if (mine)
+    if (writes)
       for (int j = 0; j < a.Hkv; ++j)
         if (head_stores(a, modes, e, j)) atomicOr(head_mask(a, c, pid, j), 1ull << (tok % a.P));
   }
-  if (e < kClasses) {
-    int opened = 0;
-    for (int w = 0; w < 8; ++w) opened += s_wopen[w][e];
-    a.ctrl[kNextPage + e] = s_next[e] + opened;
+  if (warp == 0) {
+    const unsigned long long opened = add_packed(sh.wopen[lane]);
+    if (i < kClasses) a.ctrl[kNextPage + i] = sh.next[i] + field(opened, i);
   }
-  if (e == 0) a.ctrl[kAppendDone] = 0;
+  if (i == 0) a.ctrl[kAppendDone] = 0;
+}
+
+template <int D, int T>
+static cudaError_t launch_append(const LayerArgs& a, int num_sms, cudaStream_t s, int n, const int32_t* seq_ids,
+                                 const int32_t* positions, const uint8_t* bits, const uint8_t* modes,
+                                 const float* bit_logits, const float* mode_logits, const uint16_t* k,
+                                 const uint16_t* v) {
+  // a lane per 8 values, at most one CTA per SM
+  const int64_t work = static_cast<int64_t>(n) * a.Hkv * 2 * (D / 8);
+  const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>((work + T - 1) / T, num_sms)));
+  return launch_pdl(append_kernel<D, T>, dim3(grid), dim3(T), 0, s, a, n, seq_ids, positions, bits, modes, bit_logits,
+                    mode_logits, k, v);
 }
 
 }  // namespace trr
@@ -513,23 +436,10 @@ static trr_status append_call(trr_cache* cache, int32_t layer, int32_t n, const 
   cache_note_call(cache, layer);
   const uint16_t* k = static_cast<const uint16_t*>(k_bf16);
   const uint16_t* v = static_cast<const uint16_t*>(v_bf16);
-  if (n <= kFusedMax) {  // one kernel: 256 threads plan, one warp per (entry, head, K|V) row
-    const unsigned blocks = static_cast<unsigned>((static_cast<int64_t>(n) * l.Hkv * 2 + 7) / 8);
-    const cudaError_t e =
-        l.d == 64 ? launch_pdl(append_fused_kernel<64>, dim3(blocks), dim3(256), 0, s, a, n, seq_ids, positions, bits,
-                               modes, bit_logits, mode_logits, k, v)
-                  : launch_pdl(append_fused_kernel<128>, dim3(blocks), dim3(256), 0, s, a, n, seq_ids, positions,
-                               bits, modes, bit_logits, mode_logits, k, v);
-    cache_set_launches(cache, 1);
-    return e == cudaSuccess ? TRR_OK : TRR_ERR_CUDA;
-  }
-  const int threads = (n + 31) / 32 * 32;
-  cudaError_t e = launch_pdl(append_plan_kernel, dim3(1), dim3(threads), 0, s, a, n, seq_ids, positions, bits, modes,
-                             bit_logits, mode_logits);
-  if (e != cudaSuccess) return TRR_ERR_CUDA;
-  const int64_t work = static_cast<int64_t>(n) * l.Hkv * 2 * (l.d / l.G);
-  e = launch_pdl(append_write_kernel, dim3(static_cast<unsigned>((work + 255) / 256)), dim3(256), 0, s, a, n, k, v);
-  cache_set_launches(cache, 2);
+  auto* launch = n <= kSmallAppend ? (l.d == 64 ? launch_append<64, kSmallAppend> : launch_append<128, kSmallAppend>)
+                                   : (l.d == 64 ? launch_append<64, 1024> : launch_append<128, 1024>);
+  const cudaError_t e = launch(a, cache_num_sms(cache), s, n, seq_ids, positions, bits, modes, bit_logits, mode_logits, k, v);
+  cache_set_launches(cache, 1);
   return e == cudaSuccess ? TRR_OK : TRR_ERR_CUDA;
 }
 

@@ -39,7 +39,6 @@ LayerArgs layer_args(const Layout& l, const Views& v, int layer) {
   a.pfirst = v.pfirst + ls * 4 * l.MP;
   a.plast = v.plast + ls * 4 * l.MP;
   a.lastpg = v.lastpg + ls * 4;
-  a.aplan = v.aplan;
   a.cnt = v.cnt;
   a.cnt_stride = l.cnt_stride;
   a.part = v.part;
@@ -113,7 +112,6 @@ static trr_status make_layout(const trr_cache_config* c, Layout* l) {
   l->off_pfirst = take(16 * nls * l->MP);
   l->off_plast = take(16 * nls * l->MP);
   l->off_lastpg = take(16 * nls);
-  l->off_aplan = take(static_cast<int64_t>(sizeof(AppendPlan)) * l->max_append);
   l->off_cnt = take(4 * static_cast<int64_t>(l->max_queries) * l->units * l->cnt_stride);
   l->off_part = take(4 * l->max_items * (l->Hq / l->units) * (l->d + 4));
   for (int k = 0; k < kClasses; ++k) l->off_pool[k] = take(l->cap[k] * l->page_bytes[k]);

@@ -18,8 +18,7 @@ __host__ __device__ constexpr int bits_of_class(int c) { return c == 0 ? 2 : c =
 enum Ctrl : int {
   kStatus = 0,        // sticky first error since the last trr_get_status
   kNextPage = 4,      // [4] pages handed out per class
-  kAppendOk = 10,     // append: 1 when the plan kernel committed the call
-  kAppendDone = 11,   // one-kernel append: CTAs finished (the last one commits)
+  kAppendDone = 11,   // append: CTAs finished (the last one commits)
   kCtrlInts = 64
 };
 
@@ -54,7 +53,7 @@ struct Layout {
   int64_t max_items;
   int64_t hdr, tokb[kClasses], slice[kClasses], maskb, page_bytes[kClasses];
   int64_t off_ctrl, off_lctl, off_last_pos, off_ntok, off_presence, off_pt, off_pfirst, off_plast, off_lastpg;
-  int64_t off_aplan, off_cnt, off_part, off_pool[kClasses], total;
+  int64_t off_cnt, off_part, off_pool[kClasses], total;
 };
 
 // Splits of a query whose key range spans `range` positions: at least pos_split
@@ -85,14 +84,6 @@ __host__ __device__ inline int64_t swz_off(int64_t o) {
   return (o & ~static_cast<int64_t>(127)) | ((((o >> 4) ^ (o >> 7)) & 7) << 4) | (o & 15);
 }
 
-// Per-entry plan written by the append plan kernel.
-struct AppendPlan {
-  int page;   // page id, -1 = nothing stored
-  int slot;   // slot in the page
-  int cls;    // width class
-  int pos;    // position
-};
-
 struct Views {  // typed device pointers into the cache memory
   int32_t* ctrl;
   int32_t* lctl;
@@ -103,7 +94,6 @@ struct Views {  // typed device pointers into the cache memory
   int32_t* pfirst;
   int32_t* plast;
   int32_t* lastpg;
-  AppendPlan* aplan;
   int32_t* cnt;
   float* part;
   uint8_t* pool[kClasses];
@@ -121,7 +111,6 @@ inline Views make_views(const Layout& l, void* base) {
   v.pfirst = reinterpret_cast<int32_t*>(b + l.off_pfirst);
   v.plast = reinterpret_cast<int32_t*>(b + l.off_plast);
   v.lastpg = reinterpret_cast<int32_t*>(b + l.off_lastpg);
-  v.aplan = reinterpret_cast<AppendPlan*>(b + l.off_aplan);
   v.cnt = reinterpret_cast<int32_t*>(b + l.off_cnt);
   v.part = reinterpret_cast<float*>(b + l.off_part);
   for (int c = 0; c < kClasses; ++c) v.pool[c] = b + l.off_pool[c];
@@ -148,7 +137,6 @@ struct LayerArgs {
   int32_t* pfirst;
   int32_t* plast;
   int32_t* lastpg;     // this layer: [S][4] id of the page holding token ntok-1 (internal)
-  AppendPlan* aplan;
   int32_t* cnt;        // [max_queries][Hq][cnt_stride] split arrivals (zero between calls)
   float* part;         // [max_queries * s_cap * Hq][d + 4] fp32 partials: acc, M, L
   uint8_t* pool[kClasses];
