@@ -5,14 +5,14 @@
 #include <algorithm>
 #include <climits>
 
-#include "trr_attn.cuh"
+#include "trr_row.cuh"
 
 namespace trr {
 
 // Done once per cache at creation, so that calls stay legal inside stream capture.
 cudaError_t attn_configure() {
-  cudaError_t (*const parts[])() = {configure_attn_cc, configure_attn_head_modes, configure_attn_mma,
-                                     configure_attn_step_cc, configure_attn_step_mma};
+  cudaError_t (*const parts[])() = {configure_attn_row, configure_attn_row_heads, configure_attn_row_step,
+                                     configure_attn_mma, configure_attn_step_mma};
   for (auto part : parts) {
     const cudaError_t e = part();
     if (e != cudaSuccess) return e;
@@ -42,17 +42,21 @@ static int attn_ring_bytes(const Layout& l, int n, int hpu, int scr_floats, int 
 constexpr int kMaxLaunchQueries = 1024;
 
 static cudaError_t launch_one(const Layout& l, const AttnKernelArgs& ka, int num_sms, cudaStream_t s) {
-  const bool mma = use_mma(l);
-  const int ctas = mma ? kMmaCtasPerSm : cc_ctas_per_sm(l.d);
-  const int ring = attn_ring_bytes(l, ka.n, ka.hpu, ka.scr_floats, ka.fused, attn_smem_limit(ctas));
-  if (ring < 0) return cudaErrorInvalidConfiguration;
   AttnKernelArgs k = ka;
+  if (!use_mma(l)) {  // one query head per warp: every warp's ring is an equal share
+    const int fixed = RowSmem(l.d, l.d / l.G, k.n, k.fused, 0).total;
+    k.ring_bytes = (kRowSmemLimit - fixed) / kRowWarps / 128 * 128;
+    const size_t sm = static_cast<size_t>(RowSmem(l.d, l.d / l.G, k.n, k.fused, k.ring_bytes).total);
+    const dim3 grid(kRowCtasPerSm * num_sms - num_sms / kRowSpare);
+    if (k.fused) return launch_attn_row_step(l, grid, sm, s, k);
+    return l.head_modes ? launch_attn_row_heads(l, grid, sm, s, k) : launch_attn_row(l, grid, sm, s, k);
+  }
+  const int ring = attn_ring_bytes(l, ka.n, ka.hpu, ka.scr_floats, ka.fused, attn_smem_limit(kMmaCtasPerSm));
+  if (ring < 0) return cudaErrorInvalidConfiguration;
   k.ring_bytes = ring;
   const size_t sm = static_cast<size_t>(AttnSmem(ring, k.n, k.scr_floats, k.fused).total);
-  const dim3 grid(ctas * num_sms), block(32 * (kNcw + 1));
-  if (k.fused) return mma ? launch_attn_step_mma(l, grid, block, sm, s, k) : launch_attn_step_cc(l, grid, block, sm, s, k);
-  if (mma) return launch_attn_mma(l, grid, block, sm, s, k);
-  return l.head_modes ? launch_attn_head_modes(l, grid, block, sm, s, k) : launch_attn_cc(l, grid, block, sm, s, k);
+  const dim3 grid(kMmaCtasPerSm * num_sms), block(32 * (kNcw + 1));
+  return k.fused ? launch_attn_step_mma(l, grid, block, sm, s, k) : launch_attn_mma(l, grid, block, sm, s, k);
 }
 
 // The launches of an attention call with the given scratch views in `a`; *launches

@@ -76,6 +76,7 @@ __device__ __forceinline__ void warp_count_below(const int* base, int64_t stride
       hi[i] = b;
     }
   }
+#pragma unroll 1
   for (int round = 0; round < 6; ++round) {
     bool any = false;
 #pragma unroll
@@ -110,45 +111,6 @@ __device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 
 // exact 2^e, -126 <= e <= 127 (folds to a constant for constant e)
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }
 
-// Bit offset of element i (of a lane's 16 or 32) inside the word it is extracted from.
-__host__ __device__ constexpr int ex_of(int B, int i) {
-  return B == 2 ? ((i % 16) < 11 ? 2 * (i % 16) : 2 * (i % 16 - 11))
-                : B == 4 ? ((i % 8) < 5 ? 4 * (i % 8) : 4 * (i % 8 - 5)) : 0;
-}
-// Pre-scale exponent of the query in class B.
-__host__ __device__ constexpr int qe_of(int B, int i) { return B == 16 ? 0 : 100 - ex_of(B, i); }
-
-// Element i as c * 2^(ex-149): the code left in place, read as a subnormal.
-template <int B>
-__device__ __forceinline__ float code_at(const uint32_t* w, const uint32_t* h, int i) {
-  if (B == 2) {
-    const int j = i % 16;
-    return __uint_as_float(j < 11 ? (w[i / 16] & (3u << (2 * j))) : (h[i / 16] & (3u << (2 * (j - 11)))));
-  } else if (B == 4) {
-    const int j = i % 8;
-    return __uint_as_float(j < 5 ? (w[i / 8] & (15u << (4 * j))) : (h[i / 8] & (15u << (4 * (j - 5)))));
-  } else {
-    return __uint_as_float(__byte_perm(w[i / 4], 0u, 0x4440u | (i % 4)));
-  }
-}
-// d = a * b + c on two fp32 lanes at once (packed fp32 FMA, round to nearest).
-__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-
-// The words' high parts (codes past the binary32 mantissa, shifted down); NW words.
-template <int B, int NW>
-__device__ __forceinline__ void high_parts(const uint32_t* w, uint32_t* h) {
-  constexpr int sh = B == 2 ? 22 : B == 4 ? 20 : 16;
-#pragma unroll
-  for (int k = 0; k < NW; ++k) h[k] = w[k] >> sh;
-}
-
-// x *= f on pairs of fp32 lanes (packed multiply)
-__device__ __forceinline__ void fmul2_inplace(float& x0, float& x1, float f0, float f1) {
-  const float2 r = __fmul2_rn(make_float2(x0, x1), make_float2(f0, f1));
-  x0 = r.x;
-  x1 = r.y;
-}
-
 // 2^x with the hardware approximation (relative error about 2^-22; results below the
 // binary32 normal range flush to zero, far below a softmax sum's resolution).
 __device__ __forceinline__ float fast_exp2(float x) {
@@ -156,12 +118,6 @@ __device__ __forceinline__ float fast_exp2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-
-template <int E>
-struct LaneState {
-  float m, l, zacc;  // running max (log2), sum of weights, sum of p*z (V zero points)
-  float acc[E];      // sum of p*v over the lane's E dims, scaled by 2^-49
-};
 
 // Shared-memory loads at 32-bit shared addresses.  Volatile: they stay after the
 // mbarrier wait that makes the bytes valid.
@@ -187,241 +143,6 @@ __device__ __forceinline__ uint32_t lds32(uint32_t a) {
   uint32_t v;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
   return v;
-}
-
-// The factors that move a lane's query and V accumulators between the domains of two
-// width classes, element by element (E = 32 elements per lane): row from * 4 + to.  One
-// table read by every class change keeps a single copy of the code in the consumer's
-// loop (a switch over templated copies made the loop several kilobytes larger).  Each
-// CTA of the CUDA-core kernels writes the table into its shared memory before the wait
-// on the previous kernel, and a class change reads its row with warp-wide broadcast
-// loads (from constant memory, whose cache misses, a switch took about 470 cycles).
-struct RescaleTable {
-  float q[16][32];    // query: 2^(qe(to, i) - qe(from, i))
-  float acc[16][32];  // V accumulators: 2^(ex(to, i) - ex(from, i)), ex = 0 at width 16
-};
-constexpr int kRescaleFloats = static_cast<int>(sizeof(RescaleTable) / 4);
-
-// Entry k of the table (k < kRescaleFloats), as the struct lays it out.
-__device__ __forceinline__ float rescale_entry(int k) {
-  const bool is_acc = k >= 16 * 32;
-  const int row = (k >> 5) & 15, i = k & 31, bf = bits_of_class(row >> 2), bt = bits_of_class(row & 3);
-  const int e = is_acc ? (bt == 16 ? 0 : ex_of(bt, i)) - (bf == 16 ? 0 : ex_of(bf, i)) : qe_of(bt, i) - qe_of(bf, i);
-  return pow2f(e);
-}
-
-// qp and acc from the domain of class `from` to that of class `to`; tbl: the table's
-// shared-memory address.
-template <int E>
-__device__ __forceinline__ void rescale_dyn(float (&qp)[E], float (&acc)[E], int from, int to, uint32_t tbl) {
-  static_assert(E == 32, "one factor per element of a lane's 32");
-  const uint32_t qf = tbl + (from * 4 + to) * 128, af = qf + 16 * 32 * 4;
-#pragma unroll
-  for (int i = 0; i < E; i += 4) {
-    const uint4 fq = lds128(qf + 4 * i), fa = lds128(af + 4 * i);
-    fmul2_inplace(qp[i], qp[i + 1], __uint_as_float(fq.x), __uint_as_float(fq.y));
-    fmul2_inplace(qp[i + 2], qp[i + 3], __uint_as_float(fq.z), __uint_as_float(fq.w));
-    fmul2_inplace(acc[i], acc[i + 1], __uint_as_float(fa.x), __uint_as_float(fa.y));
-    fmul2_inplace(acc[i + 2], acc[i + 3], __uint_as_float(fa.z), __uint_as_float(fa.w));
-  }
-}
-// acc from class `from`'s domain back to class 16's (the common one of the merge)
-template <int E>
-__device__ __forceinline__ void acc_to_neutral(float (&acc)[E], int from, uint32_t tbl) {
-  const uint32_t af = tbl + 16 * 32 * 4 + (from * 4 + 3) * 128;
-#pragma unroll
-  for (int i = 0; i < E; i += 4) {
-    const uint4 fa = lds128(af + 4 * i);
-    fmul2_inplace(acc[i], acc[i + 1], __uint_as_float(fa.x), __uint_as_float(fa.y));
-    fmul2_inplace(acc[i + 2], acc[i + 3], __uint_as_float(fa.z), __uint_as_float(fa.w));
-  }
-}
-
-
-// The NW words of a lane's codes at shared address a (4 NW-byte aligned), in as few
-// loads as possible (one 4-, 8- or 16-byte load per row part keeps the warp's request
-// conflict-free).
-template <int NW>
-__device__ __forceinline__ void lds_codes(uint32_t a, uint32_t* w) {
-  if (NW == 1) {
-    w[0] = lds32(a);
-  } else if (NW == 2) {
-    const uint2 u = lds64(a);
-    w[0] = u.x; w[1] = u.y;
-  } else {
-#pragma unroll
-    for (int k = 0; k < NW; k += 4) {
-      const uint4 u = lds128(a + 4 * k);
-      w[k] = u.x; w[k + 1] = u.y; w[k + 2] = u.z; w[k + 3] = u.w;
-    }
-  }
-}
-
-// One page of width class B (P = NIT * keys per iteration tokens) at shared address s0;
-// lane -> (key kl, 32-dim part).  Keys past `fill` are empty slots; with positions at
-// spos (masked pages), keys outside [lo, hi] are masked too.
-// A lane's q-th 16-byte chunk of a key's 8- or 16-bit row in a swizzled slice: the row
-// part it reads starts at chunk c0 of its 128-byte line, whose chunks are stored in the
-// order chunk ^ xm (xm: the line's index mod 8; see swz_off).
-__device__ __forceinline__ uint32_t swz_chunk(uint32_t a, int c0, int xm, int q) {
-  return a + static_cast<uint32_t>((((c0 + q) ^ xm) - c0) * 16);
-}
-
-// q.k of one key at shared address ka (this lane's E dims) in class B, with its (s, z)
-// word at kszaddr for B < 16: s * sum(q_i c_i) + z * sum(q_i) in the domain of qp.
-template <int B, int E>
-__device__ __forceinline__ float k_dot(uint32_t ka, uint32_t kszaddr, const float (&qp)[E], float sumq, int c0, int xm) {
-  float2 d2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  if (B == 16) {
-#pragma unroll
-    for (int q = 0; q < E / 8; ++q) {
-      const uint4 u = lds128(swz_chunk(ka, c0, xm, q));
-      d2[0] = ffma2(make_float2(qp[8 * q + 0], qp[8 * q + 1]), make_float2(bf_lo(u.x), bf_hi(u.x)), d2[0]);
-      d2[1] = ffma2(make_float2(qp[8 * q + 2], qp[8 * q + 3]), make_float2(bf_lo(u.y), bf_hi(u.y)), d2[1]);
-      d2[0] = ffma2(make_float2(qp[8 * q + 4], qp[8 * q + 5]), make_float2(bf_lo(u.z), bf_hi(u.z)), d2[0]);
-      d2[1] = ffma2(make_float2(qp[8 * q + 6], qp[8 * q + 7]), make_float2(bf_lo(u.w), bf_hi(u.w)), d2[1]);
-    }
-    return (d2[0].x + d2[0].y) + (d2[1].x + d2[1].y);
-  }
-  constexpr int NW = E * B / 32;
-  uint32_t w[NW], h[NW];
-  if (B == 8) {  // two chunks of the swizzled row
-#pragma unroll
-    for (int q = 0; q < NW / 4; ++q) {
-      const uint4 u = lds128(swz_chunk(ka, c0, xm, q));
-      w[4 * q] = u.x; w[4 * q + 1] = u.y; w[4 * q + 2] = u.z; w[4 * q + 3] = u.w;
-    }
-  } else {
-    lds_codes<NW>(ka, w);
-  }
-  if (B != 8) high_parts<B, NW>(w, h);
-  const uint32_t szw = lds32(kszaddr);
-#pragma unroll
-  for (int i = 0; i < E / 2; ++i)
-    d2[i & 1] = ffma2(make_float2(qp[2 * i], qp[2 * i + 1]),
-                      make_float2(code_at<B>(w, h, 2 * i), code_at<B>(w, h, 2 * i + 1)), d2[i & 1]);
-  const float2 sz = __half22float2(*reinterpret_cast<const __half2*>(&szw));  // (s, z)
-  return fmaf(sz.x * pow2f(49), (d2[0].x + d2[0].y) + (d2[1].x + d2[1].y), sz.y * sumq);
-}
-
-// acc += p * v for one key's V at shared address va (this lane's E dims) in class B,
-// with its (s, z) word at vszaddr for B < 16.
-template <int B, int E>
-__device__ __forceinline__ void v_acc(uint32_t va, uint32_t vszaddr, float p, LaneState<E>& st, int c0, int xm) {
-  if (B == 16) {
-    const float wv = p * pow2f(-49);
-    const float2 w2 = make_float2(wv, wv);
-#pragma unroll
-    for (int q = 0; q < E / 8; ++q) {
-      const uint4 u = lds128(swz_chunk(va, c0, xm, q));
-      const uint32_t uw[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const int i = 8 * q + 2 * h;
-        const float2 r = ffma2(w2, make_float2(bf_lo(uw[h]), bf_hi(uw[h])), make_float2(st.acc[i], st.acc[i + 1]));
-        st.acc[i] = r.x;
-        st.acc[i + 1] = r.y;
-      }
-    }
-    return;
-  }
-  constexpr int NW = E * B / 32;
-  uint32_t w[NW], h[NW];
-  if (B == 8) {  // two chunks of the swizzled row
-#pragma unroll
-    for (int q = 0; q < NW / 4; ++q) {
-      const uint4 u = lds128(swz_chunk(va, c0, xm, q));
-      w[4 * q] = u.x; w[4 * q + 1] = u.y; w[4 * q + 2] = u.z; w[4 * q + 3] = u.w;
-    }
-  } else {
-    lds_codes<NW>(va, w);
-  }
-  if (B != 8) high_parts<B, NW>(w, h);
-  const uint32_t szw = lds32(vszaddr);
-  const float2 sz = __half22float2(*reinterpret_cast<const __half2*>(&szw));  // (s, z)
-  const float wb = p * sz.x * pow2f(100);
-  const float2 w2 = make_float2(wb, wb);
-#pragma unroll
-  for (int i = 0; i < E; i += 2) {
-    const float2 r = ffma2(w2, make_float2(code_at<B>(w, h, i), code_at<B>(w, h, i + 1)),
-                           make_float2(st.acc[i], st.acc[i + 1]));
-    st.acc[i] = r.x;
-    st.acc[i + 1] = r.y;
-  }
-  st.zacc = fmaf(p, sz.y, st.zacc);
-}
-
-// One page of width class B (P = NIT * keys per iteration tokens) at shared address s0;
-// lane -> (key kl, E-dim part), and two keys per lane per iteration (kl and kl + KPI)
-// when NIT is even, so that their dependency chains overlap.  Keys past `fill` are
-// empty slots; with positions at spos (masked pages), keys outside [lo, hi] are masked,
-// and with HM (per-head modes) the slots whose bit in pm is clear (the token does not
-// store this KV head).
-template <int D, int B, int NIT, int E, bool HM>
-__device__ __forceinline__ void consume_page(uint32_t s0, uint32_t spos, bool masked, uint64_t pm, int G, int fill,
-                                             int lo, int hi, const float (&qp)[E], float sumq, LaneState<E>& st,
-                                             int lane) {
-  constexpr int LPK = D / E;
-  constexpr int KPI = 32 / LPK;
-  constexpr int P = NIT * KPI;
-  constexpr int KP = 1;  // keys per lane per iteration (one: half the code of two, which the
-                         // instruction cache favours over the second key's overlap)
-  constexpr int rowb = B == 16 ? 2 * D : D * B / 8;  // bytes of one key's row of K (or V)
-  const int part = lane % LPK, kl = lane / LPK;
-  const int lg = __ffs(G) - 1;  // G is a power of two: shifts, not divisions
-  const int ng = D >> lg;
-  const int grp = (part * E) >> lg;
-  const uint32_t krow = s0 + kl * rowb + part * (E * B / 8);   // this lane's K bytes, key kl
-  // 8- and 16-bit rows are swizzled (every cache of this consumer): the lane's first chunk
-  // in its line and the line's index mod 8 (the same for every key it reads, as a key
-  // group spans a multiple of 8 lines, and for the V rows, which start on such a line)
-  const int o0 = kl * rowb + part * (E * B / 8);
-  const int c0 = (o0 >> 4) & 7, xm = B >= 8 ? (o0 >> 7) & 7 : 0;
-  const uint32_t ksz = s0 + 2 * P * rowb + (kl * ng + grp) * 4;  // its (s, z), key kl
-  const uint32_t szstep = KPI * ng * 4;
-#pragma unroll 1
-  for (int it = 0; it < NIT && it * KPI < fill; it += KP) {  // key groups past the fill hold nothing
-    bool valid[KP];
-    float dot[KP];
-#pragma unroll
-    for (int k = 0; k < KP; ++k) {
-      const int key = (it + k) * KPI + kl;
-      valid[k] = key < fill;
-      if (HM) valid[k] = valid[k] && ((pm >> key) & 1ull);
-      if (masked) {
-        const int pos = static_cast<int>(lds32(spos + 4 * key));
-        valid[k] = valid[k] && pos >= lo && pos <= hi;
-      }
-      dot[k] = k_dot<B, E>(krow + (it + k) * KPI * rowb, ksz + (it + k) * szstep, qp, sumq, c0, xm);
-    }
-#pragma unroll
-    for (int k = 0; k < KP; ++k) {
-#pragma unroll
-      for (int o = 1; o < LPK; o <<= 1) dot[k] += __shfl_xor_sync(0xffffffffu, dot[k], o);
-    }
-    // online softmax over the lane's keys: one lazy rescale for both
-    float top = kNegInf;
-#pragma unroll
-    for (int k = 0; k < KP; ++k)
-      if (valid[k]) top = fmaxf(top, dot[k]);
-    if (top > st.m + kTau) {
-      const float alpha = fast_exp2(st.m - top);  // 0 when m = -inf
-#pragma unroll
-      for (int j = 0; j < E; ++j) st.acc[j] *= alpha;
-      st.l *= alpha;
-      st.zacc *= alpha;
-      st.m = top;
-    }
-#pragma unroll
-    for (int k = 0; k < KP; ++k) {
-      if (valid[k]) {
-        const float p = fast_exp2(dot[k] - st.m);
-        st.l += p;
-        const uint32_t va = krow + (it + k) * KPI * rowb + P * rowb;
-        v_acc<B, E>(va, ksz + (it + k) * szstep + P * ng * 4, p, st, c0, xm);
-      }
-    }
-  }
 }
 
 // -------------------------------------------------------------------- kernel --
@@ -534,6 +255,7 @@ __device__ __forceinline__ int query_mode(const AttnKernelArgs& ka, int q, bool&
   const uint8_t* row = ka.modes + static_cast<int64_t>(q) * ka.a.Hq;
   int m = 0;
   any_local = false;
+#pragma unroll 1
   for (int h = 0; h < ka.a.Hq; ++h) {
     const int v = row[h];
     m = max(m, v);
@@ -559,7 +281,7 @@ __device__ __forceinline__ int query_range(int t, int mode, int w) {
 // (mbarriers need 8, bulk-copy destinations 16).
 __host__ __device__ constexpr int align16(int x) { return (x + 15) & ~15; }
 struct AttnSmem {
-  int ring, recs, sbytes, full, empty, scr, pre, ent, red, resc, flag, total;
+  int ring, recs, sbytes, full, empty, scr, pre, ent, red, flag, total;
   __host__ __device__ AttnSmem(int ring_bytes, int n, int scr_floats, int fused)
       : ring(0),
         recs(align16(ring_bytes)),
@@ -570,9 +292,7 @@ struct AttnSmem {
         pre(scr + align16(kNcw * scr_floats * 4)),
         ent(pre + align16(4 * (n + 2))),
         red(ent + (fused ? align16(4 * step_ints(n)) : 0)),
-        resc(red + 16 * 8),  // the class-change factors (CUDA-core consumers, which have no scratch)
-        flag(resc + (scr_floats == 0 ? 4 * kRescaleFloats : 0)),  // the abort flag; at flag + 8
-                                                                    // the entry table's readiness mbarrier
+        flag(red + 16 * 8),  // the abort flag; at flag + 8 the entry table's readiness mbarrier
         total(flag + 16) {}
 };
 
@@ -605,7 +325,7 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
 }
 
 // Pages of split sp (of ns) of a query of sequence seq over key positions [lo, t]:
-// returns their number T (<= kItemMaxPages + 4); lane j < T gets page j's id in wid,
+// returns their number T (<= kItemMaxTiles); lane j < T gets page j's id in wid,
 // class | fill << 2 | kMask in wmeta and, when wfirst / wlast are given, the page's first
 // and last positions.  Pages are listed class by class, each class's in
 // position order; split sp of ns takes np / ns of a class's np pages in range, one more
@@ -620,7 +340,7 @@ __device__ __forceinline__ int plan_split(const LayerArgs& a, int P, int seq, in
   int pages[kClasses], first[kClasses], end[kClasses];
 #pragma unroll
   for (int c = 0; c < kClasses; ++c) {
-    pages[c] = (nt[c] + P - 1) / P;
+    pages[c] = (nt[c] + P - 1) >> (__ffs(P) - 1);  // P: a power of two
     first[c] = 0;
     end[c] = pages[c];
   }
@@ -636,17 +356,26 @@ __device__ __forceinline__ int plan_split(const LayerArgs& a, int P, int seq, in
   if (lo > 0) warp_count_below<kClasses>(a.plast + row0, a.MP, pages, lo, first, lane);
   if (upper_mask) warp_count_below<kClasses>(a.pfirst + row0, a.MP, pages, t + 1, end, lane);
   int beg[kClasses], tc[kClasses], npr[kClasses];
+  const float rns = 1.f / static_cast<float>(ns);
   int T = 0;
 #pragma unroll
   for (int c = 0; c < kClasses; ++c) {
     npr[c] = max(0, end[c] - first[c]);
-    const unsigned each = static_cast<unsigned>(npr[c]) / static_cast<unsigned>(ns);
-    const int extra = npr[c] - static_cast<int>(each) * ns;
-    beg[c] = first[c] + sp * static_cast<int>(each) + min(sp, extra);
-    tc[c] = static_cast<int>(each) + (sp < extra ? 1 : 0);
+    // npr / ns: the binary32 quotient is within one of it (npr < 2^20)
+    int each = static_cast<int>(static_cast<float>(npr[c]) * rns);
+    int extra = npr[c] - each * ns;
+    if (extra < 0) {
+      --each;
+      extra += ns;
+    } else if (extra >= ns) {
+      ++each;
+      extra -= ns;
+    }
+    beg[c] = first[c] + sp * each + min(sp, extra);
+    tc[c] = each + (sp < extra ? 1 : 0);
     T += tc[c];
   }
-  T = min(T, kItemMaxPages + kClasses);  // the split bound keeps T within this
+  T = min(T, kItemMaxTiles);  // the split bound keeps T within this
   wid = -1;
   wmeta = 0;
   // lanes take the pages class by class from the widest (bf16) down: the largest copies
@@ -746,7 +475,7 @@ __device__ __forceinline__ void plan_units(const AttnKernelArgs& ka, int P, int 
   const int q0 = min(n, static_cast<int>(threadIdx.x) * chunk), q1 = min(n, q0 + chunk);
   int mine = 0;
   for (int q = q0; q < q1; ++q) {  // pre[q] becomes the query's split count
-    const int ns = splits_of(pre[q], pos_split, P, a.s_cap);
+    const int ns = splits_of(pre[q], pos_split, a.split_keys, a.split_extra, a.split_most, a.s_cap);
     pre[q] = ns;
     mine += ns;
   }
@@ -880,19 +609,25 @@ static __device__ void plan_entries(const AttnKernelArgs& ka, int* ent) {
   consumers_sync();
 }
 
+// One warp, the pools' page counters known: the first opener beyond its pool's capacity
+// (OUT_OF_PAGES) as a call error.
+__device__ __forceinline__ void step_pages_error(const AttnKernelArgs& ka, int* ent, int lane) {
+  int* sc = ent + 6 * ka.n;
+  for (int e = lane; e < ka.n; e += 32) {
+    const int tok = ent[2 * e], info = ent[2 * e + 1], c = info & 3;
+    if (tok >= 0 && (info & 4) && sc[kSNextPage + c] + (info >> 3) >= ka.a.cap[c])
+      atomicMin(&sc[kSErr], e * 16 + TRR_ERR_OUT_OF_PAGES);
+  }
+}
+
 // One warp, after the wait on the previous kernel: the pools' page counters, and the
 // first opener beyond its pool's capacity (OUT_OF_PAGES) as a call error.
 __device__ __forceinline__ void step_after_wait(const AttnKernelArgs& ka, int* ent, int lane) {
   const LayerArgs& a = ka.a;
-  const int n = ka.n;
-  int* sc = ent + 6 * n;
+  int* sc = ent + 6 * ka.n;
   if (lane < 4) sc[kSNextPage + lane] = a.ctrl[kNextPage + lane];
   __syncwarp();
-  for (int e = lane; e < n; e += 32) {
-    const int tok = ent[2 * e], info = ent[2 * e + 1], c = info & 3;
-    if (tok >= 0 && (info & 4) && sc[kSNextPage + c] + (info >> 3) >= a.cap[c])
-      atomicMin(&sc[kSErr], e * 16 + TRR_ERR_OUT_OF_PAGES);
-  }
+  step_pages_error(ka, ent, lane);
   __syncwarp();
 }
 
@@ -976,7 +711,8 @@ __device__ __forceinline__ void step_token_rows(const AttnKernelArgs& ka, uint2 
   bool bad = false;
 #pragma unroll 1
   for (int kv = 0; kv < 2; ++kv) {
-    const RowCodes r = quantise_row_codes<D>(kv ? rv : rk, b, a.G, lane);
+    float xq[D / 32];
+    const RowCodes r = quantise_row_codes<D>(kv ? rv : rk, b, a.G, lane, xq);
     bad |= r.bad;
     const int coff = (kv * P + slot) * rowb, soff = 2 * P * rowb + kv * P * ng * 4;
     if (own) {
@@ -1063,7 +799,6 @@ struct CtaRing {
   uint64_t* empty;
   volatile int* abort_flag;
   uint64_t* ent_ready;  // decode step: completes when the consumers have built the entry table
-  uint32_t resc;        // shared address of the class-change factors (CUDA-core kernels)
   int R;
 };
 
@@ -1288,7 +1023,7 @@ __device__ __forceinline__ void run_producer(const AttnKernelArgs& ka, int P, in
       // per-head modes, a block of local and skip heads in a query whose widest head is
       // full: the block's own split count, from its window; its splits past that have
       // nothing to do, and its heads merge that many partials
-      ns = min(ns, splits_of(query_range(t, TRR_MODE_LOCAL, w), pre[n + 1], P, a.s_cap));
+      ns = min(ns, splits_of(query_range(t, TRR_MODE_LOCAL, w), pre[n + 1], a.split_keys, a.split_extra, a.split_most, a.s_cap));
       if (sp >= ns) {
         __syncwarp();
         take_next();
@@ -1573,11 +1308,12 @@ __device__ __forceinline__ void merge_partials(const float* p0, int64_t stride, 
   // Chunks of CH partials: each chunk's (max, sum) words and rows are loaded together
   // (one round trip to L2 for up to CH splits), then folded into the running result;
   // CH keeps the rows within the registers the consumers have free at this point.
-  constexpr int DPL = D / 32, CH = D == 64 ? 8 : 4;
+  constexpr int DPL = D / 32, CH = D == 64 ? 16 : 8;
   Mx = kNegInf;
   float lsum = 0.f;  // lane s: the weighted sums of the partials it reads the words of
 #pragma unroll
   for (int j = 0; j < DPL; ++j) acc_o[j] = 0.f;
+#pragma unroll 1
   for (int s0 = 0; s0 < count; s0 += CH) {
     const int cnt = min(CH, count - s0);
     float2 ml = make_float2(kNegInf, 0.f);
@@ -1674,189 +1410,6 @@ __device__ __forceinline__ void store_or_merge(const AttnKernelArgs& ka, const f
   for (int j = 0; j < DPL; j += 2)
     *reinterpret_cast<__nv_bfloat162*>(ka.out + orow + lane * DPL + j) =
         __floats2bfloat162_rn(acc_o[j] * inv, acc_o[j + 1] * inv);
-}
-
-// ------------------------------------------------- CUDA-core consumer (MHA) --
-// Warp cw computes query head (block * kNcw + cw): lane pair (key, half) of a 64-wide
-// head (four lanes for 128) dequantises in registers and keeps its own online softmax.
-
-// The end of a unit for a CUDA-core consumer: merge the lanes' states, then store.
-template <int D, int E>
-__device__ __forceinline__ void finish_unit(const AttnKernelArgs& ka, LaneState<E>& st, int cur_cls, int sp, int qi,
-                                            int qh, int nsplit, int base, uint32_t tbl, int lane) {
-  constexpr int LPK = D / E;   // lanes per key
-  constexpr int DPL = D / 32;  // dimensions per lane after the merge
-  const int part = lane % LPK, kl = lane / LPK;
-  // rescale to the common maximum, then reduce-scatter over the key lanes: each
-  // halving step keeps half of the 32 dims and sends the other half to the partner
-  acc_to_neutral(st.acc, cur_cls, tbl);
-  float M = st.m;
-#pragma unroll
-  for (int o = LPK; o < 32; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-  const float f = (st.m == kNegInf) ? 0.f : fast_exp2(st.m - M);
-  float L = st.l * f;
-#pragma unroll
-  for (int o = LPK; o < 32; o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-  {
-    const float2 s49 = make_float2(pow2f(49) * f, pow2f(49) * f), zf = make_float2(st.zacc * f, st.zacc * f);
-#pragma unroll
-    for (int j = 0; j < E; j += 2) {
-      const float2 r = __ffma2_rn(make_float2(st.acc[j], st.acc[j + 1]), s49, zf);
-      st.acc[j] = r.x;
-      st.acc[j + 1] = r.y;
-    }
-  }
-#pragma unroll
-  for (int width = E / 2, o = 16; o >= LPK; width >>= 1, o >>= 1) {
-    const bool upper = lane & o;
-#pragma unroll
-    for (int i = 0; i < E / 2; ++i) {
-      if (i < width) {
-        const float keep = upper ? st.acc[width + i] : st.acc[i];
-        const float give = upper ? st.acc[i] : st.acc[width + i];
-        st.acc[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-      }
-    }
-  }
-  // lane (kl, part) now holds dims part*E + DPL*kl .. + DPL-1 in acc[0 .. DPL-1]
-  store_or_merge<D>(ka, st.acc, part * E + DPL * kl, M, L, sp, qi, qh, nsplit, base, lane);
-}
-
-template <int D, int P, int E, bool HM, bool STEP>
-__device__ __forceinline__ void run_consumer_cc(const AttnKernelArgs& ka, const CtaRing& cr, const int* ent, int cw,
-                                                int lane) {
-  constexpr int LPK = D / E;     // lanes per key
-  constexpr int KPI = 32 / LPK;  // keys per warp iteration
-  const LayerArgs& a = ka.a;
-  const int g = a.Hq / a.Hkv;
-  const int part = lane % LPK;
-  LaneState<E> st;
-  float qp[E];
-  float sumq = 0.f;
-  int cur_cls = 3;
-  st.m = kNegInf;
-  st.l = 0.f;
-  st.zacc = 0.f;
-#pragma unroll
-  for (int j = 0; j < E; ++j) st.acc[j] = 0.f;
-  // the current unit
-  int u_q = 0, u_h = 0, u_kvi = 0, u_lo = 0, u_hi = 0, u_sp = 0, u_ns = 1, u_base = 0;
-  bool u_local = false;  // per-head modes: this warp's head is local (it skips early pages)
-  bool active = false;
-  for (uint32_t s = 0;; ++s) {
-    const uint32_t slot = s % kStages;
-    const bool arrived = mbar_wait_or(&cr.full[slot], (s / kStages) & 1, cr.abort_flag, a.wait_ns);
-    if (!__all_sync(0xffffffffu, arrived)) {  // give up together, never half a warp
-      if (lane == 0) {
-        *cr.abort_flag = 1;
-        set_status(a.ctrl, TRR_ERR_TIMEOUT);
-        atomicExch(&a.lctl[kAborted], 1);
-      }
-      break;
-    }
-    const uint32_t rec = smem_u32(cr.recs) + slot * 48;
-    const int4 ra = lds128i(rec);
-    const int meta = ra.x;
-    if (meta & kEnd) break;
-    if (meta & kQRows) {
-      const int4 rb = lds128i(rec + 16);
-      const int qb = (meta >> 16) & 0x7fff;
-      u_h = qb * kNcw + cw;
-      active = u_h < a.Hq;
-      if (HM && active) {  // the head of this warp's slot (ranked by mode; or h0 + slot)
-        const int hsel = lds128i(rec + 32).w;
-        if (hsel >= 0) u_h = (hsel >> (8 * cw)) & 255;
-      }
-      u_kvi = u_h / g - (qb * kNcw) / g;
-      u_q = ra.z;
-      u_lo = ra.w;
-      u_hi = rb.x;
-      u_sp = rb.y;
-      u_ns = rb.z;
-      u_base = rb.w;
-      u_local = false;
-      if (STEP && active && u_sp == u_ns - 1) step_prefetch_rows<D>(ka, u_q, u_h / g, lane);
-      if (HM && active) {  // this head's own mode: {head modes, local lo}
-        const int4 rq = lds128i(rec + 32);
-        const int hm = (rq.x >> (2 * cw)) & 3;
-        if (hm == TRR_MODE_SKIP) {  // a zero row (written once, by split 0), no merge
-          if (u_sp == 0 && lane < D / 8)
-            reinterpret_cast<uint4*>(ka.out + (static_cast<int64_t>(u_q) * a.Hq + u_h) * D)[lane] =
-                make_uint4(0, 0, 0, 0);
-          active = false;
-        } else if (hm == TRR_MODE_LOCAL) {
-          u_lo = rq.y;
-          u_local = true;
-        }
-      }
-      cur_cls = 3;  // the neutral scale is class 16's
-      st.m = kNegInf;
-      st.l = 0.f;
-      st.zacc = 0.f;
-#pragma unroll
-      for (int j = 0; j < E; ++j) st.acc[j] = 0.f;
-      if (active && !(meta & kNoPage)) {
-        const uint32_t qa = smem_u32(cr.ring + ra.y + cw * D * 2 + part * E * 2);
-        const float2 qs2 = make_float2(ka.qscale, ka.qscale);
-        float2 sq2 = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int qq = 0; qq < E / 8; ++qq) {
-          const uint4 uq = lds128(qa + 16 * qq);
-          const uint32_t wv[4] = {uq.x, uq.y, uq.z, uq.w};
-#pragma unroll
-          for (int h = 0; h < 4; ++h) {
-            const float2 r = __fmul2_rn(make_float2(bf_lo(wv[h]), bf_hi(wv[h])), qs2);
-            qp[8 * qq + 2 * h] = r.x;
-            qp[8 * qq + 2 * h + 1] = r.y;
-            sq2 = __fadd2_rn(sq2, r);
-          }
-        }
-        sumq = sq2.x + sq2.y;
-      }
-    } else if (active) {
-      const int4 rc = lds128i(rec + 32);
-      const int nks = rc.y & 255, npg = rc.y >> 8;  // KV slices per page, pages of the stage
-      // per-head modes: the stage brings one slice per slot of its mask (rc.x), in slot
-      // order; otherwise KV slices rc.x .. rc.x + nks - 1 of the block
-      const bool mine = HM ? ((static_cast<unsigned>(rc.x) >> cw) & 1u) != 0 : (u_kvi >= rc.x && u_kvi < rc.x + nks);
-      if (mine && !(HM && u_local && (meta & kEarly))) {
-        const int cls = meta & 3, fill = (meta >> 2) & 127;  // the last page's fill; the others are full
-        if (STEP && rc.z == kNewRows) {  // the query's own token: this warp's KV head (warps that
-                                         // share a KV head write the same bytes); the keys past
-                                         // the fill that consume_page reads are never used
-          const int j = u_h / g;
-          step_new_rows<D>(ka, ent, u_q, j, j * g >= u_h - cw, smem_u32(cr.ring + ra.y + (u_kvi - rc.x) * rc.w), lane);
-        }
-        if (cls != cur_cls) {
-          rescale_dyn(qp, st.acc, cur_cls, cls, cr.resc);
-          cur_cls = cls;
-        }
-        const bool masked = meta & kMask;
-        for (int pg = 0; pg < npg; ++pg) {
-          const int idx = HM ? __popc(static_cast<unsigned>(rc.x) & ((1u << cw) - 1u)) : u_kvi - rc.x;
-          const uint32_t s0 = smem_u32(cr.ring + ra.y + (pg * nks + idx) * rc.w);
-          const int f = pg == npg - 1 ? fill : P;
-          const uint32_t sp = masked ? smem_u32(cr.ring + rc.z) : s0;
-          uint64_t pm = ~0ull;  // per-head modes: this KV head's presence mask, which ends
-                                // its slice
-          if (HM) {
-            const uint2 m2 = lds64(s0 + rc.w - a.maskb);
-            pm = (static_cast<uint64_t>(m2.y) << 32) | m2.x;
-          }
-          switch (cls) {
-            case 0: consume_page<D, 2, P / KPI, E, HM>(s0, sp, masked, pm, a.G, f, u_lo, u_hi, qp, sumq, st, lane); break;
-            case 1: consume_page<D, 4, P / KPI, E, HM>(s0, sp, masked, pm, a.G, f, u_lo, u_hi, qp, sumq, st, lane); break;
-            case 2: consume_page<D, 8, P / KPI, E, HM>(s0, sp, masked, pm, a.G, f, u_lo, u_hi, qp, sumq, st, lane); break;
-            default: consume_page<D, 16, P / KPI, E, HM>(s0, sp, masked, pm, a.G, f, u_lo, u_hi, qp, sumq, st, lane); break;
-          }
-        }
-      }
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&cr.empty[slot]);  // the stage's bytes are read
-    if ((meta & kLast) && active)
-      finish_unit<D, E>(ka, st, cur_cls, u_sp, u_q, u_h, u_ns, u_base, cr.resc, lane);
-  }
 }
 
 // ------------------------------------------------ tensor-core consumer (GQA) --
@@ -2404,14 +1957,8 @@ __device__ __forceinline__ CtaRing attn_prologue(const AttnKernelArgs& ka, uint8
   cr.empty = reinterpret_cast<uint64_t*>(smem + lay.empty);
   cr.abort_flag = reinterpret_cast<volatile int*>(smem + lay.flag);
   cr.ent_ready = reinterpret_cast<uint64_t*>(smem + lay.flag + 8);
-  cr.resc = smem_u32(smem + lay.resc);
   cr.R = ka.ring_bytes;
   pre = reinterpret_cast<int*>(smem + lay.pre);
-  if (ka.scr_floats == 0) {  // the CUDA-core consumers' class-change factors (the unit plan's
-                             // barriers order these writes before any read)
-    float* t = reinterpret_cast<float*>(smem + lay.resc);
-    for (int k = threadIdx.x; k < kRescaleFloats; k += blockDim.x) t[k] = rescale_entry(k);
-  }
   if (threadIdx.x == 0) {
 #pragma unroll 1
     for (int i = 0; i < kStages; ++i) {
@@ -2475,21 +2022,6 @@ __device__ __forceinline__ void attn_epilogue(const AttnKernelArgs& ka, const in
     }
   }
   if (!s_aborted) step_commit(ka, ent);  // a call that gave up a wait stores nothing
-}
-
-// CUDA-core path: units of kNcw query heads, one per consumer warp; HM: per-head modes
-// (presence masks read with every page).
-template <int D, int P, bool HM, bool STEP>
-__global__ void __launch_bounds__(32 * (kNcw + 1), cc_ctas_per_sm(D))
-    attn_kernel(const __grid_constant__ AttnKernelArgs ka) {
-  extern __shared__ __align__(128) uint8_t smem[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int NQB = (ka.a.Hq + ka.hpu - 1) / ka.hpu;
-  int *pre, *ent;
-  const CtaRing cr = attn_prologue<STEP>(ka, smem, P, NQB, pre, ent);
-  if (warp == 0) run_producer<D, STEP, HM>(ka, P, NQB, pre, ent, cr, lane);
-  else run_consumer_cc<D, P, cc_elems(D), HM, STEP>(ka, cr, ent, warp - 1, lane);
-  attn_epilogue<STEP>(ka, ent);
 }
 
 // Tensor-core path: units of kNcw KV heads with all their query heads.
@@ -2598,23 +2130,21 @@ __global__ void __launch_bounds__(32 * kCombineWarps) attn_combine_kernel(const 
 // ------------------------------------------------------------- launchers --
 // One translation unit per kernel family (compiled side by side): each launches its
 // instances with programmatic dependent launch and sets their shared-memory limit.
-//   attn_cc:          CUDA-core kernels of trr_decode_attn (one mode per query)
-//   attn_head_modes:  CUDA-core kernels of caches with per-head modes
-//   attn_mma:         tensor-core kernels of trr_decode_attn and the combine kernel
-//   attn_step_cc / attn_step_mma: the decode-step kernels (trr_decode_step)
-cudaError_t launch_attn_cc(const Layout& l, dim3 grid, dim3 block, size_t smem, cudaStream_t s, const AttnKernelArgs& k);
-cudaError_t launch_attn_head_modes(const Layout& l, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                   const AttnKernelArgs& k);
+//   attn_row, attn_row_heads, attn_row_step: one query head per warp (trr_row.cuh), for
+//                     trr_decode_attn, caches with per-head modes and trr_decode_step
+//   attn_mma:         query-group kernels of trr_decode_attn and the combine kernel
+//   attn_step_mma:    query-group kernels of trr_decode_step
+cudaError_t launch_attn_row(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k);
+cudaError_t launch_attn_row_heads(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k);
+cudaError_t launch_attn_row_step(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k);
 cudaError_t launch_attn_mma(const Layout& l, dim3 grid, dim3 block, size_t smem, cudaStream_t s, const AttnKernelArgs& k);
-cudaError_t launch_attn_step_cc(const Layout& l, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                const AttnKernelArgs& k);
 cudaError_t launch_attn_step_mma(const Layout& l, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                  const AttnKernelArgs& k);
 cudaError_t launch_attn_combine(int d, dim3 grid, dim3 block, cudaStream_t s, const CombineArgs& ca);
-cudaError_t configure_attn_cc();
-cudaError_t configure_attn_head_modes();
+cudaError_t configure_attn_row();
+cudaError_t configure_attn_row_heads();
+cudaError_t configure_attn_row_step();
 cudaError_t configure_attn_mma();
-cudaError_t configure_attn_step_cc();
 cudaError_t configure_attn_step_mma();
 
 }  // namespace trr

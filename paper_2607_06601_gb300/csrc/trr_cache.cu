@@ -19,6 +19,7 @@ LayerArgs layer_args(const Layout& l, const Views& v, int layer) {
   a.S = l.S; a.Hq = l.Hq; a.Hkv = l.Hkv; a.d = l.d; a.G = l.G; a.P = l.P;
   a.maxctx = l.maxctx; a.MP = l.MP; a.W32 = l.W32; a.units = l.units; a.pos_split = l.pos_split;
   a.s_cap = l.s_cap;
+  a.split_keys = l.split_keys; a.split_extra = l.split_extra; a.split_most = l.split_most;
   a.split_bytes = l.split_bytes; a.skip_writes_kv = l.skip_writes_kv;
   a.head_modes = l.head_modes; a.maskb = static_cast<int>(l.maskb); a.swz = l.swz;
   a.hdr = static_cast<int>(l.hdr);
@@ -92,7 +93,18 @@ static trr_status make_layout(const trr_cache_config* c, Layout* l) {
   // tokens), and few enough pages per split for any range up to max_context
   l->pos_split = static_cast<int>(std::max<int64_t>(l->P, l->split_bytes / l->tokb[2]));
   l->s_cap = 1 << 30;
-  l->s_cap = std::max(splits_of(l->maxctx, l->pos_split, l->P, l->s_cap), 1);
+  // tiles: whole pages, or with one query head per warp up to 32 keys of one (16 of the
+  // widest rows)
+  l->split_keys = l->P;
+  l->split_extra = kClasses;
+  l->split_most = kItemMaxTiles - kClasses;
+  if (l->swz) {
+    const int most = std::min(l->P, 32), wide = std::min(l->P, l->d == 128 ? 16 : 32);
+    l->split_keys = wide;
+    l->split_extra = 3 * (l->P / most) + l->P / wide;
+    l->split_most = kItemMaxTiles - l->split_extra;
+  }
+  l->s_cap = std::max(splits_of(l->maxctx, l->pos_split, l->split_keys, l->split_extra, l->split_most, l->s_cap), 1);
   l->cnt_stride = 1 + (l->s_cap + kMergeGroup - 1) / kMergeGroup;
   l->max_items = static_cast<int64_t>(l->max_queries) * l->units * l->s_cap;
 

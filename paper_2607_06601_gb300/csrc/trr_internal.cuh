@@ -32,13 +32,13 @@ enum LayerCtrl : int {
   kLayerCtrlInts = 4
 };
 
-// Splits of one attention work unit are sized to hold at most this many pages (+ one
-// partial page per class), so that a warp holds an item's page ids one per lane.
-constexpr int kItemMaxPages = 28;
+// An attention work unit holds at most this many tiles (a page's keys, split_keys at a time),
+// so that a warp holds one per lane.
+constexpr int kItemMaxTiles = 32;
 
 // Split partials are merged in groups of this many (then the groups): a query with
 // ns splits per head has 1 + ceil(ns / kMergeGroup) arrival counters per head.
-constexpr int kMergeGroup = 16;
+constexpr int kMergeGroup = 32;
 
 // Byte layout of one cache (see include/trr.h for the documented part).
 struct Layout {
@@ -48,6 +48,8 @@ struct Layout {
   int swz;        // 8- and 16-bit code rows stored swizzled (caches of the CUDA-core consumer)
   int units;      // attention work units per query split (one per query head)
   int pos_split;  // key positions per split at least (split_bytes of 8-bit tokens)
+  int split_keys, split_extra, split_most;  // keys of a tile; tiles a range may have above what its
+                                            // keys fill; a split's share at most (splits_of)
   int s_cap;      // most splits one query is cut into
   int cnt_stride; // arrival counters per (query, head): 1 + ceil(s_cap / kMergeGroup)
   int64_t max_items;
@@ -56,14 +58,16 @@ struct Layout {
   int64_t off_cnt, off_part, off_pool[kClasses], total;
 };
 
-// Splits of a query whose key range spans `range` positions: at least pos_split
-// positions each, enough that no split holds more than kItemMaxPages + 4 pages, at most
-// s_cap (which covers the page bound for any range up to max_context).
-__host__ __device__ inline int splits_of(int range, int pos_split, int P, int s_cap) {
+// Splits of a query whose key range spans `range` positions: at least pos_split positions
+// each, enough that no split holds more than kItemMaxTiles tiles of `keys` keys, at most s_cap
+// (which covers that bound for any range up to max_context).  A range has up to 2 `extra`
+// tiles more than its keys fill (partly filled and cut pages of each class), a split up to
+// `most` of them: its share and what rounding adds.
+__host__ __device__ inline int splits_of(int range, int pos_split, int keys, int extra, int most, int s_cap) {
   if (range <= 0) return 1;
   const int by_len = (range + pos_split - 1) / pos_split;
-  const int by_pages = ((range + P - 1) / P + 2 * kClasses + kItemMaxPages - 1) / kItemMaxPages;
-  const int ns = by_len > by_pages ? by_len : by_pages;
+  const int by_tiles = ((range + keys - 1) / keys + 2 * extra + most - 1) / most;
+  const int ns = by_len > by_tiles ? by_len : by_tiles;
   return ns < s_cap ? ns : s_cap;
 }
 
@@ -119,7 +123,7 @@ inline Views make_views(const Layout& l, void* base) {
 
 // Everything a kernel needs about one layer of one cache, passed by value.
 struct LayerArgs {
-  int layer, S, Hq, Hkv, d, G, P, maxctx, MP, W32, units, pos_split, s_cap, cnt_stride, split_bytes, skip_writes_kv;
+  int layer, S, Hq, Hkv, d, G, P, maxctx, MP, W32, units, pos_split, split_keys, split_extra, split_most, s_cap, cnt_stride, split_bytes, skip_writes_kv;
   int head_modes;      // modes are [n][Hq]; each KV head's slice ends with its presence mask
   int swz;             // 8- and 16-bit code rows stored swizzled (see swz_off)
   uint64_t wait_ns;    // bound of an in-kernel wait before the kernel reports TRR_ERR_TIMEOUT
@@ -228,11 +232,14 @@ __device__ __forceinline__ bool mbar_test_at(uint32_t addr, uint32_t parity) {
   return done != 0;
 }
 
+// Limits below this are polled instead of waited for.
+constexpr uint64_t kShortWaitNs = 20000;
+
 // One try of a wait bounded by limit_ns: a suspending try (a try may last until the
 // phase completes), or, for a limit below the 20 us hint, a test that returns at once,
 // so that a short limit is kept.
 __device__ __forceinline__ bool mbar_poll(uint32_t addr, uint32_t parity, uint64_t limit_ns) {
-  return limit_ns >= 20000 ? mbar_try(addr, parity, 20000u) : mbar_test_at(addr, parity);
+  return limit_ns >= kShortWaitNs ? mbar_try(addr, parity, static_cast<uint32_t>(kShortWaitNs)) : mbar_test_at(addr, parity);
 }
 
 // Bounded wait for phase `parity` of `bar`: returns false once limit_ns have passed
@@ -310,8 +317,9 @@ struct RowCodes {
   int code_idx, sz_idx;
   bool bad;
 };
+// xq: the lane's values as stored (z + c * s), in binary32.
 template <int D>
-__device__ __forceinline__ RowCodes quantise_row_codes(const uint2 w, int b, int G, int lane) {
+__device__ __forceinline__ RowCodes quantise_row_codes(const uint2 w, int b, int G, int lane, float (&xq)[D / 32]) {
   constexpr int EPL = D / 32;
   float x[EPL];
   x[0] = bf16lo(w.x);
@@ -337,13 +345,18 @@ __device__ __forceinline__ RowCodes quantise_row_codes(const uint2 w, int b, int
   }
   const int levels = (1 << b) - 1;
   uint32_t val = 0, szw = 0;
+#pragma unroll
+  for (int i = 0; i < EPL; ++i) xq[i] = 0.f;
   if (!bad) {
     const __half z16 = __float2half_rn(mn);                                                    // z = min(x)
     const __half s16 = __float2half_rn(__fdiv_rn(__fsub_rn(mx, mn), static_cast<float>(levels)));  // s
     const float z = __half2float(z16), s = __half2float(s16), rs = __frcp_rn(s);
 #pragma unroll
-    for (int i = 0; i < EPL; ++i)
-      val |= static_cast<uint32_t>(s != 0.f ? code_of(x[i], z, s, rs, levels) : 0) << (i * b);
+    for (int i = 0; i < EPL; ++i) {
+      const int c = s != 0.f ? code_of(x[i], z, s, rs, levels) : 0;
+      val |= static_cast<uint32_t>(c) << (i * b);
+      xq[i] = fmaf(static_cast<float>(c), s, z);
+    }
     szw = static_cast<uint32_t>(__half_as_ushort(s16)) | (static_cast<uint32_t>(__half_as_ushort(z16)) << 16);
   }
   const int lpw = 5 - (__ffs(EPL * b) - 1), LPW = 1 << lpw;  // lanes sharing one 32-bit word of codes

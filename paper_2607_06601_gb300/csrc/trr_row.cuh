@@ -1,0 +1,1341 @@
+#pragma once
+// trr_row.cuh - the attention kernels of one query head per warp (MHA, wide query groups
+// and per-head modes): mode-routed split-K decode attention over the mixed-precision paged
+// cache (Sec. 3.2(A), Eq. 2; Sec. 3.8; Sec. 7).
+//
+// A work unit is (query, query head, split) and belongs to one warp from its plan to its
+// row: the warp plans the unit (trr_attn.cuh, plan_split), streams its pages' KV slices
+// through a ring of shared memory of its own with 1-D bulk copies (one per page as a rule,
+// cp.async.bulk + mbarrier), and computes on them.  Nothing but the call's start and end
+// synchronises warps: a producer warp that fed four consumer warps through one ring, as
+// the kernels had before, kept two stages in flight and held every stage until the slowest
+// of the four was done with it.
+//
+// One CTA of eight warps per SM takes less than half of its shared memory and registers, so
+// that the next layer's kernel is resident while this one runs: its plans and its first
+// page copies come before its wait on this kernel.
+//
+// The arithmetic runs on the tensor cores (mma.sync m16n8k16, f32 accumulation) though only
+// one query head shares a key, because the codes then need one mask per two elements (a
+// pair of codes in the halves of a word, read as f16 subnormals) in place of one per
+// element, and the multiply-adds come free:
+//   q.k   A = 16 keys' codes, B = the query row, its column n holding quantiser group
+//         n % NG (zero outside it); each lane then takes one key of a tile of 32 and adds
+//         up s * (group sum) + z * (group's query sum) in binary32.
+//   P.V   A = V^T codes paired along keys, B = p * s of the tile's keys, exchanged through
+//         shared memory: column (group, hi | lo), the weight split into two f16 parts
+//         (22 bits and the sign; scaled by a power of two per unit so that the largest
+//         parts are far from f16's limits), so that weights keep binary32's accuracy.
+//         Width 16 uses m16n8k8 with tf32 operands (bf16 values are exact in tf32), its
+//         weights split the same way.
+// The running maximum is the warp's, raised only when a score exceeds it by 2^8.
+#include <type_traits>
+
+#include "trr_attn.cuh"
+
+namespace trr {
+
+constexpr int kRowWarps = 8;   // warps per CTA
+constexpr int kRowSlots = 8;   // tiles a warp may have in flight
+constexpr int kRowCtasPerSm = 2;
+// A grid leaves num_sms / kRowSpare places of the chip free: the next layer's kernel then
+// starts, and plans, while the last CTAs of this one still run (with a full grid its last CTA
+// started, and planned for 3 us, only when this kernel had ended: 160M step 18.2 -> 16.8 us).
+constexpr int kRowSpare = 32;
+constexpr int kRowSmemLimit = 110 * 1024;
+constexpr float kLoScale = 2048.f;  // the low part of a weight is stored times 2^11
+
+constexpr int kRowRed = 8 * kRowWarps * 2 + 4 * 32;  // plan_rows' sums and counts
+struct RowSmem {  // byte offsets of one CTA's shared memory
+  int full, fac, q, w, pre, qinf, ord, red, ent, flag, ring, total;
+  __host__ __device__ RowSmem(int D, int NG, int n, int step, int ring_bytes)
+      : full(0),
+        fac(full + kRowWarps * kRowSlots * 8),
+        q(fac + 16 * (D / 8) * 4),
+        w(q + kRowWarps * D * 2),
+        pre(w + kRowWarps * row_w_bytes(NG)),
+        qinf(pre + align16(4 * (n + 2))),
+        ord(qinf + 16 * n),
+        red(ord + align16(2 * n)),
+        ent(red + kRowRed),
+        flag(ent + (step ? align16(4 * step_ints(n)) : 0)),
+        ring((flag + 16 + 127) & ~127),
+        total(ring + kRowWarps * ring_bytes) {}
+  // the weights of a tile: 32 rows of 8 f16 (width 16: of 2 tf32)
+  __host__ __device__ static constexpr int row_w_bytes(int) { return 512; }
+};
+
+// Rows (work units per query split): full heads, local heads and the others of a query.
+struct HeadCounts {
+  int full, local, skip;
+};
+__device__ __forceinline__ HeadCounts head_counts(const AttnKernelArgs& ka, int q) {
+  const uint8_t* row = ka.modes + static_cast<int64_t>(q) * ka.a.Hq;
+  HeadCounts c{0, 0, 0};
+#pragma unroll 1
+  for (int h = 0; h < ka.a.Hq; ++h) {
+    c.full += row[h] == TRR_MODE_FULL;
+    c.local += row[h] == TRR_MODE_LOCAL;
+  }
+  c.skip = ka.a.Hq - c.full - c.local;
+  return c;
+}
+
+// x / y for 0 <= x < 2^24, 0 < y < 2^24: the binary32 quotient is within one of it.
+__device__ __forceinline__ int div24(int x, int y) {
+  const int q = static_cast<int>(__fdividef(static_cast<float>(x), static_cast<float>(y)));
+  const int r = x - q * y;
+  return r < 0 ? q - 1 : r >= y ? q + 1 : q;
+}
+
+// The work units of a call, computed the same way by every CTA.  Queries are taken in the
+// order of their units' size (those that read everything, those that read a window, zero
+// rows), so that units handed out on demand end with short ones: place k holds query ord[k];
+// pre[k] numbers its first unit, pre[n] counts them all, pre[n + 1] is the call's key
+// positions per split; qinf[k] = {sequence, position, first key position (per-head modes: of
+// a local head), splits of a row (per-head modes: of a full head) | query error << 24 | zero
+// row << 28}.  A query has one unit per (row, split); with per-head modes each head its own
+// splits (one for a skip head, which writes its zero row).
+template <bool HM>
+__device__ __forceinline__ void plan_rows(const AttnKernelArgs& ka, int* pre, int4* qinf, uint16_t* ord, long long* red) {
+  const LayerArgs& a = ka.a;
+  const int n = ka.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int* counts = reinterpret_cast<int*>(red + 2 * kRowWarps);  // per 32 queries: full | local << 16
+  auto facts = [&](int q, int4& qi, int& r) -> int {  // returns the query's class: 0 full, 1 local, 2 zero
+    bool any_local;
+    const int seq = ka.seq_ids[q], t = ka.q_positions[q], mode = query_mode(ka, q, any_local);
+    const int w = ka.windows ? ka.windows[q] : ka.window_scalar;
+    const int err = query_error(a, seq, t, mode, any_local, w);
+    r = err ? 0 : query_range(t, mode, w);
+    const bool local_lo = HM ? any_local : mode == TRR_MODE_LOCAL;
+    qi = make_int4(seq, t, local_lo ? max(0, t - w + 1) : 0, err << 24 | (r == 0) << 28);
+    return r == 0 ? 2 : mode == TRR_MODE_LOCAL ? 1 : 0;
+  };
+  if (threadIdx.x < 32) counts[threadIdx.x] = 0;
+  __syncthreads();
+  long long rsum = 0;
+  int4 qi;
+  int r = 0, cls = 3;
+#pragma unroll 1
+  for (int q0 = 0; q0 < n; q0 += 32 * kRowWarps) {
+    const int q = q0 + threadIdx.x;
+    cls = 3;
+    if (q < n) {
+      cls = facts(q, qi, r);
+      if (HM && r > 0) {
+        const HeadCounts c = head_counts(ka, q);
+        rsum += static_cast<long long>(c.full) * (qi.y + 1) + static_cast<long long>(c.local) * (qi.y + 1 - qi.z);
+      } else {
+        rsum += static_cast<long long>(r) * a.Hq;
+      }
+    }
+    const unsigned f = __ballot_sync(0xffffffffu, cls == 0), l = __ballot_sync(0xffffffffu, cls == 1);
+    if (lane == 0) counts[(q0 >> 5) + warp] = __popc(f) | __popc(l) << 16;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) rsum += __shfl_xor_sync(0xffffffffu, rsum, o);
+  if (lane == 0) red[warp] = rsum;
+  __syncthreads();
+  int incl = counts[lane];  // counts of each class in the query blocks before lane's
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  const int all = __shfl_sync(0xffffffffu, incl, 31), nf = all & 0xffff, nl = all >> 16;
+#pragma unroll 1
+  for (int q0 = 0; q0 < n; q0 += 32 * kRowWarps) {
+    const int q = q0 + threadIdx.x, blk = (q0 >> 5) + warp;
+    if (n > 32 * kRowWarps) cls = q < n ? facts(q, qi, r) : 3;
+    const unsigned f = __ballot_sync(0xffffffffu, cls == 0), l = __ballot_sync(0xffffffffu, cls == 1);
+    const unsigned below = (1u << lane) - 1u;
+    const int before = __shfl_sync(0xffffffffu, incl, blk) - (__popc(f) | __popc(l) << 16);
+    const int bf = (before & 0xffff) + __popc(f & below), bl = (before >> 16) + __popc(l & below);
+    const int k = cls == 0 ? bf : cls == 1 ? nf + bl : nf + nl + q - bf - bl;
+    if (q < n) {
+      ord[k] = static_cast<uint16_t>(q);
+      qinf[k] = qi;
+      pre[k] = r;
+    }
+  }
+  __syncthreads();
+  rsum = 0;
+#pragma unroll
+  for (int k = 0; k < kRowWarps; ++k) rsum += red[k];
+  // Split size: about one unit per warp while a unit then stays short, else up to three per
+  // warp, of 700 positions at least, handed out on demand; never below pos_split.  (1.3B
+  // shape, batch 64, contexts to 8192: 637 us for 8 layer calls; one unit per warp only up to
+  // 768 positions 704, units from 512 positions 689, five per warp 768.)  Binary32
+  // arithmetic: the same result in every CTA, and it only sizes the splits.
+  const float warps = static_cast<float>(gridDim.x * kRowWarps), rs = static_cast<float>(rsum);
+  const float one = rs / (0.85f * warps);
+  const float by_work = ceilf(one > 1000.f ? fmaxf(700.f, rs / (3.f * warps)) : one);
+  const int pos_split = by_work > static_cast<float>(a.pos_split) ? static_cast<int>(fminf(by_work, 1073741824.f))
+                                                                   : a.pos_split;
+  const int chunk = (n + 32 * kRowWarps - 1) / (32 * kRowWarps);
+  const int q0 = min(n, static_cast<int>(threadIdx.x) * chunk), q1 = min(n, q0 + chunk);
+  int mine = 0;
+#pragma unroll 1
+  for (int k = q0; k < q1; ++k) {  // pre[k] becomes the query's unit count
+    const int range = pre[k];
+    int ns = 1, units = a.Hq;
+    if (range > 0) {
+      ns = splits_of(range, pos_split, a.split_keys, a.split_extra, a.split_most, a.s_cap);
+      units = a.Hq * ns;
+      if (HM) {
+        const HeadCounts c = head_counts(ka, ord[k]);
+        const int4 x = qinf[k];
+        ns = splits_of(x.y + 1, pos_split, a.split_keys, a.split_extra, a.split_most, a.s_cap);
+        units = c.full * ns + c.skip +
+                c.local * splits_of(x.y + 1 - x.z, pos_split, a.split_keys, a.split_extra, a.split_most, a.s_cap);
+      }
+    }
+    qinf[k].w |= ns;
+    pre[k] = units;
+    mine += units;
+  }
+  incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) red[8 + warp] = incl;
+  __syncthreads();
+  int off = incl - mine;
+#pragma unroll 1
+  for (int k = 0; k < warp; ++k) off += static_cast<int>(red[8 + k]);
+#pragma unroll 1
+  for (int q = q0; q < q1; ++q) {
+    const int units = pre[q];
+    pre[q] = off;
+    off += units;
+  }
+  if (threadIdx.x == 32 * kRowWarps - 1) {
+    pre[n] = off;
+    pre[n + 1] = pos_split;
+  }
+  __syncthreads();
+}
+
+// mbar_wait_or out of line: a tile that has arrived is found by one test.
+static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort, uint64_t limit_ns) {
+  return mbar_wait_or(bar, parity, abort, limit_ns);
+}
+
+// One unit as its warp plans it.
+struct RowUnit {
+  int q, h;         // query, query head
+  int sp, ns;       // split, splits of the row
+  int base;         // the row's first partial
+  int t, lo;        // key range [lo, t]
+  int err;          // the query's error: a zero row
+  int T;            // pages; none for a zero row
+  bool zero;        // a skip head or a failed query
+};
+
+// A split's share of a row is a run of its pages, listed from the widest class down and each
+// class's in position order: the row's tiles (and kNewTiles for the query's own token of a
+// decode step at the end) are cut evenly, at page boundaries.  So a split meets one or two
+// classes (a share of every class made four switches a unit), and the warps of a CTA, which
+// as a rule have the same split of neighbouring heads, run the same class's code at a time.
+constexpr int kNewTiles = 3;
+
+// Pages of split sp (of ns) of a query of sequence seq over key positions [lo, t]: returns
+// their number (<= kItemMaxTiles); lane j below it gets page j's id in wid and class |
+// fill << 2 | kMask in wmeta.  own: whether the query's own token joins the last split.
+// Eight lanes per class: a rolled nine-way search of the pages' first or last positions where
+// the range needs it (small code: a unit's plan competes with its tiles for the instruction
+// cache).
+__device__ __forceinline__ int plan_pages(const LayerArgs& a, int seq, int lo, int t, int sp, int ns, bool own,
+                                          int kt_most, int kt_wide, int lane, int& wid, int& wmeta) {
+  const int c8 = lane >> 3, sub = lane & 7, lg = __ffs(a.P) - 1;
+  const int nt = a.ntok[seq * 4 + c8];
+  const bool upper_mask = t < a.last_pos[seq];  // keys after t may be stored
+  const int pages = (nt + a.P - 1) >> lg;
+  const int64_t row0 = (static_cast<int64_t>(seq) * 4 + c8) * a.MP;
+  int first = 0, end = pages;
+#pragma unroll 1
+  for (int side = lo > 0 ? 0 : 1; side < (upper_mask ? 2 : 1); ++side) {
+    const int* arr = (side ? a.pfirst : a.plast) + row0;
+    const int x = side ? t + 1 : lo;  // entries below x
+    int l = 0, h = pages;             // the count lies in [l, h]
+    int probe = max(0, pages - 8) + sub, step = 1;  // first the last 8 pages: decode queries look there
+#pragma unroll 1
+    while (__any_sync(0xffffffffu, l < h)) {
+      const bool below = probe < h && arr[probe] < x;
+      const int cnt = __popc((__ballot_sync(0xffffffffu, below) >> (8 * c8)) & 255u);
+      const int p0 = probe - sub * step;
+      if (l < h) {
+        if (cnt < 8) h = min(h, p0 + cnt * step);  // probe cnt is not below (or past the end)
+        if (cnt > 0) l = max(l, p0 + (cnt - 1) * step + 1);
+      }
+      step = max(1, (h - l + 8) / 9);
+      probe = l + sub * step + (step > 1 ? step - 1 : 0);
+    }
+    if (side) end = l;
+    else first = l;
+  }
+  const int npr = max(0, end - first);
+  const int lw = lg + 1 - __ffs(c8 == 3 ? kt_wide : kt_most), w = 1 << lw, mass = npr << lw;  // tiles of a page
+  int before = 0, all = own ? kNewTiles : 0;  // tiles of the wider classes; of the row
+#pragma unroll
+  for (int k = 0; k < kClasses; ++k) {
+    const int m = __shfl_sync(0xffffffffu, mass, 8 * k);
+    all += m;
+    before += k > c8 ? m : 0;
+  }
+  // the split's pages: those that start in its share [b0, b1) of the tiles, all / ns and one
+  // more for the first all % ns splits (all < 2^24)
+  const int each = div24(all, ns), extra = all - each * ns;
+  const int b0 = sp * each + min(sp, extra), b1 = b0 + each + (sp < extra ? 1 : 0);
+  const int beg = min(npr, max(0, (b0 - before + w - 1) >> lw));
+  const int tc = min(npr, max(0, (b1 - before + w - 1) >> lw)) - beg;
+  const int t1 = __shfl_sync(0xffffffffu, tc, 24), t2 = t1 + __shfl_sync(0xffffffffu, tc, 16);
+  const int t3 = t2 + __shfl_sync(0xffffffffu, tc, 8);
+  const int T = min(t3 + __shfl_sync(0xffffffffu, tc, 0), kItemMaxTiles);  // (the split bound keeps it within)
+  const int r = (lane >= t1) + (lane >= t2) + (lane >= t3), c = 3 - r;
+  const int kid = __shfl_sync(0xffffffffu, first + beg, 8 * c) + lane - (r == 0 ? 0 : r == 1 ? t1 : r == 2 ? t2 : t3);
+  const int f = __shfl_sync(0xffffffffu, first, 8 * c), e = __shfl_sync(0xffffffffu, end, 8 * c);
+  const int ntc = __shfl_sync(0xffffffffu, nt, 8 * c);
+  wid = 0;
+  wmeta = 0;
+  if (lane < T) {
+    wid = a.pt[(static_cast<int64_t>(seq) * 4 + c) * a.MP + kid];
+    // slot positions are needed on a page that may hold keys outside [lo, t]
+    const bool mask = (lo > 0 && kid == f) || (upper_mask && kid == e - 1);
+    wmeta = c | (min(a.P, ntc - kid * a.P) << 2) | (mask ? kMask : 0);
+  }
+  return T;
+}
+
+// ------------------------------------------------------------------- tile arithmetic --
+
+// c = a * b with a zero accumulator
+template <int B>
+__device__ __forceinline__ void mma_cls0(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+  if (B == 16)
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+  else
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+}
+
+// The eight keys i = 0 .. 7 of a tile whose V rows a lane (its lane % 4 = tig) reads, chosen
+// per row length so that the lanes' rows fall into different banks; the first four are keys
+// below 16 in each map.  (Key order is free in P.V as long as the weights follow it.)
+__host__ __device__ constexpr int row_map(int D, int B) { return B == 16 || (D == 128 && B == 8) ? 2 : B == 8 ? 1 : 0; }
+template <int MAP>
+__device__ __forceinline__ int v_key(int tig, int i) {
+  return MAP == 0 ? tig + 4 * i : MAP == 1 ? 4 * tig + (i & 3) + 16 * (i >> 2) : 2 * tig + (i & 1) + 8 * (i >> 1);
+}
+// A tile's weights lie in shared memory as one 16-byte row of eight f16 per key (columns
+// group * 2 + (hi | lo)), read as the mma's B operands by one ldmatrix.x4.trans: lane l gives
+// the address of row l % 8 of matrix l / 8, the key that this place of the contraction has.
+template <int MAP>
+__device__ __forceinline__ int w_row(int lane) {
+  const int r = lane & 7, m = lane >> 3;  // matrices: keys i = 0, 1 | 2, 3 | 4, 5 | 6, 7 of lanes r / 2
+  return v_key<MAP>(r >> 1, 2 * m + (r & 1));
+}
+__device__ __forceinline__ void ldmatrix4_trans(uint32_t (&r)[4], const uint8_t* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(smem_u32(p))
+               : "memory");
+}
+
+// Where a lane's bytes lie in a tile's K rows (rows gid + 8 h + 16 u, dims tig D/4 ..) and V
+// rows (row v_key(tig, i), dims gid D/8 ..): a lane offset, then per load one exclusive-or of
+// a constant (8- and 16-bit rows keep the chunks of a line in the order chunk ^ (line % 8))
+// and a constant to add.  q, hf: the 16-byte chunk of a lane's part.
+template <int D, int B>
+__device__ __forceinline__ uint32_t k_lane(int gid, int tig) {
+  constexpr int rowb = D * B / 8;
+  if (B < 8) return gid * rowb + tig * (rowb / 4);
+  if (rowb == 64) return (gid >> 1) * 128 + (((((gid & 1) << 2) | tig) ^ (gid >> 1)) << 4);
+  if (rowb == 128) return gid * 128 + (((2 * tig) ^ gid) << 4);
+  return (2 * gid + (tig >> 1)) * 128 + ((((tig & 1) << 2) ^ ((2 * gid + (tig >> 1)) & 7)) << 4);
+}
+template <int D, int B>
+__device__ __forceinline__ uint32_t k_off(uint32_t lane_off, int h, int u, int q) {
+  constexpr int rowb = D * B / 8;
+  const uint32_t x = B < 8 ? lane_off : lane_off ^ (rowb == 64 ? h << 6 : q << 4);
+  return x + (8 * h + 16 * u) * rowb + (B < 8 ? 16 * q : 0);
+}
+template <int D, int B>
+__device__ __forceinline__ uint32_t v_lane(int gid, int tig) {
+  constexpr int rowb = D * B / 8;
+  if (B < 8) return tig * rowb + (rowb >= 32 ? gid * (rowb / 8) : (gid * (rowb / 8)) & ~3);
+  if (rowb == 64) return tig * 256 + (((gid >> 1) ^ (2 * tig)) << 4) + ((gid & 1) << 3);
+  if (rowb == 128) return tig * 256 + ((gid ^ (2 * tig)) << 4);
+  return (4 * tig + (gid >> 2)) * 128 + ((((gid & 3) << 1) ^ ((4 * tig) & 7) ^ (gid >> 2)) << 4);
+}
+template <int D, int B>
+__device__ __forceinline__ uint32_t v_off(uint32_t lane_off, int i, int hf) {
+  constexpr int rowb = D * B / 8;
+  if (B < 8) return lane_off + 4 * i * rowb;
+  if (rowb == 64) return (lane_off ^ ((((i & 1) << 2) | ((i >> 1) & 1)) << 4)) + ((i & 3) >> 1) * 128 + (i >> 2) * 1024;
+  if (rowb == 128) return (lane_off ^ ((i & 1) << 4)) + (i & 1) * 128 + (i >> 1) * 1024;
+  return (lane_off ^ (((2 * (i & 1)) ^ hf) << 4)) + (i & 1) * 256 + (i >> 1) * 2048;
+}
+
+// NW words at p (a shared-memory pointer, aligned for one load of up to 16 bytes).
+template <int NW>
+__device__ __forceinline__ void load_words(const uint8_t* p, uint32_t* w) {
+  if (NW % 4 == 0) {
+#pragma unroll
+    for (int k = 0; k < NW; k += 4) {
+      const uint4 u = *reinterpret_cast<const uint4*>(p + 4 * k);
+      w[k] = u.x; w[k + 1] = u.y; w[k + 2] = u.z; w[k + 3] = u.w;
+    }
+  } else if (NW == 2) {
+    const uint2 u = *reinterpret_cast<const uint2*>(p);
+    w[0] = u.x; w[1] = u.y;
+  } else {
+    w[0] = *reinterpret_cast<const uint32_t*>(p);
+  }
+}
+
+__device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+template <int D, int NG>
+struct RowState {
+  static constexpr int NP = D / 8, MT = D / 16;
+  uint32_t kb[NP];    // the query as q.k's B operand in the current class
+  float acc[MT][4];   // V sums: dims gid D/8 + 2 t (+ 1) x columns (group tig % NG, hi | lo),
+                      // times 2^(vfac_log2 + F) for codes, 1 for width 16
+  float qsum[NG];     // softmax scale * log2(e) * sum of the query over each group
+  float m, l;         // running maximum (the warp's, log2 units); this lane's sum of weights
+  float zacc[NG];     // this lane's sums of p * z
+  float slim;         // largest V scale that F allows: 2^(7 - F)
+  float wscale;       // 2^F
+  float kfac;         // the current class's factor of the group sums
+  uint32_t kl, vl;    // the current class's lane offsets (k_lane, v_lane)
+  int wl;             // the byte offset of the lane's row of weights as ldmatrix reads it
+  int zoff;           // the offset in a tile of the V scales of the lane's key
+  int F;              // codes' weights are p * s * 2^F
+  int fset;           // F has been chosen
+  int E;              // codes' queries are q * 2^-E (in f16 range)
+  int cls;
+};
+
+// The query row in the order and scale of class cls's B operand, to qs: widths 2, 4 and 8 as
+// f16 pairs at the codes' bit offsets, times 2^-E (f16 range); width 16 the bf16 values.
+// Lane holds dims lane * D/32 .. (raw, bf16).
+template <int D>
+__device__ __forceinline__ void store_query_row(uint8_t* qs, uint2 raw, int cls, int E, int lane) {
+  constexpr int DPL = D / 32;
+  const int d0 = lane * DPL, part = d0 / (D / 4), dd0 = d0 % (D / 4);
+  uint8_t* row = qs + part * (D / 2);
+  if (cls == 3) {
+    if (D == 64) *reinterpret_cast<uint32_t*>(row + 2 * dd0) = raw.x;
+    else *reinterpret_cast<uint2*>(row + 2 * dd0) = raw;
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < DPL; ++j) {
+    const uint32_t w = j < 2 ? raw.x : raw.y;
+    const int dd = dd0 + j;
+    // the word and half of dim dd, and the bit offset of its code: width 8 pairs (2 i, 2 i + 1);
+    // width 4 (8 k + i, + 4), offset 4 (i % 2); width 2 (16 k + i, + 8), offset 2 (i < 5 ? i : i - 5)
+    const int lg = cls == 0 ? 3 : 2, i = dd & ((1 << lg) - 1);
+    const int word = cls == 2 ? dd >> 1 : ((dd >> (lg + 1)) << lg) + i, half = cls == 2 ? dd & 1 : (dd >> lg) & 1;
+    const int e = cls == 2 ? 0 : cls == 1 ? 4 - 4 * (i & 1) : 8 - 2 * (i < 5 ? i : i - 5);
+    const float v = ((j & 1) ? bf_hi(w) : bf_lo(w)) * __int_as_float((127 - E + e) << 23);
+    *reinterpret_cast<__half*>(row + 4 * word + 2 * half) = __float2half_rn(v);
+  }
+}
+
+// log2 of the factor the accumulators of dim j (of a lane's D/8) carry in class c, without
+// the codes' 2^F
+__host__ __device__ constexpr int row_fac(int c, int j) { return c == 3 ? 0 : vfac_log2(c, j); }
+
+// What a lane keeps of class B while it works on its tiles.
+template <int D, int NG, int B>
+__device__ __forceinline__ void row_class(RowState<D, NG>& st, float qscale, int lane) {
+  st.kfac = B == 16 ? qscale : __int_as_float((127 + 24 - smax_of<B>() + st.E) << 23) * qscale;
+  st.kl = k_lane<D, B>(lane >> 2, lane & 3);
+  st.vl = v_lane<D, B>(lane >> 2, lane & 3);
+  st.wl = 16 * w_row<row_map(D, B)>(lane);
+}
+
+// Class st.cls -> to: the query's operand (lane (gid, tig) holds dims tig D/4 .. of group
+// gid % NG), the accumulators' factors (fac: a table [from][to][dim of the lane]).
+template <int D, int NG>
+__device__ __forceinline__ void row_switch(RowState<D, NG>& st, int to, bool fresh, uint8_t* qs, uint2 qraw, const float* fac,
+                                           float qscale, int kt, int lane) {
+  constexpr int NP = D / 8, MT = D / 16;
+  const int gid = lane >> 2, tig = lane & 3;
+  const bool ok = (tig * NG) / 4 == gid % NG;
+  switch (to) {
+    case 0: row_class<D, NG, 2>(st, qscale, lane); break;
+    case 1: row_class<D, NG, 4>(st, qscale, lane); break;
+    case 2: row_class<D, NG, 8>(st, qscale, lane); break;
+    default: row_class<D, NG, 16>(st, qscale, lane); break;
+  }
+  const int b = bits_of_class(to);
+  st.zoff = kt * (2 * (D * b / 8) + 4 * NG) + min(8 * tig + gid, kt - 1) * NG * 4;
+  store_query_row<D>(qs, qraw, to, st.E, lane);
+  __syncwarp();
+  load_words<NP>(qs + tig * (D / 2), st.kb);
+#pragma unroll
+  for (int i = 0; i < NP; ++i) st.kb[i] = ok ? st.kb[i] : 0u;
+  // (width 16 weighs p itself: its wscale is 1, and its scale never asks for another F)
+  st.wscale = to == 3 ? 1.f : __int_as_float((127 + st.F) << 23);
+  st.slim = to == 3 ? 3e38f : st.cls == 3 && st.fset == 0 ? 0.f : __int_as_float((127 + 7 - st.F) << 23);
+  if (!fresh) {
+    const int e = (to == 3 ? 0 : st.F) - (st.cls == 3 ? 0 : st.F);
+    const float g = __int_as_float((127 + e) << 23);
+    float f[2 * MT];
+    load_words<2 * MT>(reinterpret_cast<const uint8_t*>(fac + (st.cls * 4 + to) * (D / 8)), reinterpret_cast<uint32_t*>(f));
+#pragma unroll
+    for (int t = 0; t < MT; ++t) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const float x = f[2 * t + r] * g;
+        st.acc[t][2 * r] *= x;
+        st.acc[t][2 * r + 1] *= x;
+      }
+    }
+  }
+  st.cls = to;
+}
+
+// A tile: kt (16 or 32) rows at `tile` (K rows, V rows, K (s, z), V (s, z)).  Its work is in
+// three parts, so that only what depends on the width has a copy per width (the four widths'
+// loops and the rest of the kernel compete for the instruction cache: with whole tiles per
+// width a seventh of the fetches missed it).
+
+// The A operands of P.V of 16 keys (half u of the tile) and this lane's D/8 dims.
+template <int D, int NG, int B>
+__device__ __forceinline__ void value_words(const RowState<D, NG>& st, const uint8_t* v0, int u, uint32_t* va, int lane) {
+  constexpr int MT = D / 16;
+  constexpr int VB = D * B / 64;   // V bytes per lane and key (D/8 dims)
+  constexpr int VW = VB >= 4 ? VB / 4 : 1;
+  uint32_t x[4][VW];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    load_words<VW>(v0 + v_off<D, B>(st.vl, 4 * u + i, 0), x[i]);
+    if (VB < 4) x[i][0] >>= (((lane >> 2) * VB) & 3) * 8;
+  }
+#pragma unroll
+  for (int t = 0; t < MT; ++t) {
+    va[4 * t] = v_pair<B>(x[0], x[1], 2 * t);
+    va[4 * t + 1] = v_pair<B>(x[0], x[1], 2 * t + 1);
+    va[4 * t + 2] = v_pair<B>(x[2], x[3], 2 * t);
+    va[4 * t + 3] = v_pair<B>(x[2], x[3], 2 * t + 1);
+  }
+}
+
+// 1. The group sums of q.c of the lane's key: lane (gid, tig) takes key 8 tig + gid, which is
+// in half tig % 2 of the 16 keys tig / 2.
+template <int D, int NG, int B>
+__device__ __forceinline__ void tile_scores(const RowState<D, NG>& st, const uint8_t* tile, int kt, float (&g)[NG], int lane) {
+  constexpr int KS = D / 16;
+  constexpr int KW = D * B / 128;  // K words per lane and key (D/4 dims)
+  const int tig = lane & 3;
+  const bool h1 = tig & 1, u1 = tig & 2;
+  float o0 = 0.f, o1 = 0.f;  // NG = 4: the partner's key, this lane's groups
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    if (u == 1 && kt == 16) break;
+    float c[4], c2[4];
+    constexpr int KH = KW >= 8 ? KW / 4 : 1, KWH = KW / KH, KSH = KS / KH;  // 16 bytes of a row at a time when long
+#pragma unroll
+    for (int hf = 0; hf < KH; ++hf) {
+      uint32_t k1[KWH], k2[KWH];
+      load_words<KWH>(tile + k_off<D, B>(st.kl, 0, u, hf), k1);
+      load_words<KWH>(tile + k_off<D, B>(st.kl, 1, u, hf), k2);
+#pragma unroll
+      for (int s = hf * KSH; s < (hf + 1) * KSH; ++s) {
+        const int i0 = 2 * (s - hf * KSH);
+        const uint32_t a0 = k_pair<B>(k1, i0), a1 = k_pair<B>(k2, i0), a2 = k_pair<B>(k1, i0 + 1), a3 = k_pair<B>(k2, i0 + 1);
+        if (s == 0) mma_cls0<B>(c, a0, a1, a2, a3, st.kb[0], st.kb[1]);
+        else if (D == 128 && s == 1) mma_cls0<B>(c2, a0, a1, a2, a3, st.kb[2], st.kb[3]);
+        else mma_cls<B>((D == 128 && (s & 1)) ? c2 : c, a0, a1, a2, a3, st.kb[2 * s], st.kb[2 * s + 1]);
+      }
+    }
+    if (D == 128) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) c[i] += c2[i];
+    }
+    if (u == 0 || u1) {
+      g[0] = h1 ? c[2] : c[0];
+      if (NG > 1) g[NG > 1 ? 1 : 0] = h1 ? c[3] : c[1];
+      if (NG == 4) {
+        o0 = h1 ? c[0] : c[2];
+        o1 = h1 ? c[1] : c[3];
+      }
+    }
+  }
+  if (NG == 4) {  // this lane's columns are groups 0 and 1 (tig even) or 2 and 3: trade with tig ^ 1
+    const float x0 = __shfl_xor_sync(0xffffffffu, o0, 1), x1 = __shfl_xor_sync(0xffffffffu, o1, 1);
+    g[NG > 2 ? 2 : 0] = h1 ? g[0] : x0;
+    g[NG > 3 ? 3 : 0] = h1 ? g[NG > 1 ? 1 : 0] : x1;
+    g[0] = h1 ? x0 : g[0];
+    g[NG > 1 ? 1 : 0] = h1 ? x1 : g[NG > 1 ? 1 : 0];
+  }
+}
+
+// 2. The key's weight (ok: it counts): the score from the group sums, the running maximum and
+// F raised and lowered when a key asks for it, p, and p * s as the operand rows at wb.
+// kw, zw: the key's K and V (s, z); (1, 0) where the width has none (has_sz).
+template <int D, int NG>
+__device__ __forceinline__ void tile_weights(RowState<D, NG>& st, float (&g)[NG], bool ok, bool has_sz,
+                                             const uint32_t (&kw)[NG], uint32_t (&zw)[NG], int key, uint8_t* wb) {
+  constexpr int MT = D / 16;
+  float sc = 0.f, smax = 0.f;
+  float2 vz[NG];
+#pragma unroll
+  for (int i = 0; i < NG; ++i) {
+    const float2 sz = __half22float2(*reinterpret_cast<const __half2*>(&kw[i]));
+    sc = fmaf(sz.x * st.kfac, g[i], fmaf(sz.y, st.qsum[i], sc));
+    if (!ok) zw[i] = 0u;  // a slot that does not count may hold any bytes
+    vz[i] = __half22float2(*reinterpret_cast<const __half2*>(&zw[i]));
+    smax = fmaxf(smax, vz[i].x);
+  }
+  if (!ok) sc = kNegInf;
+  if (__any_sync(0xffffffffu, sc > st.m + kTau || smax > st.slim)) {
+    float top = sc, big = smax;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+      big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+    }
+    top = fmaxf(top, st.m);
+    const float alpha = top == st.m ? 1.f : fast_exp2(st.m - top);
+    float f = alpha;
+    if (big > st.slim) {
+      // big * 2^F < 2^6 (width 2), 2^3, 2^0 (width 8): the scales of the narrower classes that
+      // follow are larger by the ratio of the levels, and shall seldom ask again
+      const int room = 5 - 3 * st.cls;
+      const int F = min(24, room - (static_cast<int>(__float_as_uint(big) >> 23) - 127));
+      f *= __int_as_float((127 + F - st.F) << 23);
+      st.F = F;
+      st.fset = 1;
+      st.wscale = __int_as_float((127 + F) << 23);
+      st.slim = __int_as_float((127 + 7 - F) << 23);
+    }
+    st.l *= alpha;
+#pragma unroll
+    for (int i = 0; i < NG; ++i) st.zacc[i] *= alpha;
+#pragma unroll
+    for (int t = 0; t < MT; ++t)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) st.acc[t][i] *= f;
+    st.m = top;
+  }
+  const float p = fast_exp2(sc - st.m);  // 0 for a key that does not count
+  st.l += p;
+  const float pf = p * st.wscale;
+  if (has_sz) {
+    uint32_t w2[NG];
+#pragma unroll
+    for (int i = 0; i < NG; ++i) {
+      st.zacc[i] = fmaf(p, vz[i].y, st.zacc[i]);
+      const float w = pf * vz[i].x, wh = __half2float(__float2half_rn(w));
+      w2[i] = pack_f16x2(wh, (w - wh) * kLoScale);
+    }
+    uint32_t* at = reinterpret_cast<uint32_t*>(wb + 16 * key);
+    if (NG == 1) at[0] = w2[0];
+    else if (NG == 2) *reinterpret_cast<uint2*>(at) = make_uint2(w2[0], w2[NG > 1 ? 1 : 0]);
+    else *reinterpret_cast<uint4*>(at) = make_uint4(w2[0], w2[NG > 1 ? 1 : 0], w2[NG > 2 ? 2 : 0], w2[NG > 3 ? 3 : 0]);
+  } else {
+    const uint32_t hi = __float_as_uint(p) & 0xffffe000u;  // 11 bits, exact remainder
+    *reinterpret_cast<float2*>(wb + 8 * key) = make_float2(__uint_as_float(hi), (p - __uint_as_float(hi)) * kLoScale);
+  }
+}
+
+// 3. P.V of a tile of width B < 16.
+template <int D, int NG, int B>
+__device__ __forceinline__ void tile_values(RowState<D, NG>& st, const uint8_t* tile, int kt, const uint8_t* wb, int lane) {
+  constexpr int MT = D / 16;
+  uint32_t w[4];
+  ldmatrix4_trans(w, wb + st.wl);
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    if (u == 1 && kt == 16) break;
+    uint32_t x[4 * MT];
+    value_words<D, NG, B>(st, tile + kt * (D * B / 8), u, x, lane);
+#pragma unroll
+    for (int t = 0; t < MT; ++t) mma_f16(st.acc[t], x[4 * t], x[4 * t + 1], x[4 * t + 2], x[4 * t + 3], w[2 * u], w[2 * u + 1]);
+  }
+}
+
+// The same for width 16.  all: lanes whose key counts (part: not every one does).
+template <int D, int NG>
+__device__ __forceinline__ void tile_values16(RowState<D, NG>& st, const uint8_t* tile, int kt, bool part, unsigned all,
+                                              const uint8_t* wb, int lane) {
+  constexpr int VB = D / 4, MAP = row_map(D, 16);  // V bytes per lane and key (D/8 dims)
+  const int gid = lane >> 2, tig = lane & 3;
+  const uint8_t* v0 = tile + kt * 2 * D;
+  const uint8_t* wa = wb + (gid & 1) * 4;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {  // 8 keys
+    if (s == 2 && kt == 16) break;
+    const int ka = v_key<MAP>(tig, 2 * s), kb = v_key<MAP>(tig, 2 * s + 1);
+    const uint32_t wx = *reinterpret_cast<const uint32_t*>(wa + 8 * ka), wy = *reinterpret_cast<const uint32_t*>(wa + 8 * kb);
+#pragma unroll
+    for (int hf = 0; hf < VB / 16; ++hf) {
+      uint32_t x[4], y[4];
+      load_words<4>(v0 + v_off<D, 16>(st.vl, 2 * s, hf), x);
+      load_words<4>(v0 + v_off<D, 16>(st.vl, 2 * s + 1, hf), y);
+      if (part) {  // values of keys that do not count read as 0 (they may be NaN)
+        const bool oka = (all >> ((ka & 7) * 4 + (ka >> 3))) & 1u, okb = (all >> ((kb & 7) * 4 + (kb >> 3))) & 1u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (!oka) x[i] = 0u;
+          if (!okb) y[i] = 0u;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        mma_tf32(st.acc[hf * 4 + i], x[i] << 16, x[i] & 0xffff0000u, y[i] << 16, y[i] & 0xffff0000u, wx, wy);
+    }
+  }
+}
+
+// --------------------------------------------------------------------------- rows --
+
+// A row at its unit's end (lane holds dims lane * D/32 .. of the unnormalised sum, relative to
+// max M, with weight sum L).  One split: the bf16 row.  Otherwise the split's fp32 partial,
+// partial base + sp, merged in two levels: the last split of each group of kMergeGroup to
+// arrive folds the group into its first partial, and the last group to arrive merges the
+// groups into the row (one level when ns <= kMergeGroup).
+template <int D>
+__device__ __forceinline__ void store_row(const AttnKernelArgs& ka, float (&v)[D / 32], float M, float L, int sp, int qi,
+                                          int qh, int ns, int base, int lane) {
+  constexpr int DPL = D / 32;
+  constexpr int64_t kRow = D + 4;
+  const LayerArgs& a = ka.a;
+  if (ns > 1) {
+    float* p0 = a.part + static_cast<int64_t>(base) * kRow;  // the level's first partial
+    int* counters = a.cnt + (static_cast<int64_t>(qi) * a.Hq + qh) * a.cnt_stride;
+    const bool two = ns > kMergeGroup;
+    const int gr = two ? sp / kMergeGroup : 0;
+    int* counter = two ? counters + 1 + gr : counters;       // the group's arrivals, then the row's
+    int count = two ? min(kMergeGroup, ns - gr * kMergeGroup) : ns, stride = 1;
+    float* from = two ? p0 + gr * kMergeGroup * kRow : p0;
+    float* pp = p0 + sp * kRow;
+#pragma unroll 1
+    for (int level = two ? 0 : 1; level < 2; ++level) {
+#pragma unroll
+      for (int j = 0; j < DPL; j += 2) __stcg(reinterpret_cast<float2*>(pp + lane * DPL + j), make_float2(v[j], v[j + 1]));
+      if (lane == 0) __stcg(reinterpret_cast<float2*>(pp + D), make_float2(M, L));
+      if (!arrive_last(counter, count, lane)) return;
+      merge_partials<D>(from, kRow * stride, count, lane, M, L, v);
+      __syncwarp();  // every lane has read the group's rows before the first is overwritten
+      pp = from;
+      from = p0;
+      counter = counters;
+      count = (ns + kMergeGroup - 1) / kMergeGroup;
+      stride = kMergeGroup;
+    }
+  }
+  __nv_bfloat162* out =
+      reinterpret_cast<__nv_bfloat162*>(ka.out + (static_cast<int64_t>(qi) * a.Hq + qh) * D + lane * DPL);
+  const float inv = L > 0.f ? 1.f / L : 0.f;
+#pragma unroll
+  for (int j = 0; j < DPL; j += 2) out[j / 2] = __floats2bfloat162_rn(v[j] * inv, v[j + 1] * inv);
+}
+
+// The accumulators of a unit as lane's dims lane * D/32 .., with the zero points added.
+template <int D, int NG>
+__device__ __forceinline__ void row_values(RowState<D, NG>& st, float (&v)[D / 32], const float* fac, int lane) {
+  constexpr int DPL = D / 32, MT = D / 16;
+  const int gid = lane >> 2, tig = lane & 3, grp = gid * NG / 8;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    st.l += __shfl_xor_sync(0xffffffffu, st.l, o);
+#pragma unroll
+    for (int i = 0; i < NG; ++i) st.zacc[i] += __shfl_xor_sync(0xffffffffu, st.zacc[i], o);
+  }
+  float z = st.zacc[0];
+#pragma unroll
+  for (int i = 1; i < NG; ++i)
+    if (grp == i) z = st.zacc[i];
+  // dims gid D/8 + 2 t + r are in lane (gid, grp)'s acc[t][2 r] (hi) and [2 r + 1] (lo);
+  // this lane wants t = tig DPL/2 ..
+  const float g = __int_as_float((127 - (st.cls == 3 ? 0 : st.F)) << 23);
+  float f[2 * MT];
+  load_words<2 * MT>(reinterpret_cast<const uint8_t*>(fac + (st.cls * 4 + 3) * (D / 8)), reinterpret_cast<uint32_t*>(f));
+#pragma unroll
+  for (int t = 0; t < MT; ++t) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const float inv = f[2 * t + r] * g;
+      const float hi = st.acc[t][2 * r], lo = st.acc[t][2 * r + 1];
+      // an infinite sum (16-bit values may be infinite) has no low part
+      const float x = (fabsf(hi) <= 3.4028235e38f ? fmaf(lo, 1.f / kLoScale, hi) : hi) * inv;
+      const float got = __shfl_sync(0xffffffffu, x, (lane & ~3) + grp);
+      if (t / (DPL / 2) == tig) v[(t % (DPL / 2)) * 2 + r] = got + z;
+    }
+  }
+}
+
+// ----------------------------------------------------------------------- new token --
+
+// Decode step: K or V row (raw: this lane's D/32 bf16 values) of entry e's KV head j at class
+// c: stored to slot `slot` of page pid when `own`; x: the values as stored, in binary32.
+template <int D>
+__device__ __forceinline__ void step_row(const AttnKernelArgs& ka, uint2 raw, int kv, int j, int c, int pid, int slot,
+                                         bool own, float (&x)[D / 32], int lane) {
+  const LayerArgs& a = ka.a;
+  const int P = a.P, b = bits_of_class(c), rowb = D * b / 8, ng = D >> (__ffs(a.G) - 1);
+  uint8_t* sl = a.pool[c] + static_cast<int64_t>(pid) * a.page_bytes[c] + a.hdr + static_cast<int64_t>(j) * a.slice[c];
+  const int64_t off = static_cast<int64_t>(kv * P + slot) * rowb;
+  const bool sw = a.swz && b >= 8;
+  if (b == 16) {
+    x[0] = bf16lo(raw.x);
+    x[1] = bf16hi(raw.x);
+    if (D == 128) {
+      x[D == 128 ? 2 : 0] = bf16lo(raw.y);
+      x[D == 128 ? 3 : 1] = bf16hi(raw.y);
+    }
+    if (own) {
+      const int64_t o = off + lane * (D / 16);
+      uint8_t* dst = sl + (sw ? swz_off(o) : o);
+      if (D == 64) *reinterpret_cast<uint32_t*>(dst) = raw.x;
+      else *reinterpret_cast<uint2*>(dst) = raw;
+    }
+    return;
+  }
+  const RowCodes r = quantise_row_codes<D>(raw, b, a.G, lane, x);
+  if (own) {
+    const int64_t o = off + 4 * r.code_idx;
+    if (r.code_idx >= 0) *reinterpret_cast<uint32_t*>(sl + (sw ? swz_off(o) : o)) = r.code_word;
+    if (r.sz_idx >= 0)
+      reinterpret_cast<uint32_t*>(sl + 2 * static_cast<int64_t>(P) * rowb + static_cast<int64_t>(kv * P + slot) * ng * 4)[r.sz_idx] =
+          r.sz_word;
+    if (__any_sync(0xffffffffu, r.bad) && lane == 0) set_status(a.ctrl, TRR_ERR_BAD_VALUE);
+  }
+}
+
+template <int D>
+__device__ __forceinline__ uint2 load_row(const uint16_t* src, int lane) {
+  uint2 r = make_uint2(0, 0);
+  if (D == 64) r.x = reinterpret_cast<const uint32_t*>(src)[lane];
+  else r = reinterpret_cast<const uint2*>(src)[lane];
+  return r;
+}
+
+// The per-entry table of a decode-step call (see plan_entries in trr_attn.cuh for what it
+// checks and holds), built by every CTA with one thread per entry (n <= kStepMax threads).
+__device__ __forceinline__ void plan_entries_cta(const AttnKernelArgs& ka, int* ent) {
+  const LayerArgs& a = ka.a;
+  const int n = ka.n, e = threadIdx.x, lane = e & 31, warp = e >> 5, H = 2 * n;
+  static_assert(kStepMax <= 32 * kRowWarps, "one thread per entry");
+  int* hs = ent + 2 * n;  // [H][2]: sequence + 1, lowest entry index naming it
+  int* sc = ent + 6 * n;
+#pragma unroll 1
+  for (int i = e; i < 2 * H; i += 32 * kRowWarps) hs[i] = (i & 1) ? INT_MAX : 0;
+  if (e < kSScalars) sc[e] = e == kSErr ? INT_MAX : 0;
+  const bool act = e < n;
+  int seq = -1, pos = 0, m = 0, b = 0, w = 0;
+  if (act) {
+    seq = ka.seq_ids[e];
+    pos = ka.q_positions[e];
+    m = ka.modes[e];
+    b = ka.bits[e];
+    w = ka.windows ? ka.windows[e] : ka.window_scalar;
+  }
+  const bool in = act && seq >= 0 && seq < a.S;
+  const int c = b == 2 ? 0 : b == 4 ? 1 : b == 8 ? 2 : b == 16 ? 3 : -1;
+  int last = -1, tok = -1, lp = -1;
+  if (in) {
+    last = a.last_pos[seq];
+    if (c >= 0) {
+      tok = a.ntok[seq * 4 + c];
+      lp = a.lastpg[seq * 4 + c];
+    }
+  }
+  __syncthreads();
+  unsigned h = 0;
+  if (in) {
+    h = seq_hash(seq, H);
+#pragma unroll 1
+    for (int probe = 0; probe < H; ++probe) {
+      const int old = atomicCAS(&hs[2 * h], 0, seq + 1);
+      if (old == 0 || old == seq + 1) {
+        atomicMin(&hs[2 * h + 1], e);
+        break;
+      }
+      h = h + 1 == static_cast<unsigned>(H) ? 0u : h + 1;
+    }
+  }
+  __syncthreads();
+  int err = 0;
+  if (act) {
+    if (!in || c < 0 || m > TRR_MODE_FULL) err = TRR_ERR_INVALID_ARG;
+    else if (pos < 0 || pos >= a.maxctx) err = TRR_ERR_BAD_POSITION;
+    else if (hs[2 * h + 1] != e) err = TRR_ERR_INVALID_ARG;
+    else if (pos <= last) err = TRR_ERR_BAD_POSITION;
+    else if (m == TRR_MODE_LOCAL && w < 1) err = TRR_ERR_INVALID_ARG;
+  }
+  const bool stores = act && !err && (m != TRR_MODE_SKIP || a.skip_writes_kv);
+  const bool opens = stores && tok % a.P == 0;
+  if (act && err) atomicMin(&sc[kSErr], e * 16 + err);
+  int before = 0, mine = 0;  // openers of the class in earlier lanes; of class `lane` in the warp
+#pragma unroll
+  for (int cc = 0; cc < kClasses; ++cc) {
+    const unsigned bal = __ballot_sync(0xffffffffu, opens && c == cc);
+    if (c == cc) before = __popc(bal & ((1u << lane) - 1u));
+    if (lane == cc) mine = __popc(bal);
+  }
+  if (lane < kClasses && mine) atomicAdd(&sc[kSOpeners + lane], mine);
+  __syncthreads();  // the hash is read no more
+  if (act) {
+    ent[2 * e] = stores ? tok : -1;
+    hs[e] = lp;
+  }
+  if (n > 32 && lane < kClasses && 32 * warp < n) hs[n + 4 * warp + lane] = mine;
+  __syncthreads();
+  if (act) {
+    if (opens)
+#pragma unroll 1
+      for (int w2 = 0; w2 < warp; ++w2) before += hs[n + 4 * w2 + c];
+    ent[2 * e + 1] = (c & 3) | (opens ? 4 | (before << 3) : 0);
+  }
+  __syncthreads();
+}
+
+// ------------------------------------------------------------------------- kernel --
+
+template <int D, int NG, bool HM, bool STEP>
+__global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_constant__ AttnKernelArgs ka) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  constexpr int DPL = D / 32;
+  const LayerArgs& a = ka.a;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = ka.n, P = a.P, R = ka.ring_bytes;
+  const RowSmem lay(D, NG, n, STEP, R);
+  int* pre = reinterpret_cast<int*>(smem + lay.pre);
+  int* ent = reinterpret_cast<int*>(smem + lay.ent);
+  int* sc = ent + 6 * n;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + lay.flag);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + lay.full) + warp * kRowSlots;
+  uint8_t* ring = smem + lay.ring + warp * R;
+  uint8_t* qs = smem + lay.q + warp * D * 2;
+  float* fac = reinterpret_cast<float*>(smem + lay.fac);
+#pragma unroll 1
+  for (int i = threadIdx.x; i < 16 * (D / 8); i += 32 * kRowWarps) {
+    const int j = i % (D / 8), from = i / (4 * (D / 8)), to = (i / (D / 8)) & 3;
+    fac[i] = __int_as_float((127 + row_fac(to, j) - row_fac(from, j)) << 23);
+  }
+  uint8_t* wb = smem + lay.w + warp * RowSmem::row_w_bytes(NG);
+  if (threadIdx.x < kRowWarps * kRowSlots) mbar_init(reinterpret_cast<uint64_t*>(smem + lay.full) + threadIdx.x, 1);
+  if (threadIdx.x == 0) *abort_flag = 0;
+  fence_barrier_init();
+  // The unit plan reads only the call's own index arrays, which no kernel of this library
+  // writes, so it overlaps the previous kernel of the stream.  The layer's cache state is
+  // read before the wait only when `early` says that no kernel still running can write it.
+  int4* qinf = reinterpret_cast<int4*>(smem + lay.qinf);
+  uint16_t* ord = reinterpret_cast<uint16_t*>(smem + lay.ord);
+  plan_rows<HM>(ka, pre, qinf, ord, reinterpret_cast<long long*>(smem + lay.red));
+  bool waited = !(STEP && ka.early);
+  if (waited) {
+    pdl_wait();
+    pdl_trigger();
+  }
+  const int total = pre[n], nwarps = gridDim.x * kRowWarps;
+
+  // ------------------------------------------------------------------- unit and ring state
+  // A unit's tiles (a page's keys, 32 at a time) are worked out once, one per lane: what to
+  // copy, where in the ring, and how far the ring is used up to the tile's end (the ring
+  // is filled and freed in tile order; a tile that would pass its end starts at 0).
+  RowUnit un = {};
+  uint64_t wsrc = 0;                  // lane j: tile j: its page's slice of the unit's KV head
+  uint32_t wgeo = 0;                  // class | keys << 2 | kMask | ring offset / 128 << 10 | first key / 16 << 20
+  int wbytes = 0, wcum = 0;           // bytes to copy; ring bytes used from the unit's start to the tile's end
+  uint32_t base = 0;                  // tiles of the units before
+  int inext = 0;                      // next tile to issue
+  bool good = true;                   // no wait gave up
+  const int g = a.Hq / a.Hkv;
+  int kvh = 0;                        // the unit's KV head
+  const int kt_most = min(P, 32), kt_wide = min(P, D == 128 ? 16 : 32);
+  auto tile_keys = [&](int cls) { return D == 128 && cls == 3 ? kt_wide : kt_most; };
+  auto tile_rows = [&](int cls) {     // bytes of a tile: rows, scales, presence mask
+    const int b = bits_of_class(cls);
+    return tile_keys(cls) * (b == 16 ? 4 * D : 2 * (D * b / 8) + 8 * NG) + (HM ? 16 : 0);
+  };
+  // issues the copies of the tiles that fit, each by its lane: tile c is the next to be
+  // consumed, `freed` the ring bytes used up to the end of tile c - 1 (tile c itself always
+  // fits: the ring is empty then)
+  auto issue = [&](int c, int freed) {
+    const bool can = lane >= inext && lane < min(un.T, c + kRowSlots) && (wcum - freed <= R || lane == c);
+    inext += __popc(__ballot_sync(0xffffffffu, can));
+    if (can) {
+      const int cls = wgeo & 3, kt = tile_keys(cls);
+      uint64_t* bar = &full[(base + lane) % kRowSlots];
+      uint8_t* dst = ring + ((wgeo >> 3) & (1023u << 7));
+      const uint8_t* sl = reinterpret_cast<const uint8_t*>(wsrc);
+      mbar_arrive_expect_tx(bar, wbytes);
+      const int posb = (wgeo & kMask) ? 4 * kt : 0, key0 = static_cast<int>(wgeo >> 20) << 4;
+      if (kt == P) {  // the whole slice
+        bulk_g2s(dst, sl, wbytes - posb, bar);
+      } else {  // kt of the page's keys: K rows, V rows, their scales, the presence mask
+        const int b = bits_of_class(cls), rowb = D * b / 8, szb = kt * NG * 4;
+        bulk_g2s(dst, sl + key0 * rowb, kt * rowb, bar);
+        bulk_g2s(dst + kt * rowb, sl + (P + key0) * rowb, kt * rowb, bar);
+        if (b != 16) {
+          bulk_g2s(dst + 2 * kt * rowb, sl + 2 * P * rowb + key0 * NG * 4, szb, bar);
+          bulk_g2s(dst + 2 * kt * rowb + szb, sl + 2 * P * rowb + (P + key0) * NG * 4, szb, bar);
+        }
+        if (HM) bulk_g2s(dst + tile_rows(cls) - 16, sl + a.slice[cls] - 16, 16, bar);
+      }
+      if (posb) bulk_g2s(dst + ((tile_rows(cls) + 127) & ~127), sl - a.hdr - kvh * a.slice[cls] + 4 * key0, posb, bar);
+    }
+  };
+  // the unit u: its query, head, split and pages
+  auto plan = [&](int u) {
+    int q = 0, span = n;  // the query's place: pre[q] <= u < pre[q + 1]
+#pragma unroll 1
+    while (span > 1) {
+      const int step = (span + 31) >> 5, at = q + lane * step;
+      q += (__popc(__ballot_sync(0xffffffffu, lane * step < span && pre[at] <= u)) - 1) * step;
+      span = min(step, n - q);
+    }
+    const int4 qi = qinf[q];
+    un.q = ord[q];
+    un.t = qi.y;
+    un.lo = qi.z;
+    un.ns = qi.w & 0xffffff;
+    un.err = (qi.w >> 24) & 15;
+    un.zero = qi.w >> 28;
+    const int r = u - pre[q];
+    if (HM && !un.err) {
+      // full heads first, then local, then skip ones: the k-th head of its mode
+      HeadCounts c{0, 0, 0};
+      const uint8_t* row = ka.modes + static_cast<int64_t>(un.q) * a.Hq;
+#pragma unroll 1
+      for (int h0 = 0; h0 < a.Hq; h0 += 32) {
+        const int hm = h0 + lane < a.Hq ? row[h0 + lane] : -1;
+        c.full += __popc(__ballot_sync(0xffffffffu, hm == TRR_MODE_FULL));
+        c.local += __popc(__ballot_sync(0xffffffffu, hm == TRR_MODE_LOCAL));
+      }
+      const int nsf = un.ns;
+      const int nsl = c.local ? splits_of(un.t + 1 - un.lo, pre[n + 1], a.split_keys, a.split_extra, a.split_most, a.s_cap) : 1;
+      int k, first = 0, hmode;
+      if (r < c.full * nsf) {
+        hmode = TRR_MODE_FULL;
+        un.lo = 0;
+        un.sp = div24(r, c.full);
+        k = r - un.sp * c.full;
+      } else if (r < c.full * nsf + c.local * nsl) {
+        first = c.full * nsf;
+        hmode = TRR_MODE_LOCAL;
+        un.ns = nsl;
+        un.sp = div24(r - first, c.local);
+        k = r - first - un.sp * c.local;
+      } else {
+        first = c.full * nsf + c.local * nsl;
+        hmode = TRR_MODE_SKIP;
+        un.ns = 1;
+        un.sp = 0;
+        k = r - first;
+      }
+      un.base = pre[q] + first + k * un.ns;
+      un.h = 0;
+#pragma unroll 1
+      for (int h0 = 0; h0 < a.Hq; h0 += 32) {
+        const int hm = h0 + lane < a.Hq ? row[h0 + lane] : -1;
+        const unsigned same = __ballot_sync(0xffffffffu, hm == hmode);
+        const int cnt = __popc(same);
+        const unsigned hit =
+            __ballot_sync(0xffffffffu, hm == hmode && __popc(same & ((1u << lane) - 1u)) == k);  // its k-th
+        if (hit) un.h = h0 + __ffs(hit) - 1;
+        k -= cnt;
+        if (k < 0) break;
+      }
+      un.zero = hmode == TRR_MODE_SKIP;
+    } else {
+      un.sp = div24(r, a.Hq);
+      un.h = r - un.sp * a.Hq;
+      un.base = pre[q] + un.h * un.ns;
+    }
+    kvh = g == 1 ? un.h : div24(un.h, g);
+    int wid = -1, wmeta = 0;
+    un.T = un.zero ? 0 : plan_pages(a, qi.x, un.lo, un.t, un.sp, un.ns, STEP, kt_most, kt_wide, lane, wid, wmeta);
+    if (kt_wide < P || kt_most < P) {  // pages to tiles
+      const int kt = tile_keys(wmeta & 3), nt = lane < un.T ? (((wmeta >> 2) & 127) + kt - 1) / kt : 0;
+      int incl = nt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      int page = 0, key0 = 0;
+#pragma unroll 1
+      for (int p = 0; p < un.T; ++p) {
+        const int e = __shfl_sync(0xffffffffu, incl, p), m = __shfl_sync(0xffffffffu, nt, p);
+        if (lane >= e - m && lane < e) {
+          page = p;
+          key0 = lane - (e - m);
+        }
+      }
+      un.T = min(32, __shfl_sync(0xffffffffu, incl, 31));  // (the split bound keeps it within 32)
+      wid = __shfl_sync(0xffffffffu, wid, page);
+      const int pm = __shfl_sync(0xffffffffu, wmeta, page), k = tile_keys(pm & 3);
+      key0 *= k;
+      wmeta = (pm & ~(127 << 2)) | min(k, ((pm >> 2) & 127) - key0) << 2 | (key0 >> 4) << 20;
+    }
+    const int cls = wmeta & 3, rows = tile_rows(cls), posb = (wmeta & kMask) ? 4 * tile_keys(cls) : 0;
+    const int need = ((rows + 127) & ~127) + ((posb + 127) & ~127);
+    if (lane < un.T)
+      wsrc = reinterpret_cast<uint64_t>(a.pool[cls] + static_cast<int64_t>(wid) * a.page_bytes[cls] + a.hdr +
+                                        static_cast<int64_t>(kvh) * a.slice[cls]);
+    wbytes = rows + posb;
+    int off = 0, cum = 0, woff = 0;
+#pragma unroll 1
+    for (int j = 0; j < un.T; ++j) {
+      const int nd = __shfl_sync(0xffffffffu, need, j);
+      if (off + nd > R) {
+        cum += R - off;
+        off = 0;
+      }
+      cum += nd;
+      if (lane == j) {
+        woff = off;
+        wcum = cum;
+      }
+      off += nd;
+    }
+    wgeo = static_cast<uint32_t>(wmeta) | static_cast<uint32_t>(woff >> 7) << 10;
+    inext = 0;
+    issue(0, 0);
+    // a limit shorter than a suspended wait covers the first copies from here on
+    if (a.wait_ns < kShortWaitNs && un.T > 0)
+      good = __all_sync(0xffffffffu, mbar_wait_slow(&full[base % kRowSlots], (base / kRowSlots) & 1, abort_flag, a.wait_ns));
+  };
+
+  // The first unit is planned and its copies issued before the rest of the call's start.
+  int u = blockIdx.x * kRowWarps + warp;
+  int consumed = 0;      // tiles of the unit
+  int next_page = 0;     // decode step: the pools' counters (lanes 0 .. 3)
+  bool failed = false;   // and whether the call fails (it then stores nothing, and the last
+                         // CTA zeroes every row)
+  bool started = false;
+#pragma unroll 1
+  for (;;) {
+    if (u < total && good) plan(u);
+    if (!started) {
+      started = true;
+      if (STEP) plan_entries_cta(ka, ent);
+      if (!waited) {
+        pdl_wait();
+        pdl_trigger();
+      }
+      if (STEP) {
+        next_page = lane < 4 ? a.ctrl[kNextPage + lane] : 0;
+        const int lim = lane == 0 ? a.cap[0] : lane == 1 ? a.cap[1] : lane == 2 ? a.cap[2] : a.cap[3];
+        failed = sc[kSErr] != INT_MAX || __any_sync(0xffffffffu, lane < 4 && sc[kSOpeners + (lane & 3)] > 0 &&
+                                                                      next_page + sc[kSOpeners + (lane & 3)] > lim);
+      }
+    }
+    if (u >= total || !good) break;
+    int u_next = total;
+    if (total > nwarps && lane == 0) u_next = nwarps + atomicAdd(&a.lctl[kNextUnit], 1);  // read at the unit's end
+    const bool own = un.h == kvh * g;  // stores a new token's rows of its KV head
+    // decode step: the entry's own token joins the row's last split; a skip token that
+    // stores KV is written by its zero row's unit
+    const bool has_new = STEP && !failed && un.sp == un.ns - 1 && ent[2 * un.q] >= 0 && (!un.zero || own);
+    uint2 rk = make_uint2(0, 0), rv = rk;
+    if (has_new) {
+      const int64_t src = (static_cast<int64_t>(un.q) * a.Hkv + kvh) * D;
+      rk = load_row<D>(ka.k + src, lane);
+      rv = load_row<D>(ka.v + src, lane);
+    }
+    const int64_t qrow = (static_cast<int64_t>(un.q) * a.Hq + un.h) * D;
+    uint2 qraw = make_uint2(0, 0);
+    if (!un.zero) qraw = load_row<D>(ka.q + qrow, lane);
+    float kx[DPL] = {}, vx[DPL] = {}, new_score = kNegInf;
+    if (has_new) {
+      const int tok = ent[2 * un.q], info = ent[2 * un.q + 1], c = info & 3;
+      const int np = __shfl_sync(0xffffffffu, next_page, c);
+      const int pid = (info & 4) ? np + (info >> 3) : ent[2 * n + un.q];
+#pragma unroll 1
+      for (int kv = 0; kv < 2; ++kv) {  // one copy of the quantiser (its code runs once a unit)
+        float y[DPL];
+        step_row<D>(ka, kv ? rv : rk, kv, kvh, c, pid, tok % P, own, y, lane);
+#pragma unroll
+        for (int j = 0; j < DPL; ++j) {
+          kx[j] = kv ? kx[j] : y[j];
+          vx[j] = y[j];
+        }
+      }
+    }
+    if (un.zero) {
+      if (un.sp == 0) {
+        uint32_t* o = reinterpret_cast<uint32_t*>(ka.out + qrow);
+        o[lane] = 0u;
+        if (D == 128) o[32 + lane] = 0u;
+      }
+      if (!STEP && un.err && un.sp == 0 && lane == 0) atomicMin(&a.lctl[kFirstBadQuery], (ka.q0 + un.q) * 16 + un.err);
+    } else {
+      // the query row to shared memory; its largest exponent, the sums over its groups
+      float x[DPL];
+      x[0] = bf_lo(qraw.x);
+      x[1] = bf_hi(qraw.x);
+      if (D == 128) {
+        x[D == 128 ? 2 : 0] = bf_lo(qraw.y);
+        x[D == 128 ? 3 : 1] = bf_hi(qraw.y);
+      }
+      float qmax = 0.f, qsum = 0.f, dot = 0.f;
+#pragma unroll
+      for (int j = 0; j < DPL; ++j) {
+        qmax = fmaxf(qmax, fabsf(x[j]));
+        qsum += x[j];
+        if (has_new) dot = fmaf(x[j], kx[j], dot);
+      }
+      const int gl = 32 / NG;  // lanes of a group
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
+        if (o < gl) qsum += __shfl_xor_sync(0xffffffffu, qsum, o);
+      }
+      RowState<D, NG> st;
+#pragma unroll
+      for (int i = 0; i < NG; ++i) {
+        st.qsum[i] = __shfl_sync(0xffffffffu, qsum, i * gl) * ka.qscale;
+        st.zacc[i] = 0.f;
+      }
+      if (has_new) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+        new_score = dot * ka.qscale;
+      }
+      st.E = min(100, max(-100, static_cast<int>((__float_as_uint(qmax) >> 23) & 0xff) - 127 - 6));
+      st.F = st.fset = 0;
+      st.slim = 0.f;
+      st.wscale = 1.f;
+      st.m = -1e30f;  // below any score, and finite: a key that does not count weighs 0
+      st.l = 0.f;
+      st.cls = 3;
+#pragma unroll
+      for (int t = 0; t < D / 16; ++t) st.acc[t][0] = st.acc[t][1] = st.acc[t][2] = st.acc[t][3] = 0.f;
+      __syncwarp();
+      int c = 0;  // next tile to consume
+#pragma unroll 1
+      for (; c < un.T; ++c) {
+        const uint32_t geo = __shfl_sync(0xffffffffu, wgeo, c);
+        const int cls = geo & 3, kt = tile_keys(cls);
+        if (c == 0 || cls != st.cls) row_switch<D, NG>(st, cls, c == 0, qs, qraw, fac, ka.qscale, kt, lane);
+        const uint32_t slot = (base + c) % kRowSlots, parity = ((base + c) / kRowSlots) & 1;
+        bool arrived = mbar_test_at(smem_u32(&full[slot]), parity);
+        if (!arrived) arrived = mbar_wait_slow(&full[slot], parity, abort_flag, a.wait_ns);
+        if (!__all_sync(0xffffffffu, arrived)) {  // give up together, never half a warp
+          good = false;
+          break;
+        }
+        const uint8_t* tile = ring + ((geo >> 3) & (1023u << 7));
+        uint32_t there = 0xffffffffu;
+        if (HM) {  // the KV head's presence mask, which ends the tile's rows
+          const uint2 m2 = *reinterpret_cast<const uint2*>(tile + tile_rows(cls) - 16);
+          there = static_cast<uint32_t>(((static_cast<uint64_t>(m2.y) << 32) | m2.x) >> ((geo >> 20) << 4));
+        }
+        uint32_t kw[NG], zw[NG];
+#pragma unroll
+        for (int i = 0; i < NG; ++i) kw[i] = zw[i] = 0x3c00u;  // s = 1, z = 0
+        if (cls != 3) {
+          load_words<NG>(tile + st.zoff - kt * NG * 4, kw);
+          load_words<NG>(tile + st.zoff, zw);
+        }
+        float gs[NG];
+        switch (cls) {
+          case 0: tile_scores<D, NG, 2>(st, tile, kt, gs, lane); break;
+          case 1: tile_scores<D, NG, 4>(st, tile, kt, gs, lane); break;
+          case 2: tile_scores<D, NG, 8>(st, tile, kt, gs, lane); break;
+          default: tile_scores<D, NG, 16>(st, tile, kt, gs, lane); break;
+        }
+        const int key = 8 * (lane & 3) + (lane >> 2);
+        bool ok = key < ((geo >> 2) & 127) && ((there >> key) & 1u);
+        if (geo & kMask) {  // the page may hold keys outside [lo, t]: positions follow the rows
+          const int pos = reinterpret_cast<const int*>(tile + ((tile_rows(cls) + 127) & ~127))[min(key, kt - 1)];
+          ok = ok && pos >= un.lo && pos <= un.t;
+        }
+        const unsigned all = __ballot_sync(0xffffffffu, ok);
+        tile_weights<D, NG>(st, gs, ok, cls != 3, kw, zw, key, wb);
+        __syncwarp();
+        if (cls == 3) {
+          tile_values16<D, NG>(st, tile, kt, all != (kt == 32 ? 0xffffffffu : 0x33333333u), all, wb, lane);
+        } else {
+          switch (cls) {
+            case 0: tile_values<D, NG, 2>(st, tile, kt, wb, lane); break;
+            case 1: tile_values<D, NG, 4>(st, tile, kt, wb, lane); break;
+            default: tile_values<D, NG, 8>(st, tile, kt, wb, lane); break;
+          }
+        }
+        __syncwarp();  // the tile's bytes and weights are read
+        if (inext < un.T) issue(c + 1, __shfl_sync(0xffffffffu, wcum, c));
+      }
+      consumed = c;
+      if (!good) break;
+      float v[DPL];
+      row_values<D, NG>(st, v, fac, lane);
+      float M = st.m, L = st.l;
+      if (has_new) {  // fold the new token in
+        M = fmaxf(st.m, new_score);
+        const float f = fast_exp2(st.m - M), fn = fast_exp2(new_score - M);
+        L = fmaf(L, f, fn);
+#pragma unroll
+        for (int j = 0; j < DPL; ++j) v[j] = fmaf(v[j], f, fn * vx[j]);
+      }
+      store_row<D>(ka, v, M, L, un.sp, un.q, un.h, un.ns, un.base, lane);
+    }
+    u = __shfl_sync(0xffffffffu, u_next, 0);
+    base += un.T;
+    un.T = inext = consumed = 0;
+  }
+  if (!good) {  // a wait gave up: stop the CTA's warps, then let this one's copies land
+    if (lane == 0) {
+      *abort_flag = 1;
+      set_status(a.ctrl, TRR_ERR_TIMEOUT);
+      atomicExch(&a.lctl[kAborted], 1);
+    }
+    // copies in flight always land (they only read memory): the default bound
+#pragma unroll 1
+    for (uint32_t s = base + consumed; s < base + inext; ++s) mbar_wait(&full[s % kRowSlots], (s / kRowSlots) & 1);
+  }
+
+  // The last CTA to finish records the error of the lowest failing query, readies the
+  // layer's counters for the next call and, for a decode step, commits the tokens' metadata.
+  // Its arrival tells it all: the count of CTAs, with 2^16 added by each that gave up a wait.
+  __shared__ int s_done;
+  __syncthreads();
+  if (threadIdx.x == 0) s_done = atom_add_acq_rel(&a.lctl[kDoneCtas], *abort_flag ? 0x10001 : 1) + (*abort_flag ? 0x10001 : 1);
+  if (STEP && warp == 0) {
+    if (lane < 4) sc[kSNextPage + lane] = next_page;
+    __syncwarp();
+    step_pages_error(ka, ent, lane);
+  }
+  __syncthreads();
+  const int done = s_done;
+  if ((done & 0xffff) != static_cast<int>(gridDim.x)) return;
+  if (threadIdx.x == 0) {
+    a.lctl[kDoneCtas] = 0;
+    a.lctl[kNextUnit] = 0;
+    a.lctl[kAborted] = 0;
+    if (!STEP) {
+      const int bad = atomicExch(&a.lctl[kFirstBadQuery], INT_MAX);
+      if (bad != INT_MAX) set_status(a.ctrl, bad & 15);
+    }
+  }
+  if (!STEP) return;
+  if (sc[kSErr] != INT_MAX) {  // a call error: every row zero
+    uint4* o = reinterpret_cast<uint4*>(ka.out);
+    const int64_t n16 = static_cast<int64_t>(n) * a.Hq * D / 8;
+#pragma unroll 1
+    for (int64_t i = threadIdx.x; i < n16; i += blockDim.x) o[i] = make_uint4(0, 0, 0, 0);
+  }
+  if (done < 0x10000) step_commit(ka, ent);  // a call that gave up a wait stores nothing
+}
+
+}  // namespace trr
