@@ -1,7 +1,7 @@
 // trr_attn.cu - the attention entry points: trr_decode_attn, trr_decode_step,
 // trr_decode_attn_routed and trr_decode_attn_static (Sec. 3.2(A), Eq. 2; Sec. 3.8;
 // Sec. 7).  The host side of a call: its launches, their shared memory and scratch
-// views; the kernels are in trr_attn.cuh, instantiated by the trr_attn_*.cu files.
+// views; the kernels are in trr_row.cuh and trr_attn.cuh, instantiated by the trr_attn_*.cu files.
 #include <algorithm>
 #include <climits>
 
@@ -12,7 +12,7 @@ namespace trr {
 // Done once per cache at creation, so that calls stay legal inside stream capture.
 cudaError_t attn_configure() {
   cudaError_t (*const parts[])() = {configure_attn_row, configure_attn_row_heads, configure_attn_row_step,
-                                     configure_attn_mma, configure_attn_step_mma};
+                                     configure_attn_group, configure_attn_group_step};
   for (auto part : parts) {
     const cudaError_t e = part();
     if (e != cudaSuccess) return e;
@@ -20,43 +20,28 @@ cudaError_t attn_configure() {
   return cudaSuccess;
 }
 
-// The tensor-core path serves query groups (g >= 2) whose (head, group) columns fit
-// one 8-wide mma tile.
-static bool use_mma(const Layout& l) {  // per-head modes: one warp per query head
+// Whether a warp takes a KV head and its query group (else a query head).
+static bool use_mma(const Layout& l) {
   return uses_mma(l.Hq, l.Hkv, l.d, l.G, l.head_modes);
 }
 
-// Ring bytes an attention call with n queries gets, or -1 when one stage of the
-// widest page (one KV slice, its positions) or of the query rows would not fit.
-static int attn_ring_bytes(const Layout& l, int n, int hpu, int scr_floats, int fused, int limit) {
-  const int fixed = AttnSmem(0, n, scr_floats, fused).total;
-  const int ring = (limit - fixed) / 128 * 128;
-  const int widest = static_cast<int>(l.slice[3]) + 4 * l.P;
-  const int qrows = hpu * 2 * l.d;
-  if (ring < std::max(widest, qrows)) return -1;
-  return ring;
-}
-
 // Queries per launch: their unit tables live in the CTAs' shared memory; a call with
-// more queries is cut into launches of this many, chained on the stream.
-constexpr int kMaxLaunchQueries = 1024;
+// more queries is cut into launches of this many, chained on the stream.  A query group's
+// rows take shared memory too, and its largest tile (8 KB at d 128) must fit a warp's ring.
+static int launch_queries(const Layout& l) { return use_mma(l) ? 512 : 1024; }
 
 static cudaError_t launch_one(const Layout& l, const AttnKernelArgs& ka, int num_sms, cudaStream_t s) {
   AttnKernelArgs k = ka;
-  if (!use_mma(l)) {  // one query head per warp: every warp's ring is an equal share
-    const int fixed = RowSmem(l.d, l.d / l.G, k.n, k.fused, 0).total;
-    k.ring_bytes = (kRowSmemLimit - fixed) / kRowWarps / 128 * 128;
-    const size_t sm = static_cast<size_t>(RowSmem(l.d, l.d / l.G, k.n, k.fused, k.ring_bytes).total);
-    const dim3 grid(kRowCtasPerSm * num_sms - num_sms / kRowSpare);
-    if (k.fused) return launch_attn_row_step(l, grid, sm, s, k);
-    return l.head_modes ? launch_attn_row_heads(l, grid, sm, s, k) : launch_attn_row(l, grid, sm, s, k);
-  }
-  const int ring = attn_ring_bytes(l, ka.n, ka.hpu, ka.scr_floats, ka.fused, attn_smem_limit(kMmaCtasPerSm));
-  if (ring < 0) return cudaErrorInvalidConfiguration;
-  k.ring_bytes = ring;
-  const size_t sm = static_cast<size_t>(AttnSmem(ring, k.n, k.scr_floats, k.fused).total);
-  const dim3 grid(kMmaCtasPerSm * num_sms), block(32 * (kNcw + 1));
-  return k.fused ? launch_attn_step_mma(l, grid, block, sm, s, k) : launch_attn_mma(l, grid, block, sm, s, k);
+  const int heads = use_mma(l) ? l.Hq / l.Hkv : 1;
+  // every warp's ring is an equal share of what the call's tables leave
+  const int fixed = RowSmem(l.d, heads, k.n, k.fused, 0).total;
+  k.ring_bytes = (kRowSmemLimit - fixed) / kRowWarps / 128 * 128;
+  if (k.ring_bytes < row_tile_bytes(l.d, l.d / l.G)) return cudaErrorInvalidConfiguration;
+  const size_t sm = static_cast<size_t>(RowSmem(l.d, heads, k.n, k.fused, k.ring_bytes).total);
+  const dim3 grid(kRowCtasPerSm * num_sms - num_sms / kRowSpare);
+  if (use_mma(l)) return k.fused ? launch_attn_group_step(l, grid, sm, s, k) : launch_attn_group(l, grid, sm, s, k);
+  if (k.fused) return launch_attn_row_step(l, grid, sm, s, k);
+  return l.head_modes ? launch_attn_row_heads(l, grid, sm, s, k) : launch_attn_row(l, grid, sm, s, k);
 }
 
 // The launches of an attention call with the given scratch views in `a`; *launches
@@ -86,16 +71,12 @@ static cudaError_t launch_attention(const Layout& l, const LayerArgs& a, int num
   ka.bits = step ? step->bits : nullptr;
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.f / sqrtf(static_cast<float>(l.d));
   ka.qscale = scale * 1.4426950408889634f;
-  const bool mma = use_mma(l);
-  const int g = l.Hq / l.Hkv;
-  ka.hpu = mma ? kNcw * g : kNcw;
-  ka.defer_merge = mma ? 1 : 0;
-  // tensor-core scratch per consumer warp: the query's bf16 words (4 d floats), later
-  // the unit's rows (g (d + 4) floats)
-  ka.scr_floats = mma ? std::max(4 * l.d, g * (l.d + 4)) : 0;
+  // the combine kernel follows a query-group launch whose queries can have several splits
+  ka.defer_merge = use_mma(l) && l.s_cap > 1 ? 1 : 0;
   const int64_t row = static_cast<int64_t>(l.Hq) * l.d;  // bf16 elements per query
-  for (int q0 = 0; q0 < n; q0 += kMaxLaunchQueries) {
-    ka.n = std::min(kMaxLaunchQueries, n - q0);
+  const int most = launch_queries(l);
+  for (int q0 = 0; q0 < n; q0 += most) {
+    ka.n = std::min(most, n - q0);
     ka.q0 = q0;
     ka.seq_ids = seq_ids + q0;
     ka.q_positions = q_positions + q0;
@@ -109,14 +90,16 @@ static cudaError_t launch_attention(const Layout& l, const LayerArgs& a, int num
     cudaError_t e = launch_one(l, ka, num_sms, s);
     if (e != cudaSuccess) return e;
     ++*launches;
-    if (mma) {  // the tensor-core path's splits are merged by the combine kernel
+    if (ka.defer_merge) {
       CombineArgs ca;
       ca.part = a.part;
       ca.qtab = reinterpret_cast<const int2*>(ka.a.cnt);
       ca.out = ka.out;
       ca.Hq = l.Hq;
-      const dim3 cgrid(ka.n * l.Hq), cblock(32 * kCombineWarps);
-      e = launch_attn_combine(l.d, cgrid, cblock, s, ca);
+      ca.rows = ka.n * l.Hq;
+      ca.wpr = kCombineWarps;
+      while (ca.wpr > 1 && ca.rows * ca.wpr > kCombineWarps * kCombineWarps * num_sms) ca.wpr /= 2;
+      e = launch_attn_combine(l.d, (ca.rows * ca.wpr + kCombineWarps - 1) / kCombineWarps, s, ca);
       if (e != cudaSuccess) return e;
       ++*launches;
     }

@@ -1,12 +1,13 @@
 // trr_attn_row.cu - the kernels of trr_decode_attn with one query head per warp
-// (one mode per query): one instance per head size and groups per head.
+// (one mode per query): one instance per head size and groups
+// per head.
 #include "trr_row.cuh"
 
 namespace trr {
 
 template <int D, int NG>
 static cudaError_t launch(dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k) {
-  return launch_pdl(row_kernel<D, NG, false, false>, grid, dim3(32 * kRowWarps), smem, s, k);
+  return launch_pdl(row_kernel<D, NG, false, false, false>, grid, dim3(32 * kRowWarps), smem, s, k);
 }
 
 cudaError_t launch_attn_row(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k) {
@@ -17,11 +18,11 @@ cudaError_t launch_attn_row(const Layout& l, dim3 grid, size_t smem, cudaStream_
 }
 
 cudaError_t configure_attn_row() {
-  const void* ks[] = {reinterpret_cast<const void*>(row_kernel<64, 1, false, false>),
-                      reinterpret_cast<const void*>(row_kernel<64, 2, false, false>),
-                      reinterpret_cast<const void*>(row_kernel<128, 1, false, false>),
-                      reinterpret_cast<const void*>(row_kernel<128, 2, false, false>),
-                      reinterpret_cast<const void*>(row_kernel<128, 4, false, false>)};
+  const void* ks[] = {reinterpret_cast<const void*>(row_kernel<64, 1, false, false, false>),
+                      reinterpret_cast<const void*>(row_kernel<64, 2, false, false, false>),
+                      reinterpret_cast<const void*>(row_kernel<128, 1, false, false, false>),
+                      reinterpret_cast<const void*>(row_kernel<128, 2, false, false, false>),
+                      reinterpret_cast<const void*>(row_kernel<128, 4, false, false, false>)};
   for (const void* f : ks) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemLimit);
     if (e != cudaSuccess) return e;

@@ -1,12 +1,13 @@
 // trr_attn_row_heads.cu - the kernels of caches with per-head modes (presence masks
-// read with every page): one instance per head size and groups per head.
+// read with every page): one instance per head size and groups
+// per head.
 #include "trr_row.cuh"
 
 namespace trr {
 
 template <int D, int NG>
 static cudaError_t launch(dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k) {
-  return launch_pdl(row_kernel<D, NG, true, false>, grid, dim3(32 * kRowWarps), smem, s, k);
+  return launch_pdl(row_kernel<D, NG, true, false, false>, grid, dim3(32 * kRowWarps), smem, s, k);
 }
 
 cudaError_t launch_attn_row_heads(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k) {
@@ -17,11 +18,11 @@ cudaError_t launch_attn_row_heads(const Layout& l, dim3 grid, size_t smem, cudaS
 }
 
 cudaError_t configure_attn_row_heads() {
-  const void* ks[] = {reinterpret_cast<const void*>(row_kernel<64, 1, true, false>),
-                      reinterpret_cast<const void*>(row_kernel<64, 2, true, false>),
-                      reinterpret_cast<const void*>(row_kernel<128, 1, true, false>),
-                      reinterpret_cast<const void*>(row_kernel<128, 2, true, false>),
-                      reinterpret_cast<const void*>(row_kernel<128, 4, true, false>)};
+  const void* ks[] = {reinterpret_cast<const void*>(row_kernel<64, 1, true, false, false>),
+                      reinterpret_cast<const void*>(row_kernel<64, 2, true, false, false>),
+                      reinterpret_cast<const void*>(row_kernel<128, 1, true, false, false>),
+                      reinterpret_cast<const void*>(row_kernel<128, 2, true, false, false>),
+                      reinterpret_cast<const void*>(row_kernel<128, 4, true, false, false>)};
   for (const void* f : ks) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemLimit);
     if (e != cudaSuccess) return e;

@@ -93,17 +93,11 @@ static trr_status make_layout(const trr_cache_config* c, Layout* l) {
   // tokens), and few enough pages per split for any range up to max_context
   l->pos_split = static_cast<int>(std::max<int64_t>(l->P, l->split_bytes / l->tokb[2]));
   l->s_cap = 1 << 30;
-  // tiles: whole pages, or with one query head per warp up to 32 keys of one (16 of the
-  // widest rows)
-  l->split_keys = l->P;
-  l->split_extra = kClasses;
-  l->split_most = kItemMaxTiles - kClasses;
-  if (l->swz) {
-    const int most = std::min(l->P, 32), wide = std::min(l->P, l->d == 128 ? 16 : 32);
-    l->split_keys = wide;
-    l->split_extra = 3 * (l->P / most) + l->P / wide;
-    l->split_most = kItemMaxTiles - l->split_extra;
-  }
+  // tiles: up to 32 keys of a page (16 of the widest rows)
+  const int tile = std::min(l->P, 32), wide = std::min(l->P, l->d == 128 ? 16 : 32);
+  l->split_keys = wide;
+  l->split_extra = 3 * (l->P / tile) + l->P / wide;
+  l->split_most = kItemMaxTiles - l->split_extra;
   l->s_cap = std::max(splits_of(l->maxctx, l->pos_split, l->split_keys, l->split_extra, l->split_most, l->s_cap), 1);
   l->cnt_stride = 1 + (l->s_cap + kMergeGroup - 1) / kMergeGroup;
   l->max_items = static_cast<int64_t>(l->max_queries) * l->units * l->s_cap;

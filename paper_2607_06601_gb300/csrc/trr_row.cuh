@@ -1,22 +1,29 @@
 #pragma once
-// trr_row.cuh - the attention kernels of one query head per warp (MHA, wide query groups
-// and per-head modes): mode-routed split-K decode attention over the mixed-precision paged
-// cache (Sec. 3.2(A), Eq. 2; Sec. 3.8; Sec. 7).
+// trr_row.cuh - the attention kernels: mode-routed split-K decode attention over the
+// mixed-precision paged cache (Sec. 3.2(A), Eq. 2; Sec. 3.8; Sec. 7).
 //
-// A work unit is (query, query head, split) and belongs to one warp from its plan to its
-// row: the warp plans the unit (trr_attn.cuh, plan_split), streams its pages' KV slices
-// through a ring of shared memory of its own with 1-D bulk copies (one per page as a rule,
-// cp.async.bulk + mbarrier), and computes on them.  Nothing but the call's start and end
-// synchronises warps: a producer warp that fed four consumer warps through one ring, as
-// the kernels had before, kept two stages in flight and held every stage until the slowest
-// of the four was done with it.
+// A work unit is a split of a query for one query head (MHA, wide query groups, per-head
+// modes) or for one KV head and its query group, and belongs to one warp from its plan to its
+// row: the warp plans the unit (plan_pages), streams its pages' KV slices through a ring of
+// shared memory of its own with 1-D bulk copies (one per page as a rule, cp.async.bulk +
+// mbarrier), and computes on them.  Nothing but the call's start and end synchronises warps: a
+// producer warp that fed four consumer warps through one ring, as the kernels had before, kept
+// two stages in flight and held every stage until the slowest of the four was done with it.
+// The kernels are bound by instructions issued and by the latency of a unit's chain (plan,
+// copies, tiles, merge), not by memory: batch 256 of the sweep shape streams at 5.9 TB/s
+// with the tile arithmetic left out, at 3.8 TB/s with it.
 //
-// One CTA of eight warps per SM takes less than half of its shared memory and registers, so
-// that the next layer's kernel is resident while this one runs: its plans and its first
-// page copies come before its wait on this kernel.
+// Two CTAs of eight warps fill an SM; while some of the places are free or a CTA has ended,
+// the next layer's kernel is resident, so that its plans and its first page copies come before
+// its wait on this kernel.
 //
-// The arithmetic runs on the tensor cores (mma.sync m16n8k16, f32 accumulation) though only
-// one query head shares a key, because the codes then need one mask per two elements (a
+// Query groups (a producer warp and four consumer warps, then this kernel): two sequences of
+// 37 and 130 tokens generated with 4 heads on 2 1971 -> 1397 us; 32 heads on 8 of 128, 24
+// layers, batch 1, context 4096, 1106 -> 838; batch 16, context 32768, 380 -> 289 (most of it
+// the combine kernel).
+//
+// One query head per warp: the arithmetic runs on the tensor cores (mma.sync m16n8k16, f32
+// accumulation) though only one query head shares a key, because the codes then need one mask per two elements (a
 // pair of codes in the halves of a word, read as f16 subnormals) in place of one per
 // element, and the multiply-adds come free:
 //   q.k   A = 16 keys' codes, B = the query row, its column n holding quantiser group
@@ -48,12 +55,13 @@ constexpr float kLoScale = 2048.f;  // the low part of a weight is stored times 
 constexpr int kRowRed = 8 * kRowWarps * 2 + 4 * 32;  // plan_rows' sums and counts
 struct RowSmem {  // byte offsets of one CTA's shared memory
   int full, fac, q, w, pre, qinf, ord, red, ent, flag, ring, total;
-  __host__ __device__ RowSmem(int D, int NG, int n, int step, int ring_bytes)
+  // heads: query heads of a unit (query groups)
+  __host__ __device__ RowSmem(int D, int heads, int n, int step, int ring_bytes)
       : full(0),
         fac(full + kRowWarps * kRowSlots * 8),
         q(fac + 16 * (D / 8) * 4),
-        w(q + kRowWarps * D * 2),
-        pre(w + kRowWarps * row_w_bytes(NG)),
+        w(q + kRowWarps * heads * D * 2),
+        pre(w + kRowWarps * row_w_bytes(heads)),
         qinf(pre + align16(4 * (n + 2))),
         ord(qinf + 16 * n),
         red(ord + align16(2 * n)),
@@ -61,9 +69,17 @@ struct RowSmem {  // byte offsets of one CTA's shared memory
         flag(ent + (step ? align16(4 * step_ints(n)) : 0)),
         ring((flag + 16 + 127) & ~127),
         total(ring + kRowWarps * ring_bytes) {}
-  // the weights of a tile: 32 rows of 8 f16 (width 16: of 2 tf32)
-  __host__ __device__ static constexpr int row_w_bytes(int) { return 512; }
+  // the weights of a tile: 32 rows of 8 f16 (width 16: of 2 tf32; query groups: of 8 bf16,
+  // high parts, then low parts)
+  __host__ __device__ static constexpr int row_w_bytes(int heads) { return heads > 1 ? 1024 : 512; }
 };
+
+// The largest tile in a ring: 16-bit rows (at d 128 sixteen of them) or 32 8-bit ones, with a
+// presence mask and positions.
+constexpr int row_tile_bytes(int D, int NG) {
+  const int wide = (D == 64 ? 32 : 16) * 4 * D, b8 = 32 * (2 * D + 8 * NG);
+  return (((wide > b8 ? wide : b8) + 16 + 127) & ~127) + 128;
+}
 
 // Rows (work units per query split): full heads, local heads and the others of a query.
 struct HeadCounts {
@@ -96,8 +112,8 @@ __device__ __forceinline__ int div24(int x, int y) {
 // a local head), splits of a row (per-head modes: of a full head) | query error << 24 | zero
 // row << 28}.  A query has one unit per (row, split); with per-head modes each head its own
 // splits (one for a skip head, which writes its zero row).
-template <bool HM>
-__device__ __forceinline__ void plan_rows(const AttnKernelArgs& ka, int* pre, int4* qinf, uint16_t* ord, long long* red) {
+template <bool HM, bool GQ>
+__device__ __forceinline__ void plan_rows(const AttnKernelArgs& ka, int rows, int* pre, int4* qinf, uint16_t* ord, long long* red) {
   const LayerArgs& a = ka.a;
   const int n = ka.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int* counts = reinterpret_cast<int*>(red + 2 * kRowWarps);  // per 32 queries: full | local << 16
@@ -126,7 +142,7 @@ __device__ __forceinline__ void plan_rows(const AttnKernelArgs& ka, int* pre, in
         const HeadCounts c = head_counts(ka, q);
         rsum += static_cast<long long>(c.full) * (qi.y + 1) + static_cast<long long>(c.local) * (qi.y + 1 - qi.z);
       } else {
-        rsum += static_cast<long long>(r) * a.Hq;
+        rsum += static_cast<long long>(r) * rows;
       }
     }
     const unsigned f = __ballot_sync(0xffffffffu, cls == 0), l = __ballot_sync(0xffffffffu, cls == 1);
@@ -165,11 +181,14 @@ __device__ __forceinline__ void plan_rows(const AttnKernelArgs& ka, int* pre, in
   // Split size: about one unit per warp while a unit then stays short, else up to three per
   // warp, of 700 positions at least, handed out on demand; never below pos_split.  (1.3B
   // shape, batch 64, contexts to 8192: 637 us for 8 layer calls; one unit per warp only up to
-  // 768 positions 704, units from 512 positions 689, five per warp 768.)  Binary32
-  // arithmetic: the same result in every CTA, and it only sizes the splits.
+  // 768 positions 704, units from 512 positions 689, five per warp 768.  A query group's
+  // positions weigh about twice as much: gqa_long shape 412 us for 6 layer calls, 468 with units
+  // from 250 positions.)  Binary32 arithmetic: the same result in every CTA, and it only sizes
+  // the splits.
   const float warps = static_cast<float>(gridDim.x * kRowWarps), rs = static_cast<float>(rsum);
   const float one = rs / (0.85f * warps);
-  const float by_work = ceilf(one > 1000.f ? fmaxf(700.f, rs / (3.f * warps)) : one);
+  const float most = GQ ? 600.f : 1000.f, least = GQ ? 350.f : 700.f;
+  const float by_work = ceilf(one > most ? fmaxf(least, rs / (3.f * warps)) : one);
   const int pos_split = by_work > static_cast<float>(a.pos_split) ? static_cast<int>(fminf(by_work, 1073741824.f))
                                                                    : a.pos_split;
   const int chunk = (n + 32 * kRowWarps - 1) / (32 * kRowWarps);
@@ -178,10 +197,10 @@ __device__ __forceinline__ void plan_rows(const AttnKernelArgs& ka, int* pre, in
 #pragma unroll 1
   for (int k = q0; k < q1; ++k) {  // pre[k] becomes the query's unit count
     const int range = pre[k];
-    int ns = 1, units = a.Hq;
+    int ns = 1, units = rows;
     if (range > 0) {
       ns = splits_of(range, pos_split, a.split_keys, a.split_extra, a.split_most, a.s_cap);
-      units = a.Hq * ns;
+      units = rows * ns;
       if (HM) {
         const HeadCounts c = head_counts(ka, ord[k]);
         const int4 x = qinf[k];
@@ -260,7 +279,9 @@ __device__ __forceinline__ int plan_pages(const LayerArgs& a, int seq, int lo, i
     const int* arr = (side ? a.pfirst : a.plast) + row0;
     const int x = side ? t + 1 : lo;  // entries below x
     int l = 0, h = pages;             // the count lies in [l, h]
-    int probe = max(0, pages - 8) + sub, step = 1;  // first the last 8 pages: decode queries look there
+    // first the end of the list, where decode queries look: a window's pages and a few more
+    int step = side ? 1 : (((t + 1 - lo) >> lg) + 8) >> 3, p1 = max(0, pages - 8 * step);
+    int probe = p1 + sub * step;
 #pragma unroll 1
     while (__any_sync(0xffffffffu, l < h)) {
       const bool below = probe < h && arr[probe] < x;
@@ -704,6 +725,245 @@ __device__ __forceinline__ void tile_values16(RowState<D, NG>& st, const uint8_t
   }
 }
 
+// ------------------------------------------------------------------- query groups --
+//
+// A KV head with its g >= 2 query heads (g * NG <= 8) per unit: column n of the B operands is
+// head n / NG and quantiser group n % NG, so that lane (gid, tig) has the scores of keys
+// gid + 8 h + 16 u for its columns 2 tig and 2 tig + 1 (two groups of a head, or two heads at
+// NG = 1).  Weights p * s are one f16, width 16's p two bf16 parts.  A running maximum is
+// raised when a score exceeds it by 2^3 (any excess where a scale could then take p * s out
+// of f16's range): raised at every new maximum, as before, nine tiles in ten rescaled the
+// accumulators.  These caches' rows are stored plainly.
+constexpr float kGroupTau = 3.f, kGroupWide = 8000.f;
+template <int D, int NG>
+struct GroupState {
+  static constexpr int NP = D / 8, MT = D / 16;
+  uint32_t kb[NP];
+  float acc[MT][4];  // dims gid D/8 + 2 t (+ 1) x the lane's columns, times 2^vfac_log2
+  float qsum[2], m[2], l[2], zacc[2];  // per column (m: of its head)
+  float kfac;
+  uint32_t kl, vl;
+  int wl, zoff, E, cls;
+};
+
+template <int D, int NG, int B>
+__device__ __forceinline__ void group_class(GroupState<D, NG>& st, const uint8_t* qs, int heads, float qscale, int lane) {
+  constexpr int NP = D / 8, rowb = D * B / 8;
+  const int gid = lane >> 2, tig = lane & 3, r = gid / NG;
+  const bool ok = r < heads && (tig * NG) / 4 == gid % NG;
+  uint32_t raw[NP];
+  load_words<NP>(qs + (r < heads ? r : 0) * D * 2 + tig * (D / 2), raw);
+  const float escale = __int_as_float((127 - st.E) << 23);
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    uint32_t w = raw[i];
+    if (B != 16) {
+      const int lo = kp_lo<B>(i), hi = kp_hi<B>(i);
+      const float f = pow2f(smax_of<B>() - kp_pos<B>(i)) * escale;
+      w = pack_f16x2(((lo & 1) ? bf_hi(raw[lo >> 1]) : bf_lo(raw[lo >> 1])) * f,
+                     ((hi & 1) ? bf_hi(raw[hi >> 1]) : bf_lo(raw[hi >> 1])) * f);
+    }
+    st.kb[i] = ok ? w : 0u;
+  }
+  st.kfac = B == 16 ? qscale : __int_as_float((127 + 24 - smax_of<B>() + st.E) << 23) * qscale;
+  st.kl = gid * rowb + tig * (rowb / 4);
+  st.vl = tig * rowb + (rowb >= 32 ? gid * (rowb / 8) : (gid * (rowb / 8)) & ~3);
+}
+
+template <int D, int NG>
+__device__ __forceinline__ void group_switch(GroupState<D, NG>& st, int to, bool fresh, const uint8_t* qs, int heads,
+                                             const float* fac, float qscale, int kt, int lane) {
+  constexpr int MT = D / 16;
+  switch (to) {
+    case 0: group_class<D, NG, 2>(st, qs, heads, qscale, lane); break;
+    case 1: group_class<D, NG, 4>(st, qs, heads, qscale, lane); break;
+    case 2: group_class<D, NG, 8>(st, qs, heads, qscale, lane); break;
+    default: group_class<D, NG, 16>(st, qs, heads, qscale, lane); break;
+  }
+  st.wl = 16 * w_row<0>(lane);
+  st.zoff = kt * (2 * (D * bits_of_class(to) / 8) + 4 * NG) + (lane >> 2) * NG * 4 + (NG == 4 ? (lane & 1) * 8 : 0);
+  if (!fresh) {
+    float f[2 * MT];
+    load_words<2 * MT>(reinterpret_cast<const uint8_t*>(fac + (st.cls * 4 + to) * (D / 8)), reinterpret_cast<uint32_t*>(f));
+#pragma unroll
+    for (int t = 0; t < MT; ++t) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) st.acc[t][i] *= f[2 * t + (i >> 1)];
+    }
+  }
+  st.cls = to;
+}
+
+// 1. The columns' group sums of q.c: c[u][2 h + j] is key gid + 8 h + 16 u, column 2 tig + j.
+template <int D, int NG, int B>
+__device__ __forceinline__ void group_scores(const GroupState<D, NG>& st, const uint8_t* tile, int kt, float (&c)[2][4]) {
+  constexpr int KS = D / 16, rowb = D * B / 8;
+  constexpr int KW = D * B / 128;  // K words per lane and key (D/4 dims)
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    if (u == 1 && kt == 16) break;
+    float c2[4];
+    constexpr int KH = KW >= 8 ? KW / 4 : 1, KWH = KW / KH, KSH = KS / KH;
+#pragma unroll
+    for (int hf = 0; hf < KH; ++hf) {
+      uint32_t k1[KWH], k2[KWH];
+      load_words<KWH>(tile + st.kl + 16 * u * rowb + 16 * hf, k1);
+      load_words<KWH>(tile + st.kl + (16 * u + 8) * rowb + 16 * hf, k2);
+#pragma unroll
+      for (int s = hf * KSH; s < (hf + 1) * KSH; ++s) {
+        const int i0 = 2 * (s - hf * KSH);
+        const uint32_t a0 = k_pair<B>(k1, i0), a1 = k_pair<B>(k2, i0), a2 = k_pair<B>(k1, i0 + 1), a3 = k_pair<B>(k2, i0 + 1);
+        if (s == 0) mma_cls0<B>(c[u], a0, a1, a2, a3, st.kb[0], st.kb[1]);
+        else if (D == 128 && s == 1) mma_cls0<B>(c2, a0, a1, a2, a3, st.kb[2], st.kb[3]);
+        else mma_cls<B>((D == 128 && (s & 1)) ? c2 : c[u], a0, a1, a2, a3, st.kb[2 * s], st.kb[2 * s + 1]);
+      }
+    }
+    if (D == 128) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) c[u][i] += c2[i];
+    }
+  }
+}
+
+// 2. The weights of the lane's four keys (ok: bit 2 u + h) for its columns, as operand rows at
+// wb.  has_sz: the width has scales (at sz: the key gid's V scales, K's kt keys before).
+template <int D, int NG>
+__device__ __forceinline__ void group_weights(GroupState<D, NG>& st, const float (&c)[2][4], unsigned ok, bool has_sz,
+                                              const uint8_t* sz, int kt, int heads, uint8_t* wb, int lane) {
+  constexpr int MT = D / 16, J = NG == 1 ? 2 : 1;  // heads of a lane
+  const int gid = lane >> 2, tig = lane & 3;
+  float sc[4][J], big = 0.f;
+  uint32_t zw[4][2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {  // key gid + 8 k
+    uint32_t kw[2] = {0x3c00u, 0x3c00u};
+    zw[k][0] = zw[k][1] = 0x3c00u;
+    const bool good = (ok >> k) & 1u;
+    if (has_sz && (k < 2 || kt > 16)) {
+      if (NG == 1) {
+        load_words<1>(sz + (8 * k - kt) * NG * 4, kw);
+        load_words<1>(sz + 8 * k * NG * 4, zw[k]);
+        kw[1] = kw[0];
+        zw[k][1] = zw[k][0];
+      } else {
+        load_words<2>(sz + (8 * k - kt) * NG * 4, kw);
+        load_words<2>(sz + 8 * k * NG * 4, zw[k]);
+      }
+    }
+    float cp[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&kw[j]));
+      cp[j] = fmaf(f.x * st.kfac, c[k >> 1][2 * (k & 1) + j], f.y * st.qsum[j]);
+      if (!good) zw[k][j] = 0u;  // a slot that does not count may hold any bytes
+    }
+    if (NG == 1) {
+      sc[k][0] = cp[0];
+      sc[k][J - 1] = cp[1];
+    } else {
+      sc[k][0] = cp[0] + cp[1];
+      if (NG == 4) sc[k][0] += __shfl_xor_sync(0xffffffffu, sc[k][0], 1);
+    }
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      if (!good || (2 * tig + j) / NG >= heads) sc[k][j] = kNegInf;
+    }
+  }
+  float over = kNegInf;  // the largest excess over the lane's maxima
+#pragma unroll
+  for (int j = 0; j < J; ++j)
+    over = fmaxf(over, fmaxf(fmaxf(sc[0][j], sc[1][j]), fmaxf(sc[2][j], sc[3][j])) - st.m[j]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    big = fmaxf(big, fmaxf(__half2float(__ushort_as_half(zw[k][0] & 0xffff)), __half2float(__ushort_as_half(zw[k][1] & 0xffff))));
+  if (__any_sync(0xffffffffu, over > kGroupTau || (over > 0.f && big > kGroupWide))) {  // (the keys' lanes share a maximum)
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      float mx = fmaxf(fmaxf(sc[0][j], sc[1][j]), fmaxf(sc[2][j], sc[3][j]));
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      mx = fmaxf(mx, st.m[j]);
+      const float alpha = fast_exp2(st.m[j] - mx);
+      st.m[j] = mx;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        if (NG == 1 && i != j) continue;
+        st.l[i] *= alpha;
+        st.zacc[i] *= alpha;
+#pragma unroll
+        for (int t = 0; t < MT; ++t) {
+          st.acc[t][i] *= alpha;
+          st.acc[t][i + 2] *= alpha;
+        }
+      }
+      if (NG > 1) st.m[1] = mx;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float p[2], w[2];
+    p[0] = fast_exp2(sc[k][0] - st.m[0]);
+    p[1] = NG == 1 ? fast_exp2(sc[k][J - 1] - st.m[1]) : p[0];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&zw[k][j]));
+      st.l[j] += p[j];
+      st.zacc[j] = fmaf(p[j], f.y, st.zacc[j]);
+      w[j] = p[j] * f.x;
+    }
+    uint32_t* at = reinterpret_cast<uint32_t*>(wb + 16 * (gid + 8 * k)) + tig;
+    if (has_sz) {
+      at[0] = pack_f16x2(w[0], w[1]);
+    } else {
+      const uint32_t hi = pack_bf16x2(w[0], w[1]);
+      at[0] = hi;
+      at[128] = pack_bf16x2(w[0] - bf_lo(hi), w[1] - bf_hi(hi));
+    }
+  }
+}
+
+// 3. P.V.  all[k]: lanes whose key gid + 8 k counts (width 16: other keys' values read as 0).
+template <int D, int NG, int B>
+__device__ __forceinline__ void group_values(GroupState<D, NG>& st, const uint8_t* tile, int kt, bool part,
+                                             const unsigned (&all)[4], const uint8_t* wb, int lane) {
+  constexpr int MT = D / 16, rowb = D * B / 8;
+  constexpr int VB = D * B / 64, VW = VB >= 4 ? VB / 4 : 1;  // V bytes per lane and key (D/8 dims)
+  constexpr int VH = VW > 4 ? VW / 4 : 1, VWH = VW / VH, MTH = MT / VH;
+  const int gid = lane >> 2, tig = lane & 3;
+  const uint8_t* v0 = tile + kt * rowb + st.vl;
+  uint32_t w[4], wlo[4];
+  ldmatrix4_trans(w, wb + st.wl);
+  if (B == 16) ldmatrix4_trans(wlo, wb + 512 + st.wl);
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    if (u == 1 && kt == 16) break;
+#pragma unroll
+    for (int hf = 0; hf < VH; ++hf) {
+      uint32_t x[4][VWH];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        load_words<VWH>(v0 + 4 * (4 * u + i) * rowb + 16 * hf, x[i]);  // key tig + 4 (4 u + i)
+        if (VB < 4) x[i][0] >>= ((gid * VB) & 3) * 8;
+        if (B == 16 && part) {
+          const int key = tig + 4 * (4 * u + i);  // its ok: lane 4 (key % 8)'s bit of all[key / 8]
+          const unsigned bits = key & 16 ? (key & 8 ? all[3] : all[2]) : (key & 8 ? all[1] : all[0]);
+          if (!((bits >> (4 * (key & 7))) & 1u)) {
+#pragma unroll
+            for (int y = 0; y < VWH; ++y) x[i][y] = 0u;
+          }
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < MTH; ++t) {
+        const uint32_t a0 = v_pair<B>(x[0], x[1], 2 * t), a1 = v_pair<B>(x[0], x[1], 2 * t + 1);
+        const uint32_t a2 = v_pair<B>(x[2], x[3], 2 * t), a3 = v_pair<B>(x[2], x[3], 2 * t + 1);
+        mma_cls<B>(st.acc[hf * MTH + t], a0, a1, a2, a3, w[2 * u], w[2 * u + 1]);
+        if (B == 16) mma_bf16(st.acc[hf * MTH + t], a0, a1, a2, a3, wlo[2 * u], wlo[2 * u + 1]);
+      }
+    }
+  }
+}
+
 // --------------------------------------------------------------------------- rows --
 
 // A row at its unit's end (lane holds dims lane * D/32 .. of the unnormalised sum, relative to
@@ -828,8 +1088,13 @@ __device__ __forceinline__ uint2 load_row(const uint16_t* src, int lane) {
   return r;
 }
 
-// The per-entry table of a decode-step call (see plan_entries in trr_attn.cuh for what it
-// checks and holds), built by every CTA with one thread per entry (n <= kStepMax threads).
+// Every CTA: validates the entries and plans where each token goes (the same plan as the
+// append kernels: the token takes index ntok of its (sequence, class) list; index % P == 0
+// opens a page, whose id is next_page + the class's openers before it).  Errors, lowest
+// entry first: sequence id, bit-width or mode not allowed, or a sequence named by an
+// earlier entry (INVALID_ARG); position outside [0, max_context) or not above the
+// sequence's last one (BAD_POSITION); a local query with a window below 1 (INVALID_ARG).
+// Built with one thread per entry (n <= kStepMax threads).
 __device__ __forceinline__ void plan_entries_cta(const AttnKernelArgs& ka, int* ent) {
   const LayerArgs& a = ka.a;
   const int n = ka.n, e = threadIdx.x, lane = e & 31, warp = e >> 5, H = 2 * n;
@@ -910,27 +1175,29 @@ __device__ __forceinline__ void plan_entries_cta(const AttnKernelArgs& ka, int* 
 
 // ------------------------------------------------------------------------- kernel --
 
-template <int D, int NG, bool HM, bool STEP>
+// GQ: a unit is a KV head and its query group, and the combine kernel merges its splits.
+template <int D, int NG, bool HM, bool STEP, bool GQ>
 __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_constant__ AttnKernelArgs ka) {
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr int DPL = D / 32;
   const LayerArgs& a = ka.a;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = ka.n, P = a.P, R = ka.ring_bytes;
-  const RowSmem lay(D, NG, n, STEP, R);
+  const int g = a.Hq / a.Hkv, heads = GQ ? g : 1, rows = GQ ? a.Hkv : a.Hq;  // of a unit; of a query
+  const RowSmem lay(D, heads, n, STEP, R);
   int* pre = reinterpret_cast<int*>(smem + lay.pre);
   int* ent = reinterpret_cast<int*>(smem + lay.ent);
   int* sc = ent + 6 * n;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + lay.flag);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + lay.full) + warp * kRowSlots;
   uint8_t* ring = smem + lay.ring + warp * R;
-  uint8_t* qs = smem + lay.q + warp * D * 2;
+  uint8_t* qs = smem + lay.q + warp * heads * D * 2;
   float* fac = reinterpret_cast<float*>(smem + lay.fac);
 #pragma unroll 1
   for (int i = threadIdx.x; i < 16 * (D / 8); i += 32 * kRowWarps) {
     const int j = i % (D / 8), from = i / (4 * (D / 8)), to = (i / (D / 8)) & 3;
     fac[i] = __int_as_float((127 + row_fac(to, j) - row_fac(from, j)) << 23);
   }
-  uint8_t* wb = smem + lay.w + warp * RowSmem::row_w_bytes(NG);
+  uint8_t* wb = smem + lay.w + warp * RowSmem::row_w_bytes(GQ ? 2 : 1);
   if (threadIdx.x < kRowWarps * kRowSlots) mbar_init(reinterpret_cast<uint64_t*>(smem + lay.full) + threadIdx.x, 1);
   if (threadIdx.x == 0) *abort_flag = 0;
   fence_barrier_init();
@@ -939,7 +1206,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
   // read before the wait only when `early` says that no kernel still running can write it.
   int4* qinf = reinterpret_cast<int4*>(smem + lay.qinf);
   uint16_t* ord = reinterpret_cast<uint16_t*>(smem + lay.ord);
-  plan_rows<HM>(ka, pre, qinf, ord, reinterpret_cast<long long*>(smem + lay.red));
+  plan_rows<HM, GQ>(ka, rows, pre, qinf, ord, reinterpret_cast<long long*>(smem + lay.red));
   bool waited = !(STEP && ka.early);
   if (waited) {
     pdl_wait();
@@ -958,7 +1225,6 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
   uint32_t base = 0;                  // tiles of the units before
   int inext = 0;                      // next tile to issue
   bool good = true;                   // no wait gave up
-  const int g = a.Hq / a.Hkv;
   int kvh = 0;                        // the unit's KV head
   const int kt_most = min(P, 32), kt_wide = min(P, D == 128 ? 16 : 32);
   auto tile_keys = [&](int cls) { return D == 128 && cls == 3 ? kt_wide : kt_most; };
@@ -993,6 +1259,14 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       }
       if (posb) bulk_g2s(dst + ((tile_rows(cls) + 127) & ~127), sl - a.hdr - kvh * a.slice[cls] + 4 * key0, posb, bar);
     }
+  };
+  // waits for tile c's copies; false (and not good) when the wait gave up
+  auto tile_in = [&](int c) -> bool {
+    const uint32_t slot = (base + c) % kRowSlots, parity = ((base + c) / kRowSlots) & 1;
+    bool arrived = mbar_test_at(smem_u32(&full[slot]), parity);
+    if (!arrived) arrived = mbar_wait_slow(&full[slot], parity, abort_flag, a.wait_ns);
+    good = __all_sync(0xffffffffu, arrived);  // give up together, never half a warp
+    return good;
   };
   // the unit u: its query, head, split and pages
   auto plan = [&](int u) {
@@ -1057,11 +1331,11 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       }
       un.zero = hmode == TRR_MODE_SKIP;
     } else {
-      un.sp = div24(r, a.Hq);
-      un.h = r - un.sp * a.Hq;
-      un.base = pre[q] + un.h * un.ns;
+      un.sp = div24(r, rows);
+      un.h = r - un.sp * rows;
+      un.base = (pre[q] + un.h * un.ns) * heads;
     }
-    kvh = g == 1 ? un.h : div24(un.h, g);
+    kvh = GQ || g == 1 ? un.h : div24(un.h, g);
     int wid = -1, wmeta = 0;
     un.T = un.zero ? 0 : plan_pages(a, qi.x, un.lo, un.t, un.sp, un.ns, STEP, kt_most, kt_wide, lane, wid, wmeta);
     if (kt_wide < P || kt_most < P) {  // pages to tiles
@@ -1126,7 +1400,8 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
 #pragma unroll 1
   for (;;) {
     if (u < total && good) plan(u);
-    if (!started) {
+    const bool first = !started;
+    if (first) {
       started = true;
       if (STEP) plan_entries_cta(ka, ent);
       if (!waited) {
@@ -1140,10 +1415,15 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
                                                                       next_page + sc[kSOpeners + (lane & 3)] > lim);
       }
     }
+    if (GQ && ka.defer_merge && first && blockIdx.x == 0) {  // for the combine kernel: a query's first partial, splits
+      int2* qtab = reinterpret_cast<int2*>(a.cnt);
+#pragma unroll 1
+      for (int k = threadIdx.x; k < n; k += 32 * kRowWarps) qtab[ord[k]] = make_int2(pre[k] * heads, qinf[k].w & 0xffffff);
+    }
     if (u >= total || !good) break;
     int u_next = total;
     if (total > nwarps && lane == 0) u_next = nwarps + atomicAdd(&a.lctl[kNextUnit], 1);  // read at the unit's end
-    const bool own = un.h == kvh * g;  // stores a new token's rows of its KV head
+    const bool own = GQ || un.h == kvh * g;  // stores a new token's rows of its KV head
     // decode step: the entry's own token joins the row's last split; a skip token that
     // stores KV is written by its zero row's unit
     const bool has_new = STEP && !failed && un.sp == un.ns - 1 && ent[2 * un.q] >= 0 && (!un.zero || own);
@@ -1153,9 +1433,9 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       rk = load_row<D>(ka.k + src, lane);
       rv = load_row<D>(ka.v + src, lane);
     }
-    const int64_t qrow = (static_cast<int64_t>(un.q) * a.Hq + un.h) * D;
+    const int64_t qrow = (static_cast<int64_t>(un.q) * a.Hq + un.h * heads) * D;  // its first head's
     uint2 qraw = make_uint2(0, 0);
-    if (!un.zero) qraw = load_row<D>(ka.q + qrow, lane);
+    if (!GQ && !un.zero) qraw = load_row<D>(ka.q + qrow, lane);
     float kx[DPL] = {}, vx[DPL] = {}, new_score = kNegInf;
     if (has_new) {
       const int tok = ent[2 * un.q], info = ent[2 * un.q + 1], c = info & 3;
@@ -1175,10 +1455,163 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
     if (un.zero) {
       if (un.sp == 0) {
         uint32_t* o = reinterpret_cast<uint32_t*>(ka.out + qrow);
-        o[lane] = 0u;
-        if (D == 128) o[32 + lane] = 0u;
+#pragma unroll 1
+        for (int i = lane; i < heads * D / 2; i += 32) o[i] = 0u;
       }
       if (!STEP && un.err && un.sp == 0 && lane == 0) atomicMin(&a.lctl[kFirstBadQuery], (ka.q0 + un.q) * 16 + un.err);
+    } else if constexpr (GQ) {
+      // the group's query rows to shared memory; their largest exponent, each column's sum
+      GroupState<D, NG> st;
+      const int gid = lane >> 2, tig = lane & 3;
+      float qmax = 0.f, new_score[2] = {kNegInf, kNegInf};
+      st.qsum[0] = st.qsum[1] = 0.f;
+      constexpr int kMost = 8 / NG;  // heads of a group, at most
+      uint2 raws[kMost];
+#pragma unroll
+      for (int r = 0; r < kMost; ++r)
+        raws[r] = r < heads ? load_row<D>(ka.q + qrow + r * D, lane) : make_uint2(0, 0);
+#pragma unroll
+      for (int r = 0; r < kMost; ++r) {
+        if (r >= heads) break;
+        const uint2 raw = raws[r];
+        float x[DPL], sum = 0.f, dot = 0.f;
+        x[0] = bf_lo(raw.x);
+        x[1] = bf_hi(raw.x);
+        if (D == 128) {
+          x[D == 128 ? 2 : 0] = bf_lo(raw.y);
+          x[D == 128 ? 3 : 1] = bf_hi(raw.y);
+          reinterpret_cast<uint2*>(qs + r * D * 2)[lane] = raw;
+        } else {
+          reinterpret_cast<uint32_t*>(qs + r * D * 2)[lane] = raw.x;
+        }
+#pragma unroll
+        for (int j = 0; j < DPL; ++j) {
+          qmax = fmaxf(qmax, fabsf(x[j]));
+          sum += x[j];
+          dot = fmaf(x[j], kx[j], dot);
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          if (o < 32 / NG) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+          dot += __shfl_xor_sync(0xffffffffu, dot, o);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const float v = __shfl_sync(0xffffffffu, sum, ((2 * tig + j) % NG) * (32 / NG));
+          if ((2 * tig + j) / NG == r) {
+            st.qsum[j] = v * ka.qscale;
+            new_score[j] = has_new ? dot * ka.qscale : kNegInf;
+          }
+        }
+      }
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
+      st.E = min(100, max(-100, static_cast<int>((__float_as_uint(qmax) >> 23) & 0xff) - 127 - 6));
+      st.cls = 3;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        st.m[j] = -1e30f;
+        st.l[j] = st.zacc[j] = 0.f;
+      }
+#pragma unroll
+      for (int t = 0; t < D / 16; ++t) st.acc[t][0] = st.acc[t][1] = st.acc[t][2] = st.acc[t][3] = 0.f;
+      __syncwarp();
+      int c = 0;  // next tile to consume
+#pragma unroll 1
+      for (; c < un.T; ++c) {
+        const uint32_t geo = __shfl_sync(0xffffffffu, wgeo, c);
+        const int cls = geo & 3, kt = tile_keys(cls);
+        if (c == 0 || cls != st.cls) group_switch<D, NG>(st, cls, c == 0, qs, heads, fac, ka.qscale, kt, lane);
+        if (!tile_in(c)) break;
+        const uint8_t* tile = ring + ((geo >> 3) & (1023u << 7));
+        const int fill = (geo >> 2) & 127;
+        unsigned ok = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) ok |= static_cast<unsigned>(gid + 8 * k < fill) << k;
+        if (geo & kMask) {
+          const int* pos = reinterpret_cast<const int*>(tile + ((tile_rows(cls) + 127) & ~127));
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int p = pos[min(gid + 8 * k, kt - 1)];
+            if (p < un.lo || p > un.t) ok &= ~(1u << k);
+          }
+        }
+        float sc[2][4] = {};
+        switch (cls) {
+          case 0: group_scores<D, NG, 2>(st, tile, kt, sc); break;
+          case 1: group_scores<D, NG, 4>(st, tile, kt, sc); break;
+          case 2: group_scores<D, NG, 8>(st, tile, kt, sc); break;
+          default: group_scores<D, NG, 16>(st, tile, kt, sc); break;
+        }
+        group_weights<D, NG>(st, sc, ok, cls != 3, tile + st.zoff, kt, heads, wb, lane);
+        unsigned all[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) all[k] = __ballot_sync(0xffffffffu, (ok >> k) & 1u);
+        __syncwarp();
+        switch (cls) {
+          case 0: group_values<D, NG, 2>(st, tile, kt, false, all, wb, lane); break;
+          case 1: group_values<D, NG, 4>(st, tile, kt, false, all, wb, lane); break;
+          case 2: group_values<D, NG, 8>(st, tile, kt, false, all, wb, lane); break;
+          default: group_values<D, NG, 16>(st, tile, kt, fill < kt || (geo & kMask), all, wb, lane); break;
+        }
+        __syncwarp();  // the tile's bytes and weights are read
+        if (inext < un.T) issue(c + 1, __shfl_sync(0xffffffffu, wcum, c));
+      }
+      consumed = c;
+      if (!good) break;
+      // the heads' rows: lane (gid, tig) has dims gid D/8 .. of the columns whose group they are in
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+          st.l[j] += __shfl_xor_sync(0xffffffffu, st.l[j], o);
+          st.zacc[j] += __shfl_xor_sync(0xffffffffu, st.zacc[j], o);
+        }
+      }
+      float* vnew = reinterpret_cast<float*>(wb);  // the new token's V row
+      if (has_new) {
+#pragma unroll
+        for (int j = 0; j < DPL; ++j) vnew[lane * DPL + j] = vx[j];
+      }
+      __syncwarp();
+      float f[D / 8];
+      load_words<D / 8>(reinterpret_cast<const uint8_t*>(fac + (st.cls * 4 + 3) * (D / 8)), reinterpret_cast<uint32_t*>(f));
+      auto finish = [&](auto column) {
+        constexpr int j = decltype(column)::value;
+        const int r = (2 * tig + j) / NG, gi = (2 * tig + j) % NG;
+        float M = st.m[j], L = st.l[j], fo = 1.f, fn = 0.f;
+        if (has_new) {  // fold the new token in
+          M = fmaxf(st.m[j], new_score[j]);
+          fo = fast_exp2(st.m[j] - M);
+          fn = fast_exp2(new_score[j] - M);
+          L = fmaf(L, fo, fn);
+        }
+        if (r >= heads || gid * NG / 8 != gi) return;
+        const float inv = un.ns > 1 ? 1.f : L > 0.f ? 1.f / L : 0.f;
+        float y[D / 8];
+#pragma unroll
+        for (int i = 0; i < D / 8; ++i) {
+          float v = fmaf(st.acc[i / 2][2 * (i % 2) + j], f[i], st.zacc[j]) * fo;
+          if (has_new) v = fmaf(fn, vnew[gid * (D / 8) + i], v);
+          y[i] = v * inv;
+        }
+        if (un.ns == 1) {
+          uint4* o = reinterpret_cast<uint4*>(ka.out + qrow + r * D + gid * (D / 8));
+#pragma unroll
+          for (int i = 0; i < D / 8; i += 8)
+            o[i / 8] = make_uint4(pack_bf16x2(y[i], y[i + 1]), pack_bf16x2(y[i + 2], y[i + 3]), pack_bf16x2(y[i + 4], y[i + 5]),
+                                  pack_bf16x2(y[i + 6], y[i + 7]));
+        } else {  // the split's partial; the combine kernel merges them
+          float* pp = a.part + static_cast<int64_t>(un.base + r * un.ns + un.sp) * (D + 4);
+#pragma unroll
+          for (int i = 0; i < D / 8; i += 4)
+            *reinterpret_cast<float4*>(pp + gid * (D / 8) + i) = make_float4(y[i], y[i + 1], y[i + 2], y[i + 3]);
+          if (gid == 0) *reinterpret_cast<float2*>(pp + D) = make_float2(M, L);  // (group 0's column)
+        }
+      };
+      finish(std::integral_constant<int, 0>());
+      finish(std::integral_constant<int, 1>());
+      __syncwarp();  // vnew is read
     } else {
       // the query row to shared memory; its largest exponent, the sums over its groups
       float x[DPL];
@@ -1228,13 +1661,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
         const uint32_t geo = __shfl_sync(0xffffffffu, wgeo, c);
         const int cls = geo & 3, kt = tile_keys(cls);
         if (c == 0 || cls != st.cls) row_switch<D, NG>(st, cls, c == 0, qs, qraw, fac, ka.qscale, kt, lane);
-        const uint32_t slot = (base + c) % kRowSlots, parity = ((base + c) / kRowSlots) & 1;
-        bool arrived = mbar_test_at(smem_u32(&full[slot]), parity);
-        if (!arrived) arrived = mbar_wait_slow(&full[slot], parity, abort_flag, a.wait_ns);
-        if (!__all_sync(0xffffffffu, arrived)) {  // give up together, never half a warp
-          good = false;
-          break;
-        }
+        if (!tile_in(c)) break;
         const uint8_t* tile = ring + ((geo >> 3) & (1023u << 7));
         uint32_t there = 0xffffffffu;
         if (HM) {  // the KV head's presence mask, which ends the tile's rows
@@ -1334,6 +1761,11 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
     const int64_t n16 = static_cast<int64_t>(n) * a.Hq * D / 8;
 #pragma unroll 1
     for (int64_t i = threadIdx.x; i < n16; i += blockDim.x) o[i] = make_uint4(0, 0, 0, 0);
+    if (GQ && ka.defer_merge) {  // nothing to merge
+      int2* qtab = reinterpret_cast<int2*>(a.cnt);
+#pragma unroll 1
+      for (int q = threadIdx.x; q < n; q += blockDim.x) qtab[q] = make_int2(0, 1);
+    }
   }
   if (done < 0x10000) step_commit(ka, ent);  // a call that gave up a wait stores nothing
 }

@@ -104,3 +104,28 @@ def test_infinite_values_stay_in_their_rows():
     want = np.isinf(np.zeros_like(out))
     want[1, 1, 7] = True
     assert np.array_equal(np.isinf(out), want) and not np.isnan(out).any() and out[1, 1, 7] > 0
+
+
+GROUPS = [  # d, G, P, Hq, Hkv: read by the kernels with a KV head and its query group per warp
+    (64, 32, 32, 4, 2), (64, 64, 16, 8, 1), (64, 64, 64, 12, 4), (128, 128, 32, 10, 2), (128, 64, 64, 8, 2),
+    (128, 32, 16, 4, 2),
+]
+
+
+@pytest.mark.parametrize("bits", [(2,), (4,), (8,), (16,), (2, 4, 8, 16)])
+@pytest.mark.parametrize("d,G,P,Hq,Hkv", GROUPS)
+def test_group_tile_edges(d, G, P, Hq, Hkv, bits):
+    test_tile_edges(d, G, P, Hq, Hkv, bits)
+
+
+@pytest.mark.parametrize("n", [2, 50, 100, 200])
+def test_rows_of_several_splits(n):
+    """Calls of 64 to 6400 (query, head) rows with up to a dozen splits each: the kernel that
+    merges them gives a row 8, 4, 2 and 1 warps."""
+    rng = np.random.default_rng(n)
+    d, G, P, Hq, Hkv, S, ctx = 64, 64, 16, 32, 8, 2, 3000
+    pair = Pair(1, S, Hq, Hkv, d, G, P, ctx, [S * (ctx // P + 2)] * 4, max_queries=n)
+    _fill(pair, rng, [ctx] * S, Hkv, d, (2, 4, 8, 16), modes=lambda m: rng.choice(3, size=m))
+    q = wl.bf16_bits(rng.standard_normal((n, Hq, d), dtype=np.float32))
+    pair.attend(0, rng.integers(0, S, n), np.r_[ctx - 1, rng.integers(0, ctx, n - 1)], q, rng.choice(3, size=n),
+                windows=rng.integers(1, 900, n))
