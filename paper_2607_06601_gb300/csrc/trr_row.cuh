@@ -1391,7 +1391,19 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
   };
 
   // The first unit is planned and its copies issued before the rest of the call's start.
-  int u = blockIdx.x * kRowWarps + warp;
+  // Units that do not fill half of the CTAs, one per SM, are dealt evenly to these; more fill
+  // CTA after CTA, which leaves places for the next layer's kernel.  (Without the deal a 24
+  // layer step of batch 1, context 4096, took 1180 us in place of 1130, 12 heads, batch 20, in
+  // pages of 16 389 in place of 363; dealing up to a unit per warp evenly to all CTAs cost the
+  // 160M step 850 us in place of 813.)
+  const int cta = static_cast<int>(blockIdx.x), half = (gridDim.x + 1) / 2;
+  int per = kRowWarps, more = 0;
+  if (total < half * kRowWarps) {
+    per = div24(total, half);
+    more = total - per * half;
+    if (cta >= half) per = more = 0;
+  }
+  int u = warp < per + (cta < more) ? cta * per + min(cta, more) + warp : total;
   int consumed = 0;      // tiles of the unit
   int next_page = 0;     // decode step: the pools' counters (lanes 0 .. 3)
   bool failed = false;   // and whether the call fails (it then stores nothing, and the last
