@@ -730,7 +730,9 @@ __device__ __forceinline__ void tile_values16(RowState<D, NG>& st, const uint8_t
 // A KV head with its g >= 2 query heads (g * NG <= 8) per unit: column n of the B operands is
 // head n / NG and quantiser group n % NG, so that lane (gid, tig) has the scores of keys
 // gid + 8 h + 16 u for its columns 2 tig and 2 tig + 1 (two groups of a head, or two heads at
-// NG = 1).  Weights p * s are one f16, width 16's p two bf16 parts.  A running maximum is
+// NG = 1).  Weights p * s are two f16 parts, width 16's p two bf16 parts (one f16 part, as
+// before, rounds by 2^-12: rows were 0.6 to 2% further off than with a maximum raised at every
+// score; two parts are closer than that was, for 1 to 4% of the time).  A running maximum is
 // raised when a score exceeds it by 2^3 (any excess where a scale could then take p * s out
 // of f16's range): raised at every new maximum, as before, nine tiles in ten rescaled the
 // accumulators.  These caches' rows are stored plainly.
@@ -912,8 +914,11 @@ __device__ __forceinline__ void group_weights(GroupState<D, NG>& st, const float
       w[j] = p[j] * f.x;
     }
     uint32_t* at = reinterpret_cast<uint32_t*>(wb + 16 * (gid + 8 * k)) + tig;
-    if (has_sz) {
-      at[0] = pack_f16x2(w[0], w[1]);
+    if (has_sz) {  // high and low part (finite: p <= 1 where a scale is above kGroupWide)
+      const uint32_t hi = pack_f16x2(w[0], w[1]);
+      const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&hi));
+      at[0] = hi;
+      at[128] = pack_f16x2(w[0] - h.x, w[1] - h.y);
     } else {
       const uint32_t hi = pack_bf16x2(w[0], w[1]);
       at[0] = hi;
@@ -933,7 +938,7 @@ __device__ __forceinline__ void group_values(GroupState<D, NG>& st, const uint8_
   const uint8_t* v0 = tile + kt * rowb + st.vl;
   uint32_t w[4], wlo[4];
   ldmatrix4_trans(w, wb + st.wl);
-  if (B == 16) ldmatrix4_trans(wlo, wb + 512 + st.wl);
+  ldmatrix4_trans(wlo, wb + 512 + st.wl);
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     if (u == 1 && kt == 16) break;
@@ -958,7 +963,7 @@ __device__ __forceinline__ void group_values(GroupState<D, NG>& st, const uint8_
         const uint32_t a0 = v_pair<B>(x[0], x[1], 2 * t), a1 = v_pair<B>(x[0], x[1], 2 * t + 1);
         const uint32_t a2 = v_pair<B>(x[2], x[3], 2 * t), a3 = v_pair<B>(x[2], x[3], 2 * t + 1);
         mma_cls<B>(st.acc[hf * MTH + t], a0, a1, a2, a3, w[2 * u], w[2 * u + 1]);
-        if (B == 16) mma_bf16(st.acc[hf * MTH + t], a0, a1, a2, a3, wlo[2 * u], wlo[2 * u + 1]);
+        mma_cls<B>(st.acc[hf * MTH + t], a0, a1, a2, a3, wlo[2 * u], wlo[2 * u + 1]);
       }
     }
   }
