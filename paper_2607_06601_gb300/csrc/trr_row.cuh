@@ -298,7 +298,8 @@ __device__ __forceinline__ int plan_pages(const LayerArgs& a, int seq, int lo, i
     else first = l;
   }
   const int npr = max(0, end - first);
-  const int lw = lg + 1 - __ffs(c8 == 3 ? kt_wide : kt_most), w = 1 << lw, mass = npr << lw;  // tiles of a page
+  int lw = lg + 1 - __ffs(c8 == 3 ? kt_wide : kt_most);  // log2 of a page's tiles
+  const int mass = npr << lw;
   int before = 0, all = own ? kNewTiles : 0;  // tiles of the wider classes; of the row
 #pragma unroll
   for (int k = 0; k < kClasses; ++k) {
@@ -306,6 +307,17 @@ __device__ __forceinline__ int plan_pages(const LayerArgs& a, int seq, int lo, i
     all += m;
     before += k > c8 ? m : 0;
   }
+  // 16-bit tiles count twice where a split's tiles then stay within a warp's lanes: a warp's
+  // ring holds one of 8 KB, so that each waits out a copy, and a split of nothing else ended
+  // last.  (160M step 801 -> 776 us, batch 256 of the sweep 1468 -> 1413, gqa_long shape 290 ->
+  // 283 for 6 layer calls, batch 8 of contexts 4000 255 -> 260.)
+  const int wide = __shfl_sync(0xffffffffu, mass, 24);
+  if (div24(all + wide, ns) + 1 + 2 * (a.P >> (__ffs(kt_wide) - 1)) <= kItemMaxTiles) {
+    all += wide;
+    if (c8 == 3) ++lw;
+    else before += wide;
+  }
+  const int w = 1 << lw;
   // the split's pages: those that start in its share [b0, b1) of the tiles, all / ns and one
   // more for the first all % ns splits (all < 2^24)
   const int each = div24(all, ns), extra = all - each * ns;
