@@ -11,7 +11,7 @@
 // two stages in flight and held every stage until the slowest of the four was done with it.
 // The kernels are bound by instructions issued and by the latency of a unit's chain (plan,
 // copies, tiles, merge), not by memory: batch 256 of the sweep shape streams at 5.9 TB/s
-// with the tile arithmetic left out, at 3.8 TB/s with it.
+// with the tile arithmetic left out, at 4 TB/s with it.
 //
 // Two CTAs of eight warps fill an SM; while some of the places are free or a CTA has ended,
 // the next layer's kernel is resident, so that its plans and its first page copies come before
