@@ -360,7 +360,13 @@ template <int B> __host__ __device__ constexpr int kp_pos(int i) {
 template <int B> __host__ __device__ constexpr int smax_of() { return B == 2 ? 8 : B == 4 ? 4 : 0; }
 
 // V side: dim j of the thread's D/8 dims for keys (a, b) as an A-operand word (key a
-// in the low half).
+// in the low half).  The tensor core lines products up by their operands' exponents, and all
+// subnormals have the same: what a product has below 2^-24 of the largest operand exponents is
+// cut off, which costs a code at bit offset 0 ten bits.  Codes of 2 and 4 bits are therefore
+// moved up to offsets 4, 6, 8 and 2, 6, two shifts a half word in place of one (offsets 0, 2, ..
+// and 0, 4: rows of 2-bit tokens with outlier channels were 1e-4 to 3e-4 of their size off
+// before rounding, of 4-bit ones 7e-5 to 2e-4).
+__host__ __device__ constexpr int v2_pos(int k) { return 4 + 2 * ((k + 1) % 3); }  // width 2: field k of 8
 template <int B>
 __device__ __forceinline__ uint32_t v_pair(const uint32_t* wa, const uint32_t* wb, int j) {
   if (B == 16) return __byte_perm(wa[j >> 1], wb[j >> 1], (j & 1) ? 0x7632 : 0x5410);
@@ -372,18 +378,19 @@ __device__ __forceinline__ uint32_t v_pair(const uint32_t* wa, const uint32_t* w
   if (B == 4) {
     const int k = j & 7;
     uint32_t x = __byte_perm(wa[j >> 3], wb[j >> 3], k < 4 ? 0x5410 : 0x7632);
-    if ((k & 3) >= 2) x >>= 8;
-    return x & ((k & 1) ? 0x00F000F0u : 0x000F000Fu);
+    x = (k & 3) < 2 ? x << 2 : x >> 6;
+    return x & ((k & 1) ? 0x03C003C0u : 0x003C003Cu);
   }
   const int k = j & 15, kk = k & 7;
   uint32_t x = __byte_perm(wa[j >> 4], wb[j >> 4], k < 8 ? 0x5410 : 0x7632);
-  if (kk >= 5) x >>= 10;
-  return x & (0x00030003u << (2 * (kk < 5 ? kk : kk - 5)));
+  if (kk < 2) x <<= 6;
+  if (kk >= 5) x >>= 6;
+  return x & (0x00030003u << v2_pos(kk));
 }
 // log2 of the factor a V accumulator row carries in class index c (dim j of the
 // thread's D/8): 2^(pos - 24) for codes, 1 for bf16
 __host__ __device__ constexpr int vfac_log2(int c, int j) {
-  return c == 3 ? 0 : c == 2 ? -24 : c == 1 ? 4 * (j & 1) - 24 : 2 * ((j & 7) < 5 ? (j & 7) : (j & 7) - 5) - 24;
+  return c == 3 ? 0 : c == 2 ? -24 : c == 1 ? 2 + 4 * (j & 1) - 24 : v2_pos(j & 7) - 24;
 }
 
 // ------------------------------------------------------------------ combine --
