@@ -981,6 +981,38 @@ __device__ __forceinline__ void group_values(GroupState<D, NG>& st, const uint8_
   }
 }
 
+// The tensor core truncates its sums, and codes are not negative: running sums of p * s * c come
+// out low by up to 2^-23 of themselves per 16 keys, and p * z, about as large with the other sign,
+// leaves that in a row a hundred times smaller.  The zero points are therefore added every
+// kFoldTiles tiles, so that the running sums stay near the row itself.  (8-bit tokens, 670 keys a
+// split: 1.1e-4 of the row off before its rounding, 2.4e-5 so.  Batch 256 of the sweep 1467 -> 1525
+// us; every 4 or 16 tiles takes as long; sums begun at zero for each tile 1720, and codes made
+// normal and centred 1740.)
+constexpr int kFoldTiles = 8;
+template <int D, int NG>
+__device__ __forceinline__ void fold_zero_points(RowState<D, NG>& st, const float* fac, int lane) {
+  constexpr int MT = D / 16;
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int i = 0; i < NG; ++i) st.zacc[i] += __shfl_xor_sync(0xffffffffu, st.zacc[i], o);
+  }
+  float z = st.zacc[0];
+#pragma unroll
+  for (int i = 0; i < NG; ++i) {
+    if ((lane & 3) % NG == i) z = st.zacc[i];
+    st.zacc[i] = 0.f;
+  }
+  z *= st.wscale;  // (1 in width 16, as its sums are kept)
+  float f[2 * MT];
+  load_words<2 * MT>(reinterpret_cast<const uint8_t*>(fac + (12 + st.cls) * (D / 8)), reinterpret_cast<uint32_t*>(f));
+#pragma unroll
+  for (int t = 0; t < MT; ++t) {
+    st.acc[t][0] = fmaf(z, f[2 * t], st.acc[t][0]);
+    st.acc[t][2] = fmaf(z, f[2 * t + 1], st.acc[t][2]);
+  }
+}
+
 // --------------------------------------------------------------------------- rows --
 
 // A row at its unit's end (lane holds dims lane * D/32 .. of the unnormalised sum, relative to
@@ -1731,6 +1763,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
         }
         __syncwarp();  // the tile's bytes and weights are read
         if (inext < un.T) issue(c + 1, __shfl_sync(0xffffffffu, wcum, c));
+        if (c % kFoldTiles == kFoldTiles - 1) fold_zero_points<D, NG>(st, fac, lane);
       }
       consumed = c;
       if (!good) break;

@@ -19,7 +19,7 @@ def _cuda():
     torch.cuda.set_device(0)
 
 
-@pytest.mark.parametrize("bits,outliers", [(2, True), (4, True)])
+@pytest.mark.parametrize("bits,outliers", [(2, True), (4, True), (8, False), (2, False)])
 @pytest.mark.parametrize("d,G,P,H", [(64, 32, 32, 16), (128, 128, 32, 8)])
 def test_sums_add_nothing_to_the_rounding(d, G, P, H, bits, outliers):
     """Rows of 2000 keys in few splits, whose sums of p * s * c and of p * z are a hundred times
