@@ -24,6 +24,8 @@
 namespace trr {
 
 #define kNegInf (-__int_as_float(0x7f800000))
+constexpr float kNoMax = -3.4028235e38f;  // a running maximum before the first key: no score is below
+                                          // it, and finite (a key that does not count weighs 0)
 constexpr float kTau = 8.f;    // lazy rescale threshold (log2 units)
 
 __device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }

@@ -1571,7 +1571,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       st.cls = 3;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        st.m[j] = -1e30f;
+        st.m[j] = kNoMax;
         st.l[j] = st.zacc[j] = 0.f;
       }
 #pragma unroll
@@ -1710,7 +1710,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       st.F = st.fset = 0;
       st.slim = 0.f;
       st.wscale = 1.f;
-      st.m = -1e30f;  // below any score, and finite: a key that does not count weighs 0
+      st.m = kNoMax;
       st.l = 0.f;
       st.cls = 3;
 #pragma unroll

@@ -1,5 +1,5 @@
 """What the tensor cores' operands and sums keep of the attention's binary32 arithmetic: sums
-whose codes cancel against the zero points."""
+whose codes cancel against the zero points, scores far below zero."""
 import numpy as np
 import pytest
 import torch
@@ -44,3 +44,33 @@ def test_sums_add_nothing_to_the_rounding(d, G, P, H, bits, outliers):
     rounded = torch.from_numpy(ref).bfloat16().double().numpy()
     ratio = np.sqrt(((got - ref) ** 2).mean() / ((rounded - ref) ** 2).mean())
     assert ratio <= 1.0006 + 0.0016, f"{ratio:.5f} times the error of rounding the exact rows"
+
+
+@pytest.mark.parametrize("d,G,P,Hq,Hkv", [(64, 32, 32, 4, 4), (64, 64, 16, 10, 1), (128, 64, 32, 8, 2)])
+@pytest.mark.parametrize("bits", [8, 16])
+@pytest.mark.parametrize("step", [False, True])
+def test_every_score_far_below_zero(d, G, P, Hq, Hkv, bits, step):
+    """Finite inputs whose scores all lie between -1e30 and -3.4e38: the largest one decides.
+    (16-bit keys of 2^55 and queries of 2^55; 8-bit keys of 2^10 and queries of 2^98.)  Different
+    keys' scores differ by 2^-8 of themselves at least, far above binary32's rounding and far
+    beyond the softmax's reach, and the largest is one key's."""
+    rng = np.random.default_rng(bits + d)
+    ctx = 100
+    pair = Pair(1, 2, Hq, Hkv, d, G, P, ctx + 8, [2 * ctx // P + 8] * 4)
+    size = 2.0 ** 55 if bits == 16 else 2.0 ** 10
+    qsize = 2.0 ** 55 if bits == 16 else 2.0 ** 98
+
+    def rows(frac):  # every value of a key the same and negative: a constant group, scale 0
+        k = np.broadcast_to((-size * (1 + frac)).astype(np.float32)[:, None, None], (len(frac), Hkv, d))
+        return wl.bf16_bits(np.ascontiguousarray(k)), wl.bf16_bits(rng.standard_normal((len(frac), Hkv, d), dtype=np.float32))
+
+    frac = (np.arange(ctx) + 20) * 37 % 101 / 101.0
+    for s in range(2):
+        pair.append(0, np.full(ctx, s), np.arange(ctx), *rows(frac), np.full(ctx, bits), np.full(ctx, FULL))
+    q = wl.bf16_bits(np.full((2, Hq, d), qsize, dtype=np.float32))
+    if step:
+        # sequence 0's own token is above every key, sequence 1's below most
+        _, ref = pair.step(0, [0, 1], [ctx, ctx + 1], *rows(np.array([-0.1, 0.9])), [bits, bits], [FULL, FULL], q)
+    else:
+        _, ref = pair.attend(0, [0, 1], [ctx - 1, 50], q, [FULL, FULL])
+    assert (np.abs(ref).max(axis=-1) > 0).all()
