@@ -524,7 +524,7 @@ __device__ __forceinline__ void row_switch(RowState<D, NG>& st, int to, bool fre
   for (int i = 0; i < NP; ++i) st.kb[i] = ok ? st.kb[i] : 0u;
   // (width 16 weighs p itself: its wscale is 1, and its scale never asks for another F)
   st.wscale = to == 3 ? 1.f : __int_as_float((127 + st.F) << 23);
-  st.slim = to == 3 ? 3e38f : st.cls == 3 && st.fset == 0 ? 0.f : __int_as_float((127 + 7 - st.F) << 23);
+  st.slim = to == 3 ? 3e38f : st.fset == 0 ? 0.f : __int_as_float((127 + 7 - st.F) << 23);
   if (!fresh) {
     const int e = (to == 3 ? 0 : st.F) - (st.cls == 3 ? 0 : st.F);
     const float g = __int_as_float((127 + e) << 23);
