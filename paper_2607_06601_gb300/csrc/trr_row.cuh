@@ -31,8 +31,8 @@
 //         up s * (group sum) + z * (group's query sum) in binary32.
 //   P.V   A = V^T codes paired along keys, B = p * s of the tile's keys, exchanged through
 //         shared memory: column (group, hi | lo), the weight split into two f16 parts
-//         (22 bits and the sign; scaled by a power of two per unit so that the largest
-//         parts are far from f16's limits), so that weights keep binary32's accuracy.
+//         (22 bits and the sign, as many as exp2's approximation has; scaled by a power of
+//         two per group that follows the weights, far from f16's limits).
 //         Width 16 uses m16n8k8 with tf32 operands (bf16 values are exact in tf32), its
 //         weights split the same way.
 // The running maximum is the warp's, raised only when a score exceeds it by 2^8.
@@ -445,18 +445,15 @@ struct RowState {
   static constexpr int NP = D / 8, MT = D / 16;
   uint32_t kb[NP];    // the query as q.k's B operand in the current class
   float acc[MT][4];   // V sums: dims gid D/8 + 2 t (+ 1) x columns (group tig % NG, hi | lo),
-                      // times 2^(vfac_log2 + F) for codes, 1 for width 16
+                      // times 2^vfac_log2 and the group's ws for codes, 1 for width 16
   float qsum[NG];     // softmax scale * log2(e) * sum of the query over each group
   float m, l;         // running maximum (the warp's, log2 units); this lane's sum of weights
   float zacc[NG];     // this lane's sums of p * z
-  float slim;         // largest V scale that F allows: 2^(7 - F)
-  float wscale;       // 2^F
+  float ws[NG];       // codes' weights are p * s * ws (a power of two per group)
   float kfac;         // the current class's factor of the group sums
   uint32_t kl, vl;    // the current class's lane offsets (k_lane, v_lane)
   int wl;             // the byte offset of the lane's row of weights as ldmatrix reads it
   int zoff;           // the offset in a tile of the V scales of the lane's key
-  int F;              // codes' weights are p * s * 2^F
-  int fset;           // F has been chosen
   int E;              // codes' queries are q * 2^-E (in f16 range)
   int cls;
 };
@@ -489,8 +486,25 @@ __device__ __forceinline__ void store_query_row(uint8_t* qs, uint2 raw, int cls,
 }
 
 // log2 of the factor the accumulators of dim j (of a lane's D/8) carry in class c, without
-// the codes' 2^F
+// the codes' ws
 __host__ __device__ constexpr int row_fac(int c, int j) { return c == 3 ? 0 : vfac_log2(c, j); }
+
+// What a code's weight p * s * ws may reach (f16 ends at 2^16), and the largest ws: with the
+// largest factor of a code's bit offset it takes sums of width 16 into a code's domain unchanged.
+constexpr float kWeightTop = 32768.f;
+constexpr int kWeightScale = 16;  // log2
+
+// The element of a per-group array for the group whose columns this lane's accumulators have.
+template <int NG>
+__device__ __forceinline__ float lane_group(const float (&x)[NG], int lane) {
+  float r = x[0];
+#pragma unroll
+  for (int i = 1; i < NG; ++i)
+    if ((lane & 3) % NG == i) r = x[i];
+  return r;
+}
+// 1 / x of a power of two
+__device__ __forceinline__ float pow2_inverse(float x) { return __int_as_float((254 << 23) - __float_as_int(x)); }
 
 // What a lane keeps of class B while it works on its tiles.
 template <int D, int NG, int B>
@@ -522,12 +536,9 @@ __device__ __forceinline__ void row_switch(RowState<D, NG>& st, int to, bool fre
   load_words<NP>(qs + tig * (D / 2), st.kb);
 #pragma unroll
   for (int i = 0; i < NP; ++i) st.kb[i] = ok ? st.kb[i] : 0u;
-  // (width 16 weighs p itself: its wscale is 1, and its scale never asks for another F)
-  st.wscale = to == 3 ? 1.f : __int_as_float((127 + st.F) << 23);
-  st.slim = to == 3 ? 3e38f : st.fset == 0 ? 0.f : __int_as_float((127 + 7 - st.F) << 23);
   if (!fresh) {
-    const int e = (to == 3 ? 0 : st.F) - (st.cls == 3 ? 0 : st.F);
-    const float g = __int_as_float((127 + e) << 23);
+    const float ws = lane_group<NG>(st.ws, lane);
+    const float g = (to == 3) == (st.cls == 3) ? 1.f : to == 3 ? pow2_inverse(ws) : ws;
     float f[2 * MT];
     load_words<2 * MT>(reinterpret_cast<const uint8_t*>(fac + (st.cls * 4 + to) * (D / 8)), reinterpret_cast<uint32_t*>(f));
 #pragma unroll
@@ -619,14 +630,17 @@ __device__ __forceinline__ void tile_scores(const RowState<D, NG>& st, const uin
   }
 }
 
-// 2. The key's weight (ok: it counts): the score from the group sums, the running maximum and
-// F raised and lowered when a key asks for it, p, and p * s as the operand rows at wb.
+// 2. The key's weight (ok: it counts): the score from the group sums, p, and p * s * ws as the
+// operand rows at wb.  The running maximum and the groups' ws are set anew when a key asks for it:
+// its score is above the maximum by more than kTau, or its weight in a group above kWeightTop.  ws
+// follows the weights, not the scales alone, and each group its own: a group with scales 2^26 below
+// another's, or keys with such scales beside one of no weight, keep all of their bits.
 // kw, zw: the key's K and V (s, z); (1, 0) where the width has none (has_sz).
 template <int D, int NG>
 __device__ __forceinline__ void tile_weights(RowState<D, NG>& st, float (&g)[NG], bool ok, bool has_sz,
-                                             const uint32_t (&kw)[NG], uint32_t (&zw)[NG], int key, uint8_t* wb) {
+                                             const uint32_t (&kw)[NG], uint32_t (&zw)[NG], int key, uint8_t* wb, int lane) {
   constexpr int MT = D / 16;
-  float sc = 0.f, smax = 0.f;
+  float sc = 0.f, w[NG];
   float2 vz[NG];
 #pragma unroll
   for (int i = 0; i < NG; ++i) {
@@ -634,49 +648,57 @@ __device__ __forceinline__ void tile_weights(RowState<D, NG>& st, float (&g)[NG]
     sc = fmaf(sz.x * st.kfac, g[i], fmaf(sz.y, st.qsum[i], sc));
     if (!ok) zw[i] = 0u;  // a slot that does not count may hold any bytes
     vz[i] = __half22float2(*reinterpret_cast<const __half2*>(&zw[i]));
-    smax = fmaxf(smax, vz[i].x);
   }
   if (!ok) sc = kNegInf;
-  if (__any_sync(0xffffffffu, sc > st.m + kTau || smax > st.slim)) {
-    float top = sc, big = smax;
+  float p = fast_exp2(sc - st.m);  // 0 for a key that does not count
+  bool ask = p > 256.f;            // 2^kTau
+  if (has_sz) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
-      big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+    for (int i = 0; i < NG; ++i) {
+      w[i] = p * vz[i].x * st.ws[i];
+      ask |= w[i] > kWeightTop;
     }
+  }
+  if (__any_sync(0xffffffffu, ask)) {
+    float top = sc;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
     top = fmaxf(top, st.m);
     const float alpha = top == st.m ? 1.f : fast_exp2(st.m - top);
     float f = alpha;
-    if (big > st.slim) {
-      // big * 2^F < 2^6 (width 2), 2^3, 2^0 (width 8): the scales of the narrower classes that
-      // follow are larger by the ratio of the levels, and shall seldom ask again
-      const int room = 5 - 3 * st.cls;
-      const int F = min(24, room - (static_cast<int>(__float_as_uint(big) >> 23) - 127));
-      f *= __int_as_float((127 + F - st.F) << 23);
-      st.F = F;
-      st.fset = 1;
-      st.wscale = __int_as_float((127 + F) << 23);
-      st.slim = __int_as_float((127 + 7 - F) << 23);
-    }
+    st.m = top;
+    p = fast_exp2(sc - top);
     st.l *= alpha;
 #pragma unroll
     for (int i = 0; i < NG; ++i) st.zacc[i] *= alpha;
+    if (has_sz) {
+      const float before = lane_group<NG>(st.ws, lane);
+#pragma unroll
+      for (int i = 0; i < NG; ++i) {
+        float big = p * vz[i].x;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+        // big * ws < 2^6 (width 2), 2^3, 2^0 (width 8): p may rise by 2^8, and the scales of the
+        // narrower classes that follow are larger by the ratio of the levels
+        const int e = 5 - 3 * st.cls - (static_cast<int>(__float_as_uint(big) >> 23) - 127);
+        if (big > 0.f) st.ws[i] = __int_as_float((127 + min(kWeightScale, e)) << 23);
+        w[i] = p * vz[i].x * st.ws[i];
+      }
+      f *= lane_group<NG>(st.ws, lane) * pow2_inverse(before);
+    }
 #pragma unroll
     for (int t = 0; t < MT; ++t)
 #pragma unroll
       for (int i = 0; i < 4; ++i) st.acc[t][i] *= f;
-    st.m = top;
   }
-  const float p = fast_exp2(sc - st.m);  // 0 for a key that does not count
   st.l += p;
-  const float pf = p * st.wscale;
   if (has_sz) {
     uint32_t w2[NG];
 #pragma unroll
     for (int i = 0; i < NG; ++i) {
       st.zacc[i] = fmaf(p, vz[i].y, st.zacc[i]);
-      const float w = pf * vz[i].x, wh = __half2float(__float2half_rn(w));
-      w2[i] = pack_f16x2(wh, (w - wh) * kLoScale);
+      const float wh = __half2float(__float2half_rn(w[i]));
+      w2[i] = pack_f16x2(wh, (w[i] - wh) * kLoScale);
     }
     uint32_t* at = reinterpret_cast<uint32_t*>(wb + 16 * key);
     if (NG == 1) at[0] = w2[0];
@@ -997,13 +1019,10 @@ __device__ __forceinline__ void fold_zero_points(RowState<D, NG>& st, const floa
 #pragma unroll
     for (int i = 0; i < NG; ++i) st.zacc[i] += __shfl_xor_sync(0xffffffffu, st.zacc[i], o);
   }
-  float z = st.zacc[0];
+  float z = lane_group<NG>(st.zacc, lane);
 #pragma unroll
-  for (int i = 0; i < NG; ++i) {
-    if ((lane & 3) % NG == i) z = st.zacc[i];
-    st.zacc[i] = 0.f;
-  }
-  z *= st.wscale;  // (1 in width 16, as its sums are kept)
+  for (int i = 0; i < NG; ++i) st.zacc[i] = 0.f;
+  if (st.cls != 3) z *= lane_group<NG>(st.ws, lane);
   float f[2 * MT];
   load_words<2 * MT>(reinterpret_cast<const uint8_t*>(fac + (12 + st.cls) * (D / 8)), reinterpret_cast<uint32_t*>(f));
 #pragma unroll
@@ -1074,7 +1093,7 @@ __device__ __forceinline__ void row_values(RowState<D, NG>& st, float (&v)[D / 3
     if (grp == i) z = st.zacc[i];
   // dims gid D/8 + 2 t + r are in lane (gid, grp)'s acc[t][2 r] (hi) and [2 r + 1] (lo);
   // this lane wants t = tig DPL/2 ..
-  const float g = __int_as_float((127 - (st.cls == 3 ? 0 : st.F)) << 23);
+  const float g = st.cls == 3 ? 1.f : pow2_inverse(lane_group<NG>(st.ws, lane));
   float f[2 * MT];
   load_words<2 * MT>(reinterpret_cast<const uint8_t*>(fac + (st.cls * 4 + 3) * (D / 8)), reinterpret_cast<uint32_t*>(f));
 #pragma unroll
@@ -1700,6 +1719,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       for (int i = 0; i < NG; ++i) {
         st.qsum[i] = __shfl_sync(0xffffffffu, qsum, i * gl) * ka.qscale;
         st.zacc[i] = 0.f;
+        st.ws[i] = pow2f(kWeightScale);
       }
       if (has_new) {
 #pragma unroll
@@ -1707,9 +1727,6 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
         new_score = dot * ka.qscale;
       }
       st.E = min(100, max(-100, static_cast<int>((__float_as_uint(qmax) >> 23) & 0xff) - 127 - 6));
-      st.F = st.fset = 0;
-      st.slim = 0.f;
-      st.wscale = 1.f;
       st.m = kNoMax;
       st.l = 0.f;
       st.cls = 3;
@@ -1750,7 +1767,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
           ok = ok && pos >= un.lo && pos <= un.t;
         }
         const unsigned all = __ballot_sync(0xffffffffu, ok);
-        tile_weights<D, NG>(st, gs, ok, cls != 3, kw, zw, key, wb);
+        tile_weights<D, NG>(st, gs, ok, cls != 3, kw, zw, key, wb, lane);
         __syncwarp();
         if (cls == 3) {
           tile_values16<D, NG>(st, tile, kt, all != (kt == 32 ? 0xffffffffu : 0x33333333u), all, wb, lane);

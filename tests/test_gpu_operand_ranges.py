@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from paper_2607_06601_gb300 import workloads as wl
-from tests._parity import Pair
+from tests._parity import Pair, dev
 
 pytestmark = pytest.mark.gpu
 
@@ -88,6 +88,24 @@ def test_every_score_far_below_zero(d, G, P, Hq, Hkv, bits, step):
 MIXED = 1.002 + 0.006
 
 
+def _rows(pair, seqs, ts, q):
+    """Full queries' rows and the oracle's.  (Not Pair.attend: its absolute bound of 2e-2 beyond the
+    rounding is for values of order 1; of rows of 2^13 it is 2^-18.6, which only the binary32 sums of
+    a few keys would meet.)"""
+    seqs, ts, modes = np.asarray(seqs, np.int32), np.asarray(ts, np.int32), np.full(len(seqs), FULL, np.uint8)
+    out = pair.gpu.decode_attn(0, dev(seqs, torch.int32), dev(ts, torch.int32), dev(q, torch.bfloat16),
+                               dev(modes, torch.uint8))
+    st, ref = pair.orc.decode_attn(0, seqs, ts, q, modes)
+    assert st == 0 and pair.gpu.status() == 0
+    return out.double().cpu().numpy(), ref
+
+
+def _mixed(pair, rng, ctx, Hkv, d, bits, kscale=1.0, vscale=1.0):
+    """ctx tokens of one sequence; bits, kscale and vscale per token (the scales per dimension too)."""
+    k, v = (rng.standard_normal((ctx, Hkv, d)) * x for x in (kscale, vscale))
+    pair.append(0, np.zeros(ctx), np.arange(ctx), wl.bf16_bits(k), wl.bf16_bits(v), bits, np.full(ctx, FULL))
+
+
 def test_constant_groups_then_tiny_scales():
     """Every 8-bit token's V groups are constant (scale 0), the 4- and 2-bit tokens that follow them
     have the smallest scales: the weights' power of two is chosen by the first scale that is not 0."""
@@ -100,4 +118,34 @@ def test_constant_groups_then_tiny_scales():
     pair.append(0, np.zeros(ctx), np.arange(ctx), wl.bf16_bits(k), wl.bf16_bits(v), bits, np.full(ctx, FULL))
     q = wl.bf16_bits(3 * rng.standard_normal((1, H, d)))
     got, ref = pair.attend(0, [0], [ctx - 1], q, [FULL])
+    assert _ratio(got, ref) <= MIXED, _ratio(got, ref)
+
+
+@pytest.mark.parametrize("d,G,H", [(64, 32, 64), (128, 32, 32)])
+def test_groups_with_scales_far_apart(d, G, H):
+    """V's first quantiser group is 2^26 times as large as the others."""
+    rng = np.random.default_rng(22)
+    ctx = 800
+    pair = Pair(1, 1, H, H, d, G, 32, ctx, [ctx // 32 + 2] * 4, split_bytes=100000)
+    size = np.where(np.arange(d) < G, 2.0 ** 12, 2.0 ** -14)
+    _mixed(pair, rng, ctx, H, d, rng.choice((2, 4, 8), size=ctx), vscale=size)
+    q = wl.bf16_bits(3 * rng.standard_normal((1, H, d)))
+    got, ref = _rows(pair, [0], [ctx - 1], q)
+    for part in (slice(0, G), slice(G, d)):
+        assert _ratio(got[..., part], ref[..., part]) <= MIXED, _ratio(got[..., part], ref[..., part])
+
+
+def test_large_scales_of_keys_without_weight():
+    """Every 16th token has V scales 2^26 times as large as the others' and scores some 100 below
+    theirs (e^-100 of the weight)."""
+    rng = np.random.default_rng(23)
+    d, G, H, ctx = 64, 32, 64, 800
+    pair = Pair(1, 1, H, H, d, G, 32, ctx, [ctx // 32 + 2] * 4, split_bytes=100000)
+    odd = np.arange(ctx) % 16 == 3
+    q = np.abs(rng.standard_normal((1, H, d))) + 0.5
+    k = rng.standard_normal((ctx, H, d)) + np.where(odd, -16.0, 0.0)[:, None, None]
+    v = rng.standard_normal((ctx, H, d)) * np.where(odd, 2.0 ** 12, 2.0 ** -14)[:, None, None]
+    pair.append(0, np.zeros(ctx), np.arange(ctx), wl.bf16_bits(k), wl.bf16_bits(v), rng.choice((2, 4, 8), size=ctx),
+                np.full(ctx, FULL))
+    got, ref = pair.attend(0, [0], [ctx - 1], wl.bf16_bits(q), [FULL])
     assert _ratio(got, ref) <= MIXED, _ratio(got, ref)
