@@ -60,7 +60,7 @@ struct RowSmem {  // byte offsets of one CTA's shared memory
       : full(0),
         fac(full + kRowWarps * kRowSlots * 8),
         q(fac + 16 * (D / 8) * 4),
-        w(q + kRowWarps * heads * D * 2),
+        w(q + kRowWarps * row_q_bytes(D, heads)),
         pre(w + kRowWarps * row_w_bytes(heads)),
         qinf(pre + align16(4 * (n + 2))),
         ord(qinf + 16 * n),
@@ -69,6 +69,8 @@ struct RowSmem {  // byte offsets of one CTA's shared memory
         flag(ent + (step ? align16(4 * step_ints(n)) : 0)),
         ring((flag + 16 + 127) & ~127),
         total(ring + kRowWarps * ring_bytes) {}
+  // a unit's query rows; one head: the row as the class's operand, as given, its groups' exponents
+  __host__ __device__ static constexpr int row_q_bytes(int D, int heads) { return heads > 1 ? heads * D * 2 : 4 * D + 16; }
   // the weights of a tile: 32 rows of 8 f16 (width 16: of 2 tf32; query groups: of 8 bf16,
   // high parts, then low parts)
   __host__ __device__ static constexpr int row_w_bytes(int heads) { return heads > 1 ? 1024 : 512; }
@@ -450,16 +452,16 @@ struct RowState {
   float m, l;         // running maximum (the warp's, log2 units); this lane's sum of weights
   float zacc[NG];     // this lane's sums of p * z
   float ws[NG];       // codes' weights are p * s * ws (a power of two per group)
-  float kfac;         // the current class's factor of the group sums
+  float kfac[NG];     // the current class's factors of the group sums
   uint32_t kl, vl;    // the current class's lane offsets (k_lane, v_lane)
   int wl;             // the byte offset of the lane's row of weights as ldmatrix reads it
   int zoff;           // the offset in a tile of the V scales of the lane's key
-  int E;              // codes' queries are q * 2^-E (in f16 range)
   int cls;
 };
 
 // The query row in the order and scale of class cls's B operand, to qs: widths 2, 4 and 8 as
-// f16 pairs at the codes' bit offsets, times 2^-E (f16 range); width 16 the bf16 values.
+// f16 pairs times 2^(15 - E - the code's bit offset), E of the values' group: the largest are just
+// below f16's end, and what is 2^-24 of them still has all of its 8 bits; width 16 the bf16 values.
 // Lane holds dims lane * D/32 .. (raw, bf16).
 template <int D>
 __device__ __forceinline__ void store_query_row(uint8_t* qs, uint2 raw, int cls, int E, int lane) {
@@ -479,8 +481,8 @@ __device__ __forceinline__ void store_query_row(uint8_t* qs, uint2 raw, int cls,
     // width 4 (8 k + i, + 4), offset 4 (i % 2); width 2 (16 k + i, + 8), offset 2 (i < 5 ? i : i - 5)
     const int lg = cls == 0 ? 3 : 2, i = dd & ((1 << lg) - 1);
     const int word = cls == 2 ? dd >> 1 : ((dd >> (lg + 1)) << lg) + i, half = cls == 2 ? dd & 1 : (dd >> lg) & 1;
-    const int e = cls == 2 ? 0 : cls == 1 ? 4 - 4 * (i & 1) : 8 - 2 * (i < 5 ? i : i - 5);
-    const float v = ((j & 1) ? bf_hi(w) : bf_lo(w)) * __int_as_float((127 - E + e) << 23);
+    const int pos = cls == 2 ? 0 : cls == 1 ? 4 * (i & 1) : 2 * (i < 5 ? i : i - 5);
+    const float v = ((j & 1) ? bf_hi(w) : bf_lo(w)) * __int_as_float((127 + 15 - E - pos) << 23);
     *reinterpret_cast<__half*>(row + 4 * word + 2 * half) = __float2half_rn(v);
   }
 }
@@ -488,6 +490,14 @@ __device__ __forceinline__ void store_query_row(uint8_t* qs, uint2 raw, int cls,
 // log2 of the factor the accumulators of dim j (of a lane's D/8) carry in class c, without
 // the codes' ws
 __host__ __device__ constexpr int row_fac(int c, int j) { return c == 3 ? 0 : vfac_log2(c, j); }
+
+template <int D>
+__device__ __forceinline__ uint2 load_row(const uint16_t* src, int lane) {
+  uint2 r = make_uint2(0, 0);
+  if (D == 64) r.x = reinterpret_cast<const uint32_t*>(src)[lane];
+  else r = reinterpret_cast<const uint2*>(src)[lane];
+  return r;
+}
 
 // What a code's weight p * s * ws may reach (f16 ends at 2^16), and the largest ws: with the
 // largest factor of a code's bit offset it takes sums of width 16 into a code's domain unchanged.
@@ -508,8 +518,7 @@ __device__ __forceinline__ float pow2_inverse(float x) { return __int_as_float((
 
 // What a lane keeps of class B while it works on its tiles.
 template <int D, int NG, int B>
-__device__ __forceinline__ void row_class(RowState<D, NG>& st, float qscale, int lane) {
-  st.kfac = B == 16 ? qscale : __int_as_float((127 + 24 - smax_of<B>() + st.E) << 23) * qscale;
+__device__ __forceinline__ void row_class(RowState<D, NG>& st, int lane) {
   st.kl = k_lane<D, B>(lane >> 2, lane & 3);
   st.vl = v_lane<D, B>(lane >> 2, lane & 3);
   st.wl = 16 * w_row<row_map(D, B)>(lane);
@@ -518,20 +527,25 @@ __device__ __forceinline__ void row_class(RowState<D, NG>& st, float qscale, int
 // Class st.cls -> to: the query's operand (lane (gid, tig) holds dims tig D/4 .. of group
 // gid % NG), the accumulators' factors (fac: a table [from][to][dim of the lane]).
 template <int D, int NG>
-__device__ __forceinline__ void row_switch(RowState<D, NG>& st, int to, bool fresh, uint8_t* qs, uint2 qraw, const float* fac,
+__device__ __forceinline__ void row_switch(RowState<D, NG>& st, int to, bool fresh, uint8_t* qs, const float* fac,
                                            float qscale, int kt, int lane) {
   constexpr int NP = D / 8, MT = D / 16;
   const int gid = lane >> 2, tig = lane & 3;
   const bool ok = (tig * NG) / 4 == gid % NG;
   switch (to) {
-    case 0: row_class<D, NG, 2>(st, qscale, lane); break;
-    case 1: row_class<D, NG, 4>(st, qscale, lane); break;
-    case 2: row_class<D, NG, 8>(st, qscale, lane); break;
-    default: row_class<D, NG, 16>(st, qscale, lane); break;
+    case 0: row_class<D, NG, 2>(st, lane); break;
+    case 1: row_class<D, NG, 4>(st, lane); break;
+    case 2: row_class<D, NG, 8>(st, lane); break;
+    default: row_class<D, NG, 16>(st, lane); break;
   }
   const int b = bits_of_class(to);
   st.zoff = kt * (2 * (D * b / 8) + 4 * NG) + min(8 * tig + gid, kt - 1) * NG * 4;
-  store_query_row<D>(qs, qraw, to, st.E, lane);
+  const int* qe = reinterpret_cast<const int*>(qs + 4 * D);  // largest exponents of the groups
+  store_query_row<D>(qs, load_row<D>(reinterpret_cast<const uint16_t*>(qs + 2 * D), lane), to, qe[lane / (32 / NG)], lane);
+#pragma unroll
+  for (int i = 0; i < NG; ++i)
+    // finite: 0 * kfac of a scale of 0 is 0; above 2^118 q's scores are beyond binary32 anyway
+    st.kfac[i] = to == 3 ? qscale : fminf(__int_as_float((127 + qe[i]) << 23) * qscale * pow2f(9), 3.4028235e38f);
   __syncwarp();
   load_words<NP>(qs + tig * (D / 2), st.kb);
 #pragma unroll
@@ -645,7 +659,7 @@ __device__ __forceinline__ void tile_weights(RowState<D, NG>& st, float (&g)[NG]
 #pragma unroll
   for (int i = 0; i < NG; ++i) {
     const float2 sz = __half22float2(*reinterpret_cast<const __half2*>(&kw[i]));
-    sc = fmaf(sz.x * st.kfac, g[i], fmaf(sz.y, st.qsum[i], sc));
+    sc = fmaf(sz.x * st.kfac[i], g[i], fmaf(sz.y, st.qsum[i], sc));
     if (!ok) zw[i] = 0u;  // a slot that does not count may hold any bytes
     vz[i] = __half22float2(*reinterpret_cast<const __half2*>(&zw[i]));
   }
@@ -1148,14 +1162,6 @@ __device__ __forceinline__ void step_row(const AttnKernelArgs& ka, uint2 raw, in
   }
 }
 
-template <int D>
-__device__ __forceinline__ uint2 load_row(const uint16_t* src, int lane) {
-  uint2 r = make_uint2(0, 0);
-  if (D == 64) r.x = reinterpret_cast<const uint32_t*>(src)[lane];
-  else r = reinterpret_cast<const uint2*>(src)[lane];
-  return r;
-}
-
 // Every CTA: validates the entries and plans where each token goes (the same plan as the
 // append kernels: the token takes index ntok of its (sequence, class) list; index % P == 0
 // opens a page, whose id is next_page + the class's openers before it).  Errors, lowest
@@ -1258,7 +1264,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + lay.flag);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + lay.full) + warp * kRowSlots;
   uint8_t* ring = smem + lay.ring + warp * R;
-  uint8_t* qs = smem + lay.q + warp * heads * D * 2;
+  uint8_t* qs = smem + lay.q + warp * RowSmem::row_q_bytes(D, heads);
   float* fac = reinterpret_cast<float*>(smem + lay.fac);
 #pragma unroll 1
   for (int i = threadIdx.x; i < 16 * (D / 8); i += 32 * kRowWarps) {
@@ -1693,7 +1699,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       finish(std::integral_constant<int, 1>());
       __syncwarp();  // vnew is read
     } else {
-      // the query row to shared memory; its largest exponent, the sums over its groups
+      // the query row's largest exponents and sums per group
       float x[DPL];
       x[0] = bf_lo(qraw.x);
       x[1] = bf_hi(qraw.x);
@@ -1711,7 +1717,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       const int gl = 32 / NG;  // lanes of a group
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
+        if (o < gl) qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
         if (o < gl) qsum += __shfl_xor_sync(0xffffffffu, qsum, o);
       }
       RowState<D, NG> st;
@@ -1726,7 +1732,10 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
         for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
         new_score = dot * ka.qscale;
       }
-      st.E = min(100, max(-100, static_cast<int>((__float_as_uint(qmax) >> 23) & 0xff) - 127 - 6));
+      if (D == 64) reinterpret_cast<uint32_t*>(qs + 2 * D)[lane] = qraw.x;
+      else reinterpret_cast<uint2*>(qs + 2 * D)[lane] = qraw;
+      if (lane % gl == 0)
+        reinterpret_cast<int*>(qs + 4 * D)[lane / gl] = max(-85, static_cast<int>((__float_as_uint(qmax) >> 23) & 0xff) - 127);
       st.m = kNoMax;
       st.l = 0.f;
       st.cls = 3;
@@ -1738,7 +1747,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       for (; c < un.T; ++c) {
         const uint32_t geo = __shfl_sync(0xffffffffu, wgeo, c);
         const int cls = geo & 3, kt = tile_keys(cls);
-        if (c == 0 || cls != st.cls) row_switch<D, NG>(st, cls, c == 0, qs, qraw, fac, ka.qscale, kt, lane);
+        if (c == 0 || cls != st.cls) row_switch<D, NG>(st, cls, c == 0, qs, fac, ka.qscale, kt, lane);
         if (!tile_in(c)) break;
         const uint8_t* tile = ring + ((geo >> 3) & (1023u << 7));
         uint32_t there = 0xffffffffu;

@@ -27,8 +27,8 @@ def _ratio(got, ref):
 
 
 @pytest.mark.parametrize("bits,outliers", [(2, True), (4, True), (8, False), (2, False)])
-@pytest.mark.parametrize("d,G,P,H", [(64, 32, 32, 16), (128, 128, 32, 8)])
-def test_sums_add_nothing_to_the_rounding(d, G, P, H, bits, outliers):
+@pytest.mark.parametrize("d,G,P,H,g", [(64, 32, 32, 16, 1), (128, 128, 32, 8, 1)])
+def test_sums_add_nothing_to_the_rounding(d, G, P, H, g, bits, outliers):
     """Rows of 2000 keys in few splits, whose sums of p * s * c and of p * z are a hundred times
     the row and cancel: the error is that of rounding the exact row to bf16.  An error of 2^-23 of
     sums 100 times as large is under 1/30 of that rounding's (about 2^-9.2 of the row): in
@@ -36,17 +36,17 @@ def test_sums_add_nothing_to_the_rounding(d, G, P, H, bits, outliers):
     2 / 30."""
     rng = np.random.default_rng(100 * bits + d)
     S, ctx = 1024 // d, 2000
-    pair = Pair(1, S, H, H, d, G, P, ctx, [S * (ctx // P + 2)] * 4, split_bytes=100000)
+    pair = Pair(1, S, H * g, H, d, G, P, ctx, [S * (ctx // P + 2)] * 4, split_bytes=100000)
     chan = np.ones(H * d, dtype=np.float32)
     if outliers:
-        chan[rng.permutation(H * d)[:H * d // 100]] = 8
+        chan[rng.permutation(H * d)[:max(1, H * d // 100)]] = 8
     for s in range(S):
         for p0 in range(0, ctx, 1000):
             kv = [wl.bf16_bits(rng.standard_normal((1000, H, d), dtype=np.float32) * chan.reshape(H, d))
                   for _ in range(2)]
             pair.append(0, np.full(1000, s), np.arange(p0, p0 + 1000), kv[0], kv[1], np.full(1000, bits),
                         np.full(1000, FULL))
-    q = wl.bf16_bits(rng.standard_normal((S, H, d), dtype=np.float32))
+    q = wl.bf16_bits(rng.standard_normal((S, H * g, d), dtype=np.float32))
     got, ref = pair.attend(0, np.arange(S), [ctx - 1] * S, q, [FULL] * S)
     ratio = _ratio(got, ref)
     assert ratio <= 1.0006 + 0.0016, f"{ratio:.5f} times the error of rounding the exact rows"
@@ -148,4 +148,18 @@ def test_large_scales_of_keys_without_weight():
     pair.append(0, np.zeros(ctx), np.arange(ctx), wl.bf16_bits(k), wl.bf16_bits(v), rng.choice((2, 4, 8), size=ctx),
                 np.full(ctx, FULL))
     got, ref = pair.attend(0, [0], [ctx - 1], wl.bf16_bits(q), [FULL])
+    assert _ratio(got, ref) <= MIXED, _ratio(got, ref)
+
+
+@pytest.mark.parametrize("bits", [(2,), (4,), (8,)])
+def test_query_groups_far_apart(bits):
+    """The query's first quantiser group is 2^28 times as large as its second, whose keys are as many
+    times larger: both decide the scores."""
+    rng = np.random.default_rng(24)
+    d, G, H, ctx = 64, 32, 64, 800
+    pair = Pair(1, 1, H, H, d, G, 32, ctx, [ctx // 32 + 2] * 4, split_bytes=100000)
+    first = np.arange(d) < G
+    _mixed(pair, rng, ctx, H, d, rng.choice(bits, size=ctx), kscale=np.where(first, 2.0 ** -14, 2.0 ** 13))
+    q = wl.bf16_bits(rng.standard_normal((1, H, d)) * np.where(first, 2.0 ** 14, 2.0 ** -14))
+    got, ref = pair.attend(0, [0], [ctx - 1], q, [FULL])
     assert _ratio(got, ref) <= MIXED, _ratio(got, ref)
