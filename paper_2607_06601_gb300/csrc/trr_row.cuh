@@ -791,31 +791,31 @@ struct GroupState {
   uint32_t kb[NP];
   float acc[MT][4];  // dims gid D/8 + 2 t (+ 1) x the lane's columns, times 2^vfac_log2
   float qsum[2], m[2], l[2], zacc[2];  // per column (m: of its head)
-  float kfac;
+  float kfac[2];     // per column: the current class's factor of the group sums
   uint32_t kl, vl;
-  int wl, zoff, E, cls;
+  int wl, zoff, cls;
+  int E;             // exponent of the largest query value of the head and group of column gid
 };
 
 template <int D, int NG, int B>
-__device__ __forceinline__ void group_class(GroupState<D, NG>& st, const uint8_t* qs, int heads, float qscale, int lane) {
+__device__ __forceinline__ void group_class(GroupState<D, NG>& st, const uint8_t* qs, int heads, int lane) {
   constexpr int NP = D / 8, rowb = D * B / 8;
   const int gid = lane >> 2, tig = lane & 3, r = gid / NG;
   const bool ok = r < heads && (tig * NG) / 4 == gid % NG;
   uint32_t raw[NP];
   load_words<NP>(qs + (r < heads ? r : 0) * D * 2 + tig * (D / 2), raw);
-  const float escale = __int_as_float((127 - st.E) << 23);
+  const float escale = __int_as_float((127 + 15 - st.E) << 23);
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     uint32_t w = raw[i];
     if (B != 16) {
       const int lo = kp_lo<B>(i), hi = kp_hi<B>(i);
-      const float f = pow2f(smax_of<B>() - kp_pos<B>(i)) * escale;
+      const float f = pow2f(-kp_pos<B>(i)) * escale;
       w = pack_f16x2(((lo & 1) ? bf_hi(raw[lo >> 1]) : bf_lo(raw[lo >> 1])) * f,
                      ((hi & 1) ? bf_hi(raw[hi >> 1]) : bf_lo(raw[hi >> 1])) * f);
     }
     st.kb[i] = ok ? w : 0u;
   }
-  st.kfac = B == 16 ? qscale : __int_as_float((127 + 24 - smax_of<B>() + st.E) << 23) * qscale;
   st.kl = gid * rowb + tig * (rowb / 4);
   st.vl = tig * rowb + (rowb >= 32 ? gid * (rowb / 8) : (gid * (rowb / 8)) & ~3);
 }
@@ -825,10 +825,15 @@ __device__ __forceinline__ void group_switch(GroupState<D, NG>& st, int to, bool
                                              const float* fac, float qscale, int kt, int lane) {
   constexpr int MT = D / 16;
   switch (to) {
-    case 0: group_class<D, NG, 2>(st, qs, heads, qscale, lane); break;
-    case 1: group_class<D, NG, 4>(st, qs, heads, qscale, lane); break;
-    case 2: group_class<D, NG, 8>(st, qs, heads, qscale, lane); break;
-    default: group_class<D, NG, 16>(st, qs, heads, qscale, lane); break;
+    case 0: group_class<D, NG, 2>(st, qs, heads, lane); break;
+    case 1: group_class<D, NG, 4>(st, qs, heads, lane); break;
+    case 2: group_class<D, NG, 8>(st, qs, heads, lane); break;
+    default: group_class<D, NG, 16>(st, qs, heads, lane); break;
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {  // as in row_switch
+    const float e = __int_as_float((127 + __shfl_sync(0xffffffffu, st.E, 4 * (2 * (lane & 3) + j))) << 23);
+    st.kfac[j] = to == 3 ? qscale : fminf(e * qscale * pow2f(9), 3.4028235e38f);
   }
   st.wl = 16 * w_row<0>(lane);
   st.zoff = kt * (2 * (D * bits_of_class(to) / 8) + 4 * NG) + (lane >> 2) * NG * 4 + (NG == 4 ? (lane & 1) * 8 : 0);
@@ -904,7 +909,7 @@ __device__ __forceinline__ void group_weights(GroupState<D, NG>& st, const float
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&kw[j]));
-      cp[j] = fmaf(f.x * st.kfac, c[k >> 1][2 * (k & 1) + j], f.y * st.qsum[j]);
+      cp[j] = fmaf(f.x * st.kfac[j], c[k >> 1][2 * (k & 1) + j], f.y * st.qsum[j]);
       if (!good) zw[k][j] = 0u;  // a slot that does not count may hold any bytes
     }
     if (NG == 1) {
@@ -1546,10 +1551,11 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       }
       if (!STEP && un.err && un.sp == 0 && lane == 0) atomicMin(&a.lctl[kFirstBadQuery], (ka.q0 + un.q) * 16 + un.err);
     } else if constexpr (GQ) {
-      // the group's query rows to shared memory; their largest exponent, each column's sum
+      // the group's query rows to shared memory; each column's sum and largest exponent
       GroupState<D, NG> st;
       const int gid = lane >> 2, tig = lane & 3;
-      float qmax = 0.f, new_score[2] = {kNegInf, kNegInf};
+      float new_score[2] = {kNegInf, kNegInf};
+      st.E = -85;
       st.qsum[0] = st.qsum[1] = 0.f;
       constexpr int kMost = 8 / NG;  // heads of a group, at most
       uint2 raws[kMost];
@@ -1560,7 +1566,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       for (int r = 0; r < kMost; ++r) {
         if (r >= heads) break;
         const uint2 raw = raws[r];
-        float x[DPL], sum = 0.f, dot = 0.f;
+        float x[DPL], sum = 0.f, dot = 0.f, qmax = 0.f;
         x[0] = bf_lo(raw.x);
         x[1] = bf_hi(raw.x);
         if (D == 128) {
@@ -1579,8 +1585,11 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
           if (o < 32 / NG) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+          if (o < 32 / NG) qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
           dot += __shfl_xor_sync(0xffffffffu, dot, o);
         }
+        qmax = __shfl_sync(0xffffffffu, qmax, (gid % NG) * (32 / NG));
+        if (gid / NG == r) st.E = max(-85, static_cast<int>((__float_as_uint(qmax) >> 23) & 0xff) - 127);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           const float v = __shfl_sync(0xffffffffu, sum, ((2 * tig + j) % NG) * (32 / NG));
@@ -1590,9 +1599,6 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
           }
         }
       }
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
-      st.E = min(100, max(-100, static_cast<int>((__float_as_uint(qmax) >> 23) & 0xff) - 127 - 6));
       st.cls = 3;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {

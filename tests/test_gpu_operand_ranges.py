@@ -163,3 +163,21 @@ def test_query_groups_far_apart(bits):
     q = wl.bf16_bits(rng.standard_normal((1, H, d)) * np.where(first, 2.0 ** 14, 2.0 ** -14))
     got, ref = pair.attend(0, [0], [ctx - 1], q, [FULL])
     assert _ratio(got, ref) <= MIXED, _ratio(got, ref)
+
+
+@pytest.mark.parametrize("bits", [(2,), (4,), (8,)])
+@pytest.mark.parametrize("d,G", [(64, 64), (64, 32), (128, 64)])
+def test_query_group_with_parts_far_apart(d, G, bits):
+    """A query group: each head's quantiser groups are 2^27 apart in the query, for which the keys make
+    up, and one of the two heads is 2^28 times the other (its rows are one key's values)."""
+    rng = np.random.default_rng(25)
+    Hkv, ctx = 2048 // d, 800
+    pair = Pair(1, 1, 2 * Hkv, Hkv, d, G, 32, ctx, [ctx // 32 + 2] * 4, split_bytes=100000)
+    first = np.arange(d) < G
+    kscale = np.where(first, 2.0 ** -14, 2.0 ** 13)
+    _mixed(pair, rng, ctx, Hkv, d, rng.choice(bits, size=ctx), kscale=kscale)
+    q = rng.standard_normal((1, 2 * Hkv, d)) / kscale
+    q[:, 1::2] *= 2.0 ** 28
+    got, ref = pair.attend(0, [0], [ctx - 1], wl.bf16_bits(q), [FULL])
+    for h in (0, 1):
+        assert _ratio(got[:, h::2], ref[:, h::2]) <= MIXED, _ratio(got[:, h::2], ref[:, h::2])
