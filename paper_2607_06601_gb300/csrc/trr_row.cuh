@@ -784,13 +784,19 @@ __device__ __forceinline__ void tile_values16(RowState<D, NG>& st, const uint8_t
 // raised when a score exceeds it by 2^3 (any excess where a scale could then take p * s out
 // of f16's range): raised at every new maximum, as before, nine tiles in ten rescaled the
 // accumulators.  These caches' rows are stored plainly.
+//
+// f16 ends at 2^-25, which p * s of small values would come near: p is therefore taken relative to
+// 2^-lift of the maximum, lift (0 to 16) lowered when a larger V scale comes.  (V of size 2^-10: rows
+// 5e-3 off without it, 2^-14 8 %; gqa_long shape 630 -> 646 us for 4 steps.)
 constexpr float kGroupTau = 3.f, kGroupWide = 8000.f;
+constexpr float kLift = 16.f;  // at first
 template <int D, int NG>
 struct GroupState {
   static constexpr int NP = D / 8, MT = D / 16;
   uint32_t kb[NP];
   float acc[MT][4];  // dims gid D/8 + 2 t (+ 1) x the lane's columns, times 2^vfac_log2
-  float qsum[2], m[2], l[2], zacc[2];  // per column (m: of its head)
+  float qsum[2], m[2], l[2], zacc[2];  // per column (m: its head's maximum - lift)
+  float lift, lim;   // and the largest V scale that lift allows
   float kfac[2];     // per column: the current class's factor of the group sums
   uint32_t kl, vl;
   int wl, zoff, cls;
@@ -928,18 +934,33 @@ __device__ __forceinline__ void group_weights(GroupState<D, NG>& st, const float
 #pragma unroll
   for (int j = 0; j < J; ++j)
     over = fmaxf(over, fmaxf(fmaxf(sc[0][j], sc[1][j]), fmaxf(sc[2][j], sc[3][j])) - st.m[j]);
+  over -= st.lift;
+  if (has_sz) {
 #pragma unroll
-  for (int k = 0; k < 4; ++k)
-    big = fmaxf(big, fmaxf(__half2float(__ushort_as_half(zw[k][0] & 0xffff)), __half2float(__ushort_as_half(zw[k][1] & 0xffff))));
-  if (__any_sync(0xffffffffu, over > kGroupTau || (over > 0.f && big > kGroupWide))) {  // (the keys' lanes share a maximum)
+    for (int k = 0; k < 4; ++k)
+      big = fmaxf(big, fmaxf(__half2float(__ushort_as_half(zw[k][0] & 0xffff)), __half2float(__ushort_as_half(zw[k][1] & 0xffff))));
+  }
+  if (__any_sync(0xffffffffu, over > kGroupTau || (big > st.lim && (st.lift > 0.f || over > 0.f)))) {  // (the keys' lanes share a maximum)
+    const float lift = st.lift;
+    if (has_sz) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+      if (big > st.lim) {
+        // big * 2^lift < 2^6, 2^3, 2^0 as in tile_weights, lift >= 0; 2^(lift + 3) * lim < 2^16
+        const int e = 5 - 3 * st.cls - (static_cast<int>(__float_as_uint(big) >> 23) - 127);
+        st.lift = static_cast<float>(max(0, min(static_cast<int>(lift), e)));
+        st.lim = st.lift > 0.f ? __int_as_float((127 + 12 - static_cast<int>(st.lift)) << 23) : kGroupWide;
+      }
+    }
 #pragma unroll
     for (int j = 0; j < J; ++j) {
       float mx = fmaxf(fmaxf(sc[0][j], sc[1][j]), fmaxf(sc[2][j], sc[3][j]));
 #pragma unroll
       for (int o = 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      mx = fmaxf(mx, st.m[j]);
-      const float alpha = fast_exp2(st.m[j] - mx);
-      st.m[j] = mx;
+      mx = fmaxf(mx, __fadd_rd(st.m[j], lift));
+      const float m = __fadd_ru(mx, -st.lift);  // rounded up: p <= 2^lift also where a score's ulp is larger
+      const float alpha = fast_exp2(st.m[j] - m);
+      st.m[j] = m;
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         if (NG == 1 && i != j) continue;
@@ -951,7 +972,7 @@ __device__ __forceinline__ void group_weights(GroupState<D, NG>& st, const float
           st.acc[t][i + 2] *= alpha;
         }
       }
-      if (NG > 1) st.m[1] = mx;
+      if (NG > 1) st.m[1] = st.m[0];
     }
   }
 #pragma unroll
@@ -967,7 +988,7 @@ __device__ __forceinline__ void group_weights(GroupState<D, NG>& st, const float
       w[j] = p[j] * f.x;
     }
     uint32_t* at = reinterpret_cast<uint32_t*>(wb + 16 * (gid + 8 * k)) + tig;
-    if (has_sz) {  // high and low part (finite: p <= 1 where a scale is above kGroupWide)
+    if (has_sz) {  // high and low part (finite: p <= 1 where a scale is above kGroupWide, then lift is 0)
       const uint32_t hi = pack_f16x2(w[0], w[1]);
       const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&hi));
       at[0] = hi;
@@ -1600,6 +1621,8 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
         }
       }
       st.cls = 3;
+      st.lift = kLift;
+      st.lim = pow2f(12 - static_cast<int>(kLift));
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         st.m[j] = kNoMax;

@@ -181,3 +181,15 @@ def test_query_group_with_parts_far_apart(d, G, bits):
     got, ref = pair.attend(0, [0], [ctx - 1], wl.bf16_bits(q), [FULL])
     for h in (0, 1):
         assert _ratio(got[:, h::2], ref[:, h::2]) <= MIXED, _ratio(got[:, h::2], ref[:, h::2])
+
+
+@pytest.mark.parametrize("d,G,P,Hq,Hkv", [(64, 32, 32, 64, 32), (64, 64, 16, 64, 16), (128, 64, 64, 32, 8), (128, 32, 32, 32, 16)])
+@pytest.mark.parametrize("size", [2.0 ** -4, 2.0 ** -8, 2.0 ** -10, 2.0 ** -14, 2.0 ** -20])
+def test_query_group_small_values(d, G, P, Hq, Hkv, size):
+    """Query groups with small V: the low part of a weight is far above f16's end."""
+    rng = np.random.default_rng(26)
+    ctx = 800
+    pair = Pair(1, 1, Hq, Hkv, d, G, P, ctx, [ctx // P + 2] * 4, split_bytes=100000)
+    _mixed(pair, rng, ctx, Hkv, d, rng.choice((2, 4, 8), size=ctx), vscale=size)
+    got, ref = pair.attend(0, [0], [ctx - 1], wl.bf16_bits(3 * rng.standard_normal((1, Hq, d))), [FULL])
+    assert _ratio(got, ref) <= MIXED, _ratio(got, ref)
