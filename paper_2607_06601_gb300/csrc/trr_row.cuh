@@ -1001,6 +1001,14 @@ __device__ __forceinline__ void group_weights(GroupState<D, NG>& st, const float
   }
 }
 
+// Infinite bf16 values (and NaN) as the largest finite ones.
+__device__ __forceinline__ uint32_t finite_bf16x2(uint32_t x) {
+  const uint32_t top = 0x7f7f7f7fu, low = 0xff7fff7fu;
+  const __nv_bfloat162 m = __hmin2(*reinterpret_cast<const __nv_bfloat162*>(&x), *reinterpret_cast<const __nv_bfloat162*>(&top));
+  const __nv_bfloat162 r = __hmax2(m, *reinterpret_cast<const __nv_bfloat162*>(&low));
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
+
 // 3. P.V.  all[k]: lanes whose key gid + 8 k counts (width 16: other keys' values read as 0).
 template <int D, int NG, int B>
 __device__ __forceinline__ void group_values(GroupState<D, NG>& st, const uint8_t* tile, int kt, bool part,
@@ -1037,7 +1045,11 @@ __device__ __forceinline__ void group_values(GroupState<D, NG>& st, const uint8_
         const uint32_t a0 = v_pair<B>(x[0], x[1], 2 * t), a1 = v_pair<B>(x[0], x[1], 2 * t + 1);
         const uint32_t a2 = v_pair<B>(x[2], x[3], 2 * t), a3 = v_pair<B>(x[2], x[3], 2 * t + 1);
         mma_cls<B>(st.acc[hf * MTH + t], a0, a1, a2, a3, w[2 * u], w[2 * u + 1]);
-        mma_cls<B>(st.acc[hf * MTH + t], a0, a1, a2, a3, wlo[2 * u], wlo[2 * u + 1]);
+        if (B == 16)  // an infinite value times a low part of 0 or below would make its sum a NaN
+          mma_bf16(st.acc[hf * MTH + t], finite_bf16x2(a0), finite_bf16x2(a1), finite_bf16x2(a2), finite_bf16x2(a3),
+                   wlo[2 * u], wlo[2 * u + 1]);
+        else
+          mma_f16(st.acc[hf * MTH + t], a0, a1, a2, a3, wlo[2 * u], wlo[2 * u + 1]);
       }
     }
   }

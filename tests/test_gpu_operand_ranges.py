@@ -193,3 +193,26 @@ def test_query_group_small_values(d, G, P, Hq, Hkv, size):
     _mixed(pair, rng, ctx, Hkv, d, rng.choice((2, 4, 8), size=ctx), vscale=size)
     got, ref = pair.attend(0, [0], [ctx - 1], wl.bf16_bits(3 * rng.standard_normal((1, Hq, d))), [FULL])
     assert _ratio(got, ref) <= MIXED, _ratio(got, ref)
+
+
+@pytest.mark.parametrize("d,G,Hq,Hkv", [(64, 32, 4, 2), (128, 64, 8, 2), (64, 64, 16, 2)])
+@pytest.mark.parametrize("sign", [1, -1])
+def test_infinite_values_of_a_query_group(d, G, Hq, Hkv, sign):
+    """A 16-bit token with an infinite value in one dimension of one KV head, also as the only key of
+    a query (weight 1, whose low part is 0): infinite there, for the heads that read it, alone."""
+    rng = np.random.default_rng(28)
+    ctx, g = 200, Hq // Hkv
+    pair = Pair(1, 1, Hq, Hkv, d, G, 32, ctx, [ctx // 32 + 2] * 4)
+    k, v = (rng.standard_normal((ctx, Hkv, d)) for _ in range(2))
+    bits = np.where(np.arange(ctx) % 5 == 0, 16, rng.choice((2, 4, 8), size=ctx))
+    v[100, 1, 7] = sign * np.inf
+    pair.append(0, np.zeros(ctx), np.arange(ctx), wl.bf16_bits(k), wl.bf16_bits(v), bits, np.full(ctx, FULL))
+    q = wl.bf16_bits(rng.standard_normal((3, Hq, d)))
+    i32 = lambda x: dev(np.array(x, np.int32), torch.int32)
+    out = pair.gpu.decode_attn(0, i32([0, 0, 0]), i32([99, 100, ctx - 1]), dev(q, torch.bfloat16),
+                               dev(np.array([FULL, LOCAL, FULL], np.uint8), torch.uint8), window_scalar=1)
+    assert pair.gpu.status() == 0
+    out = out.float().cpu().numpy()
+    want = np.zeros(out.shape, dtype=bool)
+    want[1:, g:2 * g, 7] = True
+    assert np.array_equal(np.isinf(out), want) and not np.isnan(out).any() and (out[want] * sign > 0).all()
