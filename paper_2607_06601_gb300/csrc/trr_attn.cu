@@ -9,16 +9,16 @@
 
 namespace trr {
 
-// Done once per cache at creation, so that calls stay legal inside stream capture.
-cudaError_t attn_configure() {
-  cudaError_t (*const parts[])() = {configure_attn_row, configure_attn_row_heads, configure_attn_row_step,
-                                     configure_attn_group, configure_attn_group_step};
-  for (auto part : parts) {
-    const cudaError_t e = part();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
+TRR_ROW_FAMILY(extern, false, false, false, false)
+TRR_ROW_FAMILY(extern, true, false, false, false)
+TRR_ROW_FAMILY(extern, false, true, false, false)
+TRR_ROW_FAMILY(extern, false, false, true, false)
+TRR_ROW_FAMILY(extern, false, true, true, false)
+TRR_ROW_FAMILY(extern, false, false, false, true)
+TRR_ROW_FAMILY(extern, true, false, false, true)
+TRR_ROW_FAMILY(extern, false, true, false, true)
+TRR_ROW_FAMILY(extern, false, false, true, true)
+TRR_ROW_FAMILY(extern, false, true, true, true)
 
 // Whether a warp takes a KV head and its query group (else a query head).
 static bool use_mma(const Layout& l) {
@@ -30,6 +30,20 @@ static bool use_mma(const Layout& l) {
 // rows take shared memory too, and its largest tile (8 KB at d 128) must fit a warp's ring.
 static int launch_queries(const Layout& l) { return use_mma(l) ? 512 : 1024; }
 
+// Done once per cache at creation, so that calls stay legal inside stream capture: the
+// instances that the cache's calls launch.
+cudaError_t attn_configure(const Layout& l) {
+  if (use_mma(l)) {
+    const cudaError_t e = l.runs ? configure_rows<false, false, true, true>(l) : configure_rows<false, false, true, false>(l);
+    if (e != cudaSuccess) return e;
+    return l.runs ? configure_rows<false, true, true, true>(l) : configure_rows<false, true, true, false>(l);
+  }
+  if (l.head_modes) return l.runs ? configure_rows<true, false, false, true>(l) : configure_rows<true, false, false, false>(l);
+  const cudaError_t e = l.runs ? configure_rows<false, false, false, true>(l) : configure_rows<false, false, false, false>(l);
+  if (e != cudaSuccess) return e;
+  return l.runs ? configure_rows<false, true, false, true>(l) : configure_rows<false, true, false, false>(l);
+}
+
 static cudaError_t launch_one(const Layout& l, const AttnKernelArgs& ka, int num_sms, cudaStream_t s) {
   AttnKernelArgs k = ka;
   const int heads = use_mma(l) ? l.Hq / l.Hkv : 1;
@@ -39,9 +53,13 @@ static cudaError_t launch_one(const Layout& l, const AttnKernelArgs& ka, int num
   if (k.ring_bytes < row_tile_bytes(l.d, l.d / l.G)) return cudaErrorInvalidConfiguration;
   const size_t sm = static_cast<size_t>(RowSmem(l.d, heads, k.n, k.fused, k.ring_bytes).total);
   const dim3 grid(kRowCtasPerSm * num_sms - num_sms / kRowSpare);
-  if (use_mma(l)) return k.fused ? launch_attn_group_step(l, grid, sm, s, k) : launch_attn_group(l, grid, sm, s, k);
-  if (k.fused) return launch_attn_row_step(l, grid, sm, s, k);
-  return l.head_modes ? launch_attn_row_heads(l, grid, sm, s, k) : launch_attn_row(l, grid, sm, s, k);
+  if (use_mma(l)) {
+    if (k.fused) return l.runs ? launch_rows<false, true, true, true>(l, grid, sm, s, k) : launch_rows<false, true, true, false>(l, grid, sm, s, k);
+    return l.runs ? launch_rows<false, false, true, true>(l, grid, sm, s, k) : launch_rows<false, false, true, false>(l, grid, sm, s, k);
+  }
+  if (k.fused) return l.runs ? launch_rows<false, true, false, true>(l, grid, sm, s, k) : launch_rows<false, true, false, false>(l, grid, sm, s, k);
+  if (l.head_modes) return l.runs ? launch_rows<true, false, false, true>(l, grid, sm, s, k) : launch_rows<true, false, false, false>(l, grid, sm, s, k);
+  return l.runs ? launch_rows<false, false, false, true>(l, grid, sm, s, k) : launch_rows<false, false, false, false>(l, grid, sm, s, k);
 }
 
 // The launches of an attention call with the given scratch views in `a`; *launches

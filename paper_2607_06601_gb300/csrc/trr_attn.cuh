@@ -467,23 +467,6 @@ __global__ void __launch_bounds__(32 * kCombineWarps) attn_combine_kernel(const 
     *reinterpret_cast<__nv_bfloat162*>(orow + j) = __floats2bfloat162_rn(acc[j] * inv, acc[j + 1] * inv);
 }
 
-// ------------------------------------------------------------- launchers --
-// One translation unit per kernel family (compiled side by side): each launches its
-// instances with programmatic dependent launch and sets their shared-memory limit.
-//   attn_row, attn_row_heads, attn_row_step: one query head per warp (trr_row.cuh), for
-//                     trr_decode_attn, caches with per-head modes and trr_decode_step
-//   attn_group, attn_group_step: a KV head and its query group per warp, for trr_decode_attn
-//                     (with the combine kernel) and trr_decode_step
-cudaError_t launch_attn_row(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k);
-cudaError_t launch_attn_row_heads(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k);
-cudaError_t launch_attn_row_step(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k);
-cudaError_t launch_attn_group(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k);
-cudaError_t launch_attn_group_step(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k);
 cudaError_t launch_attn_combine(int d, int ctas, cudaStream_t s, const CombineArgs& ca);
-cudaError_t configure_attn_row();
-cudaError_t configure_attn_row_heads();
-cudaError_t configure_attn_row_step();
-cudaError_t configure_attn_group();
-cudaError_t configure_attn_group_step();
 
 }  // namespace trr

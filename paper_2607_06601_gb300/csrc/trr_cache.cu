@@ -89,16 +89,19 @@ static trr_status make_layout(const trr_cache_config* c, Layout* l) {
     l->page_bytes[k] = roundup(l->hdr + l->Hkv * l->slice[k], 128);
   }
   l->units = l->Hq;
-  // splits per query: at least pos_split key positions each (split_bytes of 8-bit
-  // tokens), and few enough pages per split for any range up to max_context
+  // splits per query: at least pos_split key positions each (split_bytes of 8-bit tokens)
   l->pos_split = static_cast<int>(std::max<int64_t>(l->P, l->split_bytes / l->tokb[2]));
-  l->s_cap = 1 << 30;
-  // tiles: up to 32 keys of a page (16 of the widest rows)
+  // a unit's tiles: up to 32 keys of a page (16 of the widest rows)
   const int tile = std::min(l->P, 32), wide = std::min(l->P, l->d == 128 ? 16 : 32);
   l->split_keys = wide;
   l->split_extra = 3 * (l->P / tile) + l->P / wide;
   l->split_most = kItemMaxTiles - l->split_extra;
-  l->s_cap = std::max(splits_of(l->maxctx, l->pos_split, l->split_keys, l->split_extra, l->split_most, l->s_cap), 1);
+  // most splits: one per pos_split positions, or per 28 pages where that is more.  (The tiles of a
+  // range may ask for up to five times as many where split_bytes is large; a cache's scratch, and
+  // what a call needs of the static array, do not grow with them.)
+  l->s_cap = std::max((l->maxctx + l->pos_split - 1) / l->pos_split, (l->MP + 2 * kClasses + 27) / 28);
+  // (the tiles' bound grows with the range)
+  l->runs = splits_of(l->maxctx, l->pos_split, l->split_keys, l->split_extra, l->split_most, 1 << 30) > l->s_cap;
   l->cnt_stride = 1 + (l->s_cap + kMergeGroup - 1) / kMergeGroup;
   l->max_items = static_cast<int64_t>(l->max_queries) * l->units * l->s_cap;
 
@@ -205,7 +208,7 @@ extern "C" trr_status trr_create_cache(const trr_cache_config* cfg, trr_cache** 
     }
     c->owned = true;
   }
-  if (attn_configure() != cudaSuccess) {
+  if (attn_configure(l) != cudaSuccess) {
     if (c->owned) cudaFree(c->base);
     delete c;
     return TRR_ERR_CUDA;

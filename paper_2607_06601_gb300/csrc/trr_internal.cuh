@@ -32,8 +32,8 @@ enum LayerCtrl : int {
   kLayerCtrlInts = 4
 };
 
-// An attention work unit holds at most this many tiles (a page's keys, split_keys at a time),
-// so that a warp holds one per lane.
+// An attention work unit has at most this many tiles (a page's keys, split_keys at a time) planned
+// at once, so that a warp holds one per lane.
 constexpr int kItemMaxTiles = 32;
 
 // Split partials are merged in groups of this many (then the groups): a query with
@@ -51,6 +51,7 @@ struct Layout {
   int split_keys, split_extra, split_most;  // keys of a tile; tiles a range may have above what its
                                             // keys fill; a split's share at most (splits_of)
   int s_cap;      // most splits one query is cut into
+  int runs;       // a range's tiles may ask for more splits than that: a split's come in runs
   int cnt_stride; // arrival counters per (query, head): 1 + ceil(s_cap / kMergeGroup)
   int64_t max_items;
   int64_t hdr, tokb[kClasses], slice[kClasses], maskb, page_bytes[kClasses];
@@ -59,10 +60,10 @@ struct Layout {
 };
 
 // Splits of a query whose key range spans `range` positions: at least pos_split positions
-// each, enough that no split holds more than kItemMaxTiles tiles of `keys` keys, at most s_cap
-// (which covers that bound for any range up to max_context).  A range has up to 2 `extra`
-// tiles more than its keys fill (partly filled and cut pages of each class), a split up to
-// `most` of them: its share and what rounding adds.
+// each, enough that no split holds more than kItemMaxTiles tiles of `keys` keys, at most s_cap (a
+// split then takes its tiles in several runs).  A range has up to 2 `extra` tiles more than its keys
+// fill (partly filled and cut pages of each class), a split up to `most` of them: its share and what
+// rounding adds.
 __host__ __device__ inline int splits_of(int range, int pos_split, int keys, int extra, int most, int s_cap) {
   if (range <= 0) return 1;
   const int by_len = (range + pos_split - 1) / pos_split;
@@ -162,8 +163,8 @@ bool cache_layer_settled(const trr_cache* c, int layer);
 void cache_note_call(trr_cache* c, int layer);
 uint64_t cache_wait_ns(const trr_cache* c);
 
-// One-time kernel attribute setup (defined in trr_attn.cu).
-cudaError_t attn_configure();
+// Kernel attribute setup of a cache's kernels (defined in trr_attn.cu).
+cudaError_t attn_configure(const Layout& l);
 
 // ------------------------------------------------------------------ PTX helpers --
 

@@ -67,7 +67,7 @@ struct RowSmem {  // byte offsets of one CTA's shared memory
         red(ord + align16(2 * n)),
         ent(red + kRowRed),
         flag(ent + (step ? align16(4 * step_ints(n)) : 0)),
-        ring((flag + 16 + 127) & ~127),
+        ring((flag + 16 + 8 * kRowWarps + 127) & ~127),
         total(ring + kRowWarps * ring_bytes) {}
   // a unit's query rows; one head: the row as the class's operand, as given, its groups' exponents
   __host__ __device__ static constexpr int row_q_bytes(int D, int heads) { return heads > 1 ? heads * D * 2 : 4 * D + 16; }
@@ -264,12 +264,15 @@ constexpr int kNewTiles = 3;
 
 // Pages of split sp (of ns) of a query of sequence seq over key positions [lo, t]: returns
 // their number (<= kItemMaxTiles); lane j below it gets page j's id in wid and class |
-// fill << 2 | kMask in wmeta.  own: whether the query's own token joins the last split.
+// fill << 2 | kMask in wmeta.  own: whether the query's own token joins the last split.  RUNS: a
+// split may have more tiles than a warp has lanes and comes in runs of pages; skip is where the run
+// starts in the split's share, and becomes where the next one does (0: this was the last).
 // Eight lanes per class: a rolled nine-way search of the pages' first or last positions where
 // the range needs it (small code: a unit's plan competes with its tiles for the instruction
 // cache).
+template <bool RUNS>
 __device__ __forceinline__ int plan_pages(const LayerArgs& a, int seq, int lo, int t, int sp, int ns, bool own,
-                                          int kt_most, int kt_wide, int lane, int& wid, int& wmeta) {
+                                          int kt_most, int kt_wide, int lane, int& skip, int& wid, int& wmeta) {
   const int c8 = lane >> 3, sub = lane & 7, lg = __ffs(a.P) - 1;
   const int nt = a.ntok[seq * 4 + c8];
   const bool upper_mask = t < a.last_pos[seq];  // keys after t may be stored
@@ -323,12 +326,18 @@ __device__ __forceinline__ int plan_pages(const LayerArgs& a, int seq, int lo, i
   // the split's pages: those that start in its share [b0, b1) of the tiles, all / ns and one
   // more for the first all % ns splits (all < 2^24)
   const int each = div24(all, ns), extra = all - each * ns;
-  const int b0 = sp * each + min(sp, extra), b1 = b0 + each + (sp < extra ? 1 : 0);
+  const int share = sp * each + min(sp, extra), b2 = share + each + (sp < extra ? 1 : 0);
+  int b0 = share, b1 = b2;
+  if (RUNS) {
+    b0 += skip;
+    b1 = min(b2, b0 + kItemMaxTiles + 1 - (1 << __shfl_sync(0xffffffffu, lw, 24)));  // (the widest pages are class 3's)
+    skip = b1 < b2 ? b1 - share : 0;
+  }
   const int beg = min(npr, max(0, (b0 - before + w - 1) >> lw));
   const int tc = min(npr, max(0, (b1 - before + w - 1) >> lw)) - beg;
   const int t1 = __shfl_sync(0xffffffffu, tc, 24), t2 = t1 + __shfl_sync(0xffffffffu, tc, 16);
   const int t3 = t2 + __shfl_sync(0xffffffffu, tc, 8);
-  const int T = min(t3 + __shfl_sync(0xffffffffu, tc, 0), kItemMaxTiles);  // (the split bound keeps it within)
+  const int T = min(t3 + __shfl_sync(0xffffffffu, tc, 0), kItemMaxTiles);  // (the split bound, or the run's, keeps it within)
   const int r = (lane >= t1) + (lane >= t2) + (lane >= t3), c = 3 - r;
   const int kid = __shfl_sync(0xffffffffu, first + beg, 8 * c) + lane - (r == 0 ? 0 : r == 1 ? t1 : r == 2 ? t2 : t3);
   const int f = __shfl_sync(0xffffffffu, first, 8 * c), e = __shfl_sync(0xffffffffu, end, 8 * c);
@@ -1086,6 +1095,27 @@ __device__ __forceinline__ void fold_zero_points(RowState<D, NG>& st, const floa
 
 // --------------------------------------------------------------------------- rows --
 
+// A partial: the sums (lane holds dims lane * D/32 ..), their maximum and the weights' sum.
+template <int D>
+__device__ __forceinline__ void store_partial(float* pp, const float (&v)[D / 32], float M, float L, int lane) {
+  constexpr int DPL = D / 32;
+#pragma unroll
+  for (int j = 0; j < DPL; j += 2) __stcg(reinterpret_cast<float2*>(pp + lane * DPL + j), make_float2(v[j], v[j + 1]));
+  if (lane == 0) __stcg(reinterpret_cast<float2*>(pp + D), make_float2(M, L));
+}
+// Adds one that this warp stored.
+template <int D>
+__device__ __forceinline__ void take_partial(const float* pp, float (&v)[D / 32], float& M, float& L, int lane) {
+  constexpr int DPL = D / 32;
+  const float2 ml = __ldcg(reinterpret_cast<const float2*>(pp + D));
+  const float top = fmaxf(M, ml.x), f = fast_exp2(M - top), fp = fast_exp2(ml.x - top);
+#pragma unroll
+  for (int j = 0; j < DPL; ++j) v[j] = fmaf(v[j], f, fp * __ldcg(pp + lane * DPL + j));
+  L = fmaf(L, f, fp * ml.y);
+  M = top;
+  __syncwarp();  // the sums are read before they are overwritten
+}
+
 // A row at its unit's end (lane holds dims lane * D/32 .. of the unnormalised sum, relative to
 // max M, with weight sum L).  One split: the bf16 row.  Otherwise the split's fp32 partial,
 // partial base + sp, merged in two levels: the last split of each group of kMergeGroup to
@@ -1108,9 +1138,7 @@ __device__ __forceinline__ void store_row(const AttnKernelArgs& ka, float (&v)[D
     float* pp = p0 + sp * kRow;
 #pragma unroll 1
     for (int level = two ? 0 : 1; level < 2; ++level) {
-#pragma unroll
-      for (int j = 0; j < DPL; j += 2) __stcg(reinterpret_cast<float2*>(pp + lane * DPL + j), make_float2(v[j], v[j + 1]));
-      if (lane == 0) __stcg(reinterpret_cast<float2*>(pp + D), make_float2(M, L));
+      store_partial<D>(pp, v, M, L, lane);
       if (!arrive_last(counter, count, lane)) return;
       merge_partials<D>(from, kRow * stride, count, lane, M, L, v);
       __syncwarp();  // every lane has read the group's rows before the first is overwritten
@@ -1285,10 +1313,82 @@ __device__ __forceinline__ void plan_entries_cta(const AttnKernelArgs& ka, int* 
   __syncthreads();
 }
 
+// The tiles of a unit's run of pages: their number, and per lane its tile's copy.
+struct TilePlan {
+  int T, skip;      // tiles; where the split's next run starts (plan_pages), 0: this is the last
+  uint64_t src;     // the tile's page's slice of the unit's KV head
+  uint32_t geo;     // class | keys << 2 | kMask | ring offset / 128 << 10 | first key / 16 << 20
+  int bytes, cum;   // bytes to copy; ring bytes used from the run's start to the tile's end
+};
+// Bytes of a tile of kt keys: rows, scales, presence mask.
+template <int D, int NG, bool HM>
+__device__ __forceinline__ int tile_bytes(int cls, int kt) {
+  const int b = bits_of_class(cls);
+  return kt * (b == 16 ? 4 * D : 2 * (D * b / 8) + 8 * NG) + (HM ? 16 : 0);
+}
+template <int D, int NG, bool HM, bool STEP, bool RUNS>
+__device__ __forceinline__ TilePlan plan_tiles(const AttnKernelArgs& ka, int seq, const RowUnit& un, int kvh, int skip, int lane) {
+  const LayerArgs& a = ka.a;
+  const int P = a.P, R = ka.ring_bytes;
+  const int kt_most = min(P, 32), kt_wide = min(P, D == 128 ? 16 : 32);
+  auto tile_keys = [&](int cls) { return D == 128 && cls == 3 ? kt_wide : kt_most; };
+  TilePlan tp;
+  tp.skip = skip;
+  int wid = -1, wmeta = 0;
+  tp.T = un.zero ? 0 : plan_pages<RUNS>(a, seq, un.lo, un.t, un.sp, un.ns, STEP, kt_most, kt_wide, lane, tp.skip, wid, wmeta);
+  if (kt_wide < P || kt_most < P) {  // pages to tiles
+    const int kt = tile_keys(wmeta & 3), nt = lane < tp.T ? (((wmeta >> 2) & 127) + kt - 1) / kt : 0;
+    int incl = nt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    int page = 0, key0 = 0;
+#pragma unroll 1
+    for (int p = 0; p < tp.T; ++p) {
+      const int e = __shfl_sync(0xffffffffu, incl, p), m = __shfl_sync(0xffffffffu, nt, p);
+      if (lane >= e - m && lane < e) {
+        page = p;
+        key0 = lane - (e - m);
+      }
+    }
+    tp.T = min(32, __shfl_sync(0xffffffffu, incl, 31));  // (as in plan_pages)
+    wid = __shfl_sync(0xffffffffu, wid, page);
+    const int pm = __shfl_sync(0xffffffffu, wmeta, page), k = tile_keys(pm & 3);
+    key0 *= k;
+    wmeta = (pm & ~(127 << 2)) | min(k, ((pm >> 2) & 127) - key0) << 2 | (key0 >> 4) << 20;
+  }
+  const int cls = wmeta & 3, rows = tile_bytes<D, NG, HM>(cls, tile_keys(cls)), posb = (wmeta & kMask) ? 4 * tile_keys(cls) : 0;
+  const int need = ((rows + 127) & ~127) + ((posb + 127) & ~127);
+  tp.src = 0;
+  tp.cum = 0;
+  if (lane < tp.T)
+    tp.src = reinterpret_cast<uint64_t>(a.pool[cls] + static_cast<int64_t>(wid) * a.page_bytes[cls] + a.hdr +
+                                      static_cast<int64_t>(kvh) * a.slice[cls]);
+  tp.bytes = rows + posb;
+  int off = 0, cum = 0, woff = 0;
+#pragma unroll 1
+  for (int j = 0; j < tp.T; ++j) {
+    const int nd = __shfl_sync(0xffffffffu, need, j);
+    if (off + nd > R) {
+      cum += R - off;
+      off = 0;
+    }
+    cum += nd;
+    if (lane == j) {
+      woff = off;
+      tp.cum = cum;
+    }
+    off += nd;
+  }
+  tp.geo = static_cast<uint32_t>(wmeta) | static_cast<uint32_t>(woff >> 7) << 10;
+  return tp;
+}
 // ------------------------------------------------------------------------- kernel --
 
 // GQ: a unit is a KV head and its query group, and the combine kernel merges its splits.
-template <int D, int NG, bool HM, bool STEP, bool GQ>
+template <int D, int NG, bool HM, bool STEP, bool GQ, bool RUNS>
 __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_constant__ AttnKernelArgs ka) {
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr int DPL = D / 32;
@@ -1312,6 +1412,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
   uint8_t* wb = smem + lay.w + warp * RowSmem::row_w_bytes(GQ ? 2 : 1);
   if (threadIdx.x < kRowWarps * kRowSlots) mbar_init(reinterpret_cast<uint64_t*>(smem + lay.full) + threadIdx.x, 1);
   if (threadIdx.x == 0) *abort_flag = 0;
+  if (RUNS && threadIdx.x < 2 * kRowWarps) reinterpret_cast<int*>(smem + lay.flag + 16)[threadIdx.x] = 0;
   fence_barrier_init();
   // The unit plan reads only the call's own index arrays, which no kernel of this library
   // writes, so it overlaps the previous kernel of the stream.  The layer's cache state is
@@ -1327,23 +1428,25 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
   const int total = pre[n], nwarps = gridDim.x * kRowWarps;
 
   // ------------------------------------------------------------------- unit and ring state
-  // A unit's tiles (a page's keys, 32 at a time) are worked out once, one per lane: what to
-  // copy, where in the ring, and how far the ring is used up to the tile's end (the ring
+  // A unit's tiles (a page's keys, 32 at a time) are worked out once, one per lane (TilePlan): what
+  // to copy, where in the ring, and how far the ring is used up to the tile's end (the ring
   // is filled and freed in tile order; a tile that would pass its end starts at 0).
   RowUnit un = {};
-  uint64_t wsrc = 0;                  // lane j: tile j: its page's slice of the unit's KV head
-  uint32_t wgeo = 0;                  // class | keys << 2 | kMask | ring offset / 128 << 10 | first key / 16 << 20
-  int wbytes = 0, wcum = 0;           // bytes to copy; ring bytes used from the unit's start to the tile's end
+  uint64_t wsrc = 0;                  // lane j: tile j
+  uint32_t wgeo = 0;
+  int wbytes = 0, wcum = 0;
   uint32_t base = 0;                  // tiles of the units before
   int inext = 0;                      // next tile to issue
   bool good = true;                   // no wait gave up
   int kvh = 0;                        // the unit's KV head
   const int kt_most = min(P, 32), kt_wide = min(P, D == 128 ? 16 : 32);
   auto tile_keys = [&](int cls) { return D == 128 && cls == 3 ? kt_wide : kt_most; };
-  auto tile_rows = [&](int cls) {     // bytes of a tile: rows, scales, presence mask
-    const int b = bits_of_class(cls);
-    return tile_keys(cls) * (b == 16 ? 4 * D : 2 * (D * b / 8) + 8 * NG) + (HM ? 16 : 0);
-  };
+  auto tile_rows = [&](int cls) { return tile_bytes<D, NG, HM>(cls, tile_keys(cls)); };
+  // RUNS: a split of more tiles than a warp plans at once (plan_pages) is worked on in runs, as one
+  // unit after another: every run but the last leaves its sums as the split's partial, every run but
+  // the first takes them up.  run[0]: where this run starts, run[1]: the next one (0: there is none).
+  // (Kernels of their own for the caches that can meet one: a step with them in took 3 to 8 % longer.)
+  int* run = reinterpret_cast<int*>(smem + lay.flag + 16) + 2 * warp;
   // issues the copies of the tiles that fit, each by its lane: tile c is the next to be
   // consumed, `freed` the ring bytes used up to the end of tile c - 1 (tile c itself always
   // fits: the ring is empty then)
@@ -1448,53 +1551,16 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       un.base = (pre[q] + un.h * un.ns) * heads;
     }
     kvh = GQ || g == 1 ? un.h : div24(un.h, g);
-    int wid = -1, wmeta = 0;
-    un.T = un.zero ? 0 : plan_pages(a, qi.x, un.lo, un.t, un.sp, un.ns, STEP, kt_most, kt_wide, lane, wid, wmeta);
-    if (kt_wide < P || kt_most < P) {  // pages to tiles
-      const int kt = tile_keys(wmeta & 3), nt = lane < un.T ? (((wmeta >> 2) & 127) + kt - 1) / kt : 0;
-      int incl = nt;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      int page = 0, key0 = 0;
-#pragma unroll 1
-      for (int p = 0; p < un.T; ++p) {
-        const int e = __shfl_sync(0xffffffffu, incl, p), m = __shfl_sync(0xffffffffu, nt, p);
-        if (lane >= e - m && lane < e) {
-          page = p;
-          key0 = lane - (e - m);
-        }
-      }
-      un.T = min(32, __shfl_sync(0xffffffffu, incl, 31));  // (the split bound keeps it within 32)
-      wid = __shfl_sync(0xffffffffu, wid, page);
-      const int pm = __shfl_sync(0xffffffffu, wmeta, page), k = tile_keys(pm & 3);
-      key0 *= k;
-      wmeta = (pm & ~(127 << 2)) | min(k, ((pm >> 2) & 127) - key0) << 2 | (key0 >> 4) << 20;
+    const TilePlan tp = plan_tiles<D, NG, HM, STEP, RUNS>(ka, qi.x, un, kvh, RUNS ? run[0] : 0, lane);
+    un.T = tp.T;
+    wsrc = tp.src;
+    wgeo = tp.geo;
+    wbytes = tp.bytes;
+    wcum = tp.cum;
+    if (RUNS) {
+      __syncwarp();
+      if (lane == 0) run[1] = tp.skip;
     }
-    const int cls = wmeta & 3, rows = tile_rows(cls), posb = (wmeta & kMask) ? 4 * tile_keys(cls) : 0;
-    const int need = ((rows + 127) & ~127) + ((posb + 127) & ~127);
-    if (lane < un.T)
-      wsrc = reinterpret_cast<uint64_t>(a.pool[cls] + static_cast<int64_t>(wid) * a.page_bytes[cls] + a.hdr +
-                                        static_cast<int64_t>(kvh) * a.slice[cls]);
-    wbytes = rows + posb;
-    int off = 0, cum = 0, woff = 0;
-#pragma unroll 1
-    for (int j = 0; j < un.T; ++j) {
-      const int nd = __shfl_sync(0xffffffffu, need, j);
-      if (off + nd > R) {
-        cum += R - off;
-        off = 0;
-      }
-      cum += nd;
-      if (lane == j) {
-        woff = off;
-        wcum = cum;
-      }
-      off += nd;
-    }
-    wgeo = static_cast<uint32_t>(wmeta) | static_cast<uint32_t>(woff >> 7) << 10;
     inext = 0;
     issue(0, 0);
     // a limit shorter than a suspended wait covers the first copies from here on
@@ -1545,12 +1611,14 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       for (int k = threadIdx.x; k < n; k += 32 * kRowWarps) qtab[ord[k]] = make_int2(pre[k] * heads, qinf[k].w & 0xffffff);
     }
     if (u >= total || !good) break;
+    if (RUNS) __syncwarp();
+    const bool last_run = !RUNS || run[1] == 0;
     int u_next = total;
-    if (total > nwarps && lane == 0) u_next = nwarps + atomicAdd(&a.lctl[kNextUnit], 1);  // read at the unit's end
+    if (total > nwarps && lane == 0 && last_run) u_next = nwarps + atomicAdd(&a.lctl[kNextUnit], 1);  // read at the unit's end
     const bool own = GQ || un.h == kvh * g;  // stores a new token's rows of its KV head
     // decode step: the entry's own token joins the row's last split; a skip token that
     // stores KV is written by its zero row's unit
-    const bool has_new = STEP && !failed && un.sp == un.ns - 1 && ent[2 * un.q] >= 0 && (!un.zero || own);
+    const bool has_new = STEP && !failed && last_run && un.sp == un.ns - 1 && ent[2 * un.q] >= 0 && (!un.zero || own);
     uint2 rk = make_uint2(0, 0), rv = rk;
     if (has_new) {
       const int64_t src = (static_cast<int64_t>(un.q) * a.Hkv + kvh) * D;
@@ -1703,6 +1771,17 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       __syncwarp();
       float f[D / 8];
       load_words<D / 8>(reinterpret_cast<const uint8_t*>(fac + (st.cls * 4 + 3) * (D / 8)), reinterpret_cast<uint32_t*>(f));
+      float2 old[2];  // an earlier run's maximum and sum of the lane's columns
+      if (RUNS) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          old[j] = make_float2(kNegInf, 0.f);
+          if (run[0] && (2 * tig + j) / NG < heads)
+            old[j] = __ldcg(reinterpret_cast<const float2*>(
+                a.part + static_cast<int64_t>(un.base + (2 * tig + j) / NG * un.ns + un.sp) * (D + 4) + D));
+        }
+        __syncwarp();
+      }
       auto finish = [&](auto column) {
         constexpr int j = decltype(column)::value;
         const int r = (2 * tig + j) / NG, gi = (2 * tig + j) % NG;
@@ -1714,22 +1793,34 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
           L = fmaf(L, fo, fn);
         }
         if (r >= heads || gid * NG / 8 != gi) return;
-        const float inv = un.ns > 1 ? 1.f : L > 0.f ? 1.f / L : 0.f;
+        auto partial = [&] { return a.part + static_cast<int64_t>(un.base + r * un.ns + un.sp) * (D + 4); };
+        float fp = 0.f;
+        if (RUNS && run[0]) {
+          const float top = fmaxf(M, old[j].x), d = fast_exp2(M - top);
+          fp = fast_exp2(old[j].x - top);
+          L = fmaf(L, d, fp * old[j].y);
+          fo *= d;
+          fn *= d;
+          M = top;
+        }
+        const bool part = un.ns > 1 || !last_run;
+        const float inv = part ? 1.f : L > 0.f ? 1.f / L : 0.f;
         float y[D / 8];
 #pragma unroll
         for (int i = 0; i < D / 8; ++i) {
           float v = fmaf(st.acc[i / 2][2 * (i % 2) + j], f[i], st.zacc[j]) * fo;
           if (has_new) v = fmaf(fn, vnew[gid * (D / 8) + i], v);
+          if (RUNS && run[0]) v = fmaf(fp, __ldcg(partial() + gid * (D / 8) + i), v);
           y[i] = v * inv;
         }
-        if (un.ns == 1) {
+        if (!part) {
           uint4* o = reinterpret_cast<uint4*>(ka.out + qrow + r * D + gid * (D / 8));
 #pragma unroll
           for (int i = 0; i < D / 8; i += 8)
             o[i / 8] = make_uint4(pack_bf16x2(y[i], y[i + 1]), pack_bf16x2(y[i + 2], y[i + 3]), pack_bf16x2(y[i + 4], y[i + 5]),
                                   pack_bf16x2(y[i + 6], y[i + 7]));
         } else {  // the split's partial; the combine kernel merges them
-          float* pp = a.part + static_cast<int64_t>(un.base + r * un.ns + un.sp) * (D + 4);
+          float* pp = partial();
 #pragma unroll
           for (int i = 0; i < D / 8; i += 4)
             *reinterpret_cast<float4*>(pp + gid * (D / 8) + i) = make_float4(y[i], y[i + 1], y[i + 2], y[i + 3]);
@@ -1844,11 +1935,24 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
 #pragma unroll
         for (int j = 0; j < DPL; ++j) v[j] = fmaf(v[j], f, fn * vx[j]);
       }
-      store_row<D>(ka, v, M, L, un.sp, un.q, un.h, un.ns, un.base, lane);
+      if (RUNS) {
+        float* pp = a.part + static_cast<int64_t>(un.base + un.sp) * (D + 4);
+        if (run[0]) take_partial<D>(pp, v, M, L, lane);
+        if (run[1]) store_partial<D>(pp, v, M, L, lane);
+      }
+      if (last_run) store_row<D>(ka, v, M, L, un.sp, un.q, un.h, un.ns, un.base, lane);
     }
-    u = __shfl_sync(0xffffffffu, u_next, 0);
     base += un.T;
     un.T = inext = consumed = 0;
+    if (RUNS) {
+      __syncwarp();
+      const int next = run[1];
+      __syncwarp();
+      if (lane == 0) run[0] = next;
+      __syncwarp();
+      if (next) continue;
+    }
+    u = __shfl_sync(0xffffffffu, u_next, 0);
   }
   if (!good) {  // a wait gave up: stop the CTA's warps, then let this one's copies land
     if (lane == 0) {
@@ -1898,5 +2002,32 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
   }
   if (done < 0x10000) step_commit(ka, ent);  // a call that gave up a wait stores nothing
 }
+
+// ------------------------------------------------------------------------- launch --
+// A kernel family (compiled side by side, one translation unit each): launches the instance of a
+// layout's head size and groups per head, and sets its shared-memory limit.
+
+template <bool HM, bool STEP, bool GQ, bool RUNS>
+auto row_instance(const Layout& l) {
+  using Kernel = void (*)(AttnKernelArgs);
+  const int ng = l.d / l.G;
+  if (l.d == 64) return ng == 1 ? Kernel(row_kernel<64, 1, HM, STEP, GQ, RUNS>) : Kernel(row_kernel<64, 2, HM, STEP, GQ, RUNS>);
+  return ng == 1   ? Kernel(row_kernel<128, 1, HM, STEP, GQ, RUNS>)
+         : ng == 2 ? Kernel(row_kernel<128, 2, HM, STEP, GQ, RUNS>)
+                   : Kernel(row_kernel<128, 4, HM, STEP, GQ, RUNS>);
+}
+template <bool HM, bool STEP, bool GQ, bool RUNS>
+cudaError_t launch_rows(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k) {
+  return launch_pdl(row_instance<HM, STEP, GQ, RUNS>(l), grid, dim3(32 * kRowWarps), smem, s, k);
+}
+template <bool HM, bool STEP, bool GQ, bool RUNS>
+cudaError_t configure_rows(const Layout& l) {
+  return cudaFuncSetAttribute(reinterpret_cast<const void*>(row_instance<HM, STEP, GQ, RUNS>(l)),
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemLimit);
+}
+#define TRR_ROW_FAMILY(prefix, HM, STEP, GQ, RUNS)                                                                   \
+  prefix template cudaError_t launch_rows<HM, STEP, GQ, RUNS>(const Layout&, dim3, size_t, cudaStream_t,             \
+                                                              const AttnKernelArgs&);                                \
+  prefix template cudaError_t configure_rows<HM, STEP, GQ, RUNS>(const Layout&);
 
 }  // namespace trr
