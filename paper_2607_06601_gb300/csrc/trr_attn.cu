@@ -9,57 +9,85 @@
 
 namespace trr {
 
-TRR_ROW_FAMILY(extern, false, false, false, false)
-TRR_ROW_FAMILY(extern, true, false, false, false)
-TRR_ROW_FAMILY(extern, false, true, false, false)
-TRR_ROW_FAMILY(extern, false, false, true, false)
-TRR_ROW_FAMILY(extern, false, true, true, false)
-TRR_ROW_FAMILY(extern, false, false, false, true)
-TRR_ROW_FAMILY(extern, true, false, false, true)
-TRR_ROW_FAMILY(extern, false, true, false, true)
-TRR_ROW_FAMILY(extern, false, false, true, true)
-TRR_ROW_FAMILY(extern, false, true, true, true)
+TRR_ROW_FAMILY(extern, kRow, false, false)
+TRR_ROW_FAMILY(extern, kRow, false, true)
+TRR_ROW_FAMILY(extern, kRow, true, false)
+TRR_ROW_FAMILY(extern, kRow, true, true)
+TRR_ROW_FAMILY(extern, kHeads, false, false)
+TRR_ROW_FAMILY(extern, kHeads, false, true)
+TRR_ROW_FAMILY(extern, kGroup, false, false)
+TRR_ROW_FAMILY(extern, kGroup, false, true)
+TRR_ROW_FAMILY(extern, kGroup, true, false)
+TRR_ROW_FAMILY(extern, kGroup, true, true)
+TRR_ROW_FAMILY(extern, kWide, false, false)
+TRR_ROW_FAMILY(extern, kWide, false, true)
+TRR_ROW_FAMILY(extern, kWide, true, false)
+TRR_ROW_FAMILY(extern, kWide, true, true)
 
-// Whether a warp takes a KV head and its query group (else a query head).
-static bool use_mma(const Layout& l) {
-  return uses_mma(l.Hq, l.Hkv, l.d, l.G, l.head_modes);
+// What a warp takes in a call of n queries.  With one mode per query a group's heads share their KV
+// head's pages.  Groups wider than the operand's 8 columns: calls of little work are bound by a unit's
+// chain (plan, copies, tiles, merge), which is shorter for one head; many rows, or long contexts, by
+// the copies and the unpacking that the wide unit shares.  A layer with a head per warp and with the
+// wide unit, us: 64 heads on 8 of 128, batch 1, context 4096 13 and 20, batch 8, 2048 26 and 30, batch 4,
+// 16384 78 and 44, batch 128, 100 64 and 49; 16 heads on 1 of 64, batch 64, 600 19 and 25, batch 16,
+// 16384 30 and 24; 32 on 2 of 128, batch 8, 2048 18 and 25, batch 32, 2048 47 and 34.
+static Kind kind_of(const Layout& l, int n) {
+  if (l.head_modes) return kHeads;
+  if (l.Hq == l.Hkv) return kRow;
+  if (uses_mma(l.Hq, l.Hkv, l.d, l.G, 0)) return kGroup;
+  const int64_t rows = static_cast<int64_t>(n) * l.Hq * l.d;
+  return rows >= 1 << 18 || rows * l.maxctx >= 1 << 28 ? kWide : kRow;
 }
+
+// Query heads of a unit, at most.
+static int unit_heads(const Layout& l, Kind k) { return k == kGroup ? l.Hq / l.Hkv : k == kWide ? 8 / (l.d / l.G) : 1; }
 
 // Queries per launch: their unit tables live in the CTAs' shared memory; a call with
 // more queries is cut into launches of this many, chained on the stream.  A query group's
 // rows take shared memory too, and its largest tile (8 KB at d 128) must fit a warp's ring.
-static int launch_queries(const Layout& l) { return use_mma(l) ? 512 : 1024; }
+static int launch_queries(Kind k) { return k == kGroup || k == kWide ? 512 : 1024; }
+
+template <Kind K>
+static cudaError_t configure_kind(const Layout& l) {
+  if constexpr (K != kHeads) {
+    const cudaError_t e = l.runs ? configure_rows<K, true, true>(l) : configure_rows<K, true, false>(l);
+    if (e != cudaSuccess) return e;
+  }
+  return l.runs ? configure_rows<K, false, true>(l) : configure_rows<K, false, false>(l);
+}
+template <Kind K>
+static cudaError_t launch_kind(const Layout& l, dim3 grid, size_t sm, cudaStream_t s, const AttnKernelArgs& k) {
+  if constexpr (K != kHeads) {
+    if (k.fused) return l.runs ? launch_rows<K, true, true>(l, grid, sm, s, k) : launch_rows<K, true, false>(l, grid, sm, s, k);
+  }
+  return l.runs ? launch_rows<K, false, true>(l, grid, sm, s, k) : launch_rows<K, false, false>(l, grid, sm, s, k);
+}
 
 // Done once per cache at creation, so that calls stay legal inside stream capture: the
 // instances that the cache's calls launch.
 cudaError_t attn_configure(const Layout& l) {
-  if (use_mma(l)) {
-    const cudaError_t e = l.runs ? configure_rows<false, false, true, true>(l) : configure_rows<false, false, true, false>(l);
-    if (e != cudaSuccess) return e;
-    return l.runs ? configure_rows<false, true, true, true>(l) : configure_rows<false, true, true, false>(l);
-  }
-  if (l.head_modes) return l.runs ? configure_rows<true, false, false, true>(l) : configure_rows<true, false, false, false>(l);
-  const cudaError_t e = l.runs ? configure_rows<false, false, false, true>(l) : configure_rows<false, false, false, false>(l);
-  if (e != cudaSuccess) return e;
-  return l.runs ? configure_rows<false, true, false, true>(l) : configure_rows<false, true, false, false>(l);
+  const Kind k = kind_of(l, 1);
+  if (k == kHeads) return configure_kind<kHeads>(l);
+  if (k == kGroup) return configure_kind<kGroup>(l);
+  const cudaError_t e = configure_kind<kRow>(l);
+  return e == cudaSuccess && l.Hq != l.Hkv ? configure_kind<kWide>(l) : e;
 }
 
-static cudaError_t launch_one(const Layout& l, const AttnKernelArgs& ka, int num_sms, cudaStream_t s) {
+static cudaError_t launch_one(const Layout& l, Kind kind, const AttnKernelArgs& ka, int num_sms, cudaStream_t s) {
   AttnKernelArgs k = ka;
-  const int heads = use_mma(l) ? l.Hq / l.Hkv : 1;
+  const int heads = unit_heads(l, kind);
   // every warp's ring is an equal share of what the call's tables leave
   const int fixed = RowSmem(l.d, heads, k.n, k.fused, 0).total;
   k.ring_bytes = (kRowSmemLimit - fixed) / kRowWarps / 128 * 128;
   if (k.ring_bytes < row_tile_bytes(l.d, l.d / l.G)) return cudaErrorInvalidConfiguration;
   const size_t sm = static_cast<size_t>(RowSmem(l.d, heads, k.n, k.fused, k.ring_bytes).total);
   const dim3 grid(kRowCtasPerSm * num_sms - num_sms / kRowSpare);
-  if (use_mma(l)) {
-    if (k.fused) return l.runs ? launch_rows<false, true, true, true>(l, grid, sm, s, k) : launch_rows<false, true, true, false>(l, grid, sm, s, k);
-    return l.runs ? launch_rows<false, false, true, true>(l, grid, sm, s, k) : launch_rows<false, false, true, false>(l, grid, sm, s, k);
+  switch (kind) {
+    case kRow: return launch_kind<kRow>(l, grid, sm, s, k);
+    case kHeads: return launch_kind<kHeads>(l, grid, sm, s, k);
+    case kGroup: return launch_kind<kGroup>(l, grid, sm, s, k);
+    default: return launch_kind<kWide>(l, grid, sm, s, k);
   }
-  if (k.fused) return l.runs ? launch_rows<false, true, false, true>(l, grid, sm, s, k) : launch_rows<false, true, false, false>(l, grid, sm, s, k);
-  if (l.head_modes) return l.runs ? launch_rows<true, false, false, true>(l, grid, sm, s, k) : launch_rows<true, false, false, false>(l, grid, sm, s, k);
-  return l.runs ? launch_rows<false, false, false, true>(l, grid, sm, s, k) : launch_rows<false, false, false, false>(l, grid, sm, s, k);
 }
 
 // The launches of an attention call with the given scratch views in `a`; *launches
@@ -90,9 +118,10 @@ static cudaError_t launch_attention(const Layout& l, const LayerArgs& a, int num
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.f / sqrtf(static_cast<float>(l.d));
   ka.qscale = scale * 1.4426950408889634f;
   // the combine kernel follows a query-group launch whose queries can have several splits
-  ka.defer_merge = use_mma(l) && l.s_cap > 1 ? 1 : 0;
+  const Kind kind = kind_of(l, n);
+  ka.defer_merge = unit_heads(l, kind) > 1 && l.s_cap > 1 ? 1 : 0;
   const int64_t row = static_cast<int64_t>(l.Hq) * l.d;  // bf16 elements per query
-  const int most = launch_queries(l);
+  const int most = launch_queries(kind);
   for (int q0 = 0; q0 < n; q0 += most) {
     ka.n = std::min(most, n - q0);
     ka.q0 = q0;
@@ -104,14 +133,15 @@ static cudaError_t launch_attention(const Layout& l, const LayerArgs& a, int num
     ka.q = static_cast<const uint16_t*>(q_bf16) + q0 * row;
     ka.out = static_cast<uint16_t*>(out_bf16) + q0 * row;
     ka.a.cnt = a.cnt + static_cast<int64_t>(q0) * l.Hq * l.cnt_stride;
+    ka.a.qtab = a.qtab + 2 * static_cast<int64_t>(q0);
     ka.early = step && early && q0 == 0 ? 1 : 0;  // a later launch follows one on the same layer
-    cudaError_t e = launch_one(l, ka, num_sms, s);
+    cudaError_t e = launch_one(l, kind, ka, num_sms, s);
     if (e != cudaSuccess) return e;
     ++*launches;
     if (ka.defer_merge) {
       CombineArgs ca;
       ca.part = a.part;
-      ca.qtab = reinterpret_cast<const int2*>(ka.a.cnt);
+      ca.qtab = reinterpret_cast<const int2*>(ka.a.qtab);
       ca.out = ka.out;
       ca.Hq = l.Hq;
       ca.rows = ka.n * l.Hq;
@@ -282,6 +312,7 @@ extern "C" trr_status trr_decode_attn_static(trr_cache* cache, int32_t layer, in
   a.ctrl = reinterpret_cast<int32_t*>(b);
   a.lctl = a.ctrl + kStaticLayerCtrl;
   a.cnt = reinterpret_cast<int32_t*>(b + b_ctrl);
+  a.qtab = a.cnt;  // (a call uses one of the two, and clears them first)
   a.part = reinterpret_cast<float*>(b + b_ctrl + b_cnt);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int ncnt = n * l.units * l.cnt_stride;

@@ -412,7 +412,7 @@ constexpr int kCombineWarps = 8;  // of a CTA
 struct CombineArgs {
   const float* part;  // partials of the launch: a head's splits one after another, D + 4 floats each
   const int2* qtab;   // [n] first partial and splits per head of each query (written by CTA 0 of the
-                      // attention kernel, in the arrival-counter region it does not use)
+                      // attention kernel)
   uint16_t* out;      // [n][Hq][D] bf16 rows of the launch
   int Hq, rows;       // rows: n * Hq
   int wpr;            // warps of a row: 1, 2, 4 or 8

@@ -5,7 +5,7 @@
 
 namespace trr {
 
-TRR_ROW_FAMILY(, false, false, true, false)
+TRR_ROW_FAMILY(, kGroup, false, false)
 
 cudaError_t launch_attn_combine(int d, int ctas, cudaStream_t s, const CombineArgs& ca) {
   return d == 64 ? launch_pdl(attn_combine_kernel<64>, dim3(ctas), dim3(32 * kCombineWarps), 0, s, ca)

@@ -3,5 +3,5 @@
 #include "trr_row.cuh"
 
 namespace trr {
-TRR_ROW_FAMILY(, false, false, true, true)
+TRR_ROW_FAMILY(, kGroup, false, true)
 }  // namespace trr

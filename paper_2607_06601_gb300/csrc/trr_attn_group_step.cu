@@ -2,5 +2,5 @@
 #include "trr_row.cuh"
 
 namespace trr {
-TRR_ROW_FAMILY(, false, true, true, false)
+TRR_ROW_FAMILY(, kGroup, true, false)
 }  // namespace trr

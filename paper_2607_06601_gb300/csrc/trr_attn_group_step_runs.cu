@@ -3,5 +3,5 @@
 #include "trr_row.cuh"
 
 namespace trr {
-TRR_ROW_FAMILY(, false, true, true, true)
+TRR_ROW_FAMILY(, kGroup, true, true)
 }  // namespace trr

@@ -2,5 +2,5 @@
 #include "trr_row.cuh"
 
 namespace trr {
-TRR_ROW_FAMILY(, false, false, false, false)
+TRR_ROW_FAMILY(, kRow, false, false)
 }  // namespace trr

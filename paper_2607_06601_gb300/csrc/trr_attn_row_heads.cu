@@ -2,5 +2,5 @@
 #include "trr_row.cuh"
 
 namespace trr {
-TRR_ROW_FAMILY(, true, false, false, false)
+TRR_ROW_FAMILY(, kHeads, false, false)
 }  // namespace trr

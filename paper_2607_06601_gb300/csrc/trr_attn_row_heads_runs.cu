@@ -3,5 +3,5 @@
 #include "trr_row.cuh"
 
 namespace trr {
-TRR_ROW_FAMILY(, true, false, false, true)
+TRR_ROW_FAMILY(, kHeads, false, true)
 }  // namespace trr

@@ -3,5 +3,5 @@
 #include "trr_row.cuh"
 
 namespace trr {
-TRR_ROW_FAMILY(, false, false, false, true)
+TRR_ROW_FAMILY(, kRow, false, true)
 }  // namespace trr

@@ -2,5 +2,5 @@
 #include "trr_row.cuh"
 
 namespace trr {
-TRR_ROW_FAMILY(, false, true, false, false)
+TRR_ROW_FAMILY(, kRow, true, false)
 }  // namespace trr

@@ -3,5 +3,5 @@
 #include "trr_row.cuh"
 
 namespace trr {
-TRR_ROW_FAMILY(, false, true, false, true)
+TRR_ROW_FAMILY(, kRow, true, true)
 }  // namespace trr

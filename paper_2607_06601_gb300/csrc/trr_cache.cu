@@ -41,6 +41,7 @@ LayerArgs layer_args(const Layout& l, const Views& v, int layer) {
   a.plast = v.plast + ls * 4 * l.MP;
   a.lastpg = v.lastpg + ls * 4;
   a.cnt = v.cnt;
+  a.qtab = v.qtab;
   a.cnt_stride = l.cnt_stride;
   a.part = v.part;
   return a;
@@ -122,6 +123,8 @@ static trr_status make_layout(const trr_cache_config* c, Layout* l) {
   l->off_plast = take(16 * nls * l->MP);
   l->off_lastpg = take(16 * nls);
   l->off_cnt = take(4 * static_cast<int64_t>(l->max_queries) * l->units * l->cnt_stride);
+  // (narrow query groups do not use the arrivals: their table takes the same place)
+  l->off_qtab = l->swz && l->Hq > l->Hkv && !l->head_modes ? take(8 * static_cast<int64_t>(l->max_queries)) : l->off_cnt;
   l->off_part = take(4 * l->max_items * (l->Hq / l->units) * (l->d + 4));
   for (int k = 0; k < kClasses; ++k) l->off_pool[k] = take(l->cap[k] * l->page_bytes[k]);
   l->total = off;

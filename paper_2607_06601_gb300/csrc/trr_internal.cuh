@@ -56,7 +56,7 @@ struct Layout {
   int64_t max_items;
   int64_t hdr, tokb[kClasses], slice[kClasses], maskb, page_bytes[kClasses];
   int64_t off_ctrl, off_lctl, off_last_pos, off_ntok, off_presence, off_pt, off_pfirst, off_plast, off_lastpg;
-  int64_t off_cnt, off_part, off_pool[kClasses], total;
+  int64_t off_cnt, off_qtab, off_part, off_pool[kClasses], total;
 };
 
 // Splits of a query whose key range spans `range` positions: at least pos_split positions
@@ -100,6 +100,7 @@ struct Views {  // typed device pointers into the cache memory
   int32_t* plast;
   int32_t* lastpg;
   int32_t* cnt;
+  int32_t* qtab;
   float* part;
   uint8_t* pool[kClasses];
 };
@@ -117,6 +118,7 @@ inline Views make_views(const Layout& l, void* base) {
   v.plast = reinterpret_cast<int32_t*>(b + l.off_plast);
   v.lastpg = reinterpret_cast<int32_t*>(b + l.off_lastpg);
   v.cnt = reinterpret_cast<int32_t*>(b + l.off_cnt);
+  v.qtab = reinterpret_cast<int32_t*>(b + l.off_qtab);
   v.part = reinterpret_cast<float*>(b + l.off_part);
   for (int c = 0; c < kClasses; ++c) v.pool[c] = b + l.off_pool[c];
   return v;
@@ -143,6 +145,7 @@ struct LayerArgs {
   int32_t* plast;
   int32_t* lastpg;     // this layer: [S][4] id of the page holding token ntok-1 (internal)
   int32_t* cnt;        // [max_queries][Hq][cnt_stride] split arrivals (zero between calls)
+  int32_t* qtab;       // [max_queries][2] query groups: a query's first partial and splits per head
   float* part;         // [max_queries * s_cap * Hq][d + 4] fp32 partials: acc, M, L
   uint8_t* pool[kClasses];
 };

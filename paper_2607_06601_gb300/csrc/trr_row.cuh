@@ -42,6 +42,10 @@
 
 namespace trr {
 
+// What a work unit is: a query head; a query head of a cache with per-head modes; a KV head and its
+// query group (g * d/G <= 8); a KV head and up to 8 / (d/G) heads of a wider query group.
+enum Kind { kRow, kHeads, kGroup, kWide };
+
 constexpr int kRowWarps = 8;   // warps per CTA
 constexpr int kRowSlots = 8;   // tiles a warp may have in flight
 constexpr int kRowCtasPerSm = 2;
@@ -799,21 +803,32 @@ __device__ __forceinline__ void tile_values16(RowState<D, NG>& st, const uint8_t
 // 5e-3 off without it, 2^-14 8 %; gqa_long shape 630 -> 646 us for 4 steps.)
 constexpr float kGroupTau = 3.f, kGroupWide = 8000.f;
 constexpr float kLift = 16.f;  // at first
-template <int D, int NG>
+//
+// Groups wider than the operand's 8 columns are taken 8 / NG heads at a time, so that a page is
+// copied and its codes unpacked once for those heads, where a call's work is bound by that.  (64 heads
+// on 8 of 128, batch 128, context 4096, 2 steps of 2 layers: 953 us; 1998 with a query head per warp,
+// each copying the pages for itself.)  They keep more of the weights' and sums' bits: a power of two
+// per column in place of the lift, chosen from the V scales of keys with weight, and the zero points
+// folded in.  Their rows are stored as MHA's.
+constexpr float kGroupTop = 4096.f;     // s * ws at most: p <= 2^3 keeps p * s * ws below f16's end
+constexpr float kGroupWeight = -17.f;   // log2 of the p from which on a key's scale counts: a smaller
+                                        // p takes no s * ws (at most 2^32) past f16's end
+template <int D, int NG, bool WIDE>
 struct GroupState {
   static constexpr int NP = D / 8, MT = D / 16;
   uint32_t kb[NP];
   float acc[MT][4];  // dims gid D/8 + 2 t (+ 1) x the lane's columns, times 2^vfac_log2
   float qsum[2], m[2], l[2], zacc[2];  // per column (m: its head's maximum - lift)
-  float lift, lim;   // and the largest V scale that lift allows
+  float lift, lim;   // and the largest V scale that lift allows (wide groups: 0, not used)
+  float ws[2];       // wide groups, per column: codes' weights are p * s * ws (a power of two)
   float kfac[2];     // per column: the current class's factor of the group sums
   uint32_t kl, vl;
   int wl, zoff, cls;
   int E;             // exponent of the largest query value of the head and group of column gid
 };
 
-template <int D, int NG, int B>
-__device__ __forceinline__ void group_class(GroupState<D, NG>& st, const uint8_t* qs, int heads, int lane) {
+template <int D, int NG, int B, bool WIDE>
+__device__ __forceinline__ void group_class(GroupState<D, NG, WIDE>& st, const uint8_t* qs, int heads, int lane) {
   constexpr int NP = D / 8, rowb = D * B / 8;
   const int gid = lane >> 2, tig = lane & 3, r = gid / NG;
   const bool ok = r < heads && (tig * NG) / 4 == gid % NG;
@@ -831,42 +846,46 @@ __device__ __forceinline__ void group_class(GroupState<D, NG>& st, const uint8_t
     }
     st.kb[i] = ok ? w : 0u;
   }
-  st.kl = gid * rowb + tig * (rowb / 4);
-  st.vl = tig * rowb + (rowb >= 32 ? gid * (rowb / 8) : (gid * (rowb / 8)) & ~3);
+  st.kl = WIDE ? k_lane<D, B>(gid, tig) : gid * rowb + tig * (rowb / 4);
+  st.vl = WIDE ? v_lane<D, B>(gid, tig) : tig * rowb + (rowb >= 32 ? gid * (rowb / 8) : (gid * (rowb / 8)) & ~3);
+  st.wl = 16 * w_row<WIDE ? row_map(D, B) : 0>(lane);
 }
 
-template <int D, int NG>
-__device__ __forceinline__ void group_switch(GroupState<D, NG>& st, int to, bool fresh, const uint8_t* qs, int heads,
+template <int D, int NG, bool WIDE>
+__device__ __forceinline__ void group_switch(GroupState<D, NG, WIDE>& st, int to, bool fresh, const uint8_t* qs, int heads,
                                              const float* fac, float qscale, int kt, int lane) {
   constexpr int MT = D / 16;
   switch (to) {
-    case 0: group_class<D, NG, 2>(st, qs, heads, lane); break;
-    case 1: group_class<D, NG, 4>(st, qs, heads, lane); break;
-    case 2: group_class<D, NG, 8>(st, qs, heads, lane); break;
-    default: group_class<D, NG, 16>(st, qs, heads, lane); break;
+    case 0: group_class<D, NG, 2, WIDE>(st, qs, heads, lane); break;
+    case 1: group_class<D, NG, 4, WIDE>(st, qs, heads, lane); break;
+    case 2: group_class<D, NG, 8, WIDE>(st, qs, heads, lane); break;
+    default: group_class<D, NG, 16, WIDE>(st, qs, heads, lane); break;
   }
 #pragma unroll
   for (int j = 0; j < 2; ++j) {  // as in row_switch
     const float e = __int_as_float((127 + __shfl_sync(0xffffffffu, st.E, 4 * (2 * (lane & 3) + j))) << 23);
     st.kfac[j] = to == 3 ? qscale : fminf(e * qscale * pow2f(9), 3.4028235e38f);
   }
-  st.wl = 16 * w_row<0>(lane);
   st.zoff = kt * (2 * (D * bits_of_class(to) / 8) + 4 * NG) + (lane >> 2) * NG * 4 + (NG == 4 ? (lane & 1) * 8 : 0);
   if (!fresh) {
     float f[2 * MT];
     load_words<2 * MT>(reinterpret_cast<const uint8_t*>(fac + (st.cls * 4 + to) * (D / 8)), reinterpret_cast<uint32_t*>(f));
 #pragma unroll
-    for (int t = 0; t < MT; ++t) {
+    for (int j = 0; j < 2; ++j) {
+      const float g = !WIDE || (to == 3) == (st.cls == 3) ? 1.f : to == 3 ? pow2_inverse(st.ws[j]) : st.ws[j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) st.acc[t][i] *= f[2 * t + (i >> 1)];
+      for (int t = 0; t < MT; ++t) {
+        st.acc[t][j] *= f[2 * t] * g;
+        st.acc[t][2 + j] *= f[2 * t + 1] * g;
+      }
     }
   }
   st.cls = to;
 }
 
 // 1. The columns' group sums of q.c: c[u][2 h + j] is key gid + 8 h + 16 u, column 2 tig + j.
-template <int D, int NG, int B>
-__device__ __forceinline__ void group_scores(const GroupState<D, NG>& st, const uint8_t* tile, int kt, float (&c)[2][4]) {
+template <int D, int NG, int B, bool WIDE>
+__device__ __forceinline__ void group_scores(const GroupState<D, NG, WIDE>& st, const uint8_t* tile, int kt, float (&c)[2][4]) {
   constexpr int KS = D / 16, rowb = D * B / 8;
   constexpr int KW = D * B / 128;  // K words per lane and key (D/4 dims)
 #pragma unroll
@@ -877,8 +896,8 @@ __device__ __forceinline__ void group_scores(const GroupState<D, NG>& st, const 
 #pragma unroll
     for (int hf = 0; hf < KH; ++hf) {
       uint32_t k1[KWH], k2[KWH];
-      load_words<KWH>(tile + st.kl + 16 * u * rowb + 16 * hf, k1);
-      load_words<KWH>(tile + st.kl + (16 * u + 8) * rowb + 16 * hf, k2);
+      load_words<KWH>(tile + (WIDE ? k_off<D, B>(st.kl, 0, u, hf) : st.kl + 16 * u * rowb + 16 * hf), k1);
+      load_words<KWH>(tile + (WIDE ? k_off<D, B>(st.kl, 1, u, hf) : st.kl + (16 * u + 8) * rowb + 16 * hf), k2);
 #pragma unroll
       for (int s = hf * KSH; s < (hf + 1) * KSH; ++s) {
         const int i0 = 2 * (s - hf * KSH);
@@ -897,8 +916,8 @@ __device__ __forceinline__ void group_scores(const GroupState<D, NG>& st, const 
 
 // 2. The weights of the lane's four keys (ok: bit 2 u + h) for its columns, as operand rows at
 // wb.  has_sz: the width has scales (at sz: the key gid's V scales, K's kt keys before).
-template <int D, int NG>
-__device__ __forceinline__ void group_weights(GroupState<D, NG>& st, const float (&c)[2][4], unsigned ok, bool has_sz,
+template <int D, int NG, bool WIDE>
+__device__ __forceinline__ void group_weights(GroupState<D, NG, WIDE>& st, const float (&c)[2][4], unsigned ok, bool has_sz,
                                               const uint8_t* sz, int kt, int heads, uint8_t* wb, int lane) {
   constexpr int MT = D / 16, J = NG == 1 ? 2 : 1;  // heads of a lane
   const int gid = lane >> 2, tig = lane & 3;
@@ -943,45 +962,104 @@ __device__ __forceinline__ void group_weights(GroupState<D, NG>& st, const float
 #pragma unroll
   for (int j = 0; j < J; ++j)
     over = fmaxf(over, fmaxf(fmaxf(sc[0][j], sc[1][j]), fmaxf(sc[2][j], sc[3][j])) - st.m[j]);
-  over -= st.lift;
-  if (has_sz) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      big = fmaxf(big, fmaxf(__half2float(__ushort_as_half(zw[k][0] & 0xffff)), __half2float(__ushort_as_half(zw[k][1] & 0xffff))));
-  }
-  if (__any_sync(0xffffffffu, over > kGroupTau || (big > st.lim && (st.lift > 0.f || over > 0.f)))) {  // (the keys' lanes share a maximum)
-    const float lift = st.lift;
+  if constexpr (!WIDE) {
+    over -= st.lift;
     if (has_sz) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
-      if (big > st.lim) {
-        // big * 2^lift < 2^6, 2^3, 2^0 as in tile_weights, lift >= 0; 2^(lift + 3) * lim < 2^16
-        const int e = 5 - 3 * st.cls - (static_cast<int>(__float_as_uint(big) >> 23) - 127);
-        st.lift = static_cast<float>(max(0, min(static_cast<int>(lift), e)));
-        st.lim = st.lift > 0.f ? __int_as_float((127 + 12 - static_cast<int>(st.lift)) << 23) : kGroupWide;
-      }
+      for (int k = 0; k < 4; ++k)
+        big = fmaxf(big, fmaxf(__half2float(__ushort_as_half(zw[k][0] & 0xffff)), __half2float(__ushort_as_half(zw[k][1] & 0xffff))));
     }
+    if (__any_sync(0xffffffffu, over > kGroupTau || (big > st.lim && (st.lift > 0.f || over > 0.f)))) {  // (the keys' lanes share a maximum)
+      const float lift = st.lift;
+      if (has_sz) {
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-      float mx = fmaxf(fmaxf(sc[0][j], sc[1][j]), fmaxf(sc[2][j], sc[3][j]));
-#pragma unroll
-      for (int o = 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      mx = fmaxf(mx, __fadd_rd(st.m[j], lift));
-      const float m = __fadd_ru(mx, -st.lift);  // rounded up: p <= 2^lift also where a score's ulp is larger
-      const float alpha = fast_exp2(st.m[j] - m);
-      st.m[j] = m;
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        if (NG == 1 && i != j) continue;
-        st.l[i] *= alpha;
-        st.zacc[i] *= alpha;
-#pragma unroll
-        for (int t = 0; t < MT; ++t) {
-          st.acc[t][i] *= alpha;
-          st.acc[t][i + 2] *= alpha;
+        for (int o = 16; o > 0; o >>= 1) big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+        if (big > st.lim) {
+          // big * 2^lift < 2^6, 2^3, 2^0 as in tile_weights, lift >= 0; 2^(lift + 3) * lim < 2^16
+          const int e = 5 - 3 * st.cls - (static_cast<int>(__float_as_uint(big) >> 23) - 127);
+          st.lift = static_cast<float>(max(0, min(static_cast<int>(lift), e)));
+          st.lim = st.lift > 0.f ? __int_as_float((127 + 12 - static_cast<int>(st.lift)) << 23) : kGroupWide;
         }
       }
-      if (NG > 1) st.m[1] = st.m[0];
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        float mx = fmaxf(fmaxf(sc[0][j], sc[1][j]), fmaxf(sc[2][j], sc[3][j]));
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        mx = fmaxf(mx, __fadd_rd(st.m[j], lift));
+        const float m = __fadd_ru(mx, -st.lift);  // rounded up: p <= 2^lift also where a score's ulp is larger
+        const float alpha = fast_exp2(st.m[j] - m);
+        st.m[j] = m;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if (NG == 1 && i != j) continue;
+          st.l[i] *= alpha;
+          st.zacc[i] *= alpha;
+#pragma unroll
+          for (int t = 0; t < MT; ++t) {
+            st.acc[t][i] *= alpha;
+            st.acc[t][i + 2] *= alpha;
+          }
+        }
+        if (NG > 1) st.m[1] = st.m[0];
+      }
+    }
+  } else {
+    if (__any_sync(0xffffffffu, over > kGroupTau)) {  // (the keys' lanes share a maximum)
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        float mx = fmaxf(fmaxf(sc[0][j], sc[1][j]), fmaxf(sc[2][j], sc[3][j]));
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        mx = fmaxf(mx, st.m[j]);
+        const float alpha = fast_exp2(st.m[j] - mx);
+        st.m[j] = mx;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if (NG == 1 && i != j) continue;
+          float f = alpha;
+          if (has_sz && alpha < pow2f(-12)) {  // little is left of what ws was chosen for
+            f *= pow2f(kWeightScale) * pow2_inverse(st.ws[i]);
+            st.ws[i] = pow2f(kWeightScale);
+          }
+          st.l[i] *= alpha;
+          st.zacc[i] *= alpha;
+#pragma unroll
+          for (int t = 0; t < MT; ++t) {
+            st.acc[t][i] *= f;
+            st.acc[t][i + 2] *= f;
+          }
+        }
+        if (NG > 1) st.m[1] = mx;
+      }
+    }
+    if (has_sz) {
+      float big[2] = {0.f, 0.f};  // per column: the largest V scale of a key with weight
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const float x = __half2float(__ushort_as_half(zw[k][j] & 0xffff));
+          if (sc[k][J == 2 ? j : 0] - st.m[j] > kGroupWeight) big[j] = fmaxf(big[j], x);
+        }
+      }
+      if (__any_sync(0xffffffffu, big[0] * st.ws[0] > kGroupTop || big[1] * st.ws[1] > kGroupTop)) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+#pragma unroll
+          for (int o = 4; o < 32; o <<= 1) big[j] = fmaxf(big[j], __shfl_xor_sync(0xffffffffu, big[j], o));
+          // big * ws < 2^6, 2^3, 2^0 as in tile_weights
+          const int e = 5 - 3 * st.cls - (static_cast<int>(__float_as_uint(big[j]) >> 23) - 127);
+          const float ws = big[j] > 0.f ? __int_as_float((127 + min(kWeightScale, e)) << 23) : st.ws[j];
+          const float f = ws * pow2_inverse(st.ws[j]);
+          st.ws[j] = ws;
+#pragma unroll
+          for (int t = 0; t < MT; ++t) {
+            st.acc[t][j] *= f;
+            st.acc[t][j + 2] *= f;
+          }
+        }
+      }
     }
   }
 #pragma unroll
@@ -994,7 +1072,7 @@ __device__ __forceinline__ void group_weights(GroupState<D, NG>& st, const float
       const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&zw[k][j]));
       st.l[j] += p[j];
       st.zacc[j] = fmaf(p[j], f.y, st.zacc[j]);
-      w[j] = p[j] * f.x;
+      w[j] = WIDE && has_sz ? p[j] * f.x * st.ws[j] : p[j] * f.x;
     }
     uint32_t* at = reinterpret_cast<uint32_t*>(wb + 16 * (gid + 8 * k)) + tig;
     if (has_sz) {  // high and low part (finite: p <= 1 where a scale is above kGroupWide, then lift is 0)
@@ -1019,14 +1097,15 @@ __device__ __forceinline__ uint32_t finite_bf16x2(uint32_t x) {
 }
 
 // 3. P.V.  all[k]: lanes whose key gid + 8 k counts (width 16: other keys' values read as 0).
-template <int D, int NG, int B>
-__device__ __forceinline__ void group_values(GroupState<D, NG>& st, const uint8_t* tile, int kt, bool part,
+template <int D, int NG, int B, bool WIDE>
+__device__ __forceinline__ void group_values(GroupState<D, NG, WIDE>& st, const uint8_t* tile, int kt, bool part,
                                              const unsigned (&all)[4], const uint8_t* wb, int lane) {
   constexpr int MT = D / 16, rowb = D * B / 8;
   constexpr int VB = D * B / 64, VW = VB >= 4 ? VB / 4 : 1;  // V bytes per lane and key (D/8 dims)
   constexpr int VH = VW > 4 ? VW / 4 : 1, VWH = VW / VH, MTH = MT / VH;
   const int gid = lane >> 2, tig = lane & 3;
-  const uint8_t* v0 = tile + kt * rowb + st.vl;
+  constexpr int MAP = WIDE ? row_map(D, B) : 0;
+  const uint8_t* v0 = tile + kt * rowb;
   uint32_t w[4], wlo[4];
   ldmatrix4_trans(w, wb + st.wl);
   ldmatrix4_trans(wlo, wb + 512 + st.wl);
@@ -1038,10 +1117,10 @@ __device__ __forceinline__ void group_values(GroupState<D, NG>& st, const uint8_
       uint32_t x[4][VWH];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        load_words<VWH>(v0 + 4 * (4 * u + i) * rowb + 16 * hf, x[i]);  // key tig + 4 (4 u + i)
+        load_words<VWH>(v0 + (WIDE ? v_off<D, B>(st.vl, 4 * u + i, hf) : st.vl + 4 * (4 * u + i) * rowb + 16 * hf), x[i]);
         if (VB < 4) x[i][0] >>= ((gid * VB) & 3) * 8;
         if (B == 16 && part) {
-          const int key = tig + 4 * (4 * u + i);  // its ok: lane 4 (key % 8)'s bit of all[key / 8]
+          const int key = v_key<MAP>(tig, 4 * u + i);  // its ok: lane 4 (key % 8)'s bit of all[key / 8]
           const unsigned bits = key & 16 ? (key & 8 ? all[3] : all[2]) : (key & 8 ? all[1] : all[0]);
           if (!((bits >> (4 * (key & 7))) & 1u)) {
 #pragma unroll
@@ -1090,6 +1169,26 @@ __device__ __forceinline__ void fold_zero_points(RowState<D, NG>& st, const floa
   for (int t = 0; t < MT; ++t) {
     st.acc[t][0] = fmaf(z, f[2 * t], st.acc[t][0]);
     st.acc[t][2] = fmaf(z, f[2 * t + 1], st.acc[t][2]);
+  }
+}
+
+template <int D, int NG>
+__device__ __forceinline__ void fold_zero_points(GroupState<D, NG, true>& st, const float* fac, int lane) {
+  constexpr int MT = D / 16;
+  float f[2 * MT];
+  load_words<2 * MT>(reinterpret_cast<const uint8_t*>(fac + (12 + st.cls) * (D / 8)), reinterpret_cast<uint32_t*>(f));
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    float z = st.zacc[j];
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+    st.zacc[j] = 0.f;
+    if (st.cls != 3) z *= st.ws[j];
+#pragma unroll
+    for (int t = 0; t < MT; ++t) {
+      st.acc[t][j] = fmaf(z, f[2 * t], st.acc[t][j]);
+      st.acc[t][j + 2] = fmaf(z, f[2 * t + 1], st.acc[t][j + 2]);
+    }
   }
 }
 
@@ -1387,22 +1486,25 @@ __device__ __forceinline__ TilePlan plan_tiles(const AttnKernelArgs& ka, int seq
 }
 // ------------------------------------------------------------------------- kernel --
 
-// GQ: a unit is a KV head and its query group, and the combine kernel merges its splits.
-template <int D, int NG, bool HM, bool STEP, bool GQ, bool RUNS>
+template <int D, int NG, Kind K, bool STEP, bool RUNS>
 __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_constant__ AttnKernelArgs ka) {
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr int DPL = D / 32;
+  constexpr bool HM = K == kHeads, WIDE = K == kWide;
+  constexpr bool GQ = K == kGroup || WIDE;  // the combine kernel merges a query's splits
   const LayerArgs& a = ka.a;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = ka.n, P = a.P, R = ka.ring_bytes;
-  const int g = a.Hq / a.Hkv, heads = GQ ? g : 1, rows = GQ ? a.Hkv : a.Hq;  // of a unit; of a query
-  const RowSmem lay(D, heads, n, STEP, R);
+  const int g = a.Hq / a.Hkv, hmost = WIDE ? 8 / NG : GQ ? g : 1;  // query heads of a unit, at most
+  const int blocks = WIDE ? (g + hmost - 1) / hmost : 1;           // units of a KV head's group
+  const int rows = GQ ? a.Hkv * blocks : a.Hq;                     // units of a query's split
+  const RowSmem lay(D, hmost, n, STEP, R);
   int* pre = reinterpret_cast<int*>(smem + lay.pre);
   int* ent = reinterpret_cast<int*>(smem + lay.ent);
   int* sc = ent + 6 * n;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + lay.flag);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + lay.full) + warp * kRowSlots;
   uint8_t* ring = smem + lay.ring + warp * R;
-  uint8_t* qs = smem + lay.q + warp * RowSmem::row_q_bytes(D, heads);
+  uint8_t* qs = smem + lay.q + warp * RowSmem::row_q_bytes(D, hmost);
   float* fac = reinterpret_cast<float*>(smem + lay.fac);
 #pragma unroll 1
   for (int i = threadIdx.x; i < 16 * (D / 8); i += 32 * kRowWarps) {
@@ -1548,9 +1650,11 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
     } else {
       un.sp = div24(r, rows);
       un.h = r - un.sp * rows;
-      un.base = (pre[q] + un.h * un.ns) * heads;
+      // (wide groups: the units of the queries before are `rows` for each of their splits)
+      un.base = WIDE ? pre[q] / rows * a.Hq : (pre[q] + un.h * un.ns) * hmost;
     }
-    kvh = GQ || g == 1 ? un.h : div24(un.h, g);
+    kvh = WIDE ? div24(un.h, blocks) : GQ || g == 1 ? un.h : div24(un.h, g);
+    if (WIDE) un.base += (kvh * g + (un.h - kvh * blocks) * hmost) * un.ns;
     const TilePlan tp = plan_tiles<D, NG, HM, STEP, RUNS>(ka, qi.x, un, kvh, RUNS ? run[0] : 0, lane);
     un.T = tp.T;
     wsrc = tp.src;
@@ -1606,16 +1710,19 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       }
     }
     if (GQ && ka.defer_merge && first && blockIdx.x == 0) {  // for the combine kernel: a query's first partial, splits
-      int2* qtab = reinterpret_cast<int2*>(a.cnt);
+      int2* qtab = reinterpret_cast<int2*>(a.qtab);
 #pragma unroll 1
-      for (int k = threadIdx.x; k < n; k += 32 * kRowWarps) qtab[ord[k]] = make_int2(pre[k] * heads, qinf[k].w & 0xffffff);
+      for (int k = threadIdx.x; k < n; k += 32 * kRowWarps) qtab[ord[k]] = make_int2(WIDE ? pre[k] / rows * a.Hq : pre[k] * hmost, qinf[k].w & 0xffffff);
     }
     if (u >= total || !good) break;
     if (RUNS) __syncwarp();
     const bool last_run = !RUNS || run[1] == 0;
     int u_next = total;
     if (total > nwarps && lane == 0 && last_run) u_next = nwarps + atomicAdd(&a.lctl[kNextUnit], 1);  // read at the unit's end
-    const bool own = GQ || un.h == kvh * g;  // stores a new token's rows of its KV head
+    const int blk = WIDE ? un.h - kvh * blocks : 0;
+    const int heads = WIDE ? min(hmost, g - blk * hmost) : hmost;  // of the unit, from h0 on
+    const int h0 = WIDE ? kvh * g + blk * hmost : un.h * hmost;
+    const bool own = WIDE ? blk == 0 : GQ || un.h == kvh * g;  // stores a new token's rows of its KV head
     // decode step: the entry's own token joins the row's last split; a skip token that
     // stores KV is written by its zero row's unit
     const bool has_new = STEP && !failed && last_run && un.sp == un.ns - 1 && ent[2 * un.q] >= 0 && (!un.zero || own);
@@ -1625,7 +1732,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       rk = load_row<D>(ka.k + src, lane);
       rv = load_row<D>(ka.v + src, lane);
     }
-    const int64_t qrow = (static_cast<int64_t>(un.q) * a.Hq + un.h * heads) * D;  // its first head's
+    const int64_t qrow = (static_cast<int64_t>(un.q) * a.Hq + h0) * D;  // its first head's
     uint2 qraw = make_uint2(0, 0);
     if (!GQ && !un.zero) qraw = load_row<D>(ka.q + qrow, lane);
     float kx[DPL] = {}, vx[DPL] = {}, new_score = kNegInf;
@@ -1653,7 +1760,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       if (!STEP && un.err && un.sp == 0 && lane == 0) atomicMin(&a.lctl[kFirstBadQuery], (ka.q0 + un.q) * 16 + un.err);
     } else if constexpr (GQ) {
       // the group's query rows to shared memory; each column's sum and largest exponent
-      GroupState<D, NG> st;
+      GroupState<D, NG, WIDE> st;
       const int gid = lane >> 2, tig = lane & 3;
       float new_score[2] = {kNegInf, kNegInf};
       st.E = -85;
@@ -1701,12 +1808,13 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
         }
       }
       st.cls = 3;
-      st.lift = kLift;
+      st.lift = WIDE ? 0.f : kLift;
       st.lim = pow2f(12 - static_cast<int>(kLift));
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         st.m[j] = kNoMax;
         st.l[j] = st.zacc[j] = 0.f;
+        st.ws[j] = pow2f(kWeightScale);
       }
 #pragma unroll
       for (int t = 0; t < D / 16; ++t) st.acc[t][0] = st.acc[t][1] = st.acc[t][2] = st.acc[t][3] = 0.f;
@@ -1716,7 +1824,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       for (; c < un.T; ++c) {
         const uint32_t geo = __shfl_sync(0xffffffffu, wgeo, c);
         const int cls = geo & 3, kt = tile_keys(cls);
-        if (c == 0 || cls != st.cls) group_switch<D, NG>(st, cls, c == 0, qs, heads, fac, ka.qscale, kt, lane);
+        if (c == 0 || cls != st.cls) group_switch<D, NG, WIDE>(st, cls, c == 0, qs, heads, fac, ka.qscale, kt, lane);
         if (!tile_in(c)) break;
         const uint8_t* tile = ring + ((geo >> 3) & (1023u << 7));
         const int fill = (geo >> 2) & 127;
@@ -1733,24 +1841,27 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
         }
         float sc[2][4] = {};
         switch (cls) {
-          case 0: group_scores<D, NG, 2>(st, tile, kt, sc); break;
-          case 1: group_scores<D, NG, 4>(st, tile, kt, sc); break;
-          case 2: group_scores<D, NG, 8>(st, tile, kt, sc); break;
-          default: group_scores<D, NG, 16>(st, tile, kt, sc); break;
+          case 0: group_scores<D, NG, 2, WIDE>(st, tile, kt, sc); break;
+          case 1: group_scores<D, NG, 4, WIDE>(st, tile, kt, sc); break;
+          case 2: group_scores<D, NG, 8, WIDE>(st, tile, kt, sc); break;
+          default: group_scores<D, NG, 16, WIDE>(st, tile, kt, sc); break;
         }
-        group_weights<D, NG>(st, sc, ok, cls != 3, tile + st.zoff, kt, heads, wb, lane);
+        group_weights<D, NG, WIDE>(st, sc, ok, cls != 3, tile + st.zoff, kt, heads, wb, lane);
         unsigned all[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) all[k] = __ballot_sync(0xffffffffu, (ok >> k) & 1u);
         __syncwarp();
         switch (cls) {
-          case 0: group_values<D, NG, 2>(st, tile, kt, false, all, wb, lane); break;
-          case 1: group_values<D, NG, 4>(st, tile, kt, false, all, wb, lane); break;
-          case 2: group_values<D, NG, 8>(st, tile, kt, false, all, wb, lane); break;
-          default: group_values<D, NG, 16>(st, tile, kt, fill < kt || (geo & kMask), all, wb, lane); break;
+          case 0: group_values<D, NG, 2, WIDE>(st, tile, kt, false, all, wb, lane); break;
+          case 1: group_values<D, NG, 4, WIDE>(st, tile, kt, false, all, wb, lane); break;
+          case 2: group_values<D, NG, 8, WIDE>(st, tile, kt, false, all, wb, lane); break;
+          default: group_values<D, NG, 16, WIDE>(st, tile, kt, fill < kt || (geo & kMask), all, wb, lane); break;
         }
         __syncwarp();  // the tile's bytes and weights are read
         if (inext < un.T) issue(c + 1, __shfl_sync(0xffffffffu, wcum, c));
+        if constexpr (WIDE) {
+          if (c % kFoldTiles == kFoldTiles - 1) fold_zero_points<D, NG>(st, fac, lane);
+        }
       }
       consumed = c;
       if (!good) break;
@@ -1785,6 +1896,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       auto finish = [&](auto column) {
         constexpr int j = decltype(column)::value;
         const int r = (2 * tig + j) / NG, gi = (2 * tig + j) % NG;
+        const float g = st.cls == 3 ? 1.f : pow2_inverse(st.ws[j]);
         float M = st.m[j], L = st.l[j], fo = 1.f, fn = 0.f;
         if (has_new) {  // fold the new token in
           M = fmaxf(st.m[j], new_score[j]);
@@ -1808,7 +1920,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
         float y[D / 8];
 #pragma unroll
         for (int i = 0; i < D / 8; ++i) {
-          float v = fmaf(st.acc[i / 2][2 * (i % 2) + j], f[i], st.zacc[j]) * fo;
+          float v = fmaf(st.acc[i / 2][2 * (i % 2) + j], WIDE ? f[i] * g : f[i], st.zacc[j]) * fo;
           if (has_new) v = fmaf(fn, vnew[gid * (D / 8) + i], v);
           if (RUNS && run[0]) v = fmaf(fp, __ldcg(partial() + gid * (D / 8) + i), v);
           y[i] = v * inv;
@@ -1995,7 +2107,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
 #pragma unroll 1
     for (int64_t i = threadIdx.x; i < n16; i += blockDim.x) o[i] = make_uint4(0, 0, 0, 0);
     if (GQ && ka.defer_merge) {  // nothing to merge
-      int2* qtab = reinterpret_cast<int2*>(a.cnt);
+      int2* qtab = reinterpret_cast<int2*>(a.qtab);
 #pragma unroll 1
       for (int q = threadIdx.x; q < n; q += blockDim.x) qtab[q] = make_int2(0, 1);
     }
@@ -2007,27 +2119,27 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
 // A kernel family (compiled side by side, one translation unit each): launches the instance of a
 // layout's head size and groups per head, and sets its shared-memory limit.
 
-template <bool HM, bool STEP, bool GQ, bool RUNS>
+template <Kind K, bool STEP, bool RUNS>
 auto row_instance(const Layout& l) {
   using Kernel = void (*)(AttnKernelArgs);
   const int ng = l.d / l.G;
-  if (l.d == 64) return ng == 1 ? Kernel(row_kernel<64, 1, HM, STEP, GQ, RUNS>) : Kernel(row_kernel<64, 2, HM, STEP, GQ, RUNS>);
-  return ng == 1   ? Kernel(row_kernel<128, 1, HM, STEP, GQ, RUNS>)
-         : ng == 2 ? Kernel(row_kernel<128, 2, HM, STEP, GQ, RUNS>)
-                   : Kernel(row_kernel<128, 4, HM, STEP, GQ, RUNS>);
+  if (l.d == 64) return ng == 1 ? Kernel(row_kernel<64, 1, K, STEP, RUNS>) : Kernel(row_kernel<64, 2, K, STEP, RUNS>);
+  return ng == 1   ? Kernel(row_kernel<128, 1, K, STEP, RUNS>)
+         : ng == 2 ? Kernel(row_kernel<128, 2, K, STEP, RUNS>)
+                   : Kernel(row_kernel<128, 4, K, STEP, RUNS>);
 }
-template <bool HM, bool STEP, bool GQ, bool RUNS>
+template <Kind K, bool STEP, bool RUNS>
 cudaError_t launch_rows(const Layout& l, dim3 grid, size_t smem, cudaStream_t s, const AttnKernelArgs& k) {
-  return launch_pdl(row_instance<HM, STEP, GQ, RUNS>(l), grid, dim3(32 * kRowWarps), smem, s, k);
+  return launch_pdl(row_instance<K, STEP, RUNS>(l), grid, dim3(32 * kRowWarps), smem, s, k);
 }
-template <bool HM, bool STEP, bool GQ, bool RUNS>
+template <Kind K, bool STEP, bool RUNS>
 cudaError_t configure_rows(const Layout& l) {
-  return cudaFuncSetAttribute(reinterpret_cast<const void*>(row_instance<HM, STEP, GQ, RUNS>(l)),
+  return cudaFuncSetAttribute(reinterpret_cast<const void*>(row_instance<K, STEP, RUNS>(l)),
                               cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemLimit);
 }
-#define TRR_ROW_FAMILY(prefix, HM, STEP, GQ, RUNS)                                                                   \
-  prefix template cudaError_t launch_rows<HM, STEP, GQ, RUNS>(const Layout&, dim3, size_t, cudaStream_t,             \
-                                                              const AttnKernelArgs&);                                \
-  prefix template cudaError_t configure_rows<HM, STEP, GQ, RUNS>(const Layout&);
+#define TRR_ROW_FAMILY(prefix, K, STEP, RUNS)                                                                        \
+  prefix template cudaError_t launch_rows<K, STEP, RUNS>(const Layout&, dim3, size_t, cudaStream_t,                  \
+                                                         const AttnKernelArgs&);                                     \
+  prefix template cudaError_t configure_rows<K, STEP, RUNS>(const Layout&);
 
 }  // namespace trr

@@ -57,15 +57,16 @@ def test_units_of_several_runs_give_up_a_wait():
     """The bounded waits hold in every run of tiles."""
     _cuda()
     rng = np.random.default_rng(6)
-    pair = Pair(1, 1, 2, 2, 128, 64, 64, 3200, [80] * 4, split_bytes=1 << 20)
-    _fill(pair, rng, [3000], 2, 2, 128, (2, 4, 8, 16), 0)
-    q = wl.bf16_bits(rng.standard_normal((1, 2, 128), dtype=np.float32))
-    args = [dev(np.array([x], np.int32), torch.int32) for x in (0, 2999)]
+    S, ctx = 8, 1500
+    pair = Pair(1, S, 8, 8, 128, 64, 64, ctx, [S * 26] * 4, split_bytes=1 << 20)
+    _fill(pair, rng, [ctx] * S, 8, 8, 128, (2, 4, 8, 16), 0)
+    q = wl.bf16_bits(rng.standard_normal((S, 8, 128), dtype=np.float32))
+    args = [dev(x.astype(np.int32), torch.int32) for x in (np.arange(S), np.full(S, ctx - 1))]
     pair.gpu.set_wait_limit(1)
-    pair.gpu.decode_attn(0, *args, dev(q, torch.bfloat16), dev(np.array([FULL], np.uint8), torch.uint8))
+    pair.gpu.decode_attn(0, *args, dev(q, torch.bfloat16), dev(np.full(S, FULL, np.uint8), torch.uint8))
     assert pair.gpu.status() == 8
     pair.gpu.set_wait_limit(0)
-    pair.attend(0, [0], [2999], q, [FULL])
+    pair.attend(0, np.arange(S), [ctx - 1] * S, q, [FULL] * S)
 
 
 @pytest.mark.parametrize("d,G,P,split_bytes,splits", [(128, 64, 64, 1 << 20, 19), (128, 64, 32, 1 << 20, 37),

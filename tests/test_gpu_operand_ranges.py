@@ -27,7 +27,7 @@ def _ratio(got, ref):
 
 
 @pytest.mark.parametrize("bits,outliers", [(2, True), (4, True), (8, False), (2, False)])
-@pytest.mark.parametrize("d,G,P,H,g", [(64, 32, 32, 16, 1), (128, 128, 32, 8, 1)])
+@pytest.mark.parametrize("d,G,P,H,g", [(64, 32, 32, 16, 1), (128, 128, 32, 8, 1), (64, 64, 32, 2, 10), (128, 64, 32, 2, 8)])
 def test_sums_add_nothing_to_the_rounding(d, G, P, H, g, bits, outliers):
     """Rows of 2000 keys in few splits, whose sums of p * s * c and of p * z are a hundred times
     the row and cancel: the error is that of rounding the exact row to bf16.  An error of 2^-23 of
@@ -36,7 +36,8 @@ def test_sums_add_nothing_to_the_rounding(d, G, P, H, g, bits, outliers):
     2 / 30."""
     rng = np.random.default_rng(100 * bits + d)
     S, ctx = 1024 // d, 2000
-    pair = Pair(1, S, H * g, H, d, G, P, ctx, [S * (ctx // P + 2)] * 4, split_bytes=100000)
+    # (a cache of long contexts: a wide group's calls of these sizes take the units of several heads)
+    pair = Pair(1, S, H * g, H, d, G, P, ctx if g == 1 else 8192, [S * (ctx // P + 2)] * 4, split_bytes=100000)
     chan = np.ones(H * d, dtype=np.float32)
     if outliers:
         chan[rng.permutation(H * d)[:max(1, H * d // 100)]] = 8
@@ -46,8 +47,9 @@ def test_sums_add_nothing_to_the_rounding(d, G, P, H, g, bits, outliers):
                   for _ in range(2)]
             pair.append(0, np.full(1000, s), np.arange(p0, p0 + 1000), kv[0], kv[1], np.full(1000, bits),
                         np.full(1000, FULL))
-    q = wl.bf16_bits(rng.standard_normal((S, H * g, d), dtype=np.float32))
-    got, ref = pair.attend(0, np.arange(S), [ctx - 1] * S, q, [FULL] * S)
+    seqs = np.tile(np.arange(S), 1 if g == 1 else 4)  # (four times: rows enough for a wide group's units)
+    q = wl.bf16_bits(rng.standard_normal((len(seqs), H * g, d), dtype=np.float32))
+    got, ref = pair.attend(0, seqs, [ctx - 1] * len(seqs), q, [FULL] * len(seqs))
     ratio = _ratio(got, ref)
     assert ratio <= 1.0006 + 0.0016, f"{ratio:.5f} times the error of rounding the exact rows"
 
@@ -193,6 +195,28 @@ def test_query_group_small_values(d, G, P, Hq, Hkv, size):
     _mixed(pair, rng, ctx, Hkv, d, rng.choice((2, 4, 8), size=ctx), vscale=size)
     got, ref = pair.attend(0, [0], [ctx - 1], wl.bf16_bits(3 * rng.standard_normal((1, Hq, d))), [FULL])
     assert _ratio(got, ref) <= MIXED, _ratio(got, ref)
+
+
+@pytest.mark.parametrize("d,G,Hq,Hkv", [(64, 32, 60, 10), (128, 64, 40, 8), (128, 32, 24, 8)])
+def test_wide_group_scales_far_apart(d, G, Hq, Hkv):
+    """Groups wider than 8 / (d / G) heads: V's first quantiser group is 2^26 times as large as the others, and large scales of keys
+    without weight."""
+    rng = np.random.default_rng(27)
+    ctx = 800
+    pair = Pair(1, 2, Hq, Hkv, d, G, 32, 8192, [2 * (ctx // 32 + 2)] * 4, split_bytes=100000)
+    _mixed(pair, rng, ctx, Hkv, d, rng.choice((2, 4, 8), size=ctx), vscale=np.where(np.arange(d) < G, 2.0 ** 12, 2.0 ** -14))
+    odd = (np.arange(ctx) % 16 == 3)[:, None, None]
+    k = rng.standard_normal((ctx, Hkv, d)) - 16.0 * odd
+    v = rng.standard_normal((ctx, Hkv, d)) * np.where(odd, 2.0 ** 12, 2.0 ** -14)
+    pair.append(0, np.ones(ctx), np.arange(ctx), wl.bf16_bits(k), wl.bf16_bits(v), rng.choice((2, 4, 8), size=ctx),
+                np.full(ctx, FULL))
+    n = 32768 // (Hq * d) + 1  # of each sequence: rows enough for a wide group's units
+    q = np.abs(3 * rng.standard_normal((2 * n, Hq, d))) + 0.5
+    q[:n] = rng.standard_normal((n, Hq, d))
+    got, ref = _rows(pair, [0] * n + [1] * n, [ctx - 1] * 2 * n, wl.bf16_bits(q))
+    first = slice(0, n), slice(None)
+    for part in ((*first, slice(0, G)), (*first, slice(G, d)), (slice(n, 2 * n),)):
+        assert _ratio(got[part], ref[part]) <= MIXED, _ratio(got[part], ref[part])
 
 
 @pytest.mark.parametrize("d,G,Hq,Hkv", [(64, 32, 4, 2), (128, 64, 8, 2), (64, 64, 16, 2)])
