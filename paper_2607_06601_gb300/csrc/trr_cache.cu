@@ -15,12 +15,11 @@ namespace trr {
 
 LayerArgs layer_args(const Layout& l, const Views& v, int layer) {
   LayerArgs a;
-  a.layer = layer;
   a.S = l.S; a.Hq = l.Hq; a.Hkv = l.Hkv; a.d = l.d; a.G = l.G; a.P = l.P;
-  a.maxctx = l.maxctx; a.MP = l.MP; a.W32 = l.W32; a.units = l.units; a.pos_split = l.pos_split;
+  a.maxctx = l.maxctx; a.MP = l.MP; a.W32 = l.W32; a.pos_split = l.pos_split;
   a.s_cap = l.s_cap;
   a.split_keys = l.split_keys; a.split_extra = l.split_extra; a.split_most = l.split_most;
-  a.split_bytes = l.split_bytes; a.skip_writes_kv = l.skip_writes_kv;
+  a.skip_writes_kv = l.skip_writes_kv;
   a.head_modes = l.head_modes; a.maskb = static_cast<int>(l.maskb); a.swz = l.swz;
   a.hdr = static_cast<int>(l.hdr);
   for (int c = 0; c < kClasses; ++c) {

@@ -26,10 +26,10 @@ enum Ctrl : int {
 // kernel of one layer may start while the previous layer's kernel still runs).
 enum LayerCtrl : int {
   kNextUnit = 0,      // next work unit to hand out
-  kDoneCtas = 1,      // CTAs finished (the last one records the status)
+  kDoneCtas = 1,      // CTAs finished (the last one records the status), 2^16 more for each that gave up a
+                      // wait (a decode step then commits nothing)
   kFirstBadQuery = 2, // min of (query index * 16 + error) over failing queries (INT_MAX = none)
-  kAborted = 3,       // 1 when a CTA gave up a wait (a decode step then commits nothing)
-  kLayerCtrlInts = 4
+  kLayerCtrlInts = 4  // (16 bytes a layer)
 };
 
 // An attention work unit has at most this many tiles (a page's keys, split_keys at a time) planned
@@ -126,7 +126,8 @@ inline Views make_views(const Layout& l, void* base) {
 
 // Everything a kernel needs about one layer of one cache, passed by value.
 struct LayerArgs {
-  int layer, S, Hq, Hkv, d, G, P, maxctx, MP, W32, units, pos_split, split_keys, split_extra, split_most, s_cap, cnt_stride, split_bytes, skip_writes_kv;
+  int S, Hq, Hkv, d, G, P, maxctx, MP, W32, pos_split, split_keys, split_extra, split_most, s_cap, cnt_stride;
+  int skip_writes_kv;
   int head_modes;      // modes are [n][Hq]; each KV head's slice ends with its presence mask
   int swz;             // 8- and 16-bit code rows stored swizzled (see swz_off)
   uint64_t wait_ns;    // bound of an in-kernel wait before the kernel reports TRR_ERR_TIMEOUT
@@ -181,10 +182,6 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 
 __device__ __forceinline__ void fence_barrier_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-__device__ __forceinline__ void fence_proxy_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {

@@ -2070,7 +2070,6 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
     if (lane == 0) {
       *abort_flag = 1;
       set_status(a.ctrl, TRR_ERR_TIMEOUT);
-      atomicExch(&a.lctl[kAborted], 1);
     }
     // copies in flight always land (they only read memory): the default bound
 #pragma unroll 1
@@ -2094,7 +2093,6 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
   if (threadIdx.x == 0) {
     a.lctl[kDoneCtas] = 0;
     a.lctl[kNextUnit] = 0;
-    a.lctl[kAborted] = 0;
     if (!STEP) {
       const int bad = atomicExch(&a.lctl[kFirstBadQuery], INT_MAX);
       if (bad != INT_MAX) set_status(a.ctrl, bad & 15);
