@@ -292,7 +292,7 @@ def ncu_traffic(workload):
     """Per-launch DRAM bytes of the attention kernel from the committed ncu summary,
     if it was taken on the current kernel sources (else None)."""
     digest = kernel_source_digest()
-    path = os.path.join(ROOT, "profiles", f"attn_kernel_{workload}_traffic.txt")
+    path = os.path.join(ROOT, "profiles", f"row_kernel_{workload}_traffic.txt")
     try:
         kv = dict(line.split(":", 1) for line in open(path) if ":" in line)
     except OSError:
@@ -952,8 +952,8 @@ def run_gpu(args):
                          "traffic": None if (bench.head_modes or bench.swk or bench.C > 1)
                          else ncu_traffic(args.workload),
                          "peak_kind": peak_kind,
-                         "kernel": "trr_decode_step call (attn_kernel: append and attention, one launch)" if bench.C == 1
-                         and not bench.head_modes else "trr_decode_attn call (attn_kernel, one launch)",
+                         "kernel": "trr_decode_step call (row_kernel: append and attention, one launch)" if bench.C == 1
+                         and not bench.head_modes else "trr_decode_attn call (row_kernel, one launch)",
                          "bytes_per_call": round(avg_bytes), "us_per_call": round(launch_ms * 1e3, 3),
                          "timing": "timed region / launches (one launch per layer)" if in_stream
                          else "event nodes around each call",

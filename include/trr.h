@@ -242,7 +242,8 @@ TRR_API trr_status trr_decode_step(trr_cache* cache, int32_t layer, int32_t n, c
  *   for: n is bounded by the array instead of by max_queries.
  *   The call needs 256 + n * Hq * (4 * (1 + ceil(S_cap / 32)) + S_cap * (4*d + 16))
  *   bytes (plus 256-byte rounding per region), with S_cap the most splits per query of
- *   this cache; a call above 32 MiB returns TRR_ERR_OUT_OF_MEMORY and launches nothing.
+ *   this cache: max_context over the positions whose 8-bit K and V (one KV head) take
+ *   split_bytes, or over 28 pages where that is more; a call above 32 MiB returns TRR_ERR_OUT_OF_MEMORY and launches nothing.
  *   The first call on a device looks up the array's device address (once per device,
  *   with that device current); make that first call before any stream capture.
  *   Every call clears what must start at zero and then overwrites the array, so calls

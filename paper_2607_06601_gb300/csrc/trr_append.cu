@@ -156,11 +156,10 @@ __device__ __forceinline__ void quantise_8(const uint4 raw, int b, int GL, unsig
 //
 // Bound by latency: the chain from the wait (metadata, page ids, first rows).  The second
 // row of a lane is loaded while the first is quantised, and the arrival's round trip and the
-// commit overlap the rows (13.9 -> 11.8 us a call of 1024 entries of 12 x 64 KV heads, on
-// the GPU alone).  With a plan kernel that scanned all entries for each and a second kernel
-// of one thread per group such a call took 122 us.  A call of 256 entries with its
-// attention: 97 -> 73 us.  The large instance waits before it reads its entries (as calls
-// of that size always did; reading them early would save 2.4 us).
+// commit overlap the rows: 11.8 us a call of 1024 entries of 12 x 64 KV heads, on the GPU alone
+// (13.9 without either; 122 with a plan kernel that scans all entries for each entry and a second
+// kernel of one thread per group).  The large instance waits before it reads its entries
+// (reading them early would save 2.4 us).
 template <int D, int T>
 __global__ void __launch_bounds__(T) append_kernel(LayerArgs a, int n, const int32_t* __restrict__ seq_ids,
                                                    const int32_t* __restrict__ positions,

@@ -3,7 +3,7 @@
 // mode-routed split-K decode attention over the mixed-precision paged cache (Sec. 3.2(A),
 // Eq. 2; Sec. 3.8; Sec. 7).  trr_row.cuh holds the kernel; here are its arguments, a query's
 // mode, range and errors, a decode step's token bookkeeping, the operands of the tensor-core
-// products, the merge of split partials, the combine kernel of query groups and the launchers.
+// products, the merge of split partials and the combine kernel of query groups.
 //
 // One persistent kernel per call cuts it into work units: a query gets splits from the length
 // of its key range (full: [0, t]; local: [t-w+1, t]; skip or invalid: one that writes the zero
@@ -299,11 +299,12 @@ __device__ __forceinline__ bool arrive_last(int* counter, int expected, int lane
 // holding head r's query on group gi's dimensions (zero elsewhere), so every column
 // gets its own group sum and s, z apply per group.  A code is masked in place and
 // read as an f16 subnormal c * 2^(pos - 24) (pos = its bit offset in the 16-bit half);
-// the query is pre-scaled by 2^(smax - pos) in f16 so that every product carries the
-// same factor 2^(smax - 24).  Width 16 uses bf16 operands (the query is bf16 already).
+// the query is pre-scaled in f16 by 2^(15 - E - pos), E the exponent of the column's largest
+// query value, so that every product of a column carries the same factor 2^(-9 - E).  Width 16
+// uses bf16 operands (the query is bf16 already).
 //
-// P.V: O^T[dim][col] = sum_k V^T[dim][key] W[key][col] with W = p * s (f16; bf16 hi
-// and lo parts for width 16, whose values are raw bf16).  Pairs along keys for the A
+// P.V: O^T[dim][col] = sum_k V^T[dim][key] W[key][col] with W = p * s (two f16 parts; for width 16,
+// whose values are raw bf16, two bf16 or tf32 parts).  Pairs along keys for the A
 // operand come from byte permutes of two keys' code words.  Each accumulator row keeps
 // its class's factor 2^(pos - 24) until the class changes.
 
@@ -359,7 +360,6 @@ template <int B> __host__ __device__ constexpr int kp_hi(int i) {
 template <int B> __host__ __device__ constexpr int kp_pos(int i) {
   return B >= 8 ? 0 : B == 4 ? 4 * (i % 2) : 2 * ((i % 8) < 5 ? i % 8 : i % 8 - 5);
 }
-template <int B> __host__ __device__ constexpr int smax_of() { return B == 2 ? 8 : B == 4 ? 4 : 0; }
 
 // V side: dim j of the thread's D/8 dims for keys (a, b) as an A-operand word (key a
 // in the low half).  The tensor core lines products up by their operands' exponents, and all
@@ -403,8 +403,8 @@ __host__ __device__ constexpr int vfac_log2(int c, int j) {
 // has finished, and the next layer's kernel waits for all of it, so it is bound by its round
 // trips to L2.  Each warp therefore has a chunk of rows and its (max, sum) words in flight at
 // once (merge_partials).  (gqa_long shape, 3 full queries of 16, 93 splits of 32768 positions:
-// 17 us with four warps a row that read the maxima, then the sums, then row after row; 5.2 us
-// now.)  A row gets as many warps, up to the CTA's 8, as keep the CTAs within what the chip
+// 5.2 us; 17 with four warps a row that read the maxima, then the sums, then row after row.)
+// A row gets as many warps, up to the CTA's 8, as keep the CTAs within what the chip
 // holds at once (8 per SM): with 2048 rows of 0 to 3 splits, 8 warps a row took 16 us more
 // per 6 layers than 4.
 constexpr int kCombineWarps = 8;  // of a CTA

@@ -45,7 +45,7 @@ struct Layout {
   int L, S, Hq, Hkv, d, G, P, maxctx, MP, W32;
   int cap[kClasses];
   int max_append, max_queries, split_bytes, skip_writes_kv, head_modes;
-  int swz;        // 8- and 16-bit code rows stored swizzled (caches read one query head per warp)
+  int swz;        // 8- and 16-bit code rows stored swizzled (every cache but narrow query groups)
   int units;      // attention work units per query split (one per query head)
   int pos_split;  // key positions per split at least (split_bytes of 8-bit tokens)
   int split_keys, split_extra, split_most;  // keys of a tile; tiles a range may have above what its
@@ -73,9 +73,8 @@ __host__ __device__ inline int splits_of(int range, int pos_split, int keys, int
 }
 
 // Query groups (g >= 2) whose (head, group) columns fit one 8-wide mma tile, without per-head
-// modes, are read a KV head per warp; every other cache a query head per warp, whose lanes
-// read 8- and 16-bit code rows in a pattern that the swizzle below makes free of
-// shared-memory bank conflicts.
+// modes, store their rows plainly; every other cache stores 8- and 16-bit code rows in the order
+// below, whose reading pattern is free of shared-memory bank conflicts.
 __host__ __device__ inline bool uses_mma(int Hq, int Hkv, int d, int G, int head_modes) {
   const int g = Hq / Hkv, ng = d / G;
   return !head_modes && g >= 2 && g * ng <= 8;

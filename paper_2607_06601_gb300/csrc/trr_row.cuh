@@ -2,30 +2,24 @@
 // trr_row.cuh - the attention kernels: mode-routed split-K decode attention over the
 // mixed-precision paged cache (Sec. 3.2(A), Eq. 2; Sec. 3.8; Sec. 7).
 //
-// A work unit is a split of a query for one query head (MHA, wide query groups, per-head
-// modes) or for one KV head and its query group, and belongs to one warp from its plan to its
-// row: the warp plans the unit (plan_pages), streams its pages' KV slices through a ring of
+// A work unit is a split of a query for one query head (MHA, per-head modes, small calls of wide
+// groups) or for one KV head and heads of its query group, and belongs to one warp from its plan to
+// its row: the warp plans the unit (plan_pages), streams its pages' KV slices through a ring of
 // shared memory of its own with 1-D bulk copies (one per page as a rule, cp.async.bulk +
-// mbarrier), and computes on them.  Nothing but the call's start and end synchronises warps: a
-// producer warp that fed four consumer warps through one ring, as the kernels had before, kept
-// two stages in flight and held every stage until the slowest of the four was done with it.
+// mbarrier), and computes on them.  Nothing but the call's start and end synchronises warps.
 // The kernels are bound by instructions issued and by the latency of a unit's chain (plan,
-// copies, tiles, merge), not by memory: batch 256 of the sweep shape streams at 5.9 TB/s
-// with the tile arithmetic left out, at 4 TB/s with it.
+// copies, tiles, merge), not by memory: batch 256 of the sweep shape streams at 3.8 TB/s, at 5.9
+// with the tile arithmetic left out.  (A step of 3 such layers 771 us; 817 with a producer warp that
+// fed four consumer warps through one ring and binary32 arithmetic on the CUDA cores.)
 //
 // Two CTAs of eight warps fill an SM; while some of the places are free or a CTA has ended,
 // the next layer's kernel is resident, so that its plans and its first page copies come before
 // its wait on this kernel.
 //
-// Query groups (a producer warp and four consumer warps, then this kernel): two sequences of
-// 37 and 130 tokens generated with 4 heads on 2 1971 -> 1397 us; 32 heads on 8 of 128, 24
-// layers, batch 1, context 4096, 1106 -> 838; batch 16, context 32768, 380 -> 289 (most of it
-// the combine kernel).
-//
 // One query head per warp: the arithmetic runs on the tensor cores (mma.sync m16n8k16, f32
-// accumulation) though only one query head shares a key, because the codes then need one mask per two elements (a
-// pair of codes in the halves of a word, read as f16 subnormals) in place of one per
-// element, and the multiply-adds come free:
+// accumulation) though only one query head shares a key, because the codes then need one mask per
+// two elements (a pair of codes in the halves of a word, read as f16 subnormals) in place of one
+// per element, and the multiply-adds come free:
 //   q.k   A = 16 keys' codes, B = the query row, its column n holding quantiser group
 //         n % NG (zero outside it); each lane then takes one key of a tile of 32 and adds
 //         up s * (group sum) + z * (group's query sum) in binary32.
@@ -50,8 +44,8 @@ constexpr int kRowWarps = 8;   // warps per CTA
 constexpr int kRowSlots = 8;   // tiles a warp may have in flight
 constexpr int kRowCtasPerSm = 2;
 // A grid leaves num_sms / kRowSpare places of the chip free: the next layer's kernel then
-// starts, and plans, while the last CTAs of this one still run (with a full grid its last CTA
-// started, and planned for 3 us, only when this kernel had ended: 160M step 18.2 -> 16.8 us).
+// starts, and plans, while the last CTAs of this one still run.  (160M, 4 steps 796 us, 799 with a
+// full grid; the 1.3B shape 666 and 653, per-head modes 666 and 645.)
 constexpr int kRowSpare = 32;
 constexpr int kRowSmemLimit = 110 * 1024;
 constexpr float kLoScale = 2048.f;  // the low part of a weight is stored times 2^11
@@ -185,12 +179,13 @@ __device__ __forceinline__ void plan_rows(const AttnKernelArgs& ka, int rows, in
 #pragma unroll
   for (int k = 0; k < kRowWarps; ++k) rsum += red[k];
   // Split size: about one unit per warp while a unit then stays short, else up to three per
-  // warp, of 700 positions at least, handed out on demand; never below pos_split.  (1.3B
-  // shape, batch 64, contexts to 8192: 637 us for 8 layer calls; one unit per warp only up to
-  // 768 positions 704, units from 512 positions 689, five per warp 768.  A query group's
-  // positions weigh about twice as much: gqa_long shape 412 us for 6 layer calls, 468 with units
-  // from 250 positions.)  Binary32 arithmetic: the same result in every CTA, and it only sizes
-  // the splits.
+  // warp, of 700 positions at least, handed out on demand; never below pos_split.  (1.3B shape,
+  // batch 64, contexts to 8192, 2 steps of 4 layers 666 us, units from 512 positions 685; 8 queries
+  // of 32 sequences 269 and 292.  A query group's positions weigh about twice as much: gqa_long
+  // shape 663 us for 4 steps of 3 layers, 673 with units from 250 positions.)  The tiles' bound of
+  // splits_of cuts finer where tiles are of 16 keys: at head size 128 and in pages of 16 a unit has
+  // 350 to 450 positions at most, whatever this asks for.  Binary32 arithmetic: the same result in
+  // every CTA, and it only sizes the splits.
   const float warps = static_cast<float>(gridDim.x * kRowWarps), rs = static_cast<float>(rsum);
   const float one = rs / (0.85f * warps);
   const float most = GQ ? 600.f : 1000.f, least = GQ ? 350.f : 700.f;
@@ -318,8 +313,8 @@ __device__ __forceinline__ int plan_pages(const LayerArgs& a, int seq, int lo, i
   }
   // 16-bit tiles count twice where a split's tiles then stay within a warp's lanes: a warp's
   // ring holds one of 8 KB, so that each waits out a copy, and a split of nothing else ended
-  // last.  (160M step 801 -> 776 us, batch 256 of the sweep 1468 -> 1413, gqa_long shape 290 ->
-  // 283 for 6 layer calls, batch 8 of contexts 4000 255 -> 260.)
+  // last.  (160M, 4 steps 796 us, 832 counted once; batch 256 of the sweep 1575 and 1631, 1.3B 666 and
+  // 707; head size 128, batch 64 of contexts 4000 251 and 247.)
   const int wide = __shfl_sync(0xffffffffu, mass, 24);
   if (div24(all + wide, ns) + 1 + 2 * (a.P >> (__ffs(kt_wide) - 1)) <= kItemMaxTiles) {
     all += wide;
@@ -791,16 +786,15 @@ __device__ __forceinline__ void tile_values16(RowState<D, NG>& st, const uint8_t
 // A KV head with its g >= 2 query heads (g * NG <= 8) per unit: column n of the B operands is
 // head n / NG and quantiser group n % NG, so that lane (gid, tig) has the scores of keys
 // gid + 8 h + 16 u for its columns 2 tig and 2 tig + 1 (two groups of a head, or two heads at
-// NG = 1).  Weights p * s are two f16 parts, width 16's p two bf16 parts (one f16 part, as
-// before, rounds by 2^-12: rows were 0.6 to 2% further off than with a maximum raised at every
-// score; two parts are closer than that was, for 1 to 4% of the time).  A running maximum is
-// raised when a score exceeds it by 2^3 (any excess where a scale could then take p * s out
-// of f16's range): raised at every new maximum, as before, nine tiles in ten rescaled the
-// accumulators.  These caches' rows are stored plainly.
+// NG = 1).  Weights p * s are two f16 parts, width 16's p two bf16 parts (one f16 part rounds by
+// 2^-12, which leaves rows 1 to 2 % further off; the second takes 1 to 4 % of the time).  A
+// running maximum is raised when a score exceeds it by 2^3 (any excess where a scale could then
+// take p * s out of f16's range): raised at every new maximum, nine tiles in ten would rescale
+// the accumulators.  Narrow groups' rows are stored plainly.
 //
 // f16 ends at 2^-25, which p * s of small values would come near: p is therefore taken relative to
 // 2^-lift of the maximum, lift (0 to 16) lowered when a larger V scale comes.  (V of size 2^-10: rows
-// 5e-3 off without it, 2^-14 8 %; gqa_long shape 630 -> 646 us for 4 steps.)
+// 5e-3 off without it, 2^-14 8 %; gqa_long shape 646 us for 4 steps, 630 without.)
 constexpr float kGroupTau = 3.f, kGroupWide = 8000.f;
 constexpr float kLift = 16.f;  // at first
 //
@@ -1147,9 +1141,9 @@ __device__ __forceinline__ void group_values(GroupState<D, NG, WIDE>& st, const 
 // out low by up to 2^-23 of themselves per 16 keys, and p * z, about as large with the other sign,
 // leaves that in a row a hundred times smaller.  The zero points are therefore added every
 // kFoldTiles tiles, so that the running sums stay near the row itself.  (8-bit tokens, 670 keys a
-// split: 1.1e-4 of the row off before its rounding, 2.4e-5 so.  Batch 256 of the sweep 1467 -> 1525
-// us; every 4 or 16 tiles takes as long; sums begun at zero for each tile 1720, and codes made
-// normal and centred 1740.)
+// split: 1.1e-4 of the row off before its rounding, 2.4e-5 so.  Batch 256 of the sweep 1576 us, 1524
+// without; every 4 or 16 tiles takes as long.  Sums begun at zero for each tile, or codes made
+// normal and centred, take 12 % more.)
 constexpr int kFoldTiles = 8;
 template <int D, int NG>
 __device__ __forceinline__ void fold_zero_points(RowState<D, NG>& st, const float* fac, int lane) {
@@ -1674,10 +1668,9 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
 
   // The first unit is planned and its copies issued before the rest of the call's start.
   // Units that do not fill half of the CTAs, one per SM, are dealt evenly to these; more fill
-  // CTA after CTA, which leaves places for the next layer's kernel.  (Without the deal a 24
-  // layer step of batch 1, context 4096, took 1180 us in place of 1130, 12 heads, batch 20, in
-  // pages of 16 389 in place of 363; dealing up to a unit per warp evenly to all CTAs cost the
-  // 160M step 850 us in place of 813.)
+  // CTA after CTA, which leaves places for the next layer's kernel.  (Head size 128, batch 8, 2 steps
+  // of 12 layers 392 us, 420 without the deal; a group of 4, batch 8, 440 and 466.  Dealing up to
+  // a unit per warp evenly to all CTAs: the 160M steps 847 in place of 796, pages of 16 418 for 367.)
   const int cta = static_cast<int>(blockIdx.x), half = (gridDim.x + 1) / 2;
   int per = kRowWarps, more = 0;
   if (total < half * kRowWarps) {
