@@ -1660,10 +1660,17 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) row_kernel(const __grid_con
       if (lane == 0) run[1] = tp.skip;
     }
     inext = 0;
+    // a limit shorter than a suspended wait covers the first copies from before they are issued
+    // (from after it, instructions not yet fetched may take as long as the copies)
+    const bool brief = a.wait_ns < kShortWaitNs;
+    const uint64_t t0 = brief ? global_ns() : 0;
     issue(0, 0);
-    // a limit shorter than a suspended wait covers the first copies from here on
-    if (a.wait_ns < kShortWaitNs && un.T > 0)
-      good = __all_sync(0xffffffffu, mbar_wait_slow(&full[base % kRowSlots], (base / kRowSlots) & 1, abort_flag, a.wait_ns));
+    if (brief && un.T > 0) {
+      const uint32_t bar = smem_u32(&full[base % kRowSlots]);
+      bool in = false;
+      while (!in && global_ns() - t0 < a.wait_ns) in = mbar_test_at(bar, (base / kRowSlots) & 1);
+      good = __all_sync(0xffffffffu, in);
+    }
   };
 
   // The first unit is planned and its copies issued before the rest of the call's start.
