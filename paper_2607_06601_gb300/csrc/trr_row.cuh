@@ -8,8 +8,8 @@
 // shared memory of its own with 1-D bulk copies (one per page as a rule, cp.async.bulk +
 // mbarrier), and computes on them.  Nothing but the call's start and end synchronises warps.
 // The kernels are bound by instructions issued and by the latency of a unit's chain (plan,
-// copies, tiles, merge), not by memory: batch 256 of the sweep shape streams at 3.8 TB/s, at 5.9
-// with the tile arithmetic left out.  (A step of 3 such layers 771 us; 817 with a producer warp that
+// copies, tiles, merge), not by memory: batch 256 of the sweep shape streams at 3.9 TB/s, at 5.9
+// with the tile arithmetic left out.  (A step of 3 such layers 762 us; 828 with a producer warp that
 // fed four consumer warps through one ring and binary32 arithmetic on the CUDA cores.)
 //
 // Two CTAs of eight warps fill an SM; while some of the places are free or a CTA has ended,
